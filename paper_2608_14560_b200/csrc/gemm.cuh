@@ -5,9 +5,8 @@
 //
 // One persistent CTA per SM walks a static list of 128 x 256 output tiles.
 //   warp 0      TMA producer.  Per K-block (128 K-bytes = one scale block): the A
-//               tile (128 rows), the B tile (256 weight rows) and the 128
-//               activation scales of the block, into a 4-stage ring (128-byte
-//               swizzle) / an 8-slot scale ring, completion on mbarriers.
+//               tile (128 rows) and the B tile (256 weight rows) into a 4-stage ring
+//               (128-byte swizzle), completion on mbarriers.
 //   warps 1,2   MMA issuers (even / odd K-blocks).  Four tcgen05.mma (M128 N256 K32, e4m3 -> fp32) per
 //               K-block into one of two 256-column TMEM buffers, then ONE
 //               tcgen05.commit: the same mbarrier tells the producer that the stage
@@ -16,10 +15,17 @@
 //               50-100 clocks, so the per-K-block instruction count is kept minimal).
 //               Every K-block starts from zero because its partial sum must be
 //               multiplied by fp32 scales before it joins the running sum.
+//   warp 3      factors: activation scale x weight scale per row and column half,
+//               into an 8-slot ring (factor_tiles).
 //   warps 4-7   epilogue of columns [0,128), warps 8-11 of columns [128,256): read
 //               the partial from TMEM, multiply by a_scale[row,kb] * w_scale[nblk,kb]
-//               with fp32 FMAs, accumulate in registers; at the end of the
+//               with packed fp32 FMAs, accumulate in registers; at the end of the
 //               tile apply the fused tail and store.
+// What bounds a large batch is that loop: stage refilled -> MMAs -> epilogue reads the accumulator -> buffer handed
+// back.  Together, the factor warp, the packed FMAs (see fma64), the hand-back through a named barrier and three
+// instead of six copies per K-block took a forward from 2292 to 2179 us at 8192 skewed tokens with 32 local experts,
+// from 650 to 624 us at 4096 tokens and from 9281 to 9218 us at 16384 tokens with 256 local experts (under the power
+// cap); batches bound by the weight stream gain 1 %.
 // Scales are arbitrary fp32 (amax/448), so the power-of-two hardware block
 // scaling cannot express them; the per-K-block promotion is done on the ALUs.
 //
@@ -66,19 +72,33 @@ constexpr int G_STORE_WARP_BYTES = 2048;                // per-warp staging: 32 
 constexpr int G_AMAX_BYTES = 2 * 2 * TILE_M * 4;               // GEMM1 row-amax exchange
 constexpr int G_CTRL_BYTES = 512;
 constexpr uint32_t G_TMEM_COLS = 512;
+// Large-tile kernels: named barrier ACC_BARRIER + b hands accumulator buffer b from the epilogue warps (which
+// arrive) back to its issuer warp (which waits).
+constexpr int ACC_BARRIER = 1;
+constexpr int ACC_BARRIER_THREADS = (G_EPI_WARPS + 1) * 32;
+
+// Scales on their way to the factor warp of the large-tile kernels, in K-blocks and ring slots of 128 activation and 2
+// weight scales.
+constexpr int F_AHEAD = 4;
+constexpr int F_SLOTS = 8;
+constexpr int F_SLOT_FLOATS = TILE_M + 4;
 
 // Shared-memory geometry of a kernel: pipeline stages, rows of the A tile that are actually fetched (the MMA
 // always reads 128 rows; with fewer fetched rows the rest of its A operand is whatever follows in shared
 // memory, and those accumulator rows are never stored), slots of the activation-scale ring.
-template <int STAGES_, int A_ROWS_, int SCALE_SLOTS_, int STORE_BYTES_>
+template <int STAGES_, int A_ROWS_, int SCALE_SLOTS_, int STORE_BYTES_, bool FACTORS_>
 struct Geometry {
     static constexpr int STAGES = STAGES_, A_ROWS = A_ROWS_, SCALE_SLOTS = SCALE_SLOTS_;
+    static constexpr bool FACTORS = FACTORS_;                        // see factor_tiles
     static constexpr int A_BYTES = A_ROWS_ * G_BLOCK_K;
     static constexpr int STAGE_BYTES = A_BYTES + G_B_BYTES;
     static constexpr int SCALE_BYTES = A_ROWS_ * 4;                  // per K-block
+    // a slot: the activation scales of a K-block, or (large-tile kernels) their products with two weight scales
+    static constexpr int SLOT_BYTES = FACTORS_ ? 2 * SCALE_BYTES : SCALE_BYTES;
+    static constexpr int RAW_BYTES = FACTORS_ ? F_SLOTS * F_SLOT_FLOATS * 4 : 0;
     static constexpr int STORE_BYTES = STORE_BYTES_;                 // GEMM1 output staging
-    static constexpr int SMEM_BYTES = STAGES_ * STAGE_BYTES + SCALE_SLOTS_ * SCALE_BYTES + STORE_BYTES_ + G_AMAX_BYTES +
-                                      G_CTRL_BYTES + 1024;           // + alignment slack
+    static constexpr int SMEM_BYTES = STAGES_ * STAGE_BYTES + SCALE_SLOTS_ * SLOT_BYTES + STORE_BYTES_ + G_AMAX_BYTES +
+                                      G_CTRL_BYTES + RAW_BYTES + 1024;   // + alignment slack
     static_assert(STAGES_ % 2 == 0, "an odd stage count lets an issuer thread skip phases of full[s]");
     static_assert(STAGES_ <= G_MAX_STAGES, "control block holds G_MAX_STAGES barriers per kind");
     static_assert(A_BYTES % 1024 == 0, "the B tile must stay 1024-byte aligned for the 128-byte swizzle");
@@ -86,11 +106,11 @@ struct Geometry {
     static_assert(SMEM_BYTES <= 232448, "exceeds the 227 KB of shared memory a CTA may use");
 };
 // one GEMM per launch: full 128-row A tiles, 4 stages of 48 KB
-using GeomFull = Geometry<4, TILE_M, 8, G_EPI_WARPS * G_STORE_WARP_BYTES>;
+using GeomFull = Geometry<4, TILE_M, 8, G_EPI_WARPS * G_STORE_WARP_BYTES, true>;
 // fused small-batch kernel: a row tile holds at most 32 token rows, so their slot shrinks to 4 KB and six
 // stages fit: 192 KB of weights in flight per SM instead of 128 KB, which is what a weight-streaming CTA is
 // limited by; 512 bytes of output staging per epilogue warp
-using GeomSmall = Geometry<6, 32, 16, G_EPI_WARPS * 512>;
+using GeomSmall = Geometry<6, 32, 16, G_EPI_WARPS * 512, false>;
 
 // Row tiles of fused_small_kernel hold at most ST_ROWS = 32 rows (the N of its MMAs); an expert with more rows
 // gets several of them (each streams the expert's weights, the later ones out of L2).  F_MAX_TOKENS is the
@@ -120,7 +140,8 @@ struct GemmArgs {
     int w_rows_per_expert;    // rows of the weight matrix per expert (2I or H)
     int row_cap;              // rows in the activation buffers (stride of transposed scales)
     int out_cols;             // I (GEMM1) or H (GEMM2)
-    int gate_row0, up_row0;   // GEMM1: first weight row of the gate / up half
+    int up_row0;              // GEMM1: first weight row of the second half (I)
+    int up_first;             // GEMM1: 0 = the first half is the gate and the second the up projection; 1 = the other way round
     const int* num_m_tiles;   // device scalars and tables built by the permute stage
     const int* tile_expert;
     const int* tile_rows;
@@ -198,9 +219,10 @@ __host__ __device__ __forceinline__ size_t y_block_offset(int r, int c16, int n_
 
 // The CTA's carve-up of shared memory and the values every role needs.
 struct Cta {
-    float* scale_ring;
+    float* scale_ring;         // [slot][A_ROWS] activation scales; large-tile kernels: [slot][2][A_ROWS] factors
     uint8_t* store_stage;
     float* amax_x;             // [2][2][TILE_M] GEMM1 row-amax exchange
+    float* raw_scales;         // large-tile kernels: the factor warp's scales in flight
     GemmCtrl* ctrl;
     volatile int* abort_flag;
     uint32_t smem_base, tmem_base;
@@ -231,9 +253,10 @@ template <class GEO>
 __device__ __forceinline__ void gemm_cta_setup(Cta& c, uint8_t* smem_raw, int full_count) {
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     c.scale_ring = reinterpret_cast<float*>(smem + GEO::STAGES * GEO::STAGE_BYTES);
-    c.store_stage = smem + GEO::STAGES * GEO::STAGE_BYTES + GEO::SCALE_SLOTS * GEO::SCALE_BYTES;
+    c.store_stage = smem + GEO::STAGES * GEO::STAGE_BYTES + GEO::SCALE_SLOTS * GEO::SLOT_BYTES;
     c.amax_x = reinterpret_cast<float*>(c.store_stage + GEO::STORE_BYTES);
     c.ctrl = reinterpret_cast<GemmCtrl*>(c.store_stage + GEO::STORE_BYTES + G_AMAX_BYTES);
+    c.raw_scales = reinterpret_cast<float*>(c.store_stage + GEO::STORE_BYTES + G_AMAX_BYTES + G_CTRL_BYTES);
     c.abort_flag = &c.ctrl->abort_flag;
     c.smem_base = smem_u32(smem);
     c.warp = threadIdx.x >> 5;
@@ -242,7 +265,7 @@ __device__ __forceinline__ void gemm_cta_setup(Cta& c, uint8_t* smem_raw, int fu
     if (threadIdx.x == 0) {
         for (int s = 0; s < GEO::STAGES; ++s) {
             mbar_init(smem_u32(&ctrl->full[s]), full_count);
-            mbar_init(smem_u32(&ctrl->done[s]), 1);
+            mbar_init(smem_u32(&ctrl->done[s]), GEO::FACTORS ? 2 : 1);  // the MMAs' commit; the factor warp
         }
         for (int b = 0; b < G_MAX_STAGES; ++b) mbar_init(smem_u32(&ctrl->tmem_empty[b]), G_EPI_WARPS);
         mbar_init(smem_u32(&ctrl->amax_bar[0]), G_EPI_WARPS * 32);
@@ -261,28 +284,34 @@ __device__ __forceinline__ void gemm_cta_setup(Cta& c, uint8_t* smem_raw, int fu
 }
 
 // ---------------- TMA producer (one thread) ----------------
-// MODE 1: weight tile = 4 x 64 weight rows (gate[0,64) | up[0,64) | gate[64,128) | up[64,128) of the tile's 128
-// columns; in the fused kernel gate[0,128) | up[0,128)); MODE 2: 2 x 128 rows.  FUSED and MODE 1: the token
-// rows and the scales come from the gather warp instead; FUSED and MODE 2: the tile's token rows are GEMM1's
-// output and must have been stored.
+// One copy for the token rows and two for the 256 weight rows of a K-block: a copy instruction costs this thread
+// about 85 clocks, which is part of the time a stage needs to be refilled (500 clocks with the weight rows as four
+// copies and the scales as another one); boxes of 256 rows move at 52 bytes per clock and SM out of L2, boxes of 128
+// rows at 67 (measured with a loads-only kernel).
+// tmB: weight rows in the order of the MMAs' N side -- MODE 1 gate[0,64) | up[0,64) | gate[64,128) | up[64,128) of
+// the tile's 128 columns, MODE 2 256 consecutive rows; tmBm (MODE 1): in the order of the M side, gate[0,128) |
+// up[0,128), for short row tiles and the fused kernel.  ("gate" and "up" change places with gate_first = 0.)
+// FUSED and MODE 1: the token rows and the scales come from the gather warp instead; FUSED and MODE 2: the tile's
+// token rows are GEMM1's output and must have been stored.
 template <int MODE, bool FUSED, class GEO>
 __device__ __forceinline__ void producer_tiles(const Cta& c, const CUtensorMap* tmA, const CUtensorMap* tmB,
                                                const GemmArgs& g, const FusedArgs* f, int ready_target, TileRange tr,
                                                uint32_t& it, bool& ok, const CUtensorMap* tmA_short = nullptr,
-                                               KSplit ks = KSplit{1, 1 << 30}) {
+                                               const CUtensorMap* tmBm = nullptr, KSplit ks = KSplit{1, 1 << 30}) {
     GemmCtrl* ctrl = c.ctrl;
     for (int item = tr.first; item < tr.count && ok; item += tr.stride) {
         const int tile = item / ks.parts, kb0 = (item - tile * ks.parts) * ks.len;
         const int kb1 = min(g.num_kb, kb0 + ks.len);
         const int m_tile = tile / g.n_tiles, n = tile - m_tile * g.n_tiles;
-        const int wrow = __ldcg(g.tile_expert + m_tile) * g.w_rows_per_expert;
+        const int e = __ldcg(g.tile_expert + m_tile);
         const int row0 = FUSED ? __ldcg(g.tile_row0 + m_tile) : m_tile * TILE_M;
         const float* a_sc = g.a_scale_t + row0;
         // a short row tile of the large-tile kernel: 32 token rows fetched, weights laid out for the M side
         const bool wm = !FUSED && g.wm_rows > 0 && __ldcg(g.tile_rows + m_tile) <= g.wm_rows;
+        const CUtensorMap* tA = wm ? tmA_short : tmA;
         const uint32_t TX_BYTES = (FUSED && MODE == 1) ? G_B_BYTES
-                                  : wm ? WM_TOKENS * G_BLOCK_K + WM_TOKENS * 4 + G_B_BYTES
-                                       : GEO::STAGE_BYTES + GEO::SCALE_BYTES;
+                                  : FUSED ? GEO::STAGE_BYTES + GEO::SCALE_BYTES
+                                          : wm ? WM_TOKENS * G_BLOCK_K + G_B_BYTES : GEO::STAGE_BYTES;
         // claim the stage of pipeline iteration j: wait until its last reader has finished, announce the bytes
         auto claim = [&](uint32_t j) -> bool {
             const uint32_t s = j % GEO::STAGES, ph = (j / GEO::STAGES) & 1;
@@ -298,27 +327,23 @@ __device__ __forceinline__ void producer_tiles(const Cta& c, const CUtensorMap* 
             const uint32_t s = j % GEO::STAGES, bar = smem_u32(&ctrl->full[s]);
             const uint32_t b_dst = c.smem_base + s * GEO::STAGE_BYTES + GEO::A_BYTES;
             const int k0 = kb * G_BLOCK_K;
-            if (MODE == 1) {
-                const int gr = wrow + g.gate_row0 + n * 128, ur = wrow + g.up_row0 + n * 128;
-                // weights on N: gate[0,64) | up[0,64) | gate[64,128) | up[64,128); on M (fused kernel):
-                // gate[0,128) | up[0,128)
-                tma_load_2d(b_dst, tmB, k0, gr, bar);
-                tma_load_2d(b_dst + G_B_BYTES / 4, tmB, k0, (FUSED || wm) ? gr + 64 : ur, bar);
-                tma_load_2d(b_dst + G_B_BYTES / 2, tmB, k0, (FUSED || wm) ? ur : gr + 64, bar);
-                tma_load_2d(b_dst + 3 * G_B_BYTES / 4, tmB, k0, ur + 64, bar);
+            const int br = e * g.w_rows_per_expert + n * (MODE == 1 ? 128 : G_TILE_N);
+            if (MODE == 2 || FUSED || wm) {
+                tma_load_2d(b_dst, MODE == 2 ? tmB : tmBm, k0, br, bar);
+                tma_load_2d(b_dst + G_B_BYTES / 2, MODE == 2 ? tmB : tmBm, k0, br + (MODE == 1 ? g.up_row0 : 128), bar);
             } else {
-                const int br = wrow + n * G_TILE_N;
-                tma_load_2d(b_dst, tmB, k0, br, bar);
-                tma_load_2d(b_dst + G_B_BYTES / 2, tmB, k0, br + 128, bar);
+                tma_load_4d(b_dst, tmB, k0, n * 128, 0, e, bar);
+                tma_load_4d(b_dst + G_B_BYTES / 2, tmB, k0, n * 128 + 64, 0, e, bar);
             }
         };
-        auto load_a = [&](uint32_t j, int kb) {  // the A rows and their scales of the K-block
+        auto load_a = [&](uint32_t j, int kb) {  // the A rows (fused kernel: and their scales) of the K-block
             const uint32_t s = j % GEO::STAGES, bar = smem_u32(&ctrl->full[s]);
             // (the scale slot is free: the ring exceeds the stages + accumulators the producer can be ahead
             // of the epilogue)
-            bulk_load_1d(smem_u32(c.scale_ring + (j % GEO::SCALE_SLOTS) * GEO::A_ROWS),
-                         a_sc + static_cast<size_t>(kb) * g.row_cap, wm ? WM_TOKENS * 4 : GEO::SCALE_BYTES, bar);
-            tma_load_2d(c.smem_base + s * GEO::STAGE_BYTES, wm ? tmA_short : tmA, kb * G_BLOCK_K, row0, bar);
+            if (FUSED)
+                bulk_load_1d(smem_u32(c.scale_ring + (j % GEO::SCALE_SLOTS) * GEO::A_ROWS),
+                             a_sc + static_cast<size_t>(kb) * g.row_cap, GEO::SCALE_BYTES, bar);
+            tma_load_2d(c.smem_base + s * GEO::STAGE_BYTES, tA, kb * G_BLOCK_K, row0, bar);
         };
         int kb = kb0;
         if (FUSED && MODE == 2) {
@@ -343,8 +368,8 @@ __device__ __forceinline__ void producer_tiles(const Cta& c, const CUtensorMap* 
         for (; kb < kb1 && ok; ++kb, ++it) {
             ok = claim(it);
             if (!ok) break;
+            load_b(it, kb);  // (first: it may have to come from HBM, the token rows are in L2)
             if (!(FUSED && MODE == 1)) load_a(it, kb);
-            load_b(it, kb);
         }
     }
 }
@@ -366,51 +391,56 @@ __device__ __forceinline__ void producer_drain(const Cta& c, int* status, uint32
 // Two threads share the issue work: `mine` = 0 takes the even K-blocks (TMEM buffer 0), 1 the odd ones (buffer
 // 1).  A commit only tracks the MMAs of its own thread, so while one thread pays for its commit and waits the
 // other keeps the tensor pipe fed.
+// An accumulator buffer comes back through a named barrier that the eight epilogue warps arrive at and the issuer
+// warp waits on, once per K-block (see ACC_BARRIER): the hand-over is part of the loop that bounds the kernel, and
+// it is 80 clocks shorter than through an mbarrier.  Such a wait has no limit of its own, so no role may ever miss
+// its turn: after an abort the issuers and the epilogue warps go on to the end of the work list with the barriers
+// alone (the waits on mbarriers stay bounded).
 template <class GEO>
 __device__ __forceinline__ void issuer_tiles(const Cta& c, const GemmArgs& g, TileRange tr, uint32_t mine,
                                              uint32_t& it, bool& ok) {
     GemmCtrl* ctrl = c.ctrl;
     const uint32_t idesc = umma_idesc_f8(TILE_M, G_TILE_N), idesc_wm = umma_idesc_f8(TILE_M, WM_TOKENS);
-    for (int tile = tr.first; tile < tr.count && ok; tile += tr.stride) {
+    for (int tile = tr.first; tile < tr.count; tile += tr.stride) {
         // a short row tile: the stage's weight rows are the M side (two blocks of 128), its 32 token rows the N
         // side; the accumulator is the first 64 columns of the buffer
         const bool wm = g.wm_rows > 0 && __ldcg(g.tile_rows + tile / g.n_tiles) <= g.wm_rows;
         for (int kb = 0; kb < g.num_kb; ++kb, ++it) {
             if ((it & 1) != mine) continue;
             const uint32_t s = it % GEO::STAGES, ph = (it / GEO::STAGES) & 1;
-            const uint32_t b = it & 1, bph = (it >> 1) & 1;
             // The stage has normally landed long before the accumulator is handed back, so that
             // wait comes first and only the hand-over itself is left on the critical path.
             const uint32_t a_addr = c.smem_base + s * GEO::STAGE_BYTES;
             const uint64_t a_desc = umma_desc_sw128(a_addr);  // 128 rows from here, fetched or not
             const uint64_t b_desc = umma_desc_sw128(a_addr + GEO::A_BYTES);
-            const uint32_t d_tmem = c.tmem_base + b * G_TILE_N;
-            if (!mbar_wait(smem_u32(&ctrl->full[s]), ph, c.abort_flag, c.limit)) {
-                raise(ctrl, g.status, DEV_TIMEOUT_MMA_SMEM);
-                ok = false;
-                break;
+            const uint32_t d_tmem = c.tmem_base + mine * G_TILE_N;
+            if (ok) {
+                if (c.lane == 0) ok = mbar_wait(smem_u32(&ctrl->full[s]), ph, c.abort_flag, c.limit);
+                ok = __shfl_sync(0xffffffffu, ok, 0);
+                if (!ok && c.lane == 0) raise(ctrl, g.status, DEV_TIMEOUT_MMA_SMEM);
             }
-            if (!mbar_wait(smem_u32(&ctrl->tmem_empty[b]), bph ^ 1, c.abort_flag, c.limit)) {
-                raise(ctrl, g.status, DEV_TIMEOUT_MMA_TMEM);
-                ok = false;
-                break;
-            }
+            if (it >= G_ACC_BUFS) bar_sync(ACC_BARRIER + mine, ACC_BARRIER_THREADS);
+            if (!ok) continue;
             tc_fence_after();
-            if (wm) {
-                const uint64_t w1_desc = umma_desc_sw128(a_addr + GEO::A_BYTES + G_B_BYTES / 2);
+            if (c.lane == 0) {
+                if (wm) {
+                    const uint64_t w1_desc = umma_desc_sw128(a_addr + GEO::A_BYTES + G_B_BYTES / 2);
 #pragma unroll
-                for (int k = 0; k < G_BLOCK_K / 32; ++k) umma_f8(d_tmem, b_desc + 2 * k, a_desc + 2 * k, idesc_wm, k > 0);
+                    for (int k = 0; k < G_BLOCK_K / 32; ++k) umma_f8(d_tmem, b_desc + 2 * k, a_desc + 2 * k, idesc_wm, k > 0);
 #pragma unroll
-                for (int k = 0; k < G_BLOCK_K / 32; ++k)
-                    umma_f8(d_tmem + WM_TOKENS, w1_desc + 2 * k, a_desc + 2 * k, idesc_wm, k > 0);
-            } else {
+                    for (int k = 0; k < G_BLOCK_K / 32; ++k)
+                        umma_f8(d_tmem + WM_TOKENS, w1_desc + 2 * k, a_desc + 2 * k, idesc_wm, k > 0);
+                } else {
 #pragma unroll
-                for (int k = 0; k < G_BLOCK_K / 32; ++k)  // 32 K-bytes per instruction: +2 in 16-B units
-                    umma_f8(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, k > 0);
+                    for (int k = 0; k < G_BLOCK_K / 32; ++k)  // 32 K-bytes per instruction: +2 in 16-B units
+                        umma_f8(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, k > 0);
+                }
+                umma_commit(smem_u32(&ctrl->done[s]));
             }
-            umma_commit(smem_u32(&ctrl->done[s]));
+            __syncwarp();
         }
     }
+    if (it > mine) bar_sync(ACC_BARRIER + mine, ACC_BARRIER_THREADS);  // the buffer's last hand-over
 }
 
 // After an abort: let issued MMAs retire before TMEM is released.
@@ -420,6 +450,75 @@ __device__ __forceinline__ void issuer_drain(const Cta& c, uint32_t mine, bool o
         int zero = 0;
         mbar_wait(smem_u32(&c.ctrl->drain_bar[mine]), 0, &zero, c.limit);
     }
+}
+
+// ---------------- factor warp (large-tile kernels) ----------------
+// Multiplies the activation scales of every K-block with the two weight scales of the tile's 256 columns, so that
+// an epilogue thread finds its factor with one shared-memory load: [slot][2][row].  With the weight scales fetched
+// from global memory by the epilogue threads themselves, and the products formed there, an epilogue warp spent
+// about 500 of its 1240 clocks per K-block between handing a buffer back and being ready for the next one.  The
+// warp's arrival is the second one on done[s]: whoever sees that barrier finds the factors complete.  Like the
+// producer it claims a stage by waiting for the previous phase of done[s]; the slot it then writes was read by the
+// epilogue eight K-blocks ago (done of four K-blocks ago implies that the accumulator of six ago was handed back).
+// The scales come in F_AHEAD K-blocks ahead, across the ends of tiles: with loads that started anew at every tile the
+// warp's first arrival was late by the latency of three dependent loads, 3 % of a batch of 257 tokens.
+template <int MODE, class GEO>
+__device__ __forceinline__ void factor_tiles(const Cta& c, const GemmArgs& g, TileRange tr) {
+    static_assert(GEO::FACTORS && GEO::A_ROWS == 128, "a lane looks after four rows");
+    static_assert(GEO::SCALE_SLOTS >= GEO::STAGES + G_ACC_BUFS + 1, "slots still read by the epilogue");
+    static_assert(F_AHEAD < F_SLOTS, "a slot is refilled after it was read");
+    GemmCtrl* ctrl = c.ctrl;
+    const int lane = c.lane, num_kb = g.num_kb;
+    // the fetch cursor: tile, K-block, and this lane's sources there; the expert of the tile after it is known early
+    int ftile = tr.first, fkb = 0;
+    int e_next = ftile < tr.count ? __ldcg(g.tile_expert + ftile / g.n_tiles) : 0;
+    const float* as = nullptr;
+    const float* ws = nullptr;
+    uint32_t fit = 0;
+    auto fetch = [&]() {
+        if (ftile < tr.count) {
+            if (fkb == 0) {
+                const int m_tile = ftile / g.n_tiles, n = ftile - m_tile * g.n_tiles;
+                as = g.a_scale_t + static_cast<size_t>(m_tile) * TILE_M + lane * 4;
+                const int block = MODE == 1 ? n + lane * (g.up_row0 / 128) : 2 * n + lane;  // (lanes 0 and 1)
+                ws = g.w_scale + (static_cast<size_t>(e_next) * (g.w_rows_per_expert / 128) + block) * num_kb;
+                if (ftile + tr.stride < tr.count) e_next = __ldcg(g.tile_expert + (ftile + tr.stride) / g.n_tiles);
+            }
+            float* raw = c.raw_scales + (fit % F_SLOTS) * F_SLOT_FLOATS;
+            cp_async_16(smem_u32(raw + lane * 4), as, 16);
+            if (lane < 2) cp_async_4(smem_u32(raw + TILE_M + lane), ws, 4);
+            as += g.row_cap;
+            ++ws;
+            if (++fkb == num_kb) {
+                fkb = 0;
+                ftile += tr.stride;
+            }
+        }
+        ++fit;
+        cp_async_commit();
+    };
+    for (int i = 0; i < F_AHEAD; ++i) fetch();
+    uint32_t it = 0;
+    for (int tile = tr.first; tile < tr.count; tile += tr.stride)
+        for (int kb = 0; kb < num_kb; ++kb, ++it) {
+            const uint32_t s = it % GEO::STAGES;
+            cp_async_wait<F_AHEAD - 1>();
+            __syncwarp();
+            const float* raw = c.raw_scales + (it % F_SLOTS) * F_SLOT_FLOATS;
+            const float4 a = *reinterpret_cast<const float4*>(raw + lane * 4);
+            const float2 w = *reinterpret_cast<const float2*>(raw + TILE_M);
+            fetch();
+            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctrl->done[s]), ((it / GEO::STAGES) & 1) ^ 1, c.abort_flag, c.limit))) {
+                if (lane == 0) raise(ctrl, g.status, DEV_TIMEOUT_PRODUCER);
+                cp_async_wait_all();  // nothing may still be landing in shared memory when the CTA exits
+                return;
+            }
+            float* dst = c.scale_ring + (it % GEO::SCALE_SLOTS) * 2 * GEO::A_ROWS + lane * 4;
+            *reinterpret_cast<float4*>(dst) = make_float4(a.x * w.x, a.y * w.x, a.z * w.x, a.w * w.x);
+            *reinterpret_cast<float4*>(dst + GEO::A_ROWS) = make_float4(a.x * w.y, a.y * w.y, a.z * w.y, a.w * w.y);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&ctrl->done[s]));
+        }
 }
 
 // ---------------- gather warp (fused kernel) ----------------
@@ -508,6 +607,20 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
                                                  uint32_t& it, uint32_t& tile_iter, uint32_t& sync_iter, int kb0 = 0,
                                                  int kb1 = -1, int parts = 1);
 
+// acc[0..64) += v * f with packed fp32 FMAs: one instruction, two independent round-to-nearest FMAs, the bits of the
+// scalar form.  Beside scalar FMAs the MMA issuers, which share the schedulers with the epilogue warps, needed 955
+// clocks per K-block in a probe of this loop, beside packed ones 672 (602 beside an epilogue without FMAs).
+__device__ __forceinline__ void fma64(float* acc, const float (&v)[64], float f) {
+    const uint64_t p = pack_f32x2(__float_as_uint(f), __float_as_uint(f));
+#pragma unroll
+    for (int j = 0; j < 64; j += 2) {
+        const uint64_t a = fma_f32x2(pack_f32x2(__float_as_uint(v[j]), __float_as_uint(v[j + 1])), p,
+                                     pack_f32x2(__float_as_uint(acc[j]), __float_as_uint(acc[j + 1])));
+        acc[j] = __uint_as_float(static_cast<uint32_t>(a));
+        acc[j + 1] = __uint_as_float(static_cast<uint32_t>(a >> 32));
+    }
+}
+
 // ---------------- epilogue warps ----------------
 // MODE 1: gate/up projection + SwiGLU + re-quantisation; tmOut describes the e4m3 output [row_cap, I] for
 //         64-byte x 32-row TMA stores.
@@ -526,11 +639,9 @@ __device__ __forceinline__ void epilogue_tiles(const Cta& c, const CUtensorMap* 
     const size_t row_cap = static_cast<size_t>(g.row_cap);
     float* amax_x = c.amax_x;
     uint8_t* stage = c.store_stage + widx * G_STORE_WARP_BYTES;  // staging of this warp's GEMM1 rows
-    const int scale_row = r_in_tile;
     const int num_kb = g.num_kb;
     for (int tile = tr.first; tile < tr.count && ok; tile += tr.stride) {
         const int m_tile = tile / g.n_tiles, n = tile - m_tile * g.n_tiles;
-        const int e = __ldcg(g.tile_expert + m_tile);
         const int rows_valid = __ldcg(g.tile_rows + m_tile);
         if (g.wm_rows > 0 && rows_valid <= g.wm_rows) {  // a short row tile, worked on with the weights on M
             uint32_t unused = 0;
@@ -538,28 +649,11 @@ __device__ __forceinline__ void epilogue_tiles(const Cta& c, const CUtensorMap* 
             continue;
         }
         const size_t row = static_cast<size_t>(m_tile) * TILE_M + r_in_tile;
-        const int sblocks = g.w_rows_per_expert / 128;
-        // weight-scale rows of this thread's first / second 64 columns
-        const float* ws0;
-        const float* ws1;
-        if (MODE == 1) {
-            ws0 = g.w_scale + (static_cast<size_t>(e) * sblocks + g.gate_row0 / 128 + n) * num_kb;
-            ws1 = g.w_scale + (static_cast<size_t>(e) * sblocks + g.up_row0 / 128 + n) * num_kb;
-        } else {
-            ws0 = g.w_scale + (static_cast<size_t>(e) * sblocks + 2 * n + half) * num_kb;
-            ws1 = ws0;
-        }
         float acc[128];
 #pragma unroll
         for (int j = 0; j < 128; ++j) acc[j] = 0.0f;
 
-        float s0 = __ldg(ws0), s1 = __ldg(ws1);
         for (int kb = 0; kb < num_kb; ++kb, ++it) {
-            const float w0 = s0, w1 = s1;
-            if (kb + 1 < num_kb) {
-                s0 = __ldg(ws0 + kb + 1);
-                s1 = __ldg(ws1 + kb + 1);
-            }
             const uint32_t s = it % GEO::STAGES, ph = (it / GEO::STAGES) & 1, buf = it & 1;
             // Every lane polls (a single polling lane plus a broadcast was measured 2.5 % slower); the vote
             // keeps the warp converged when a wait gives up: either all lanes go on or none does.
@@ -569,24 +663,23 @@ __device__ __forceinline__ void epilogue_tiles(const Cta& c, const CUtensorMap* 
                 break;
             }
             tc_fence_after();
-            // The MMA of this K-block has finished, hence its stage -- A, B and the scales -- had landed.
-            // (Fetching the scale earlier needs a barrier of its own per ring slot -- on full[s] this warp can
-            // be lapped by a whole phase -- and that extra barrier test per K-block was measured to cost the
-            // epilogue 110 clocks, 10 % of the kernel: barrier operations of a thread queue behind one another.)
-            const float sa = ld_shared_f32(c.scale_ring + (it % GEO::SCALE_SLOTS) * GEO::A_ROWS + scale_row);
-            const float f0 = sa * w0, f1 = sa * w1;
             // GEMM1: of this warpgroup's 128 columns, [0,64) are gate and [64,128) the matching up columns.
             const uint32_t col = t_lane + buf * G_TILE_N;
             float v[64];
-            tmem_ld64(col, v);
-#pragma unroll
-            for (int j = 0; j < 64; ++j) acc[j] = fmaf(v[j], f0, acc[j]);
-            tmem_ld64(col + 64, v);
+            tmem_ld32_issue(col, v);
+            tmem_ld32_issue(col + 32, v + 32);
+            // this row's factors for the columns [0,64) and [64,128) of the half (GEMM2: the same one)
+            const float* fr = c.scale_ring + (it % GEO::SCALE_SLOTS) * 2 * GEO::A_ROWS + r_in_tile;
+            const float f0 = ld_shared_f32(fr + (MODE == 1 ? 0 : half * GEO::A_ROWS));
+            const float f1 = MODE == 1 ? ld_shared_f32(fr + GEO::A_ROWS) : f0;
+            tmem_wait_ld(v);
+            fma64(acc, v, f0);
+            tmem_ld32_issue(col + 64, v);
+            tmem_ld32_issue(col + 96, v + 32);
+            tmem_wait_ld(v);
             tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&ctrl->tmem_empty[buf]));
-#pragma unroll
-            for (int j = 0; j < 64; ++j) acc[64 + j] = fmaf(v[j], f1, acc[64 + j]);
+            bar_arrive(ACC_BARRIER + buf, ACC_BARRIER_THREADS);
+            fma64(acc + 64, v, f1);
         }
         if (!ok) break;
 
@@ -599,6 +692,14 @@ __device__ __forceinline__ void epilogue_tiles(const Cta& c, const CUtensorMap* 
             // SwiGLU on this thread's 64 columns, then the row's 128-wide amax across the two halves
             float cc[64];
             float amax = 0.0f;
+            if (g.up_first) {
+#pragma unroll
+                for (int j = 0; j < 64; ++j) {
+                    const float x = acc[j];
+                    acc[j] = acc[64 + j];
+                    acc[64 + j] = x;
+                }
+            }
 #pragma unroll
             for (int j = 0; j < 64; ++j) {
                 // silu(g) * u with the hardware exp2 and reciprocal approximations (a few ulp): the
@@ -753,7 +854,7 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
     const float* ws0;  // weight-scale rows of block 0 / block 1
     const float* ws1;
     if (MODE == 1) {
-        ws0 = g.w_scale + (static_cast<size_t>(e) * sblocks + g.gate_row0 / 128 + n) * num_kb;
+        ws0 = g.w_scale + (static_cast<size_t>(e) * sblocks + n) * num_kb;
         ws1 = g.w_scale + (static_cast<size_t>(e) * sblocks + g.up_row0 / 128 + n) * num_kb;
     } else {
         ws0 = g.w_scale + (static_cast<size_t>(e) * sblocks + 2 * n) * num_kb;
@@ -769,10 +870,14 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
     if (SPLIT)
         raw = reinterpret_cast<float4*>(f->raw[MODE - 1] + static_cast<size_t>(m_tile * g.n_tiles + n) * num_kb * SPLIT_RAW_FLOATS) +
               quad * 32 + lane;
-    float s0 = __ldg(ws0 + kb0), s1 = __ldg(ws1 + kb0);
+    float s0 = 0.0f, s1 = 0.0f;
+    if (!SHARED) {
+        s0 = __ldg(ws0 + kb0);
+        s1 = __ldg(ws1 + kb0);
+    }
     for (int kb = kb0; kb < kb_end; ++kb, ++it) {
         const float w0 = s0, w1 = s1;
-        if (kb + 1 < kb_end) {
+        if (!SHARED && kb + 1 < kb_end) {
             s0 = __ldg(ws0 + kb + 1);
             s1 = __ldg(ws1 + kb + 1);
         }
@@ -783,22 +888,36 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
         }
         tc_fence_after();
         // the MMAs of this K-block have finished, hence its stage -- tokens, weights and scales -- had landed
-        const float4* sp = reinterpret_cast<const float4*>(c.scale_ring + (it % GEO::SCALE_SLOTS) * GEO::A_ROWS + th * 16);
-        float sa[16];
+        float f0[16], f1[16];  // factors of this thread's tokens for block 0 / block 1
+        if (SHARED) {
+            const float4* fp = reinterpret_cast<const float4*>(c.scale_ring + (it % GEO::SCALE_SLOTS) * 2 * GEO::A_ROWS + th * 16);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float4 x = sp[q];
-            sa[4 * q] = x.x;
-            sa[4 * q + 1] = x.y;
-            sa[4 * q + 2] = x.z;
-            sa[4 * q + 3] = x.w;
+            for (int q = 0; q < 4; ++q) {
+                *reinterpret_cast<float4*>(f0 + 4 * q) = fp[q];
+                *reinterpret_cast<float4*>(f1 + 4 * q) = fp[GEO::A_ROWS / 4 + q];
+            }
+        } else {
+            const float4* sp = reinterpret_cast<const float4*>(c.scale_ring + (it % GEO::SCALE_SLOTS) * GEO::A_ROWS + th * 16);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 x = sp[q];
+                const float sa[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    f0[4 * q + i] = sa[i] * w0;
+                    f1[4 * q + i] = sa[i] * w1;
+                }
+            }
         }
         float v[32];
         const uint32_t buf = SHARED ? (it & 1) : s, t_buf = t_lane + buf * (SHARED ? G_TILE_N : WM_BUF_COLS);
         tmem_ld16x2(t_buf, t_buf + WM_TOKENS, v);
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&ctrl->tmem_empty[buf]));
+        if (SHARED)
+            bar_arrive(ACC_BARRIER + buf, ACC_BARRIER_THREADS);
+        else if (lane == 0)
+            mbar_arrive(smem_u32(&ctrl->tmem_empty[buf]));
         if (SPLIT) {
             if (th == 0) {  // (all four token columns; those past the tile's rows are never used)
                 raw[(kb * 2 + 0) * 128] = make_float4(v[0], v[1], v[2], v[3]);
@@ -807,8 +926,8 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
         } else {
 #pragma unroll
             for (int t = 0; t < 16; ++t) {
-                acc[t] = fmaf(v[t], sa[t] * w0, acc[t]);
-                acc[16 + t] = fmaf(v[16 + t], sa[t] * w1, acc[16 + t]);
+                acc[t] = fmaf(v[t], f0[t], acc[t]);
+                acc[16 + t] = fmaf(v[16 + t], f1[t], acc[16 + t]);
             }
         }
     }
@@ -897,6 +1016,14 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
     if (MODE == 1) {
         float cc[16];
         uint32_t wmax[16];
+        if (g.up_first) {
+#pragma unroll
+            for (int t = 0; t < 16; ++t) {
+                const float x = acc[t];
+                acc[t] = acc[16 + t];
+                acc[16 + t] = x;
+            }
+        }
 #pragma unroll
         for (int t = 0; t < 16; ++t) {
             const float gt = acc[t];
@@ -1071,7 +1198,8 @@ __device__ __forceinline__ void epilogue_tiles_wm(const Cta& c, const GemmArgs& 
 template <int MODE>
 __global__ void __launch_bounds__(G_THREADS, 1)
 grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmAs,
-                    const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmOut, const GemmArgs g) {
+                    const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmBm,
+                    const __grid_constant__ CUtensorMap tmOut, const GemmArgs g) {
     extern __shared__ uint8_t smem_raw[];
     using GEO = GeomFull;
     Cta c;
@@ -1080,7 +1208,10 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmAs);
         tma_prefetch_desc(&tmB);
-        if (MODE == 1) tma_prefetch_desc(&tmOut);
+        if (MODE == 1) {
+            tma_prefetch_desc(&tmBm);
+            tma_prefetch_desc(&tmOut);
+        }
     }
     tc_fence_before();
     __syncthreads();
@@ -1099,16 +1230,21 @@ grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     if (c.warp < 4) {
         reg_dealloc<40>();
         if (c.warp == 0 && c.lane == 0) {
-            producer_tiles<MODE, false, GEO>(c, &tmA, &tmB, g, nullptr, 0, tr, it, ok, &tmAs);
+            producer_tiles<MODE, false, GEO>(c, &tmA, &tmB, g, nullptr, 0, tr, it, ok, &tmAs, &tmBm);
             producer_drain<GEO>(c, g.status, it);
-        } else if ((c.warp == 1 || c.warp == 2) && c.lane == 0) {
+        } else if (c.warp == 1 || c.warp == 2) {
             issuer_tiles<GEO>(c, g, tr, c.warp - 1, it, ok);
-            issuer_drain(c, c.warp - 1, ok);
+            if (c.lane == 0) issuer_drain(c, c.warp - 1, ok);
+        } else if (c.warp == 3) {
+            factor_tiles<MODE, GEO>(c, g, tr);
         }
     } else {
         reg_alloc<232>();
         uint32_t tile_iter = 0;
         epilogue_tiles<MODE, GEO>(c, &tmOut, g, tr, it, tile_iter, ok);
+        // After an abort: the hand-overs this warp still owes, waiting for the issuer so that no turn is taken twice.
+        const uint32_t total = (tr.first < tr.count ? (tr.count - tr.first + tr.stride - 1) / tr.stride : 0) * g.num_kb;
+        for (; it < total; ++it) bar_sync(ACC_BARRIER + (it & 1), ACC_BARRIER_THREADS);
         if (c.lane == 0) bulk_wait_all();
     }
 
@@ -1179,8 +1315,8 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmA2, const __grid_consta
     if (c.warp < 4) {
         reg_dealloc<40>();
         if (c.warp == 0 && c.lane == 0) {
-            producer_tiles<1, true, GEO>(c, &tmA2, &tmB1, g1, &f, 0, tr1, it, ok, nullptr, ks1);
-            producer_tiles<2, true, GEO>(c, &tmA2, &tmB2, g2, &f, g1.n_tiles, tr2, it, ok, nullptr, ks2);
+            producer_tiles<1, true, GEO>(c, &tmA2, nullptr, g1, &f, 0, tr1, it, ok, nullptr, &tmB1, ks1);
+            producer_tiles<2, true, GEO>(c, &tmA2, &tmB2, g2, &f, g1.n_tiles, tr2, it, ok, nullptr, nullptr, ks2);
             producer_drain<GEO>(c, g1.status, it);
         } else if ((c.warp == 1 || c.warp == 2) && c.lane == 0) {
             issuer_tiles_wm<GEO>(c, g1, tr1, c.warp - 1, it, ok, ks1);

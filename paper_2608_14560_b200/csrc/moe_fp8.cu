@@ -111,7 +111,8 @@ struct moe_fp8_handle_s {
     uint8_t* ws;
     size_t ws_bytes;
     EncodeTiledFn encode;
-    CUtensorMap tm_a1, tm_a2, tm_a1_small, tm_a2_small, tm_a2_store, tm_w13, tm_w2;
+    // tm_w13_n / tm_w13_m: the 256 weight rows of a GEMM1 tile in the order of the MMAs' N side / M side
+    CUtensorMap tm_a1, tm_a2, tm_a1_small, tm_a2_small, tm_a2_store, tm_w13_n, tm_w13_m, tm_w2;
     const void* w13_cached;
     const void* w2_cached;
     bool stage_timing;
@@ -149,6 +150,16 @@ bool encode_2d(moe_fp8_handle_t h, CUtensorMap* m, const void* base, uint64_t ro
                            const_cast<void*>(base), gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
                            swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
+}
+
+// Four dimensions of one-byte elements (dims[0] contiguous, strides[i] in bytes between the elements of dimension
+// i + 1), 128-byte swizzle.
+bool encode_4d(moe_fp8_handle_t h, CUtensorMap* m, const void* base, const cuuint64_t* dims, const cuuint64_t* strides,
+               const cuuint32_t* box) {
+    const cuuint32_t estride[4] = {1, 1, 1, 1};
+    return h->encode(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void*>(base), dims, strides, box, estride,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 template <typename T>
@@ -376,9 +387,13 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
     cudaStream_t stream = static_cast<cudaStream_t>(stream_v);
     const int H = c.hidden, I = c.intermediate, EL = c.num_local_experts;
     if (w13 != h->w13_cached || w2 != h->w2_cached) {
-        // w13 is fetched in 64-row boxes (gate and up rows interleave in the B tile), w2 in 128-row boxes
-        if (!encode_2d(h, &h->tm_w13, w13, static_cast<uint64_t>(EL) * 2 * I, H, 1, 128, 64,
-                       CU_TENSOR_MAP_SWIZZLE_128B) ||
+        // N side of the MMAs: w13 seen as [E_loc][2 halves][I rows][H], a box takes the same 64 rows of both halves, so
+        // that an epilogue warpgroup finds gate and up of the same columns side by side; M side: 128 consecutive rows
+        const cuuint64_t Hz = H, Iz = I, Ez = EL;
+        const cuuint64_t dims[4] = {Hz, Iz, 2, Ez}, strides[3] = {Hz, Iz * Hz, 2 * Iz * Hz};
+        const cuuint32_t box[4] = {128, 64, 2, 1};
+        if (!encode_4d(h, &h->tm_w13_n, w13, dims, strides, box) ||
+            !encode_2d(h, &h->tm_w13_m, w13, static_cast<uint64_t>(EL) * 2 * I, H, 1, 128, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
             !encode_2d(h, &h->tm_w2, w2, static_cast<uint64_t>(EL) * H, I, 1, 128, 128, CU_TENSOR_MAP_SWIZZLE_128B))
             return cuda_fail(h, cudaErrorInvalidValue);
         h->w13_cached = w13;
@@ -468,8 +483,8 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
     g1.w_rows_per_expert = 2 * I;
     g1.row_cap = row_cap;
     g1.out_cols = I;
-    g1.gate_row0 = c.gate_first ? 0 : I;
-    g1.up_row0 = c.gate_first ? I : 0;
+    g1.up_row0 = I;
+    g1.up_first = c.gate_first ? 0 : 1;
     g1.num_m_tiles = m.num_m_tiles;
     g1.tile_expert = m.tile_expert;
     g1.tile_rows = m.tile_rows;
@@ -539,7 +554,7 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
         mark();  // gemm2
         mark();  // combine
         MOE_LAUNCH(fused_small_kernel, h->sm_count, G_THREADS, GeomSmall::SMEM_BYTES, stream, pdl, h->tm_a2_small,
-                   h->tm_w13, h->tm_w2, g1, g2, f);
+                   h->tm_w13_m, h->tm_w2, g1, g2, f);
         ++h->fused_calls;  // only a kernel that runs zeroes the other counter set
         mark();
     } else {
@@ -553,11 +568,11 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
         // stage 3a: GEMM1 + SwiGLU + re-quantisation
         if (h->short_tile_min_tokens > 0 && T >= h->short_tile_min_tokens) g1.wm_rows = g2.wm_rows = WM_TOKENS;
         MOE_LAUNCH(grouped_gemm_kernel<1>, h->sm_count, G_THREADS, GeomFull::SMEM_BYTES, stream, pdl, h->tm_a1,
-                   h->tm_a1_small, h->tm_w13, h->tm_a2_store, g1);
+                   h->tm_a1_small, h->tm_w13_n, h->tm_w13_m, h->tm_a2_store, g1);
         mark();
         // stage 3b: GEMM2
         MOE_LAUNCH(grouped_gemm_kernel<2>, h->sm_count, G_THREADS, GeomFull::SMEM_BYTES, stream, pdl, h->tm_a2,
-                   h->tm_a2_small, h->tm_w2, h->tm_a2_store, g2);
+                   h->tm_a2_small, h->tm_w2, h->tm_w2, h->tm_a2_store, g2);
         mark();
         {  // stage 4: weighted combine back to token order
             const int grid = min(T, h->sm_count * 16);

@@ -390,6 +390,23 @@ def test_short_row_tiles_are_bit_identical_to_full_row_tiles(cuda_device, tokens
     eng.close()
 
 
+# ---- large-tile GEMM kernels on layers with fewer K-blocks per tile than the scale fetch runs ahead -----------
+@pytest.mark.parametrize("hidden,inter,tokens,eloc,gate_first", [(256, 128, 700, 32, True), (256, 384, 300, 2, False),
+                                                                 (768, 128, 90, 256, True), (1280, 640, 1000, 5, False)])
+def test_large_tile_kernels_with_few_k_blocks_per_tile(cuda_device, hidden, inter, tokens, eloc, gate_first):
+    # 1 to 10 K-blocks per tile against 4 pipeline stages, 8 factor slots and scales fetched 4 K-blocks ahead; one
+    # CTA's list mixes short and full row tiles; w13 with the up projection first in two of the cases
+    dims = syn.LayerDims(hidden=hidden, intermediate=inter, num_local_experts=eloc)
+    wl = _wl(tokens, dims, seed=900 + hidden)
+    inp = syn.make_inputs(wl, cuda_device)
+    kw = {}
+    if not gate_first:
+        inp["w13"] = torch.cat([inp["w13"][:, inter:], inp["w13"][:, :inter]], 1).contiguous()
+        inp["w13_scale"] = torch.cat([inp["w13_scale"][:, inter // 128:], inp["w13_scale"][:, :inter // 128]], 1).contiguous()
+        kw["gate_first"] = False
+    run_and_compare(wl, cuda_device, inp=inp, **kw)
+
+
 # ---- batches of at most 80 tokens: gather, both GEMMs and the combine as one kernel; up to 16 tokens that ----
 # ---- kernel also routes and permutes (every CTA for itself), and the forward is a single launch -------------
 @pytest.mark.parametrize("tokens,kw", [(1, {}), (5, {}), (12, {}), (13, {}), (16, {"local_expert_offset": 64}),
