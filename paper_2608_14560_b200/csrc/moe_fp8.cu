@@ -29,7 +29,7 @@ constexpr size_t WS_ALIGN = 1024;
 inline size_t align_up(size_t x, size_t a = WS_ALIGN) { return (x + a - 1) / a * a; }
 
 struct WsLayout {
-    size_t topk_idx, topk_w, block_hist, expert_count, expert_offset, padded_offset, tile_expert, tile_rows,
+    size_t topk_idx, topk_w, slot_rank, block_hist, expert_count, expert_offset, padded_offset, tile_expert, tile_rows,
         num_m_tiles, slot_to_row, row_to_slot, row_token, tok_nlocal, st_expert, st_row0, st_rows, num_st, counters, num_counters, max_st, raw1, raw2, status, a1, a1_scale_t, a2, a2_scale_t, y, stage_hidden,
         stage_scale, stage_logits, stage_out, stage2_hidden, stage2_scale, stage2_logits, stage2_out, total;
     int row_cap, max_m_tiles, max_blocks;
@@ -42,7 +42,8 @@ WsLayout make_layout(const moe_fp8_config& c) {
     size_t pad_experts = static_cast<size_t>(c.num_local_experts) < slots ? c.num_local_experts : slots;
     L.row_cap = static_cast<int>(align_up(slots + pad_experts * (TILE_M - 1), TILE_M));
     L.max_m_tiles = L.row_cap / TILE_M;
-    L.max_blocks = static_cast<int>((Tm + P_TOKENS_PER_BLOCK - 1) / P_TOKENS_PER_BLOCK);
+    // blocks of route_count_kernel: of 8 tokens up to RC_SMALL_MAX_TOKENS, of 32 above
+    L.max_blocks = static_cast<int>(std::max<size_t>((Tm + 31) / 32, (std::min<size_t>(Tm, RC_SMALL_MAX_TOKENS) + 7) / 8));
     const size_t H = c.hidden, I = c.intermediate, EL = c.num_local_experts, rc = L.row_cap;
     size_t o = 0;
     auto take = [&](size_t bytes) {
@@ -52,6 +53,7 @@ WsLayout make_layout(const moe_fp8_config& c) {
     };
     L.topk_idx = take(slots * 4);
     L.topk_w = take(slots * 4);
+    L.slot_rank = take(slots);
     L.block_hist = take(static_cast<size_t>(L.max_blocks) * EL * 4);
     L.expert_count = take(EL * 4);
     L.expert_offset = take((EL + 1) * 4);
@@ -188,6 +190,7 @@ cudaError_t launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
 PermuteMeta meta_of(moe_fp8_handle_t h) {
     PermuteMeta m;
     m.block_hist = at<int>(h, h->L.block_hist);
+    m.slot_rank = at<uint8_t>(h, h->L.slot_rank);
     m.expert_count = at<int>(h, h->L.expert_count);
     m.expert_offset = at<int>(h, h->L.expert_offset);
     m.padded_offset = at<int>(h, h->L.padded_offset);
@@ -410,7 +413,6 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
     float* a2_scale_t = at<float>(h, h->L.a2_scale_t);
     __nv_bfloat16* y = at<__nv_bfloat16>(h, h->L.y);
     const int row_cap = h->L.row_cap;
-    const int nblk = (T + P_TOKENS_PER_BLOCK - 1) / P_TOKENS_PER_BLOCK;
     int launches = 0;
     // Programmatic dependent launch between our own kernels (not across the per-kernel timing events).  It
     // removes 10-13 us of launch gaps from a small batch; on large batches the early-resident blocks of the
@@ -449,7 +451,7 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
         mark();
         mark();
         mark();
-    } else if (T <= P_TAIL_MAX_TOKENS) {  // routing in parallel blocks, the last one to finish does stage 2
+    } else if (fused) {  // routing in parallel blocks, the last one to finish does stage 2 up to the gather
         const int grid = min((T + 7) / 8, h->sm_count * 8);
         MOE_LAUNCH(route_permute_kernel, grid, P_TAIL_THREADS, route_permute_smem_bytes(T, EL), stream, false, T, EL,
                    local_expert_offset, row_cap, router_logits, static_cast<const __nv_bfloat16*>(routing_bias),
@@ -458,21 +460,14 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
         mark();
         mark();
         mark();
-    } else {
-        {  // stage 1: routing
-            const int grid = min((T + 7) / 8, h->sm_count * 8);
-            MOE_LAUNCH(route_topk_kernel, grid, 256, 0, stream, false, T, router_logits,
-                       static_cast<const __nv_bfloat16*>(routing_bias), scaling_factor, topk_idx, topk_w, status);
-            mark();
-        }
-        // stage 2: histogram, scan, placement
-        MOE_LAUNCH(count_kernel, nblk, P_TOKENS_PER_BLOCK, 0, stream, pdl, T, EL, local_expert_offset,
-                   static_cast<const int*>(topk_idx), m.block_hist);
+    } else {  // routing, counts and row tables; the placement follows with the gather
+        const int tpb = route_count_tokens_per_block(T, EL), grid = (T + tpb - 1) / tpb;
+        const auto kernel = tpb == 8 ? route_count_kernel<8> : route_count_kernel<32>;
+        MOE_LAUNCH(kernel, grid, tpb * 32, 0, stream, false, T, EL, local_expert_offset, router_logits,
+                   static_cast<const __nv_bfloat16*>(routing_bias), scaling_factor, topk_idx, topk_w, m, status + 1, status);
         mark();
-        MOE_LAUNCH(scan_kernel, 1, P_MAX_LOCAL, 0, stream, pdl, nblk, EL, m);
         mark();
-        MOE_LAUNCH(place_kernel, nblk, P_TOKENS_PER_BLOCK, 0, stream, pdl, T, EL, local_expert_offset, row_cap,
-                   static_cast<const int*>(topk_idx), m, status);
+        mark();
         mark();
     }
     // the two GEMMs' arguments
@@ -558,11 +553,11 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
         ++h->fused_calls;  // only a kernel that runs zeroes the other counter set
         mark();
     } else {
-        {  // stage 2, continued: gather
-            const long long row_bound = static_cast<long long>(T) * 8 + static_cast<long long>(EL) * (TILE_M - 1);
-            const int grid = static_cast<int>(std::min<long long>((row_bound + 7) / 8, h->sm_count * 8LL));
-            MOE_LAUNCH(gather_rows_kernel, grid, 256, 0, stream, pdl, H, row_cap, c.hidden_scale_layout, T,
-                       static_cast<const uint8_t*>(hidden_fp8), hidden_scale, m, a1, a1_scale_t);
+        {  // stage 2, continued: placement and gather
+            const int grid = min((T + 7) / 8, h->sm_count * 8);
+            MOE_LAUNCH(place_gather_kernel, grid, 256, 0, stream, pdl, T, H, EL, local_expert_offset, row_cap,
+                       route_count_tokens_per_block(T, EL), c.hidden_scale_layout, static_cast<const int*>(topk_idx),
+                       static_cast<const uint8_t*>(hidden_fp8), hidden_scale, m, a1, a1_scale_t, status);
             mark();
         }
         // stage 3a: GEMM1 + SwiGLU + re-quantisation

@@ -19,7 +19,8 @@ namespace moe {
 constexpr int TILE_M = 128;              // GEMM tile height (rows)
 
 struct PermuteMeta {
-    int* block_hist;     // [nblk, E_loc] per-block counts, turned into per-block bases by the scan
+    int* block_hist;     // [nblk, E_loc] per-block counts, turned into per-block bases by the last block
+    uint8_t* slot_rank;  // [T*8] rank of a local slot among the rows of its expert inside its block of tokens
     int* expert_count;   // [E_loc]
     int* expert_offset;  // [E_loc+1] canonical (unpadded) exclusive scan
     int* padded_offset;  // [E_loc+1] exclusive scan of counts rounded up to TILE_M
@@ -38,77 +39,46 @@ struct PermuteMeta {
 };
 constexpr int ST_ROWS = 32;
 
-// Bit t of mask[e] says: token t of this block routes to local expert e.  The
-// popcount below a token's bit is its stable rank inside the block.
-// topk_idx was written by the kernel before this one, which may still be resident (programmatic dependent
-// launch): it is read with coherent (.cg) loads, never through the read-only path.
-__device__ __forceinline__ void build_block_masks(uint32_t (*mask)[P_TOKENS_PER_BLOCK / 32], int T, int E_loc,
-                                                  int off, const int* topk_idx) {
-    for (int i = threadIdx.x; i < E_loc * (P_TOKENS_PER_BLOCK / 32); i += blockDim.x)
-        (&mask[0][0])[i] = 0u;
+// Row tables of all experts from their counts, by one thread block.  In: s_cnt[e] = rows of local expert e for
+// e < P_MAX_LOCAL (zero past E_loc).  Out: the tables of `m`; s_cnt / s_pad hold the exclusive scans of the counts and
+// of the counts rounded up to TILE_M, the totals in entry P_MAX_LOCAL.
+__device__ __forceinline__ void scan_experts(int E_loc, int* s_cnt, int* s_pad, const PermuteMeta& m) {
+    const int tid = threadIdx.x, lane = tid & 31;
     __syncthreads();
-    const int t = blockIdx.x * P_TOKENS_PER_BLOCK + threadIdx.x;
-    if (t < T) {
-        const int4 a = __ldcg(reinterpret_cast<const int4*>(topk_idx) + 2 * t);
-        const int4 b = __ldcg(reinterpret_cast<const int4*>(topk_idx) + 2 * t + 1);
-        const int ids[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    if (tid < 32) {  // lane l owns entries 8l .. 8l+7
+        int c[8], sc = 0, sq = 0;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int e = ids[j] - off;
-            if (e >= 0 && e < E_loc) atomicOr(&mask[e][threadIdx.x >> 5], 1u << (threadIdx.x & 31));
+        for (int i = 0; i < 8; ++i) {
+            c[i] = s_cnt[lane * 8 + i];
+            sc += c[i];
+            sq += (c[i] + TILE_M - 1) / TILE_M * TILE_M;
         }
-    }
-    __syncthreads();
-}
-
-__global__ void __launch_bounds__(P_TOKENS_PER_BLOCK) count_kernel(int T, int E_loc, int off,
-                                                                   const int* topk_idx,
-                                                                   int* __restrict__ block_hist) {
-    pdl_launch_dependents();
-    pdl_wait();
-    __shared__ uint32_t mask[P_MAX_LOCAL][P_TOKENS_PER_BLOCK / 32];
-    build_block_masks(mask, T, E_loc, off, topk_idx);
-    for (int e = threadIdx.x; e < E_loc; e += blockDim.x) {
-        int c = 0;
+        int ec = sc, eq = sq;
 #pragma unroll
-        for (int w = 0; w < P_TOKENS_PER_BLOCK / 32; ++w) c += __popc(mask[e][w]);
-        block_hist[blockIdx.x * E_loc + e] = c;
-    }
-}
-
-// One block.  Thread e owns local expert e.
-__global__ void __launch_bounds__(P_MAX_LOCAL) scan_kernel(int nblk, int E_loc, PermuteMeta m) {
-    pdl_launch_dependents();
-    pdl_wait();
-    __shared__ int s_cnt[P_MAX_LOCAL + 1];
-    __shared__ int s_pad[P_MAX_LOCAL + 1];
-    const int e = threadIdx.x;
-    int total = 0;
-    if (e < E_loc) {
-        for (int b = 0; b < nblk; ++b) {
-            const int c = m.block_hist[b * E_loc + e];
-            m.block_hist[b * E_loc + e] = total;  // base of block b inside expert e
-            total += c;
+        for (int d = 1; d < 32; d <<= 1) {
+            const int vc = __shfl_up_sync(0xffffffffu, ec, d), vq = __shfl_up_sync(0xffffffffu, eq, d);
+            if (lane >= d) {
+                ec += vc;
+                eq += vq;
+            }
+        }
+        int bc = ec - sc, bq = eq - sq;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            s_cnt[lane * 8 + i] = bc;
+            s_pad[lane * 8 + i] = bq;
+            bc += c[i];
+            bq += (c[i] + TILE_M - 1) / TILE_M * TILE_M;
+        }
+        if (lane == 31) {
+            s_cnt[P_MAX_LOCAL] = ec;
+            s_pad[P_MAX_LOCAL] = eq;
+            *m.num_m_tiles = eq / TILE_M;
         }
     }
-    s_cnt[e] = (e < E_loc) ? total : 0;
-    s_pad[e] = (e < E_loc) ? (total + TILE_M - 1) / TILE_M * TILE_M : 0;
     __syncthreads();
-    if (threadIdx.x == 0) {  // 256 entries: a serial scan is a few hundred cycles
-        int a = 0, p = 0;
-        for (int i = 0; i < E_loc; ++i) {
-            const int c = s_cnt[i], q = s_pad[i];
-            s_cnt[i] = a;
-            s_pad[i] = p;
-            a += c;
-            p += q;
-        }
-        s_cnt[E_loc] = a;
-        s_pad[E_loc] = p;
-        *m.num_m_tiles = p / TILE_M;
-    }
-    __syncthreads();
-    if (e < E_loc) {
+    for (int e = tid; e < E_loc; e += blockDim.x) {
+        const int total = s_cnt[e + 1] - s_cnt[e];
         m.expert_count[e] = total;
         m.expert_offset[e] = s_cnt[e];
         m.padded_offset[e] = s_pad[e];
@@ -118,50 +88,187 @@ __global__ void __launch_bounds__(P_MAX_LOCAL) scan_kernel(int nblk, int E_loc, 
             m.tile_rows[t0 + i] = min(TILE_M, total - i * TILE_M);
         }
     }
-    if (e == 0) {
+    if (tid == 0) {  // entries past E_loc count nothing, so entry E_loc already holds the totals
         m.expert_offset[E_loc] = s_cnt[E_loc];
         m.padded_offset[E_loc] = s_pad[E_loc];
     }
 }
 
-__global__ void __launch_bounds__(P_TOKENS_PER_BLOCK) place_kernel(int T, int E_loc, int off, int row_cap,
-                                                                   const int* topk_idx, PermuteMeta m,
-                                                                   int* __restrict__ status) {
+// Routing and everything of the permutation that needs all tokens, in one launch: one warp per token routes it, its
+// block counts the rows of every expert and the rank of each of its slots among them (bit w of mask[e]: the token of
+// warp w routes to local expert e; the popcount below a token's bit is its stable rank), and the block that finishes
+// last -- found with a ticket counter, nobody waits -- turns the blocks' counts into bases and builds the row tables.
+// What is left, one sum per slot, place_gather_kernel does where it copies the rows.  Bound by latency: the routing
+// of a token is a chain of about 2 us, so a block takes few tokens (8) while the blocks fit the SMs at once, and 32
+// where the counts of many blocks would make the last block's pass over them long.
+// This kernel and place_gather_kernel replaced five kernels (route, count, scan, place, gather; up to 512 tokens two, the
+// first of which placed all rows in its last block, equal in time): 23 us instead of 34 at 1024 tokens, 30 instead of
+// 39 at 4096, 305 instead of 359 at 16384 tokens with all experts local, where a row is now read once instead of
+// eight times (sums of the kernels' event times).
+// `ticket` must be zero at launch; the last block leaves it zero.
+constexpr int RC_SMALL_MAX_TOKENS = 1024;   // 128 blocks of 8 tokens; above, and with many local experts: 32 per block
+constexpr int RC_SMALL_MAX_LOCAL = 64;
+__host__ __device__ constexpr int route_count_tokens_per_block(int T, int E_loc) {
+    return T <= RC_SMALL_MAX_TOKENS && E_loc <= RC_SMALL_MAX_LOCAL ? 8 : 32;
+}
+template <int WARPS>
+__global__ void __launch_bounds__(WARPS * 32) route_count_kernel(
+    int T, int E_loc, int off, const float* __restrict__ logits, const __nv_bfloat16* __restrict__ bias, float scaling,
+    int* __restrict__ topk_idx, float* __restrict__ topk_w, PermuteMeta m, int* __restrict__ ticket,
+    int* __restrict__ status) {
     pdl_launch_dependents();
     pdl_wait();
-    __shared__ uint32_t mask[P_MAX_LOCAL][P_TOKENS_PER_BLOCK / 32];
-    build_block_masks(mask, T, E_loc, off, topk_idx);
-    const int t = blockIdx.x * P_TOKENS_PER_BLOCK + threadIdx.x;
-    if (t >= T) return;
-    const int word = threadIdx.x >> 5, bit = threadIdx.x & 31;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const int e = __ldcg(topk_idx + t * 8 + j) - off;
-        int prow = -1;
-        if (e >= 0 && e < E_loc) {
-            int rank = __popc(mask[e][word] & ((1u << bit) - 1u));
-            for (int w = 0; w < word; ++w) rank += __popc(mask[e][w]);
-            const int within = m.block_hist[blockIdx.x * E_loc + e] + rank;
-            prow = m.padded_offset[e] + within;
-            if (prow < 0 || prow >= row_cap) {
-                atomicExch(status, DEV_BAD_ROW);
-                prow = -1;
-            } else {
-                m.row_to_slot[m.expert_offset[e] + within] = t * 8 + j;
-                m.row_token[prow] = t;
+    constexpr int THREADS = WARPS * 32;
+    __shared__ uint32_t mask[P_MAX_LOCAL];
+    __shared__ int s_part[THREADS];
+    __shared__ int s_cnt[P_MAX_LOCAL + 1];
+    __shared__ int s_pad[P_MAX_LOCAL + 1];
+    __shared__ int s_last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (blockIdx.x == 0 && tid == 0) *status = DEV_OK;  // first kernel of a forward: clear the fault word
+    for (int e = tid; e < P_MAX_LOCAL; e += THREADS) mask[e] = 0u;
+    __syncthreads();
+    const int t = blockIdx.x * WARPS + warp;
+    int my_e = -1;
+    if (t < T) {
+        float bias_f[8];
+        load_bias8(bias, lane, bias_f);
+        int my_idx;
+        float my_w;
+        route_token(t, lane, logits, bias_f, scaling, my_idx, my_w);
+        if (lane < R_TOPK) {
+            topk_idx[static_cast<size_t>(t) * R_TOPK + lane] = my_idx;
+            topk_w[static_cast<size_t>(t) * R_TOPK + lane] = my_w;
+            const int e = my_idx - off;
+            if (e >= 0 && e < E_loc) {
+                my_e = e;
+                atomicOr(&mask[e], 1u << warp);
             }
         }
-        m.slot_to_row[t * 8 + j] = prow;
+    }
+    __syncthreads();
+    if (my_e >= 0)
+        m.slot_rank[static_cast<size_t>(t) * R_TOPK + lane] = static_cast<uint8_t>(__popc(mask[my_e] & ((1u << warp) - 1u)));
+    for (int e = tid; e < E_loc; e += THREADS) m.block_hist[static_cast<size_t>(blockIdx.x) * E_loc + e] = __popc(mask[e]);
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+        const int n = atomicAdd(ticket, 1);
+        s_last = (n == static_cast<int>(gridDim.x) - 1);
+        if (s_last) *ticket = 0;
+        // A counter that did not start at zero (somebody wrote into the workspace) would leave this forward
+        // without a last block and with stale tables: say so instead of returning them silently.
+        if (n < 0 || n >= static_cast<int>(gridDim.x)) {
+            atomicExch(status, DEV_BAD_TICKET);
+            *ticket = 0;
+        }
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+
+    // The counts of all blocks: thread (group q, expert e) sums a contiguous range of blocks, then replaces every
+    // count of its range by the number of rows of e in front of that block.
+    int ep = 1;
+    while (ep < E_loc) ep <<= 1;
+    const int nblk = static_cast<int>(gridDim.x);
+    const int groups = min(THREADS / ep, 32), per = (nblk + groups - 1) / groups;
+    const int e = tid & (ep - 1), q = tid / ep;
+    const bool mine = q < groups && e < E_loc;
+    const int b0 = min(nblk, q * per), b1 = min(nblk, b0 + per);
+    int sum = 0;
+    if (mine) {
+#pragma unroll 8
+        for (int b = b0; b < b1; ++b) sum += __ldcg(m.block_hist + static_cast<size_t>(b) * E_loc + e);
+    }
+    s_part[tid] = sum;
+    for (int i = tid; i < P_MAX_LOCAL; i += THREADS) s_cnt[i] = 0;
+    __syncthreads();
+    if (mine) {
+        int base = 0;
+        for (int i = 0; i < q; ++i) base += s_part[i * ep + e];
+        if (q == groups - 1) s_cnt[e] = base + sum;
+#pragma unroll 8
+        for (int b = b0; b < b1; ++b) {
+            int* h = m.block_hist + static_cast<size_t>(b) * E_loc + e;
+            const int c = __ldcg(h);
+            *h = base;
+            base += c;
+        }
+    }
+    scan_experts(E_loc, s_cnt, s_pad, m);
+}
+
+// One warp per token: the padded row of each of its local slots (base of its block inside the expert + rank inside the
+// block), the tables that depend on it, and the copy of the token's FP8 row (H bytes) and its H/128 scales to those
+// rows, read once and written up to eight times.  The scales are written transposed ([H/128, row_cap]) so the GEMM
+// epilogue reads them coalesced across the rows of a tile.  Rows past an expert's count are padding and are left
+// untouched (their results are never stored).  Bound by the writes: 7392 bytes per slot.
+__global__ void __launch_bounds__(256) place_gather_kernel(int T, int H, int E_loc, int off, int row_cap, int tokens_per_block,
+                                                           int scale_layout, const int* topk_idx,
+                                                           const uint8_t* __restrict__ hidden,
+                                                           const float* __restrict__ hidden_scale, PermuteMeta m,
+                                                           uint8_t* __restrict__ a1, float* __restrict__ a1_scale_t,
+                                                           int* __restrict__ status) {
+    pdl_launch_dependents();
+    const int lane = threadIdx.x & 31;
+    const int nwarps = gridDim.x * (blockDim.x >> 5);
+    const int chunks = H / 16, nkb = H / 128;
+    constexpr int BATCH = 7;  // 16-byte chunks of a row that a lane holds at a time (a row of 7168 bytes: two batches)
+    pdl_wait();
+    for (int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < T; t += nwarps) {
+        int prow = -1;
+        if (lane < R_TOPK) {
+            const int slot = t * R_TOPK + lane;
+            const int e = __ldcg(topk_idx + slot) - off;
+            if (e >= 0 && e < E_loc) {
+                const int within = __ldcg(m.block_hist + static_cast<size_t>(t / tokens_per_block) * E_loc + e) + __ldcg(m.slot_rank + slot);
+                prow = __ldcg(m.padded_offset + e) + within;
+                if (prow < 0 || prow >= row_cap) {
+                    atomicExch(status, DEV_BAD_ROW);
+                    prow = -1;
+                } else {
+                    m.row_to_slot[__ldcg(m.expert_offset + e) + within] = slot;
+                    m.row_token[prow] = t;
+                }
+            }
+            m.slot_to_row[slot] = prow;
+        }
+        const uint32_t local = __ballot_sync(0xffffffffu, prow >= 0);
+        if (local == 0) continue;
+        const uint4* src = reinterpret_cast<const uint4*>(hidden + static_cast<size_t>(t) * H);
+        for (int c0 = lane; c0 < chunks; c0 += 32 * BATCH) {
+            uint4 v[BATCH];
+#pragma unroll
+            for (int i = 0; i < BATCH; ++i)
+                if (c0 + i * 32 < chunks) v[i] = __ldg(src + c0 + i * 32);
+            for (uint32_t todo = local; todo; todo &= todo - 1) {
+                const int r = __shfl_sync(0xffffffffu, prow, __ffs(todo) - 1);
+                uint4* dst = reinterpret_cast<uint4*>(a1 + static_cast<size_t>(r) * H);
+#pragma unroll
+                for (int i = 0; i < BATCH; ++i)
+                    if (c0 + i * 32 < chunks) dst[c0 + i * 32] = v[i];
+            }
+        }
+        for (int kb = lane; kb < (nkb + 31) / 32 * 32; kb += 32) {
+            const float s = kb >= nkb ? 0.0f
+                            : scale_layout ? __ldg(hidden_scale + static_cast<size_t>(kb) * T + t)
+                                           : __ldg(hidden_scale + static_cast<size_t>(t) * nkb + kb);
+            for (uint32_t todo = local; todo; todo &= todo - 1) {
+                const int r = __shfl_sync(0xffffffffu, prow, __ffs(todo) - 1);
+                if (kb < nkb) a1_scale_t[static_cast<size_t>(kb) * row_cap + r] = s;
+            }
+        }
     }
 }
 
-// Batches up to P_TAIL_MAX_TOKENS: routing in parallel blocks (one warp per token), then the block that
+// In front of the fused small-batch kernel: routing in parallel blocks (one warp per token), then the block that
 // finishes last -- found with a ticket counter, nobody waits -- builds histogram, scan and placement for all
-// tokens on its own.  One launch instead of four; same arithmetic and outputs as route_topk_kernel +
-// count_kernel + scan_kernel + place_kernel.  `ticket` must be zero at launch; the last block leaves it zero
+// tokens on its own (the rows are gathered by the fused kernel).  Same arithmetic and outputs as
+// route_count_kernel + place_gather_kernel, plus the tables of sub-tiles.  `ticket` must be zero at launch; the last block leaves it zero
 // (moe_fp8_set_workspace zeroes it once, nothing else ever writes it).
 // Dynamic shared memory: E_loc * ceil(T/32) words of masks, then as many 16-bit prefix counts.
-constexpr int P_TAIL_MAX_TOKENS = 512;   // measured faster than the four kernels up to here, slower at 1024
+constexpr int P_TAIL_MAX_TOKENS = 256;   // the largest batch the fused kernel takes
 constexpr int P_TAIL_THREADS = 256;
 __host__ __device__ constexpr size_t route_permute_smem_bytes(int T, int E_loc) {
     return static_cast<size_t>(E_loc) * ((T + 31) / 32) * 6;
@@ -427,35 +534,6 @@ __device__ __forceinline__ void route_permute_in_cta(int* scratch, int T, int E_
         m.tok_nlocal[tid] = nlocal;
     }
     __syncthreads();
-}
-
-// One warp per padded row: copy the token's FP8 row (K bytes) and write its
-// K/128 scales transposed ([K/128, row_cap]) so the GEMM epilogue reads them
-// coalesced across the rows of a tile.  Rows past an expert's count are padding
-// and are left untouched (their results are never stored).
-__global__ void __launch_bounds__(256) gather_rows_kernel(int H, int row_cap, int scale_layout, int T,
-                                                          const uint8_t* __restrict__ hidden,
-                                                          const float* __restrict__ hidden_scale, PermuteMeta m,
-                                                          uint8_t* __restrict__ a1, float* __restrict__ a1_scale_t) {
-    pdl_launch_dependents();
-    pdl_wait();
-    const int lane = threadIdx.x & 31;
-    const int warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int nwarps = gridDim.x * (blockDim.x >> 5);
-    const int rows = *m.num_m_tiles * TILE_M;
-    const int chunks = H / 16, nkb = H / 128;
-    for (int r = warp; r < rows; r += nwarps) {
-        if ((r % TILE_M) >= m.tile_rows[r / TILE_M]) continue;
-        const int t = m.row_token[r];
-        const uint4* src = reinterpret_cast<const uint4*>(hidden + static_cast<size_t>(t) * H);
-        uint4* dst = reinterpret_cast<uint4*>(a1 + static_cast<size_t>(r) * H);
-        for (int c = lane; c < chunks; c += 32) dst[c] = __ldg(src + c);
-        for (int kb = lane; kb < nkb; kb += 32) {
-            const float s = scale_layout ? hidden_scale[static_cast<size_t>(kb) * T + t]
-                                         : hidden_scale[static_cast<size_t>(t) * nkb + kb];
-            a1_scale_t[static_cast<size_t>(kb) * row_cap + r] = s;
-        }
-    }
 }
 
 }  // namespace moe

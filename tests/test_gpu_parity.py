@@ -407,6 +407,21 @@ def test_large_tile_kernels_with_few_k_blocks_per_tile(cuda_device, hidden, inte
     run_and_compare(wl, cuda_device, inp=inp, **kw)
 
 
+# ---- routing + counts + row tables in one launch, placement in the gather: block sizes and group splits ---------
+@pytest.mark.parametrize("tokens,eloc,off", [(1, 32, 0), (7, 1, 3), (9, 64, 64), (129, 65, 20), (1023, 64, 0), (1024, 3, 5),
+                                             (1025, 32, 32), (1025, 200, 56), (4999, 17, 0), (8193, 256, 0)])
+def test_permutation_at_the_edges_of_its_blocks(cuda_device, tokens, eloc, off):
+    # blocks of 8 tokens (up to 1024 tokens and 64 local experts) and of 32, the last block ragged; local expert
+    # counts on both sides of a power of two split the last block's threads into 1 to 32 groups
+    dims = dataclasses.replace(syn.LayerDims(hidden=256, intermediate=128), num_local_experts=eloc)
+    wl = _wl(tokens, dims, seed=40 + tokens, local_expert_offset=off)
+    eng = make_engine(wl, cuda_device)
+    eng.set_small_batch_fusion(False)
+    run_and_compare(wl, cuda_device, eng=eng, sample_tokens=_sample(tokens, 64, tokens))
+    assert eng.last_launch_count() == 5
+    eng.close()
+
+
 # ---- batches of at most 80 tokens: gather, both GEMMs and the combine as one kernel; up to 16 tokens that ----
 # ---- kernel also routes and permutes (every CTA for itself), and the forward is a single launch -------------
 @pytest.mark.parametrize("tokens,kw", [(1, {}), (5, {}), (12, {}), (13, {}), (16, {"local_expert_offset": 64}),
