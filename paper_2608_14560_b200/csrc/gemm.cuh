@@ -30,7 +30,7 @@
 // scaling cannot express them; the per-K-block promotion is done on the ALUs.
 //
 // Two kernels are built from these roles:
-//   grouped_gemm_kernel<MODE>   one GEMM per launch (any batch size);
+//   grouped_mlp_kernel (grouped_mlp.cuh)   both GEMMs, the tiles of GEMM1 in front of those of GEMM2 (any batch size);
 //   fused_small_kernel          small batches (the host decides up to which size): the gather of stage 2, GEMM1, GEMM2
 //               and the weighted combine of stage 4 in ONE launch, with the operands swapped (weights on the
 //               M side of the MMA, the tile's at most 32 token rows on the N side; see "weights on M" below).
@@ -70,18 +70,19 @@ constexpr int G_THREADS = 384;                          // 4 control warps + 8 e
 constexpr int G_EPI_WARPS = 8;
 constexpr int G_STORE_WARP_BYTES = 2048;                // per-warp staging: 32 rows x 64 B (swizzled)
 constexpr int G_AMAX_BYTES = 2 * 2 * TILE_M * 4;               // GEMM1 row-amax exchange
-constexpr int G_CTRL_BYTES = 512;
+constexpr int G_CTRL_BYTES = 768;
 constexpr uint32_t G_TMEM_COLS = 512;
-// Large-tile kernels: named barrier ACC_BARRIER + b hands accumulator buffer b from the epilogue warps (which
+// grouped_mlp_kernel: named barrier ACC_BARRIER + b hands accumulator buffer b from the epilogue warps (which
 // arrive) back to its issuer warp (which waits).
 constexpr int ACC_BARRIER = 1;
 constexpr int ACC_BARRIER_THREADS = (G_EPI_WARPS + 1) * 32;
 
-// Scales on their way to the factor warp of the large-tile kernels, in K-blocks and ring slots of 128 activation and 2
-// weight scales.
+// Scales on their way to the factor warp of grouped_mlp_kernel: the 128 activation scales of F_AHEAD K-blocks, and the
+// weight scales, two per K-block, in runs of up to 32 K-blocks of a tile.
 constexpr int F_AHEAD = 4;
 constexpr int F_SLOTS = 8;
-constexpr int F_SLOT_FLOATS = TILE_M + 4;
+constexpr int F_RUN = 32;
+constexpr int F_RAW_FLOATS = F_SLOTS * TILE_M + F_SLOTS * F_RUN * 2;
 
 // Shared-memory geometry of a kernel: pipeline stages, rows of the A tile that are actually fetched (the MMA
 // always reads 128 rows; with fewer fetched rows the rest of its A operand is whatever follows in shared
@@ -95,7 +96,7 @@ struct Geometry {
     static constexpr int SCALE_BYTES = A_ROWS_ * 4;                  // per K-block
     // a slot: the activation scales of a K-block, or (large-tile kernels) their products with two weight scales
     static constexpr int SLOT_BYTES = FACTORS_ ? 2 * SCALE_BYTES : SCALE_BYTES;
-    static constexpr int RAW_BYTES = FACTORS_ ? F_SLOTS * F_SLOT_FLOATS * 4 : 0;
+    static constexpr int RAW_BYTES = FACTORS_ ? F_RAW_FLOATS * 4 : 0;
     static constexpr int STORE_BYTES = STORE_BYTES_;                 // GEMM1 output staging
     static constexpr int SMEM_BYTES = STAGES_ * STAGE_BYTES + SCALE_SLOTS_ * SLOT_BYTES + STORE_BYTES_ + G_AMAX_BYTES +
                                       G_CTRL_BYTES + RAW_BYTES + 1024;   // + alignment slack
@@ -105,7 +106,7 @@ struct Geometry {
     static_assert(SCALE_SLOTS_ >= STAGES_ + G_ACC_BUFS + 1, "the producer may be that far ahead of the epilogue");
     static_assert(SMEM_BYTES <= 232448, "exceeds the 227 KB of shared memory a CTA may use");
 };
-// one GEMM per launch: full 128-row A tiles, 4 stages of 48 KB
+// grouped_mlp_kernel: full 128-row A tiles, 4 stages of 48 KB
 using GeomFull = Geometry<4, TILE_M, 8, G_EPI_WARPS * G_STORE_WARP_BYTES, true>;
 // fused small-batch kernel: a row tile holds at most 32 token rows, so their slot shrinks to 4 KB and six
 // stages fit: 192 KB of weights in flight per SM instead of 128 KB, which is what a weight-streaming CTA is
@@ -146,7 +147,7 @@ struct GemmArgs {
     const int* tile_expert;
     const int* tile_rows;
     const int* tile_row0;     // fused kernel: first padded row of each (sub-)tile; else null: tile * TILE_M
-    int wm_rows;              // large-tile kernel: row tiles with at most this many rows (0 or 32) run with the
+    int wm_rows;              // grouped_mlp_kernel: row tiles with at most this many rows (0 or 32) run with the
                               // weights on the M side of the MMAs, see epilogue_tile_wm
     const float* a_scale_t;   // [num_kb, row_cap]
     const float* w_scale;     // [E_loc, w_rows/128, num_kb]
@@ -191,6 +192,18 @@ constexpr int SPLIT_MAX_TILES = 74;                       // a split needs at le
 constexpr int SPLIT_RAW_FLOATS = 2 * SPLIT_MAX_TOKENS * 128;  // per tile and K-block
 constexpr int SPLIT_MAX_KB = 64;                          // K-blocks of a GEMM whose tiles may be split
 
+// A tile of grouped_mlp_kernel's work list.
+struct __align__(16) TileInfo {
+    int key;      // row tile * 16 + flags + mode; mode 1: GEMM1, 2: GEMM2, 0: the list has ended
+    int n;        // column tile
+    int rows;     // valid rows of the row tile
+    int expert;
+    static constexpr int LAST = 4, LAST_TWO = 8;  // GEMM1: the last one / one of the last two of a list
+    __device__ __forceinline__ int mode() const { return key & 3; }
+    __device__ __forceinline__ int m_tile() const { return key >> 4; }
+};
+constexpr int SCHED_SLOTS = 16;
+
 struct GemmCtrl {
     uint64_t full[G_MAX_STAGES];   // stage filled (TMA transaction bytes)
     uint64_t done[G_MAX_STAGES];   // the MMAs that read the stage have finished: stage free AND accumulator ready
@@ -201,6 +214,9 @@ struct GemmCtrl {
     uint32_t tmem_slot;
     int abort_flag;
     int split_last;            // fused kernel, K split: this CTA stored the last part of the tile
+    uint64_t sched_full[SCHED_SLOTS];   // grouped_mlp_kernel: the work list, published tile by tile
+    uint64_t sched_rows[SCHED_SLOTS];   // the tile's token rows are in memory
+    TileInfo sched[SCHED_SLOTS];
 };
 static_assert(sizeof(GemmCtrl) <= G_CTRL_BYTES, "control block too large");
 
@@ -274,6 +290,10 @@ __device__ __forceinline__ void gemm_cta_setup(Cta& c, uint8_t* smem_raw, int fu
         mbar_init(smem_u32(&ctrl->drain_bar[1]), 1);
         mbar_init(smem_u32(&ctrl->sync_bar[0]), G_EPI_WARPS * 32);
         mbar_init(smem_u32(&ctrl->sync_bar[1]), G_EPI_WARPS * 32);
+        for (int i = 0; i < SCHED_SLOTS; ++i) {
+            mbar_init(smem_u32(&ctrl->sched_full[i]), 2);
+            mbar_init(smem_u32(&ctrl->sched_rows[i]), 1);
+        }
         ctrl->abort_flag = 0;
         mbar_fence_init();
     }
@@ -283,35 +303,23 @@ __device__ __forceinline__ void gemm_cta_setup(Cta& c, uint8_t* smem_raw, int fu
     }
 }
 
-// ---------------- TMA producer (one thread) ----------------
-// One copy for the token rows and two for the 256 weight rows of a K-block: a copy instruction costs this thread
-// about 85 clocks, which is part of the time a stage needs to be refilled (500 clocks with the weight rows as four
-// copies and the scales as another one); boxes of 256 rows move at 52 bytes per clock and SM out of L2, boxes of 128
-// rows at 67 (measured with a loads-only kernel).
-// tmB: weight rows in the order of the MMAs' N side -- MODE 1 gate[0,64) | up[0,64) | gate[64,128) | up[64,128) of
-// the tile's 128 columns, MODE 2 256 consecutive rows; tmBm (MODE 1): in the order of the M side, gate[0,128) |
-// up[0,128), for short row tiles and the fused kernel.  ("gate" and "up" change places with gate_first = 0.)
-// FUSED and MODE 1: the token rows and the scales come from the gather warp instead; FUSED and MODE 2: the tile's
-// token rows are GEMM1's output and must have been stored.
-template <int MODE, bool FUSED, class GEO>
+// ---------------- TMA producer (fused kernel, one thread) ----------------
+// tmB: boxes of 128 weight rows of [expert][half][row][K]; MODE 1 takes gate[0,128) | up[0,128) of the tile's 128 columns ("gate" and "up"
+// change places with gate_first = 0), MODE 2 256 consecutive rows.  MODE 1: the token rows and the scales come from
+// the gather warp instead; MODE 2: the tile's token rows are GEMM1's output and must have been stored.
+template <int MODE, class GEO>
 __device__ __forceinline__ void producer_tiles(const Cta& c, const CUtensorMap* tmA, const CUtensorMap* tmB,
                                                const GemmArgs& g, const FusedArgs* f, int ready_target, TileRange tr,
-                                               uint32_t& it, bool& ok, const CUtensorMap* tmA_short = nullptr,
-                                               const CUtensorMap* tmBm = nullptr, KSplit ks = KSplit{1, 1 << 30}) {
+                                               uint32_t& it, bool& ok, KSplit ks) {
     GemmCtrl* ctrl = c.ctrl;
     for (int item = tr.first; item < tr.count && ok; item += tr.stride) {
         const int tile = item / ks.parts, kb0 = (item - tile * ks.parts) * ks.len;
         const int kb1 = min(g.num_kb, kb0 + ks.len);
         const int m_tile = tile / g.n_tiles, n = tile - m_tile * g.n_tiles;
-        const int e = __ldcg(g.tile_expert + m_tile);
-        const int row0 = FUSED ? __ldcg(g.tile_row0 + m_tile) : m_tile * TILE_M;
+        const int e = __ldcg(g.tile_expert + m_tile), wrow = n * (MODE == 1 ? 128 : G_TILE_N);
+        const int row0 = __ldcg(g.tile_row0 + m_tile);
         const float* a_sc = g.a_scale_t + row0;
-        // a short row tile of the large-tile kernel: 32 token rows fetched, weights laid out for the M side
-        const bool wm = !FUSED && g.wm_rows > 0 && __ldcg(g.tile_rows + m_tile) <= g.wm_rows;
-        const CUtensorMap* tA = wm ? tmA_short : tmA;
-        const uint32_t TX_BYTES = (FUSED && MODE == 1) ? G_B_BYTES
-                                  : FUSED ? GEO::STAGE_BYTES + GEO::SCALE_BYTES
-                                          : wm ? WM_TOKENS * G_BLOCK_K + G_B_BYTES : GEO::STAGE_BYTES;
+        const uint32_t TX_BYTES = MODE == 1 ? G_B_BYTES : GEO::STAGE_BYTES + GEO::SCALE_BYTES;
         // claim the stage of pipeline iteration j: wait until its last reader has finished, announce the bytes
         auto claim = [&](uint32_t j) -> bool {
             const uint32_t s = j % GEO::STAGES, ph = (j / GEO::STAGES) & 1;
@@ -326,27 +334,19 @@ __device__ __forceinline__ void producer_tiles(const Cta& c, const CUtensorMap* 
         auto load_b = [&](uint32_t j, int kb) {
             const uint32_t s = j % GEO::STAGES, bar = smem_u32(&ctrl->full[s]);
             const uint32_t b_dst = c.smem_base + s * GEO::STAGE_BYTES + GEO::A_BYTES;
-            const int k0 = kb * G_BLOCK_K;
-            const int br = e * g.w_rows_per_expert + n * (MODE == 1 ? 128 : G_TILE_N);
-            if (MODE == 2 || FUSED || wm) {
-                tma_load_2d(b_dst, MODE == 2 ? tmB : tmBm, k0, br, bar);
-                tma_load_2d(b_dst + G_B_BYTES / 2, MODE == 2 ? tmB : tmBm, k0, br + (MODE == 1 ? g.up_row0 : 128), bar);
-            } else {
-                tma_load_4d(b_dst, tmB, k0, n * 128, 0, e, bar);
-                tma_load_4d(b_dst + G_B_BYTES / 2, tmB, k0, n * 128 + 64, 0, e, bar);
-            }
+            tma_load_4d(b_dst, tmB, kb * G_BLOCK_K, wrow, 0, e, bar);
+            tma_load_4d(b_dst + G_B_BYTES / 2, tmB, kb * G_BLOCK_K, MODE == 1 ? wrow : wrow + 128, MODE == 1 ? 1 : 0, e, bar);
         };
-        auto load_a = [&](uint32_t j, int kb) {  // the A rows (fused kernel: and their scales) of the K-block
+        auto load_a = [&](uint32_t j, int kb) {  // the A rows and their scales of the K-block
             const uint32_t s = j % GEO::STAGES, bar = smem_u32(&ctrl->full[s]);
             // (the scale slot is free: the ring exceeds the stages + accumulators the producer can be ahead
             // of the epilogue)
-            if (FUSED)
-                bulk_load_1d(smem_u32(c.scale_ring + (j % GEO::SCALE_SLOTS) * GEO::A_ROWS),
-                             a_sc + static_cast<size_t>(kb) * g.row_cap, GEO::SCALE_BYTES, bar);
-            tma_load_2d(c.smem_base + s * GEO::STAGE_BYTES, tA, kb * G_BLOCK_K, row0, bar);
+            bulk_load_1d(smem_u32(c.scale_ring + (j % GEO::SCALE_SLOTS) * GEO::A_ROWS),
+                         a_sc + static_cast<size_t>(kb) * g.row_cap, GEO::SCALE_BYTES, bar);
+            tma_load_2d(c.smem_base + s * GEO::STAGE_BYTES, tmA, kb * G_BLOCK_K, row0, bar);
         };
         int kb = kb0;
-        if (FUSED && MODE == 2) {
+        if (MODE == 2) {
             // The tile's A rows are GEMM1's output and must have been stored; its weights need not wait for
             // that, so the B tiles of the first K-blocks go out before the counter is looked at.
             const int npre = kb1 - kb0 < GEO::STAGES ? kb1 - kb0 : GEO::STAGES;
@@ -368,8 +368,8 @@ __device__ __forceinline__ void producer_tiles(const Cta& c, const CUtensorMap* 
         for (; kb < kb1 && ok; ++kb, ++it) {
             ok = claim(it);
             if (!ok) break;
-            load_b(it, kb);  // (first: it may have to come from HBM, the token rows are in L2)
-            if (!(FUSED && MODE == 1)) load_a(it, kb);
+            load_b(it, kb);
+            if (MODE == 2) load_a(it, kb);
         }
     }
 }
@@ -387,62 +387,6 @@ __device__ __forceinline__ void producer_drain(const Cta& c, int* status, uint32
             atomicCAS(status, DEV_OK, DEV_TIMEOUT_DRAIN);
 }
 
-// ---------------- MMA issuers (two threads) ----------------
-// Two threads share the issue work: `mine` = 0 takes the even K-blocks (TMEM buffer 0), 1 the odd ones (buffer
-// 1).  A commit only tracks the MMAs of its own thread, so while one thread pays for its commit and waits the
-// other keeps the tensor pipe fed.
-// An accumulator buffer comes back through a named barrier that the eight epilogue warps arrive at and the issuer
-// warp waits on, once per K-block (see ACC_BARRIER): the hand-over is part of the loop that bounds the kernel, and
-// it is 80 clocks shorter than through an mbarrier.  Such a wait has no limit of its own, so no role may ever miss
-// its turn: after an abort the issuers and the epilogue warps go on to the end of the work list with the barriers
-// alone (the waits on mbarriers stay bounded).
-template <class GEO>
-__device__ __forceinline__ void issuer_tiles(const Cta& c, const GemmArgs& g, TileRange tr, uint32_t mine,
-                                             uint32_t& it, bool& ok) {
-    GemmCtrl* ctrl = c.ctrl;
-    const uint32_t idesc = umma_idesc_f8(TILE_M, G_TILE_N), idesc_wm = umma_idesc_f8(TILE_M, WM_TOKENS);
-    for (int tile = tr.first; tile < tr.count; tile += tr.stride) {
-        // a short row tile: the stage's weight rows are the M side (two blocks of 128), its 32 token rows the N
-        // side; the accumulator is the first 64 columns of the buffer
-        const bool wm = g.wm_rows > 0 && __ldcg(g.tile_rows + tile / g.n_tiles) <= g.wm_rows;
-        for (int kb = 0; kb < g.num_kb; ++kb, ++it) {
-            if ((it & 1) != mine) continue;
-            const uint32_t s = it % GEO::STAGES, ph = (it / GEO::STAGES) & 1;
-            // The stage has normally landed long before the accumulator is handed back, so that
-            // wait comes first and only the hand-over itself is left on the critical path.
-            const uint32_t a_addr = c.smem_base + s * GEO::STAGE_BYTES;
-            const uint64_t a_desc = umma_desc_sw128(a_addr);  // 128 rows from here, fetched or not
-            const uint64_t b_desc = umma_desc_sw128(a_addr + GEO::A_BYTES);
-            const uint32_t d_tmem = c.tmem_base + mine * G_TILE_N;
-            if (ok) {
-                if (c.lane == 0) ok = mbar_wait(smem_u32(&ctrl->full[s]), ph, c.abort_flag, c.limit);
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                if (!ok && c.lane == 0) raise(ctrl, g.status, DEV_TIMEOUT_MMA_SMEM);
-            }
-            if (it >= G_ACC_BUFS) bar_sync(ACC_BARRIER + mine, ACC_BARRIER_THREADS);
-            if (!ok) continue;
-            tc_fence_after();
-            if (c.lane == 0) {
-                if (wm) {
-                    const uint64_t w1_desc = umma_desc_sw128(a_addr + GEO::A_BYTES + G_B_BYTES / 2);
-#pragma unroll
-                    for (int k = 0; k < G_BLOCK_K / 32; ++k) umma_f8(d_tmem, b_desc + 2 * k, a_desc + 2 * k, idesc_wm, k > 0);
-#pragma unroll
-                    for (int k = 0; k < G_BLOCK_K / 32; ++k)
-                        umma_f8(d_tmem + WM_TOKENS, w1_desc + 2 * k, a_desc + 2 * k, idesc_wm, k > 0);
-                } else {
-#pragma unroll
-                    for (int k = 0; k < G_BLOCK_K / 32; ++k)  // 32 K-bytes per instruction: +2 in 16-B units
-                        umma_f8(d_tmem, a_desc + 2 * k, b_desc + 2 * k, idesc, k > 0);
-                }
-                umma_commit(smem_u32(&ctrl->done[s]));
-            }
-            __syncwarp();
-        }
-    }
-    if (it > mine) bar_sync(ACC_BARRIER + mine, ACC_BARRIER_THREADS);  // the buffer's last hand-over
-}
-
 // After an abort: let issued MMAs retire before TMEM is released.
 __device__ __forceinline__ void issuer_drain(const Cta& c, uint32_t mine, bool ok) {
     if (!ok || *c.abort_flag) {
@@ -450,75 +394,6 @@ __device__ __forceinline__ void issuer_drain(const Cta& c, uint32_t mine, bool o
         int zero = 0;
         mbar_wait(smem_u32(&c.ctrl->drain_bar[mine]), 0, &zero, c.limit);
     }
-}
-
-// ---------------- factor warp (large-tile kernels) ----------------
-// Multiplies the activation scales of every K-block with the two weight scales of the tile's 256 columns, so that
-// an epilogue thread finds its factor with one shared-memory load: [slot][2][row].  With the weight scales fetched
-// from global memory by the epilogue threads themselves, and the products formed there, an epilogue warp spent
-// about 500 of its 1240 clocks per K-block between handing a buffer back and being ready for the next one.  The
-// warp's arrival is the second one on done[s]: whoever sees that barrier finds the factors complete.  Like the
-// producer it claims a stage by waiting for the previous phase of done[s]; the slot it then writes was read by the
-// epilogue eight K-blocks ago (done of four K-blocks ago implies that the accumulator of six ago was handed back).
-// The scales come in F_AHEAD K-blocks ahead, across the ends of tiles: with loads that started anew at every tile the
-// warp's first arrival was late by the latency of three dependent loads, 3 % of a batch of 257 tokens.
-template <int MODE, class GEO>
-__device__ __forceinline__ void factor_tiles(const Cta& c, const GemmArgs& g, TileRange tr) {
-    static_assert(GEO::FACTORS && GEO::A_ROWS == 128, "a lane looks after four rows");
-    static_assert(GEO::SCALE_SLOTS >= GEO::STAGES + G_ACC_BUFS + 1, "slots still read by the epilogue");
-    static_assert(F_AHEAD < F_SLOTS, "a slot is refilled after it was read");
-    GemmCtrl* ctrl = c.ctrl;
-    const int lane = c.lane, num_kb = g.num_kb;
-    // the fetch cursor: tile, K-block, and this lane's sources there; the expert of the tile after it is known early
-    int ftile = tr.first, fkb = 0;
-    int e_next = ftile < tr.count ? __ldcg(g.tile_expert + ftile / g.n_tiles) : 0;
-    const float* as = nullptr;
-    const float* ws = nullptr;
-    uint32_t fit = 0;
-    auto fetch = [&]() {
-        if (ftile < tr.count) {
-            if (fkb == 0) {
-                const int m_tile = ftile / g.n_tiles, n = ftile - m_tile * g.n_tiles;
-                as = g.a_scale_t + static_cast<size_t>(m_tile) * TILE_M + lane * 4;
-                const int block = MODE == 1 ? n + lane * (g.up_row0 / 128) : 2 * n + lane;  // (lanes 0 and 1)
-                ws = g.w_scale + (static_cast<size_t>(e_next) * (g.w_rows_per_expert / 128) + block) * num_kb;
-                if (ftile + tr.stride < tr.count) e_next = __ldcg(g.tile_expert + (ftile + tr.stride) / g.n_tiles);
-            }
-            float* raw = c.raw_scales + (fit % F_SLOTS) * F_SLOT_FLOATS;
-            cp_async_16(smem_u32(raw + lane * 4), as, 16);
-            if (lane < 2) cp_async_4(smem_u32(raw + TILE_M + lane), ws, 4);
-            as += g.row_cap;
-            ++ws;
-            if (++fkb == num_kb) {
-                fkb = 0;
-                ftile += tr.stride;
-            }
-        }
-        ++fit;
-        cp_async_commit();
-    };
-    for (int i = 0; i < F_AHEAD; ++i) fetch();
-    uint32_t it = 0;
-    for (int tile = tr.first; tile < tr.count; tile += tr.stride)
-        for (int kb = 0; kb < num_kb; ++kb, ++it) {
-            const uint32_t s = it % GEO::STAGES;
-            cp_async_wait<F_AHEAD - 1>();
-            __syncwarp();
-            const float* raw = c.raw_scales + (it % F_SLOTS) * F_SLOT_FLOATS;
-            const float4 a = *reinterpret_cast<const float4*>(raw + lane * 4);
-            const float2 w = *reinterpret_cast<const float2*>(raw + TILE_M);
-            fetch();
-            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctrl->done[s]), ((it / GEO::STAGES) & 1) ^ 1, c.abort_flag, c.limit))) {
-                if (lane == 0) raise(ctrl, g.status, DEV_TIMEOUT_PRODUCER);
-                cp_async_wait_all();  // nothing may still be landing in shared memory when the CTA exits
-                return;
-            }
-            float* dst = c.scale_ring + (it % GEO::SCALE_SLOTS) * 2 * GEO::A_ROWS + lane * 4;
-            *reinterpret_cast<float4*>(dst) = make_float4(a.x * w.x, a.y * w.x, a.z * w.x, a.w * w.x);
-            *reinterpret_cast<float4*>(dst + GEO::A_ROWS) = make_float4(a.x * w.y, a.y * w.y, a.z * w.y, a.w * w.y);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&ctrl->done[s]));
-        }
 }
 
 // ---------------- gather warp (fused kernel) ----------------
@@ -602,175 +477,6 @@ __device__ __forceinline__ bool epilogue_rendezvous(const Cta& c, uint32_t& n) {
     return ok;
 }
 
-template <int MODE, bool FUSED, class GEO, bool SHARED, bool SPLIT = false>
-__device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g, const FusedArgs* f, int m_tile, int n,
-                                                 uint32_t& it, uint32_t& tile_iter, uint32_t& sync_iter, int kb0 = 0,
-                                                 int kb1 = -1, int parts = 1);
-
-// acc[0..64) += v * f with packed fp32 FMAs: one instruction, two independent round-to-nearest FMAs, the bits of the
-// scalar form.  Beside scalar FMAs the MMA issuers, which share the schedulers with the epilogue warps, needed 955
-// clocks per K-block in a probe of this loop, beside packed ones 672 (602 beside an epilogue without FMAs).
-__device__ __forceinline__ void fma64(float* acc, const float (&v)[64], float f) {
-    const uint64_t p = pack_f32x2(__float_as_uint(f), __float_as_uint(f));
-#pragma unroll
-    for (int j = 0; j < 64; j += 2) {
-        const uint64_t a = fma_f32x2(pack_f32x2(__float_as_uint(v[j]), __float_as_uint(v[j + 1])), p,
-                                     pack_f32x2(__float_as_uint(acc[j]), __float_as_uint(acc[j + 1])));
-        acc[j] = __uint_as_float(static_cast<uint32_t>(a));
-        acc[j + 1] = __uint_as_float(static_cast<uint32_t>(a >> 32));
-    }
-}
-
-// ---------------- epilogue warps ----------------
-// MODE 1: gate/up projection + SwiGLU + re-quantisation; tmOut describes the e4m3 output [row_cap, I] for
-//         64-byte x 32-row TMA stores.
-// MODE 2: down projection, bf16 rows out in the tile-blocked layout.
-template <int MODE, class GEO>
-__device__ __forceinline__ void epilogue_tiles(const Cta& c, const CUtensorMap* tmOut, const GemmArgs& g, TileRange tr,
-                                               uint32_t& it, uint32_t& tile_iter, bool& ok) {
-    static_assert(GEO::A_ROWS == TILE_M && GEO::STORE_BYTES == G_EPI_WARPS * G_STORE_WARP_BYTES, "full row tiles");
-    GemmCtrl* ctrl = c.ctrl;
-    const int warp = c.warp, lane = c.lane;
-    const int widx = warp - 4;
-    const int half = widx >> 2;              // which 128-column half of the tile
-    const int quad = warp & 3;               // TMEM lane quadrant this warp may read
-    const int r_in_tile = quad * 32 + lane;  // accumulator row == TMEM lane
-    const uint32_t t_lane = c.tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + half * G_HALF_N;
-    const size_t row_cap = static_cast<size_t>(g.row_cap);
-    float* amax_x = c.amax_x;
-    uint8_t* stage = c.store_stage + widx * G_STORE_WARP_BYTES;  // staging of this warp's GEMM1 rows
-    const int num_kb = g.num_kb;
-    for (int tile = tr.first; tile < tr.count && ok; tile += tr.stride) {
-        const int m_tile = tile / g.n_tiles, n = tile - m_tile * g.n_tiles;
-        const int rows_valid = __ldcg(g.tile_rows + m_tile);
-        if (g.wm_rows > 0 && rows_valid <= g.wm_rows) {  // a short row tile, worked on with the weights on M
-            uint32_t unused = 0;
-            ok = epilogue_tile_wm<MODE, false, GEO, true>(c, g, nullptr, m_tile, n, it, tile_iter, unused);
-            continue;
-        }
-        const size_t row = static_cast<size_t>(m_tile) * TILE_M + r_in_tile;
-        float acc[128];
-#pragma unroll
-        for (int j = 0; j < 128; ++j) acc[j] = 0.0f;
-
-        for (int kb = 0; kb < num_kb; ++kb, ++it) {
-            const uint32_t s = it % GEO::STAGES, ph = (it / GEO::STAGES) & 1, buf = it & 1;
-            // Every lane polls (a single polling lane plus a broadcast was measured 2.5 % slower); the vote
-            // keeps the warp converged when a wait gives up: either all lanes go on or none does.
-            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctrl->done[s]), ph, c.abort_flag, c.limit))) {
-                if (lane == 0) raise(ctrl, g.status, DEV_TIMEOUT_EPILOGUE);
-                ok = false;
-                break;
-            }
-            tc_fence_after();
-            // GEMM1: of this warpgroup's 128 columns, [0,64) are gate and [64,128) the matching up columns.
-            const uint32_t col = t_lane + buf * G_TILE_N;
-            float v[64];
-            tmem_ld32_issue(col, v);
-            tmem_ld32_issue(col + 32, v + 32);
-            // this row's factors for the columns [0,64) and [64,128) of the half (GEMM2: the same one)
-            const float* fr = c.scale_ring + (it % GEO::SCALE_SLOTS) * 2 * GEO::A_ROWS + r_in_tile;
-            const float f0 = ld_shared_f32(fr + (MODE == 1 ? 0 : half * GEO::A_ROWS));
-            const float f1 = MODE == 1 ? ld_shared_f32(fr + GEO::A_ROWS) : f0;
-            tmem_wait_ld(v);
-            fma64(acc, v, f0);
-            tmem_ld32_issue(col + 64, v);
-            tmem_ld32_issue(col + 96, v + 32);
-            tmem_wait_ld(v);
-            tc_fence_before();
-            bar_arrive(ACC_BARRIER + buf, ACC_BARRIER_THREADS);
-            fma64(acc + 64, v, f1);
-        }
-        if (!ok) break;
-
-        if (MODE == 1) {
-            // The staging area of this warp was handed to the TMA engine at the end of the previous tile;
-            // by now (a whole tile later) that copy has long read it, so this wait does not stall.
-            if (lane == 0) bulk_wait_read_all();
-            __syncwarp();
-            const int sw = (lane >> 1) & 3;  // 64-byte swizzle: 16-byte chunk index ^= bits 7..8 of the address
-            // SwiGLU on this thread's 64 columns, then the row's 128-wide amax across the two halves
-            float cc[64];
-            float amax = 0.0f;
-            if (g.up_first) {
-#pragma unroll
-                for (int j = 0; j < 64; ++j) {
-                    const float x = acc[j];
-                    acc[j] = acc[64 + j];
-                    acc[64 + j] = x;
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < 64; ++j) {
-                // silu(g) * u with the hardware exp2 and reciprocal approximations (a few ulp): the
-                // tile's tail runs while the tensor pipe idles, so its instruction count matters.
-                const float gt = acc[j];
-                cc[j] = __fdividef(gt, 1.0f + __expf(-gt)) * acc[64 + j];
-                amax = fmaxf(amax, fabsf(cc[j]));
-            }
-            const uint32_t par = tile_iter & 1;
-            amax_x[(par * 2 + half) * TILE_M + r_in_tile] = amax;
-            const uint32_t xbar = smem_u32(&ctrl->amax_bar[par]);
-            mbar_arrive(xbar);
-            if (!__all_sync(0xffffffffu, mbar_wait(xbar, (tile_iter >> 1) & 1, c.abort_flag, c.limit))) {
-                if (lane == 0) raise(ctrl, g.status, DEV_TIMEOUT_EPILOGUE);
-                ok = false;
-                break;
-            }
-            ++tile_iter;
-            amax = fmaxf(amax,
-                         *reinterpret_cast<volatile float*>(&amax_x[(par * 2 + (half ^ 1)) * TILE_M + r_in_tile]));
-            const float sc = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, 448.0f);
-            const float inv_sc = __frcp_rn(sc);
-            if (quad * 32 < rows_valid) {
-                // e4m3 rows out: 32 rows x 64 bytes per warp, staged with the 64-byte swizzle, one TMA store
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    uint32_t w[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int j = q * 16 + i * 4;
-                        const uint32_t lo = __nv_cvt_float2_to_fp8x2(
-                            make_float2(cc[j] * inv_sc, cc[j + 1] * inv_sc), __NV_SATFINITE, __NV_E4M3);
-                        const uint32_t hi = __nv_cvt_float2_to_fp8x2(
-                            make_float2(cc[j + 2] * inv_sc, cc[j + 3] * inv_sc), __NV_SATFINITE, __NV_E4M3);
-                        w[i] = lo | (hi << 16);
-                    }
-                    *reinterpret_cast<uint4*>(stage + lane * 64 + ((q ^ sw) << 4)) =
-                        make_uint4(w[0], w[1], w[2], w[3]);
-                }
-                fence_async_smem();
-                __syncwarp();
-                if (lane == 0) {
-                    tma_store_2d(tmOut, smem_u32(stage), n * 128 + half * 64, m_tile * TILE_M + quad * 32);
-                    bulk_commit_group();
-                }
-                if (half == 0 && r_in_tile < rows_valid)
-                    g.out_scale_t[static_cast<size_t>(n) * row_cap + row] = sc;
-            }
-        } else {
-            // bf16 rows out in a tile-blocked layout: block (row tile, column tile, half, quadrant) holds
-            // this warp's 32 rows x 128 columns as [8 column groups][32 rows][16 bf16], so every warp
-            // store instruction writes 1 KB of contiguous memory (32 bytes per lane).
-            if (quad * 32 < rows_valid) {
-                uint8_t* blk = reinterpret_cast<uint8_t*>(g.out_bf16) +
-                               (((static_cast<size_t>(m_tile) * g.n_tiles + n) * 2 + half) * 4 + quad) * 8192 +
-                               lane * 32;
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    uint32_t w[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const __nv_bfloat162 pr = __floats2bfloat162_rn(acc[q * 16 + 2 * i], acc[q * 16 + 2 * i + 1]);
-                        w[i] = *reinterpret_cast<const uint32_t*>(&pr);
-                    }
-                    st_global_v8(blk + q * 1024, w);
-                }
-            }
-        }
-    }
-}
-
 // ================= weights on M: the roles of the fused small-batch kernel =================
 // With at most 32 token rows in a tile, a 128 x 256 accumulator holds 96 rows of padding, and the two
 // epilogue warps that own the 32 real rows (TMEM lanes) do all of the per-K-block promotion.  Here the
@@ -821,6 +527,35 @@ __device__ __forceinline__ void issuer_tiles_wm(const Cta& c, const GemmArgs& g,
     }
 }
 
+// grouped_mlp_kernel: a warp's GEMM1 tiles whose stores have been issued.  GEMM2 tiles of other CTAs start once all warps
+// of all column tiles have announced theirs in `ready`.  Waiting for the stores right after they were issued would cost
+// the epilogue 1-2 us per tile, and the fence of an announcement about 400 clocks, so tiles are announced together: those
+// before in the tails of the last two tiles of a list, the last one behind it.
+struct Announce {
+    int* ready;       // [row tiles]; null: nobody waits (one GEMM per launch)
+    int n_tiles, stride;
+    int id, count;    // tiles id, id + stride, ... (row tile * n_tiles + column tile)
+    // The whole warp; the staging of the warp's last bulk store may be written again afterwards.
+    __device__ __forceinline__ void settle(int lane, bool announce) {
+        if (!announce || count == 0) {
+            if (lane == 0) bulk_wait_read_all();
+            __syncwarp();
+            return;
+        }
+        if (lane == 0) bulk_wait_all();  // stored, not only read
+        fence_proxy_async();
+        __syncwarp();
+        __threadfence();
+        for (int k = lane; k < count; k += 32) atomicAdd(ready + (id + k * stride) / n_tiles, 1);
+        count = 0;
+    }
+    __device__ __forceinline__ void add(int tile) {
+        if (ready == nullptr) return;
+        if (count == 0) id = tile;
+        ++count;
+    }
+};
+
 // MODE 1: weight-row block 0 = 128 gate rows, block 1 = the matching 128 up rows; SwiGLU, re-quantisation per
 //         token over the tile's 128 output columns, e4m3 bytes and scales out, tile announced in f->ready.
 // MODE 2: blocks 0 / 1 = output columns [0,128) / [128,256) of the tile; bf16 out in the tile-blocked layout,
@@ -834,10 +569,11 @@ __device__ __forceinline__ void issuer_tiles_wm(const Cta& c, const GemmArgs& g,
 // yet multiplied by the scales; the CTA that stores the last part of a tile -- found with a counter, nobody
 // waits -- then runs the whole promotion from the stored partial sums, K-block after K-block in the one order
 // the unsplit tile uses, and finishes the tile.  Every fp32 operation is the one of the unsplit tile.
-template <int MODE, bool FUSED, class GEO, bool SHARED, bool SPLIT>
+template <int MODE, bool FUSED, class GEO, bool SHARED, bool SPLIT = false>
 __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g, const FusedArgs* f, int m_tile, int n,
-                                                 uint32_t& it, uint32_t& tile_iter, uint32_t& sync_iter, int kb0, int kb1,
-                                                 int parts) {
+                                                 uint32_t& it, uint32_t& tile_iter, uint32_t& sync_iter, int kb0 = 0,
+                                                 int kb1 = -1, int parts = 1, Announce* announce = nullptr,
+                                                 bool settle = false) {
     static_assert(!SPLIT || FUSED, "only the fused kernel cuts K ranges");
     GemmCtrl* ctrl = c.ctrl;
     const int warp = c.warp, lane = c.lane;
@@ -1009,8 +745,7 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
     const size_t row0 = static_cast<size_t>(tile_row0) + th * 16;  // padded row of this thread's token 0
     const uint32_t wst_off = (warp - 4) * (SHARED ? G_STORE_WARP_BYTES : 512);  // this warp's staging
     if (SHARED) {  // the warp's last TMA store may still be reading the area
-        if (lane == 0) bulk_wait_read_all();
-        __syncwarp();
+        announce->settle(lane, settle);
     }
     const int valid = min(16, rows_valid - th * 16);                     // tokens of this thread that exist
     if (MODE == 1) {
@@ -1194,68 +929,6 @@ __device__ __forceinline__ void epilogue_tiles_wm(const Cta& c, const GemmArgs& 
     }
 }
 
-// One GEMM per launch.
-template <int MODE>
-__global__ void __launch_bounds__(G_THREADS, 1)
-grouped_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmAs,
-                    const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmBm,
-                    const __grid_constant__ CUtensorMap tmOut, const GemmArgs g) {
-    extern __shared__ uint8_t smem_raw[];
-    using GEO = GeomFull;
-    Cta c;
-    gemm_cta_setup<GEO>(c, smem_raw, 1);
-    if (c.warp == 0 && c.lane == 0) {
-        tma_prefetch_desc(&tmA);
-        tma_prefetch_desc(&tmAs);
-        tma_prefetch_desc(&tmB);
-        if (MODE == 1) {
-            tma_prefetch_desc(&tmBm);
-            tma_prefetch_desc(&tmOut);
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    // Everything above touched only this CTA's shared and tensor memory; the tile tables, activations and
-    // scales below were written by the kernels before this one.
-    pdl_launch_dependents();
-    pdl_wait();
-    c.tmem_base = *reinterpret_cast<volatile uint32_t*>(&c.ctrl->tmem_slot);
-    c.limit = g.wait_limit;
-    // (the tables come from the kernels before this one, which may still be resident: coherent loads)
-    const TileRange tr = {static_cast<int>(blockIdx.x), __ldcg(g.num_m_tiles) * g.n_tiles, static_cast<int>(gridDim.x)};
-    uint32_t it = 0;
-    bool ok = true;
-
-    if (c.warp < 4) {
-        reg_dealloc<40>();
-        if (c.warp == 0 && c.lane == 0) {
-            producer_tiles<MODE, false, GEO>(c, &tmA, &tmB, g, nullptr, 0, tr, it, ok, &tmAs, &tmBm);
-            producer_drain<GEO>(c, g.status, it);
-        } else if (c.warp == 1 || c.warp == 2) {
-            issuer_tiles<GEO>(c, g, tr, c.warp - 1, it, ok);
-            if (c.lane == 0) issuer_drain(c, c.warp - 1, ok);
-        } else if (c.warp == 3) {
-            factor_tiles<MODE, GEO>(c, g, tr);
-        }
-    } else {
-        reg_alloc<232>();
-        uint32_t tile_iter = 0;
-        epilogue_tiles<MODE, GEO>(c, &tmOut, g, tr, it, tile_iter, ok);
-        // After an abort: the hand-overs this warp still owes, waiting for the issuer so that no turn is taken twice.
-        const uint32_t total = (tr.first < tr.count ? (tr.count - tr.first + tr.stride - 1) / tr.stride : 0) * g.num_kb;
-        for (; it < total; ++it) bar_sync(ACC_BARRIER + (it & 1), ACC_BARRIER_THREADS);
-        if (c.lane == 0) bulk_wait_all();
-    }
-
-    tc_fence_before();
-    __syncthreads();
-    if (c.warp == 1) {
-        __syncwarp();
-        tmem_dealloc(c.tmem_base, G_TMEM_COLS);
-    }
-}
-
 // Gather + GEMM1 + GEMM2 + combine in one launch for small batches, at most F_MAX_TOKENS tokens (see the head of
 // this file).  tmA2 describes GEMM1's output buffer for loads (32-row boxes), tmB1 / tmB2 the two weight
 // tensors.
@@ -1315,8 +988,8 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmA2, const __grid_consta
     if (c.warp < 4) {
         reg_dealloc<40>();
         if (c.warp == 0 && c.lane == 0) {
-            producer_tiles<1, true, GEO>(c, &tmA2, nullptr, g1, &f, 0, tr1, it, ok, nullptr, &tmB1, ks1);
-            producer_tiles<2, true, GEO>(c, &tmA2, &tmB2, g2, &f, g1.n_tiles, tr2, it, ok, nullptr, nullptr, ks2);
+            producer_tiles<1, GEO>(c, &tmA2, &tmB1, g1, &f, 0, tr1, it, ok, ks1);
+            producer_tiles<2, GEO>(c, &tmA2, &tmB2, g2, &f, g1.n_tiles, tr2, it, ok, ks2);
             producer_drain<GEO>(c, g1.status, it);
         } else if ((c.warp == 1 || c.warp == 2) && c.lane == 0) {
             issuer_tiles_wm<GEO>(c, g1, tr1, c.warp - 1, it, ok, ks1);

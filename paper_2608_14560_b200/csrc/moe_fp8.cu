@@ -14,6 +14,7 @@
 #include "routing.cuh"
 #include "permute.cuh"
 #include "gemm.cuh"
+#include "grouped_mlp.cuh"
 #include "combine.cuh"
 #include "router.cuh"
 
@@ -30,7 +31,7 @@ inline size_t align_up(size_t x, size_t a = WS_ALIGN) { return (x + a - 1) / a *
 
 struct WsLayout {
     size_t topk_idx, topk_w, slot_rank, block_hist, expert_count, expert_offset, padded_offset, tile_expert, tile_rows,
-        num_m_tiles, slot_to_row, row_to_slot, row_token, tok_nlocal, st_expert, st_row0, st_rows, num_st, counters, num_counters, max_st, raw1, raw2, status, a1, a1_scale_t, a2, a2_scale_t, y, stage_hidden,
+        num_m_tiles, mlp_ready, mlp_claimed, slot_to_row, row_to_slot, row_token, tok_nlocal, st_expert, st_row0, st_rows, num_st, counters, num_counters, max_st, raw1, raw2, status, a1, a1_scale_t, a2, a2_scale_t, y, stage_hidden,
         stage_scale, stage_logits, stage_out, stage2_hidden, stage2_scale, stage2_logits, stage2_out, total;
     int row_cap, max_m_tiles, max_blocks;
 };
@@ -61,6 +62,8 @@ WsLayout make_layout(const moe_fp8_config& c) {
     L.tile_expert = take(static_cast<size_t>(L.max_m_tiles) * 4);
     L.tile_rows = take(static_cast<size_t>(L.max_m_tiles) * 4);
     L.num_m_tiles = take(4);
+    L.mlp_ready = take(static_cast<size_t>(L.max_m_tiles) * 4);
+    L.mlp_claimed = take(MLP_MAX_GRID * 4);
     L.slot_to_row = take(slots * 4);
     L.row_to_slot = take(slots * 4);
     L.row_token = take(rc * 4);
@@ -101,7 +104,7 @@ WsLayout make_layout(const moe_fp8_config& c) {
 
 }  // namespace
 
-constexpr int NUM_STAGES_MAX = 9;
+constexpr int NUM_STAGES_MAX = 10;
 
 struct moe_fp8_handle_s {
     moe_fp8_config cfg;
@@ -197,6 +200,9 @@ PermuteMeta meta_of(moe_fp8_handle_t h) {
     m.tile_expert = at<int>(h, h->L.tile_expert);
     m.tile_rows = at<int>(h, h->L.tile_rows);
     m.num_m_tiles = at<int>(h, h->L.num_m_tiles);
+    m.mlp_ready = at<int>(h, h->L.mlp_ready);
+    m.mlp_claimed = at<int>(h, h->L.mlp_claimed);
+    m.mlp_grid = std::min(h->sm_count, MLP_MAX_GRID);
     m.slot_to_row = at<int>(h, h->L.slot_to_row);
     m.row_to_slot = at<int>(h, h->L.row_to_slot);
     m.row_token = at<int>(h, h->L.row_token);
@@ -209,9 +215,9 @@ PermuteMeta meta_of(moe_fp8_handle_t h) {
 }
 
 constexpr int PDL_MAX_TOKENS = 2048;
-constexpr int NUM_STAGES = 9;
+constexpr int NUM_STAGES = 10;
 const char* const STAGE_NAMES[NUM_STAGES] = {"route_topk", "count", "scan", "place", "gather_rows",
-                                             "gemm1_swiglu_quant", "gemm2", "combine", "fused_small"};
+                                             "gemm1_swiglu_quant", "gemm2", "grouped_mlp", "combine", "fused_small"};
 
 bool misaligned(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) != 0; }
 
@@ -285,9 +291,7 @@ int moe_fp8_create(const moe_fp8_config* cfg, moe_fp8_handle_t* out) {
     e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q);
     if (e != cudaSuccess || q != cudaDriverEntryPointSuccess || !fn) return MOE_FP8_ERR_CUDA;
 
-    e = cudaFuncSetAttribute(grouped_gemm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, GeomFull::SMEM_BYTES);
-    if (e != cudaSuccess) return MOE_FP8_ERR_CUDA;
-    e = cudaFuncSetAttribute(grouped_gemm_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, GeomFull::SMEM_BYTES);
+    e = cudaFuncSetAttribute(grouped_mlp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GeomFull::SMEM_BYTES);
     if (e != cudaSuccess) return MOE_FP8_ERR_CUDA;
     e = cudaFuncSetAttribute(fused_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GeomSmall::SMEM_BYTES);
     if (e != cudaSuccess) return MOE_FP8_ERR_CUDA;
@@ -390,14 +394,14 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
     cudaStream_t stream = static_cast<cudaStream_t>(stream_v);
     const int H = c.hidden, I = c.intermediate, EL = c.num_local_experts;
     if (w13 != h->w13_cached || w2 != h->w2_cached) {
-        // N side of the MMAs: w13 seen as [E_loc][2 halves][I rows][H], a box takes the same 64 rows of both halves, so
-        // that an epilogue warpgroup finds gate and up of the same columns side by side; M side: 128 consecutive rows
+        // The weights as [E_loc][half][rows][K], boxes of 128 rows: for the N side of GEMM1's MMAs the same 64 rows of
+        // both halves (an epilogue warpgroup finds gate and up of the same columns side by side), else consecutive ones
         const cuuint64_t Hz = H, Iz = I, Ez = EL;
-        const cuuint64_t dims[4] = {Hz, Iz, 2, Ez}, strides[3] = {Hz, Iz * Hz, 2 * Iz * Hz};
-        const cuuint32_t box[4] = {128, 64, 2, 1};
-        if (!encode_4d(h, &h->tm_w13_n, w13, dims, strides, box) ||
-            !encode_2d(h, &h->tm_w13_m, w13, static_cast<uint64_t>(EL) * 2 * I, H, 1, 128, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
-            !encode_2d(h, &h->tm_w2, w2, static_cast<uint64_t>(EL) * H, I, 1, 128, 128, CU_TENSOR_MAP_SWIZZLE_128B))
+        const cuuint64_t d13[4] = {Hz, Iz, 2, Ez}, s13[3] = {Hz, Iz * Hz, 2 * Iz * Hz};
+        const cuuint64_t d2[4] = {Iz, Hz, 1, Ez}, s2[3] = {Iz, Hz * Iz, Hz * Iz};
+        const cuuint32_t box_n[4] = {128, 64, 2, 1}, box_m[4] = {128, 128, 1, 1};
+        if (!encode_4d(h, &h->tm_w13_n, w13, d13, s13, box_n) || !encode_4d(h, &h->tm_w13_m, w13, d13, s13, box_m) ||
+            !encode_4d(h, &h->tm_w2, w2, d2, s2, box_m))
             return cuda_fail(h, cudaErrorInvalidValue);
         h->w13_cached = w13;
         h->w2_cached = w2;
@@ -547,6 +551,7 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
         mark();  // gather_rows
         mark();  // gemm1
         mark();  // gemm2
+        mark();  // grouped_mlp
         mark();  // combine
         MOE_LAUNCH(fused_small_kernel, h->sm_count, G_THREADS, GeomSmall::SMEM_BYTES, stream, pdl, h->tm_a2_small,
                    h->tm_w13_m, h->tm_w2, g1, g2, f);
@@ -560,15 +565,30 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
                        static_cast<const uint8_t*>(hidden_fp8), hidden_scale, m, a1, a1_scale_t, status);
             mark();
         }
-        // stage 3a: GEMM1 + SwiGLU + re-quantisation
+        // stage 3: GEMM1 + SwiGLU + re-quantisation, GEMM2
         if (h->short_tile_min_tokens > 0 && T >= h->short_tile_min_tokens) g1.wm_rows = g2.wm_rows = WM_TOKENS;
-        MOE_LAUNCH(grouped_gemm_kernel<1>, h->sm_count, G_THREADS, GeomFull::SMEM_BYTES, stream, pdl, h->tm_a1,
-                   h->tm_a1_small, h->tm_w13_n, h->tm_w13_m, h->tm_a2_store, g1);
-        mark();
-        // stage 3b: GEMM2
-        MOE_LAUNCH(grouped_gemm_kernel<2>, h->sm_count, G_THREADS, GeomFull::SMEM_BYTES, stream, pdl, h->tm_a2,
-                   h->tm_a2_small, h->tm_w2, h->tm_w2, h->tm_a2_store, g2);
-        mark();
+        MlpArgs a = {g1, g2, 3, m.mlp_claimed, m.mlp_ready};
+        auto mlp = [&](int phases) {
+            a.phases = phases;
+            return launch(grouped_mlp_kernel, m.mlp_grid, G_THREADS, GeomFull::SMEM_BYTES, stream, pdl, h->tm_a1, h->tm_a1_small,
+                          h->tm_w13_n, h->tm_w13_m, h->tm_a2_store, h->tm_a2, h->tm_a2_small, h->tm_w2, a);
+        };
+        const long long slots = static_cast<long long>(T) * R_TOPK * EL / R_EXPERTS;
+        if (T > MLP_SPLIT_MAX_TOKENS && slots <= MLP_JOINT_MAX_SLOTS) {
+            mark();  // gemm1
+            mark();  // gemm2
+            if ((lerr = mlp(3)) != cudaSuccess) return cuda_fail(h, lerr);
+            ++launches;
+            mark();
+        } else {
+            if ((lerr = mlp(1)) != cudaSuccess) return cuda_fail(h, lerr);
+            ++launches;
+            mark();
+            if ((lerr = mlp(2)) != cudaSuccess) return cuda_fail(h, lerr);
+            ++launches;
+            mark();
+            mark();  // grouped_mlp
+        }
         {  // stage 4: weighted combine back to token order
             const int grid = min(T, h->sm_count * 16);
             MOE_LAUNCH(combine_kernel, grid, 256, 0, stream, pdl, T, H, static_cast<const int*>(m.slot_to_row),

@@ -27,6 +27,9 @@ struct PermuteMeta {
     int* tile_expert;    // [max_m_tiles] local expert of each row tile
     int* tile_rows;      // [max_m_tiles] valid rows in each row tile (1..TILE_M)
     int* num_m_tiles;    // [1]
+    int* mlp_ready;      // [max_m_tiles] grouped_mlp_kernel's counters, zeroed with the tables: parts of GEMM1 stored,
+    int* mlp_claimed;    // [mlp_grid] and lists of tiles claimed
+    int mlp_grid;
     int* slot_to_row;    // [T*8] padded row of each slot, -1 when the slot's expert is not local
     int* row_to_slot;    // [T*8] canonical row -> slot id (first S entries valid)
     int* row_token;      // [row_cap] padded row -> token (valid rows only)
@@ -86,8 +89,10 @@ __device__ __forceinline__ void scan_experts(int E_loc, int* s_cnt, int* s_pad, 
         for (int i = 0; i * TILE_M < total; ++i) {
             m.tile_expert[t0 + i] = e;
             m.tile_rows[t0 + i] = min(TILE_M, total - i * TILE_M);
+            m.mlp_ready[t0 + i] = 0;
         }
     }
+    for (int v = tid; v < m.mlp_grid; v += blockDim.x) m.mlp_claimed[v] = 0;
     if (tid == 0) {  // entries past E_loc count nothing, so entry E_loc already holds the totals
         m.expert_offset[E_loc] = s_cnt[E_loc];
         m.padded_offset[E_loc] = s_pad[E_loc];
@@ -210,12 +215,13 @@ __global__ void __launch_bounds__(256) place_gather_kernel(int T, int H, int E_l
                                                            const float* __restrict__ hidden_scale, PermuteMeta m,
                                                            uint8_t* __restrict__ a1, float* __restrict__ a1_scale_t,
                                                            int* __restrict__ status) {
-    pdl_launch_dependents();
     const int lane = threadIdx.x & 31;
     const int nwarps = gridDim.x * (blockDim.x >> 5);
     const int chunks = H / 16, nkb = H / 128;
     constexpr int BATCH = 7;  // 16-byte chunks of a row that a lane holds at a time (a row of 7168 bytes: two batches)
     pdl_wait();
+    // (only now: whoever is started by this may read the row tables without waiting for this kernel)
+    pdl_launch_dependents();
     for (int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < T; t += nwarps) {
         int prow = -1;
         if (lane < R_TOPK) {
