@@ -190,6 +190,19 @@ cudaError_t launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+template <int WT, int WE, int MT, int ME, int KC, int S>
+cudaError_t set_router_smem() {
+    return cudaFuncSetAttribute(router_logits_kernel<WT, WE, MT, ME, KC, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                RouterShape<WT, WE, MT, ME, KC, S>::SMEM_BYTES);
+}
+template <int WT, int WE, int MT, int ME, int KC, int S>
+cudaError_t launch_router(int T, int H, int E, const __nv_bfloat16* x, const __nv_bfloat16* w, float* logits,
+                          cudaStream_t stream) {
+    using Shape = RouterShape<WT, WE, MT, ME, KC, S>;
+    return launch(router_logits_kernel<WT, WE, MT, ME, KC, S>, dim3((T + Shape::ROWS_T - 1) / Shape::ROWS_T, E / Shape::ROWS_E),
+                  Shape::THREADS, Shape::SMEM_BYTES, stream, false, T, H, E, x, w, logits);
+}
+
 PermuteMeta meta_of(moe_fp8_handle_t h) {
     PermuteMeta m;
     m.block_hist = at<int>(h, h->L.block_hist);
@@ -295,8 +308,9 @@ int moe_fp8_create(const moe_fp8_config* cfg, moe_fp8_handle_t* out) {
     if (e != cudaSuccess) return MOE_FP8_ERR_CUDA;
     e = cudaFuncSetAttribute(fused_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GeomSmall::SMEM_BYTES);
     if (e != cudaSuccess) return MOE_FP8_ERR_CUDA;
-    e = cudaFuncSetAttribute(router_logits_kernel<4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(router_smem_bytes(4, 4)));
+    e = set_router_smem<2, 1, 4, 4, 256, 8>();
+    if (e == cudaSuccess) e = set_router_smem<2, 2, 8, 8, 256, 2>();
+    if (e == cudaSuccess) e = set_router_smem<2, 2, 16, 8, 512, 2>();
     if (e != cudaSuccess) return MOE_FP8_ERR_CUDA;
     e = cudaFuncSetAttribute(route_permute_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(route_permute_smem_bytes(P_TAIL_MAX_TOKENS, P_MAX_LOCAL)));
@@ -728,16 +742,16 @@ int moe_fp8_forward_from_hidden(moe_fp8_handle_t h, int T, const void* hidden_bf
         const __nv_bfloat16* x = static_cast<const __nv_bfloat16*>(hidden_bf16);
         const __nv_bfloat16* wr = static_cast<const __nv_bfloat16*>(router_weight);
         cudaError_t e;
-        if (T <= 128)  // few tokens: many small CTAs, so that the router weight streams in from many SMs
-            e = launch(router_logits_kernel<1, 4>, dim3((T + 7) / 8, E / 32), 128, router_smem_bytes(1, 4), stream, false,
-                       T, H, E, x, wr, d_logits);
+        if (T <= RP_SMALL_MAX_TOKENS)
+            e = launch_router<2, 1, 4, 4, 256, 8>(T, H, E, x, wr, d_logits, stream);
+        else if (T < RP_LARGE_MIN_TOKENS || H % 512 != 0)
+            e = launch_router<2, 2, 8, 8, 256, 2>(T, H, E, x, wr, d_logits, stream);
         else
-            e = launch(router_logits_kernel<4, 4>, dim3((T + 31) / 32, E / 32), 512, router_smem_bytes(4, 4), stream,
-                       false, T, H, E, x, wr, d_logits);
+            e = launch_router<2, 2, 16, 8, 512, 2>(T, H, E, x, wr, d_logits, stream);
         if (e != cudaSuccess) return cuda_fail(h, e);
         const long long blocks = (static_cast<long long>(T) * (H / 128) + 7) / 8;
         e = launch(quantize_rows_kernel, static_cast<int>(std::min<long long>(blocks, h->sm_count * 16LL)), 256, 0, stream,
-                   false, T, H, h->cfg.hidden_scale_layout, x, d_hidden, d_scale);
+                   true, T, H, h->cfg.hidden_scale_layout, x, d_hidden, d_scale);
         if (e != cudaSuccess) return cuda_fail(h, e);
     }
     const int rc = moe_fp8_forward(h, T, d_hidden, d_scale, d_logits, routing_bias, w13, w13_scale, w2, w2_scale,

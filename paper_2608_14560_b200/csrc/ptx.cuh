@@ -305,6 +305,16 @@ __device__ __forceinline__ void ld_global_v8(const void* p, uint32_t (&w)[8]) {
                  : "memory");
 }
 
+// ---- ldmatrix -----------------------------------------------------------------
+// Four 8 x 16-byte matrices: lane 8 q + j gives the address of row j of matrix q; r[q] is the 4-byte word lane & 3 of row
+// lane >> 2 of matrix q.  With the eight rows of a matrix 16 bytes apart, r[q] is the lane's word of 128 contiguous bytes.
+__device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+
 // ---- packed fp32 ------------------------------------------------------------
 // Two fp32 values (bit patterns) in one 64-bit register: lo in bits 0..31.
 __device__ __forceinline__ uint64_t pack_f32x2(uint32_t lo, uint32_t hi) {

@@ -20,125 +20,130 @@
 
 namespace moe {
 
-constexpr int RP_KC = 256;   // K elements staged per step (4 runs of 64)
-constexpr int RP_MT = 8;     // tokens per warp tile
-constexpr int RP_ME = 8;     // experts per warp tile
+// logits[t, e] = sum_h x[t, h] * w[e, h] in the order stated above.  A warp owns MT tokens x ME experts with the K
+// dimension spread over its lanes, a CTA WT x WE such warps; rows come in through a ring of S stages of KC elements
+// (cp.async).  x [T, H] and w [E, H] bf16, H a multiple of KC, E a multiple of WE * ME.
+//
+// Large batches are bound by the fp32 pipes (2 x 7168 x 256 FLOP per token, 36 TFMA/s measured for packed and for scalar
+// FMAs) and the issue slots around the FMAs.  ldmatrix hands a lane its words of four rows in one instruction (16
+// single-word loads per 64 elements and 8 x 8 tile before, 4 now); the packed FMA does two tokens at a time.  Small ones
+// are bound by latency and the number of warps that stream the 3.7 MB of weights.  Hence three shapes (us, loads in 32
+// single words and two stages before / this kernel):
+//   8 x 8 per warp, 2 x 2 warps   many small CTAs balance the SMs: 257 tokens 73 / 36, 1024 139 / 99, 2048 270 / 186
+//   16 x 8, 2 x 2 warps           fewer words per FMA, for batches that fill the GPU anyway: 2048 tokens 182, 8192
+//                                 926 / 669 (8 x 8: 704), 61 % of the pipes
+//   4 x 4, 2 x 1 warps            eight stages in flight per warp: 16 tokens 26 / 14, 64 tokens 24 / 17
+template <int WT, int WE, int MT, int ME, int KC, int S>
+struct RouterShape {
+    static constexpr int ROWS_T = WT * MT, ROWS_E = WE * ME, THREADS = WT * WE * 32, ROWS = ROWS_T + ROWS_E;
+    static constexpr int SMEM_BYTES = S * ROWS * KC * 2;
+    static_assert(MT % 4 == 0 && ME % 4 == 0 && KC % 64 == 0, "rows are read four at a time, in runs of 64 elements");
+};
+constexpr int RP_SMALL_MAX_TOKENS = 64;    // 4 x 4 up to here
+constexpr int RP_LARGE_MIN_TOKENS = 2048;  // 16 x 8 from here
 
-__host__ __device__ constexpr size_t router_smem_bytes(int WT, int WE) {
-    return static_cast<size_t>(2) * (WT * RP_MT + WE * RP_ME) * RP_KC * 2;  // two buffers of bf16 rows
-}
-
-// logits[t, e] = sum_h x[t, h] * w[e, h] in the order stated above.  One CTA computes a
-// (WT*8 tokens) x (WE*8 experts) tile; warp (wt, we) owns an 8 x 8 block of it with the K dimension
-// spread over its lanes.  x [T, H] and w [E, H] bf16, H a multiple of 256, E a multiple of WE*8.
-template <int WT, int WE>
+template <int WT, int WE, int MT, int ME, int KC, int S>
 __global__ void __launch_bounds__(WT * WE * 32)
 router_logits_kernel(int T, int H, int E, const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ w,
                      float* __restrict__ logits) {
-    extern __shared__ __align__(16) uint8_t rp_smem[];
-    constexpr int ROWS_T = WT * RP_MT, ROWS_E = WE * RP_ME, ROWS = ROWS_T + ROWS_E;
-    constexpr int THREADS = WT * WE * 32;
-    constexpr int CHUNKS_PER_ROW = RP_KC * 2 / 16;                 // 16-byte chunks of one staged row
+    using Shape = RouterShape<WT, WE, MT, ME, KC, S>;
+    extern __shared__ __align__(128) uint8_t rp_smem[];
+    constexpr int ROWS_T = Shape::ROWS_T, ROWS = Shape::ROWS, THREADS = Shape::THREADS;
+    constexpr int CHUNKS_PER_ROW = KC / 8, ROW_BYTES = KC * 2;     // 16-byte chunks of one staged row
+    pdl_launch_dependents();  // (quantize_rows_kernel needs nothing from here)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int wt = warp / WE, we = warp % WE;
-    const int t0 = blockIdx.x * ROWS_T, e0 = blockIdx.y * ROWS_E;
+    const int t0 = blockIdx.x * ROWS_T, e0 = blockIdx.y * Shape::ROWS_E;
     const uint32_t smem0 = smem_u32(rp_smem);
+    const int nkc = H / KC;
 
-    // stage K-chunk kc of the tile's rows (tokens first, then experts) into buffer b; rows past T read as zero
-    auto stage = [&](int kc, int b) {
-        for (int c = tid; c < ROWS * CHUNKS_PER_ROW; c += THREADS) {
-            const int r = c / CHUNKS_PER_ROW, cc = c % CHUNKS_PER_ROW;
-            const __nv_bfloat16* src;
-            uint32_t bytes = 16;
-            if (r < ROWS_T) {
-                const int t = t0 + r;
-                if (t >= T) bytes = 0;
-                src = x + static_cast<size_t>(t < T ? t : 0) * H + kc * RP_KC + cc * 8;
-            } else {
-                src = w + static_cast<size_t>(e0 + r - ROWS_T) * H + kc * RP_KC + cc * 8;
+    // stage K-chunk kc of the tile's rows (tokens first, then experts); rows past T read as zero
+    auto stage = [&](int kc) {
+        if (kc < nkc) {
+            const uint32_t dst = smem0 + (kc % S) * ROWS * ROW_BYTES;
+#pragma unroll
+            for (int c = tid; c < ROWS * CHUNKS_PER_ROW; c += THREADS) {
+                const int r = c / CHUNKS_PER_ROW, cc = c % CHUNKS_PER_ROW;
+                const __nv_bfloat16* src;
+                uint32_t bytes = 16;
+                if (r < ROWS_T) {
+                    const int t = t0 + r;
+                    if (t >= T) bytes = 0;
+                    src = x + static_cast<size_t>(t < T ? t : 0) * H + kc * KC + cc * 8;
+                } else {
+                    src = w + static_cast<size_t>(e0 + r - ROWS_T) * H + kc * KC + cc * 8;
+                }
+                cp_async_16(dst + r * ROW_BYTES + cc * 16, src, bytes);
             }
-            cp_async_16(smem0 + (b * ROWS + r) * (RP_KC * 2) + cc * 16, src, bytes);
         }
         cp_async_commit();
     };
 
     // Accumulators as pairs of tokens (2 i, 2 i + 1) for the packed fp32 FMA: one instruction, two independent
     // round-to-nearest FMAs, so every sum is bit for bit the one of the scalar form.
-    uint64_t acc2[RP_MT / 2][RP_ME];
+    uint64_t acc[MT / 2][ME];
 #pragma unroll
-    for (int i = 0; i < RP_MT / 2; ++i)
+    for (int i = 0; i < MT / 2; ++i)
 #pragma unroll
-        for (int j = 0; j < RP_ME; ++j) acc2[i][j] = 0ull;
+        for (int j = 0; j < ME; ++j) acc[i][j] = 0ull;
 
-    const int nkc = H / RP_KC;
-    stage(0, 0);
+#pragma unroll
+    for (int i = 0; i < S - 1; ++i) stage(i);
+    // this lane's row addresses for ldmatrix: piece lane & 7 of row lane >> 3 of a group of four
+    const uint32_t x_off = (wt * MT + (lane >> 3)) * ROW_BYTES + (lane & 7) * 16;
+    const uint32_t w_off = (ROWS_T + we * ME + (lane >> 3)) * ROW_BYTES + (lane & 7) * 16;
     for (int kc = 0; kc < nkc; ++kc) {
-        const int b = kc & 1;
-        if (kc + 1 < nkc) {
-            stage(kc + 1, b ^ 1);
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
-        }
-        __syncthreads();
-        const uint8_t* xb = rp_smem + (b * ROWS + wt * RP_MT) * (RP_KC * 2) + lane * 4;
-        const uint8_t* wb = rp_smem + (b * ROWS + ROWS_T + we * RP_ME) * (RP_KC * 2) + lane * 4;
+        cp_async_wait<S - 2>();
+        __syncthreads();  // the chunk has landed, and everybody has left the buffer that is refilled next
+        stage(kc + S - 1);
+        const uint32_t base = smem0 + (kc % S) * ROWS * ROW_BYTES;
 #pragma unroll
-        for (int run = 0; run < RP_KC / 64; ++run) {
-            uint64_t xl2[RP_MT / 2], xh2[RP_MT / 2];  // elements 2l / 2l+1 of the run for two tokens each
+        for (int run = 0; run < KC / 64; ++run) {
+            uint64_t xl[MT / 2], xh[MT / 2];  // elements 2l / 2l+1 of the run for two tokens each
 #pragma unroll
-            for (int i = 0; i < RP_MT / 2; ++i) {
-                const uint32_t u0 = *reinterpret_cast<const uint32_t*>(xb + (2 * i) * (RP_KC * 2) + run * 128);
-                const uint32_t u1 = *reinterpret_cast<const uint32_t*>(xb + (2 * i + 1) * (RP_KC * 2) + run * 128);
-                xl2[i] = pack_f32x2(u0 << 16, u1 << 16);
-                xh2[i] = pack_f32x2(u0 & 0xffff0000u, u1 & 0xffff0000u);
+            for (int q = 0; q < MT / 4; ++q) {
+                uint32_t r[4];
+                ldmatrix_x4(base + x_off + q * 4 * ROW_BYTES + run * 128, r);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    xl[2 * q + i] = pack_f32x2(r[2 * i] << 16, r[2 * i + 1] << 16);
+                    xh[2 * q + i] = pack_f32x2(r[2 * i] & 0xffff0000u, r[2 * i + 1] & 0xffff0000u);
+                }
             }
 #pragma unroll
-            for (int j = 0; j < RP_ME; ++j) {
-                const uint32_t u = *reinterpret_cast<const uint32_t*>(wb + j * (RP_KC * 2) + run * 128);
-                const uint64_t wl2 = pack_f32x2(u << 16, u << 16), wh2 = pack_f32x2(u & 0xffff0000u, u & 0xffff0000u);
+            for (int q = 0; q < ME / 4; ++q) {
+                uint32_t r[4];
+                ldmatrix_x4(base + w_off + q * 4 * ROW_BYTES + run * 128, r);
 #pragma unroll
-                for (int i = 0; i < RP_MT / 2; ++i) acc2[i][j] = fma_f32x2(xl2[i], wl2, acc2[i][j]);  // element 2l of the run
+                for (int j = 0; j < 4; ++j) {
+                    const uint64_t wl = pack_f32x2(r[j] << 16, r[j] << 16);
+                    const uint64_t wh = pack_f32x2(r[j] & 0xffff0000u, r[j] & 0xffff0000u);
 #pragma unroll
-                for (int i = 0; i < RP_MT / 2; ++i) acc2[i][j] = fma_f32x2(xh2[i], wh2, acc2[i][j]);  // then element 2l+1
+                    for (int i = 0; i < MT / 2; ++i) acc[i][4 * q + j] = fma_f32x2(xl[i], wl, acc[i][4 * q + j]);  // element 2l
+#pragma unroll
+                    for (int i = 0; i < MT / 2; ++i) acc[i][4 * q + j] = fma_f32x2(xh[i], wh, acc[i][4 * q + j]);  // then 2l+1
+                }
             }
         }
-        __syncthreads();  // the buffer is refilled two steps from now
     }
-    float acc[RP_MT][RP_ME];
-#pragma unroll
-    for (int i = 0; i < RP_MT / 2; ++i)
-#pragma unroll
-        for (int j = 0; j < RP_ME; ++j) {
-            acc[2 * i][j] = __uint_as_float(static_cast<uint32_t>(acc2[i][j]));
-            acc[2 * i + 1][j] = __uint_as_float(static_cast<uint32_t>(acc2[i][j] >> 32));
-        }
 
-    // five pairwise rounds; afterwards every lane holds every logit of the warp tile
+    // five pairwise rounds, after which every lane holds every logit of the warp tile; the lanes store them in turn
 #pragma unroll
-    for (int i = 0; i < RP_MT; ++i)
+    for (int i = 0; i < MT; ++i)
 #pragma unroll
-        for (int j = 0; j < RP_ME; ++j) {
-            float v = acc[i][j];
+        for (int j = 0; j < ME; ++j) {
+            float v = __uint_as_float(static_cast<uint32_t>((i & 1) ? acc[i / 2][j] >> 32 : acc[i / 2][j]));
 #pragma unroll
             for (int d = 16; d >= 1; d >>= 1) v = __fadd_rn(v, __shfl_xor_sync(0xffffffffu, v, d));
-            acc[i][j] = v;
+            const int t = t0 + wt * MT + i;
+            if (lane == (i * ME + j) % 32 && t < T) logits[static_cast<size_t>(t) * E + e0 + we * ME + j] = v;
         }
-    // lane l stores the logits of token (l >> 2) for experts 2 (l & 3), 2 (l & 3) + 1
-#pragma unroll
-    for (int i = 0; i < RP_MT; ++i)
-#pragma unroll
-        for (int j = 0; j < RP_ME; j += 2)
-            if (lane == i * 4 + j / 2) {
-                const int t = t0 + wt * RP_MT + i;
-                if (t < T)
-                    *reinterpret_cast<float2*>(logits + static_cast<size_t>(t) * E + e0 + we * RP_ME + j) =
-                        make_float2(acc[i][j], acc[i][j + 1]);
-            }
 }
 
 // One warp per (token, 128-column block): amax, scale = amax / 448 (1 for an all-zero block), codes =
 // e4m3(x / scale) with IEEE division, round to nearest even, saturating.  scale_layout 0: [T, H/128], 1: [H/128, T].
+// Runs beside the router projection (programmatic dependent launch): it reads the same input and waits for that kernel
+// only at its end, so that whoever follows finds both done.
 __global__ void __launch_bounds__(256) quantize_rows_kernel(int T, int H, int scale_layout,
                                                             const __nv_bfloat16* __restrict__ x,
                                                             uint8_t* __restrict__ q, float* __restrict__ scale) {
@@ -164,6 +169,7 @@ __global__ void __launch_bounds__(256) quantize_rows_kernel(int T, int H, int sc
         *reinterpret_cast<uint32_t*>(q + t * H + b * 128 + lane * 4) = lo | (hi << 16);
         if (lane == 0) scale[scale_layout ? static_cast<long long>(b) * T + t : t * nb + b] = sc;
     }
+    pdl_wait();
 }
 
 }  // namespace moe
