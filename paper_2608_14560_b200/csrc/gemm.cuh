@@ -186,6 +186,7 @@ struct FusedArgs {
     float* raw[2];
     int* part_done[2];            // [tiles] per GEMM, zero at launch (part of the counter set)
     int split;                    // 1: the split may be used by this call
+    int ahead;                    // GEMM2 tiles that take the time of a GEMM1 tile, see seq_after
 };
 constexpr int SPLIT_MAX_TOKENS = 4;                       // rows of a tile whose K range may be split
 constexpr int SPLIT_MAX_TILES = 74;                       // a split needs at least two CTAs per tile
@@ -246,10 +247,35 @@ struct Cta {
     int warp, lane;
 };
 
-// Tiles first, first + stride, ... below count.
-struct TileRange {
-    int first, count, stride;
+// A CTA's work items in one phase of the fused kernel: at(0), at(1), ... up to the first one that is not below `count`.
+struct PlainSeq {  // the items in turn to all CTAs
+    int first, stride, count;
+    __device__ __forceinline__ int at(int j) const { return first + j * stride; }
 };
+__device__ __forceinline__ PlainSeq seq_plain(int count) {
+    return PlainSeq{static_cast<int>(blockIdx.x), static_cast<int>(gridDim.x), count};
+}
+struct AheadSeq {  // the first `rounds` rounds of items to `stride` of the CTAs, the later ones to all
+    int turn, skip, rounds, stride, grid, count;
+    __device__ __forceinline__ int at(int j) const {
+        j += skip;
+        return j < rounds ? j * stride + turn : rounds * stride + (j - rounds) * grid + turn;
+    }
+};
+// After `before` items dealt by seq_plain: the CTAs that got one item less are the first in every round, and they take up
+// to `ahead` rounds among themselves in front, as far as the items reach whose row tiles the full rounds have finished
+// (n1_tiles items before and n2_tiles new ones belong to a row tile).  (Dealt in plain rounds, 54 tokens on 23 experts left 72 CTAs with 238 K-blocks and 76
+// with 182; us per forward, plain rounds / these: 54 tokens 175 / 165, 33 tokens on 256 local experts 766 / 752, 8 and
+// 16 tokens up to 6 % less, equal where GEMM1 fills whole rounds.)
+__device__ __forceinline__ AheadSeq seq_after(int before, int ahead, int n1_tiles, int n2_tiles, int count) {
+    const int grid = static_cast<int>(gridDim.x), b = static_cast<int>(blockIdx.x);
+    int r = before, rounds = 0;
+    if (before >= grid) {  // (below, the smallest batches, no division delays the first weights of the second phase)
+        r = before % grid;
+        if (r) rounds = min(ahead, (before - r) / n1_tiles * n2_tiles / (grid - r));
+    }
+    return b < r ? AheadSeq{b - r + grid, rounds, rounds, grid - r, grid, count} : AheadSeq{b - r, 0, rounds, grid - r, grid, count};
+}
 
 // Very small batches of the fused kernel: a tile's K range is cut into `parts` pieces of `len` K-blocks that
 // different CTAs work on (see epilogue_tile_wm).  parts = 1: a work item is a whole tile.
@@ -307,12 +333,12 @@ __device__ __forceinline__ void gemm_cta_setup(Cta& c, uint8_t* smem_raw, int fu
 // tmB: boxes of 128 weight rows of [expert][half][row][K]; MODE 1 takes gate[0,128) | up[0,128) of the tile's 128 columns ("gate" and "up"
 // change places with gate_first = 0), MODE 2 256 consecutive rows.  MODE 1: the token rows and the scales come from
 // the gather warp instead; MODE 2: the tile's token rows are GEMM1's output and must have been stored.
-template <int MODE, class GEO>
+template <int MODE, class GEO, class SEQ>
 __device__ __forceinline__ void producer_tiles(const Cta& c, const CUtensorMap* tmA, const CUtensorMap* tmB,
-                                               const GemmArgs& g, const FusedArgs* f, int ready_target, TileRange tr,
+                                               const GemmArgs& g, const FusedArgs* f, int ready_target, const SEQ& seq,
                                                uint32_t& it, bool& ok, KSplit ks) {
     GemmCtrl* ctrl = c.ctrl;
-    for (int item = tr.first; item < tr.count && ok; item += tr.stride) {
+    for (int j = 0, item; ok && (item = seq.at(j)) < seq.count; ++j) {
         const int tile = item / ks.parts, kb0 = (item - tile * ks.parts) * ks.len;
         const int kb1 = min(g.num_kb, kb0 + ks.len);
         const int m_tile = tile / g.n_tiles, n = tile - m_tile * g.n_tiles;
@@ -401,14 +427,14 @@ __device__ __forceinline__ void issuer_drain(const Cta& c, uint32_t mine, bool o
 // token-major input, and the scale of row l.  The stage uses the 128-byte swizzle of the TMA tiles: chunk c of
 // row r sits at r * 128 + ((c ^ (r & 7)) << 4), and r & 7 takes only two values per lane (i even / odd).  Rows
 // past the tile's valid rows are zero-filled; the stage holds only these 32 rows (see Geometry).  Each lane's arrival on full[s] is triggered by the completion of its copies.
-template <class GEO>
-__device__ __forceinline__ void gather_tiles(const Cta& c, const GemmArgs& g, const FusedArgs& f, TileRange tr,
+template <class GEO, class SEQ>
+__device__ __forceinline__ void gather_tiles(const Cta& c, const GemmArgs& g, const FusedArgs& f, const SEQ& seq,
                                              uint32_t& it, bool& ok, KSplit ks) {
     GemmCtrl* ctrl = c.ctrl;
     const int lane = c.lane, sub = lane >> 3, chunk = lane & 7;
     const uint32_t dst_even = sub * 128 + ((chunk ^ sub) << 4);
     const uint32_t dst_odd = sub * 128 + ((chunk ^ (sub + 4)) << 4);
-    for (int item = tr.first; item < tr.count && ok; item += tr.stride) {
+    for (int j = 0, item; ok && (item = seq.at(j)) < seq.count; ++j) {
         const int tile = item / ks.parts, kb0 = (item - tile * ks.parts) * ks.len;
         const int kb1 = min(g.num_kb, kb0 + ks.len);
         const int m_tile = tile / g.n_tiles;
@@ -449,11 +475,11 @@ __device__ __forceinline__ void gather_tiles(const Cta& c, const GemmArgs& g, co
     }
 }
 // GEMM2 tiles: the producer fetches everything; the lanes only keep the arrival count of full[s] uniform.
-template <class GEO>
-__device__ __forceinline__ void gather_idle_tiles(const Cta& c, const GemmArgs& g, TileRange tr, uint32_t& it, bool& ok,
+template <class GEO, class SEQ>
+__device__ __forceinline__ void gather_idle_tiles(const Cta& c, const GemmArgs& g, const SEQ& seq, uint32_t& it, bool& ok,
                                                   KSplit ks) {
     GemmCtrl* ctrl = c.ctrl;
-    for (int item = tr.first; item < tr.count && ok; item += tr.stride) {
+    for (int j = 0, item; ok && (item = seq.at(j)) < seq.count; ++j) {
         const int kb0 = (item % ks.parts) * ks.len, kb1 = min(g.num_kb, kb0 + ks.len);
         for (int kb = kb0; kb < kb1; ++kb, ++it) {
             const uint32_t s = it % GEO::STAGES, ph = (it / GEO::STAGES) & 1;
@@ -488,14 +514,14 @@ __device__ __forceinline__ bool epilogue_rendezvous(const Cta& c, uint32_t& n) {
 // Element for element the arithmetic is the one of the other orientation.
 static_assert(G_MAX_STAGES * WM_BUF_COLS <= static_cast<int>(G_TMEM_COLS), "one accumulator buffer per stage");
 
-template <class GEO>
-__device__ __forceinline__ void issuer_tiles_wm(const Cta& c, const GemmArgs& g, TileRange tr, uint32_t mine,
+template <class GEO, class SEQ>
+__device__ __forceinline__ void issuer_tiles_wm(const Cta& c, const GemmArgs& g, const SEQ& seq, uint32_t mine,
                                                 uint32_t& it, bool& ok, KSplit ks) {
     static_assert(GEO::A_ROWS == WM_TOKENS, "the token slot of a stage is the MMA's N operand");
     static_assert(GEO::SCALE_SLOTS >= 2 * GEO::STAGES + 1, "the gather may be two pipelines ahead of the epilogue");
     GemmCtrl* ctrl = c.ctrl;
     const uint32_t idesc = umma_idesc_f8(TILE_M, WM_TOKENS);
-    for (int item = tr.first; item < tr.count && ok; item += tr.stride) {
+    for (int j = 0, item; ok && (item = seq.at(j)) < seq.count; ++j) {
         const int kb0 = (item % ks.parts) * ks.len, kb1 = min(g.num_kb, kb0 + ks.len);
         for (int kb = kb0; kb < kb1; ++kb, ++it) {
             if ((it & 1) != mine) continue;
@@ -914,11 +940,11 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
     return true;
 }
 
-template <int MODE, bool FUSED, class GEO>
-__device__ __forceinline__ void epilogue_tiles_wm(const Cta& c, const GemmArgs& g, const FusedArgs* f, TileRange tr,
+template <int MODE, bool FUSED, class GEO, class SEQ>
+__device__ __forceinline__ void epilogue_tiles_wm(const Cta& c, const GemmArgs& g, const FusedArgs* f, const SEQ& seq,
                                                   uint32_t& it, uint32_t& tile_iter, uint32_t& sync_iter, bool& ok,
                                                   KSplit ks) {
-    for (int item = tr.first; item < tr.count && ok; item += tr.stride) {
+    for (int j = 0, item; ok && (item = seq.at(j)) < seq.count; ++j) {
         const int tile = item / ks.parts, kb0 = (item - tile * ks.parts) * ks.len;
         const int m_tile = tile / g.n_tiles, n = tile - m_tile * g.n_tiles;
         // (two instantiations, so that the unsplit tile's loop carries nothing of the split)
@@ -970,8 +996,7 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmA2, const __grid_consta
             for (int i = threadIdx.x; i < f.H / 8; i += blockDim.x)
                 reinterpret_cast<uint4*>(f.out + static_cast<size_t>(t) * f.H)[i] = make_uint4(0u, 0u, 0u, 0u);
 
-    // The CTA's work list: its GEMM1 tiles, then its GEMM2 tiles; the grid-strided numbering runs on from one
-    // phase into the next, so the CTAs that had no GEMM1 tile take the first GEMM2 tiles.
+    // The CTA's work list: its GEMM1 tiles, then its GEMM2 tiles.
     // Very small batches with few tiles: a tile's K range is cut into parts for different CTAs (KSplit).
     const int grid = static_cast<int>(gridDim.x), m_tiles = __ldcg(g1.num_m_tiles);
     const bool may_split = f.split && f.T <= SPLIT_MAX_TOKENS && g1.num_kb <= SPLIT_MAX_KB && g2.num_kb <= SPLIT_MAX_KB;
@@ -980,8 +1005,9 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmA2, const __grid_consta
     // cost 5-6 us per tile, which 16 K-blocks do not win back; measured 1-2 us slower)
     const KSplit ks2 = ksplit_none(g2.num_kb);
     const int n1 = m_tiles * g1.n_tiles * ks1.parts, n2 = m_tiles * g2.n_tiles * ks2.parts;
-    const TileRange tr1 = {static_cast<int>(blockIdx.x), n1, grid};
-    const TileRange tr2 = {((static_cast<int>(blockIdx.x) - n1) % grid + grid) % grid, n2, grid};
+    const PlainSeq tr1 = seq_plain(n1);
+    // (set up behind the GEMM1 phase, where nobody waits for it)
+    auto tr2 = [&]() { return seq_after(n1, f.ahead, g1.n_tiles, g2.n_tiles, n2); };
     uint32_t it = 0;
     bool ok = true;
 
@@ -989,22 +1015,22 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmA2, const __grid_consta
         reg_dealloc<40>();
         if (c.warp == 0 && c.lane == 0) {
             producer_tiles<1, GEO>(c, &tmA2, &tmB1, g1, &f, 0, tr1, it, ok, ks1);
-            producer_tiles<2, GEO>(c, &tmA2, &tmB2, g2, &f, g1.n_tiles, tr2, it, ok, ks2);
+            producer_tiles<2, GEO>(c, &tmA2, &tmB2, g2, &f, g1.n_tiles, tr2(), it, ok, ks2);
             producer_drain<GEO>(c, g1.status, it);
         } else if ((c.warp == 1 || c.warp == 2) && c.lane == 0) {
             issuer_tiles_wm<GEO>(c, g1, tr1, c.warp - 1, it, ok, ks1);
-            issuer_tiles_wm<GEO>(c, g2, tr2, c.warp - 1, it, ok, ks2);
+            issuer_tiles_wm<GEO>(c, g2, tr2(), c.warp - 1, it, ok, ks2);
             issuer_drain(c, c.warp - 1, ok);
         } else if (c.warp == 3) {
             gather_tiles<GEO>(c, g1, f, tr1, it, ok, ks1);
-            gather_idle_tiles<GEO>(c, g2, tr2, it, ok, ks2);
+            gather_idle_tiles<GEO>(c, g2, tr2(), it, ok, ks2);
             cp_async_wait_all();  // nothing may still be landing in shared memory when the CTA exits
         }
     } else {
         reg_alloc<232>();
         uint32_t tile_iter = 0, sync_iter = 0;
         epilogue_tiles_wm<1, true, GEO>(c, g1, &f, tr1, it, tile_iter, sync_iter, ok, ks1);
-        epilogue_tiles_wm<2, true, GEO>(c, g2, &f, tr2, it, tile_iter, sync_iter, ok, ks2);
+        epilogue_tiles_wm<2, true, GEO>(c, g2, &f, tr2(), it, tile_iter, sync_iter, ok, ks2);
     }
 
     tc_fence_before();

@@ -535,6 +535,27 @@ def test_fused_kernel_with_a_raised_limit_cuts_experts_into_sub_tiles(cuda_devic
     eng.close()
 
 
+@pytest.mark.parametrize("active", [8, 73, 74, 75, 148, 149, 200])
+def test_fused_kernel_work_lists_around_full_rounds_of_ctas(cuda_device, active):
+    # two GEMM1 and two GEMM2 tiles per active expert: fewer tiles than CTAs, exactly one and two per CTA, a few more
+    dims = syn.LayerDims(hidden=512, intermediate=256, num_local_experts=256)
+    wl = _wl(30, dims, seed=880 + active)
+    inp = syn.make_inputs(wl, cuda_device)
+    inp["router_logits"][:] = -8.0
+    for t in range(30):
+        inp["router_logits"][t, [(8 * t + j) % active for j in range(8)]] = 6.0
+    eng = make_engine(wl, cuda_device)
+    eng.set_small_batch_fusion(False)
+    want = eng.forward(inp).clone()
+    eng.set_small_batch_fusion(True)
+    got = eng.forward(inp).clone()
+    torch.cuda.synchronize()
+    assert eng.status() == 0 and eng.last_launch_count() == 2
+    assert torch.equal(got.view(torch.int16), want.view(torch.int16))
+    assert int((eng.debug_export(30, rows=False)["expert_count"] > 0).sum()) == active
+    eng.close()
+
+
 @pytest.mark.parametrize("tokens,launches,eloc", [(16, 1, 32), (48, 2, 32), (3, 1, 256)])  # 3 tokens: K split
 def test_a_wait_that_runs_out_in_the_fused_small_batch_kernel(cuda_device, tokens, launches, eloc):
     wl = _wl(tokens, dataclasses.replace(SMALL, num_local_experts=eloc), seed=43)
