@@ -99,12 +99,12 @@ struct Geometry {
     static constexpr int RAW_BYTES = FACTORS_ ? F_RAW_FLOATS * 4 : 0;
     static constexpr int STORE_BYTES = STORE_BYTES_;                 // GEMM1 output staging
     static constexpr int SMEM_BYTES = STAGES_ * STAGE_BYTES + SCALE_SLOTS_ * SLOT_BYTES + STORE_BYTES_ + G_AMAX_BYTES +
-                                      G_CTRL_BYTES + RAW_BYTES + 1024;   // + alignment slack
+                                      G_CTRL_BYTES + RAW_BYTES + 1024;   // + alignment slack (the fused kernel has CtaTiles besides)
     static_assert(STAGES_ % 2 == 0, "an odd stage count lets an issuer thread skip phases of full[s]");
     static_assert(STAGES_ <= G_MAX_STAGES, "control block holds G_MAX_STAGES barriers per kind");
     static_assert(A_BYTES % 1024 == 0, "the B tile must stay 1024-byte aligned for the 128-byte swizzle");
     static_assert(SCALE_SLOTS_ >= STAGES_ + G_ACC_BUFS + 1, "the producer may be that far ahead of the epilogue");
-    static_assert(SMEM_BYTES <= 232448, "exceeds the 227 KB of shared memory a CTA may use");
+    static_assert(SMEM_BYTES + (FACTORS_ ? 0 : sizeof(CtaTiles)) <= 232448, "exceeds the 227 KB of shared memory a CTA may use");
 };
 // grouped_mlp_kernel: full 128-row A tiles, 4 stages of 48 KB
 using GeomFull = Geometry<4, TILE_M, 8, G_EPI_WARPS * G_STORE_WARP_BYTES, true>;
@@ -245,7 +245,21 @@ struct Cta {
     uint32_t smem_base, tmem_base;
     long long limit;
     int warp, lane;
+    const CtaTiles* tiles;     // fused kernel that routes by itself: its tiles, else null
 };
+// A (sub-)tile of the fused kernel: local expert, valid rows, first padded row, token of a row
+__device__ __forceinline__ int tile_expert_of(const Cta& c, const GemmArgs& g, int m) {
+    return c.tiles ? static_cast<int>(c.tiles->tile[m].x) : __ldcg(g.tile_expert + m);
+}
+__device__ __forceinline__ int tile_rows_of(const Cta& c, const GemmArgs& g, int m) {
+    return c.tiles ? __popc(c.tiles->tile[m].y) : __ldcg(g.tile_rows + m);
+}
+__device__ __forceinline__ int tile_row0_of(const Cta& c, const GemmArgs& g, int m) {
+    return c.tiles ? m * TILE_M : __ldcg(g.tile_row0 + m);
+}
+__device__ __forceinline__ int row_token_of(const Cta& c, const int* row_token, int m, int row0, int r) {
+    return c.tiles ? set_member(c.tiles->tile[m].y, r) : __ldcg(row_token + row0 + r);
+}
 
 // A CTA's work items in one phase of the fused kernel: at(0), at(1), ... up to the first one that is not below `count`.
 struct PlainSeq {  // the items in turn to all CTAs
@@ -342,8 +356,8 @@ __device__ __forceinline__ void producer_tiles(const Cta& c, const CUtensorMap* 
         const int tile = item / ks.parts, kb0 = (item - tile * ks.parts) * ks.len;
         const int kb1 = min(g.num_kb, kb0 + ks.len);
         const int m_tile = tile / g.n_tiles, n = tile - m_tile * g.n_tiles;
-        const int e = __ldcg(g.tile_expert + m_tile), wrow = n * (MODE == 1 ? 128 : G_TILE_N);
-        const int row0 = __ldcg(g.tile_row0 + m_tile);
+        const int e = tile_expert_of(c, g, m_tile), wrow = n * (MODE == 1 ? 128 : G_TILE_N);
+        const int row0 = tile_row0_of(c, g, m_tile);
         const float* a_sc = g.a_scale_t + row0;
         const uint32_t TX_BYTES = MODE == 1 ? G_B_BYTES : GEO::STAGE_BYTES + GEO::SCALE_BYTES;
         // claim the stage of pipeline iteration j: wait until its last reader has finished, announce the bytes
@@ -438,9 +452,9 @@ __device__ __forceinline__ void gather_tiles(const Cta& c, const GemmArgs& g, co
         const int tile = item / ks.parts, kb0 = (item - tile * ks.parts) * ks.len;
         const int kb1 = min(g.num_kb, kb0 + ks.len);
         const int m_tile = tile / g.n_tiles;
-        const int rows_valid = __ldcg(g.tile_rows + m_tile);
+        const int rows_valid = tile_rows_of(c, g, m_tile);
         // token of row `lane` (scale copy) and source rows of this lane's eight chunks
-        const int my_tok = lane < rows_valid ? __ldcg(f.row_token + __ldcg(g.tile_row0 + m_tile) + lane) : -1;
+        const int my_tok = lane < rows_valid ? row_token_of(c, f.row_token, m_tile, tile_row0_of(c, g, m_tile), lane) : -1;
         const uint8_t* src_row[GEO::A_ROWS / 4];
 #pragma unroll
         for (int i = 0; i < GEO::A_ROWS / 4; ++i) {
@@ -610,8 +624,8 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
     const size_t row_cap = static_cast<size_t>(g.row_cap);
     uint32_t* amax_x = reinterpret_cast<uint32_t*>(c.amax_x);   // [2 parities][256]: [2 token halves][4 quadrants][16] used
     const int num_kb = g.num_kb;
-    const int e = __ldcg(g.tile_expert + m_tile);
-    const int rows_valid = __ldcg(g.tile_rows + m_tile);
+    const int e = SHARED ? __ldcg(g.tile_expert + m_tile) : tile_expert_of(c, g, m_tile);
+    const int rows_valid = SHARED ? __ldcg(g.tile_rows + m_tile) : tile_rows_of(c, g, m_tile);
     const int sblocks = g.w_rows_per_expert / 128;
     const float* ws0;  // weight-scale rows of block 0 / block 1
     const float* ws1;
@@ -627,7 +641,7 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
     for (int j = 0; j < 32; ++j) acc[j] = 0.0f;
 
     const int kb_end = kb1 < 0 ? num_kb : kb1;
-    const int tile_row0 = SHARED ? m_tile * TILE_M : __ldcg(g.tile_row0 + m_tile);
+    const int tile_row0 = SHARED ? m_tile * TILE_M : tile_row0_of(c, g, m_tile);
     float4* raw = nullptr;  // this tile's stored partial sums (four tokens each): this thread's weight row
     if (SPLIT)
         raw = reinterpret_cast<float4*>(f->raw[MODE - 1] + static_cast<size_t>(m_tile * g.n_tiles + n) * num_kb * SPLIT_RAW_FLOATS) +
@@ -724,7 +738,7 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
             float v = 0.0f;
             if (t < rows_valid) {
                 if (MODE == 1) {
-                    const int tok = __ldcg(f->row_token + tile_row0 + t);
+                    const int tok = row_token_of(c, f->row_token, m_tile, tile_row0, t);
                     v = __ldcg(f->scale_layout ? f->hidden_scale + static_cast<size_t>(kb) * f->T + tok
                                                : f->hidden_scale + static_cast<size_t>(tok) * num_kb + kb);
                 } else {
@@ -887,7 +901,7 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
             bool last = false;
             const int r_mine = (warp - 4) + 8 * lane;
             if (lane < 4 && r_mine < rows_valid) {
-                tok = __ldcg(f->row_token + tile_row0 + r_mine);
+                tok = row_token_of(c, f->row_token, m_tile, tile_row0, r_mine);
                 __threadfence();
                 const int before = atomicAdd(f->tok_done + static_cast<size_t>(tok) * g.n_tiles + n, 1);
                 last = before == __ldcg(f->tok_nlocal + tok) - 1;
@@ -982,23 +996,26 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmA2, const __grid_consta
     // after this one.
     if (blockIdx.x == 0)
         for (int i = threadIdx.x; i < f.num_counters; i += blockDim.x) f.counters_next[i] = 0;
+    __shared__ CtaTiles s_tiles;
+    c.tiles = nullptr;
     if (f.route) {
         // Stages 1 and 2, by every CTA for itself, in the not yet used pipeline stages.
         if (blockIdx.x == 0 && threadIdx.x == 0) *g1.status = DEV_OK;  // first kernel of a forward: clear the fault word
         int* scratch = reinterpret_cast<int*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-        route_permute_in_cta(scratch, f.T, f.E_loc, f.expert_offset, f.row_cap, f.logits, f.bias, f.scaling, f.topk_idx,
+        route_permute_in_cta(scratch, s_tiles, f.T, f.E_loc, f.expert_offset, f.row_cap, f.logits, f.bias, f.scaling, f.topk_idx,
                              f.topk_w_out, f.meta, g1.status);
+        c.tiles = &s_tiles;
     }
 
     // tokens without a local expert: their output rows are zeros, written here by the CTAs in turn
     for (int t = blockIdx.x; t < f.T; t += gridDim.x)
-        if (__ldcg(f.tok_nlocal + t) == 0)
+        if (f.route ? ((s_tiles.none_local >> t) & 1) != 0 : __ldcg(f.tok_nlocal + t) == 0)
             for (int i = threadIdx.x; i < f.H / 8; i += blockDim.x)
                 reinterpret_cast<uint4*>(f.out + static_cast<size_t>(t) * f.H)[i] = make_uint4(0u, 0u, 0u, 0u);
 
     // The CTA's work list: its GEMM1 tiles, then its GEMM2 tiles.
     // Very small batches with few tiles: a tile's K range is cut into parts for different CTAs (KSplit).
-    const int grid = static_cast<int>(gridDim.x), m_tiles = __ldcg(g1.num_m_tiles);
+    const int grid = static_cast<int>(gridDim.x), m_tiles = f.route ? s_tiles.count : __ldcg(g1.num_m_tiles);
     const bool may_split = f.split && f.T <= SPLIT_MAX_TOKENS && g1.num_kb <= SPLIT_MAX_KB && g2.num_kb <= SPLIT_MAX_KB;
     const KSplit ks1 = ksplit_for(g1.num_kb, m_tiles * g1.n_tiles, grid, may_split && m_tiles * g1.n_tiles <= SPLIT_MAX_TILES);
     // (GEMM2's K range is too short for it: counting the parts and the finisher's pass over the stored partial sums

@@ -423,15 +423,27 @@ __global__ void __launch_bounds__(P_TAIL_THREADS) route_permute_kernel(
 static_assert(P_TAIL_THREADS == P_MAX_LOCAL && P_TAIL_THREADS >= P_TAIL_MAX_TOKENS, "a thread per expert, and per token");
 static_assert(TILE_M % ST_ROWS == 0, "sub-tiles do not straddle row tiles");
 
-// Stages 1 and 2 for a batch of at most 32 tokens, computed by ONE thread block for itself: every CTA of the
+// Stages 1 and 2 for a batch of at most 16 tokens, computed by ONE thread block for itself: every CTA of the
 // fused small-batch kernel runs this on the same inputs and writes the same tables (to the same addresses, with
 // the same values), so no CTA ever waits for another one and no separate routing launch is needed.  Same
 // arithmetic and outputs as route_permute_kernel.  `scratch` is RP_CTA_SCRATCH_INTS ints of shared memory;
 // the block needs at least P_MAX_LOCAL threads and T warps are busy at a time.  Ends with a block barrier after
 // which every thread of the block may read the tables.
-constexpr int RP_CTA_MAX_TOKENS = 32;
+// The tiles also stay in shared memory (CtaTiles): read back from global memory, each table cost the roles a round trip to
+// L2 in a chain of three or four before their first loads.
+constexpr int RP_CTA_MAX_TOKENS = 16;
+struct CtaTiles {
+    uint2 tile[RP_CTA_MAX_TOKENS * 8];  // local expert; the set of its tokens, which are its rows in order
+    int count;
+    uint32_t none_local;                // the set of tokens without a local expert
+};
+// the r-th token of a set
+__device__ __forceinline__ int set_member(uint32_t set, int r) {
+    for (; r > 0; --r) set &= set - 1;
+    return __ffs(set) - 1;
+}
 constexpr int RP_CTA_SCRATCH_INTS = RP_CTA_MAX_TOKENS * 8 + P_MAX_LOCAL + 2 * (P_MAX_LOCAL + 1);
-__device__ __forceinline__ void route_permute_in_cta(int* scratch, int T, int E_loc, int off, int row_cap,
+__device__ __forceinline__ void route_permute_in_cta(int* scratch, CtaTiles& tiles, int T, int E_loc, int off, int row_cap,
                                                      const float* __restrict__ logits,
                                                      const __nv_bfloat16* __restrict__ bias, float scaling,
                                                      int* topk_idx, float* topk_w, const PermuteMeta& m, int* status) {
@@ -441,6 +453,7 @@ __device__ __forceinline__ void route_permute_in_cta(int* scratch, int T, int E_
     int* s_pad = s_cnt + P_MAX_LOCAL + 1;                                  // [P_MAX_LOCAL + 1]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     if (tid < P_MAX_LOCAL) mask[tid] = 0u;
+    if (tid == 0) tiles.none_local = 0u;
     {
         float bias_f[8];
         load_bias8(bias, lane, bias_f);
@@ -507,9 +520,10 @@ __device__ __forceinline__ void route_permute_in_cta(int* scratch, int T, int E_
         m.expert_count[tid] = total;
         m.expert_offset[tid] = s_cnt[tid];
         m.padded_offset[tid] = s_pad[tid];
-        // at most RP_CTA_MAX_TOKENS = 32 rows per expert: one row tile, which is also its only sub-tile
+        // at most RP_CTA_MAX_TOKENS rows per expert: one row tile, which is also its only sub-tile
         const int t0 = s_pad[tid] / TILE_M;
         if (total > 0) {
+            tiles.tile[t0] = make_uint2(tid, mask[tid]);
             m.tile_expert[t0] = tid;
             m.tile_rows[t0] = total;
             m.st_expert[t0] = tid;
@@ -518,6 +532,7 @@ __device__ __forceinline__ void route_permute_in_cta(int* scratch, int T, int E_
         }
     }
     if (tid == 0) {  // entries past E_loc count nothing, so entry E_loc already holds the totals
+        tiles.count = s_pad[E_loc] / TILE_M;
         *m.num_m_tiles = s_pad[E_loc] / TILE_M;
         *m.num_st = s_pad[E_loc] / TILE_M;
         m.expert_offset[E_loc] = s_cnt[E_loc];
@@ -544,6 +559,7 @@ __device__ __forceinline__ void route_permute_in_cta(int* scratch, int T, int E_
             m.slot_to_row[tid * 8 + j] = prow;
         }
         m.tok_nlocal[tid] = nlocal;
+        if (nlocal == 0) atomicOr(&tiles.none_local, 1u << tid);
     }
     __syncthreads();
 }
