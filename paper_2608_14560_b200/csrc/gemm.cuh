@@ -278,7 +278,9 @@ struct AheadSeq {  // the first `rounds` rounds of items to `stride` of the CTAs
 };
 // After `before` items dealt by seq_plain: the CTAs that got one item less are the first in every round, and they take up
 // to `ahead` rounds among themselves in front, as far as the items reach whose row tiles the full rounds have finished
-// (n1_tiles items before and n2_tiles new ones belong to a row tile).  (Dealt in plain rounds, 54 tokens on 23 experts left 72 CTAs with 238 K-blocks and 76
+// (n1_tiles items before and n2_tiles new ones belong to a row tile).  Only where the last round before has few items: a
+// CTA streams up to 64 GB/s, so a hundred of them saturate the memory and the idle time of the others costs nothing (with 108
+// or 140 such items a forward took 6 % longer, with 24 or 40 it takes 4-10 % less).  (Dealt in plain rounds, 54 tokens on 23 experts left 72 CTAs with 238 K-blocks and 76
 // with 182; us per forward, plain rounds / these: 54 tokens 175 / 165, 33 tokens on 256 local experts 766 / 752, 8 and
 // 16 tokens up to 6 % less, equal where GEMM1 fills whole rounds.)
 __device__ __forceinline__ AheadSeq seq_after(int before, int ahead, int n1_tiles, int n2_tiles, int count) {
@@ -286,7 +288,7 @@ __device__ __forceinline__ AheadSeq seq_after(int before, int ahead, int n1_tile
     int r = before, rounds = 0;
     if (before >= grid) {  // (below, the smallest batches, no division delays the first weights of the second phase)
         r = before % grid;
-        if (r) rounds = min(ahead, (before - r) / n1_tiles * n2_tiles / (grid - r));
+        if (r && r * 16 <= grid * 9) rounds = min(ahead, (before - r) / n1_tiles * n2_tiles / (grid - r));
     }
     return b < r ? AheadSeq{b - r + grid, rounds, rounds, grid - r, grid, count} : AheadSeq{b - r, 0, rounds, grid - r, grid, count};
 }
