@@ -255,7 +255,8 @@ __global__ void __launch_bounds__(256) place_gather_kernel(int T, int H, int E_l
         const uint32_t local = __ballot_sync(0xffffffffu, prow >= 0);
         if (local == 0) continue;
         const uint4* src = reinterpret_cast<const uint4*>(hidden + static_cast<size_t>(t) * H);
-        for (int c0 = lane; c0 < chunks; c0 += 32 * BATCH) {
+        for (int cb = 0; cb < chunks; cb += 32 * BATCH) {  // (the same number of rounds for all lanes: they shuffle)
+            const int c0 = cb + lane;
             uint4 v[BATCH];
 #pragma unroll
             for (int i = 0; i < BATCH; ++i)

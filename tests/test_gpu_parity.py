@@ -474,6 +474,19 @@ def test_permutation_at_the_edges_of_its_blocks(cuda_device, tokens, eloc, off):
     eng.close()
 
 
+@pytest.mark.parametrize("hidden", [256, 3840, 7424])  # 16, 240 and 464 16-byte chunks in a row
+def test_gather_of_rows_whose_last_round_of_copies_is_half_a_warp(cuda_device, hidden):
+    # a warp copies a row 224 chunks at a time; these leave 16 chunks, half a warp's, for the last round, in which
+    # all lanes still take part in the exchange of the destination rows.  Every gathered byte and scale feeds GEMM1.
+    dims = syn.LayerDims(hidden=hidden, intermediate=128, num_local_experts=64)
+    for layout in (0, 1):
+        wl = _wl(331, dims, seed=hidden + layout, skew=True)
+        inp = syn.make_inputs(wl, cuda_device)
+        if layout:
+            inp["hidden_scale"] = inp["hidden_scale"].t().contiguous()
+        run_and_compare(wl, cuda_device, inp=inp, hidden_scale_layout=layout)
+
+
 # ---- batches of at most 80 tokens: gather, both GEMMs and the combine as one kernel; up to 16 tokens that ----
 # ---- kernel also routes and permutes (every CTA for itself), and the forward is a single launch -------------
 @pytest.mark.parametrize("tokens,kw", [(1, {}), (5, {}), (12, {}), (13, {}), (16, {"local_expert_offset": 64}),
