@@ -134,10 +134,6 @@ struct moe_fp8_handle_s {
     unsigned pipe_calls;
     cudaStream_t s_in, s_out;
     cudaEvent_t ev_in[2], ev_compute[2], ev_out[2];
-    // moe_fp8_forward_host: the stream that brings in the activations beside the routing, and its ordering events
-    bool rows_ready;
-    cudaStream_t s_rows;
-    cudaEvent_t ev_rows[2];
 };
 
 namespace {
@@ -351,12 +347,6 @@ int moe_fp8_destroy(moe_fp8_handle_t h) {
         cudaStreamDestroy(h->s_in);
         cudaStreamDestroy(h->s_out);
     }
-    if (h->rows_ready) {
-        cudaStreamSynchronize(h->s_rows);
-        cudaEventDestroy(h->ev_rows[0]);
-        cudaEventDestroy(h->ev_rows[1]);
-        cudaStreamDestroy(h->s_rows);
-    }
     delete h;
     return MOE_FP8_OK;
 }
@@ -395,11 +385,10 @@ int moe_fp8_set_workspace(moe_fp8_handle_t h, void* ws, size_t bytes) {
 int moe_fp8_last_cuda_error(moe_fp8_handle_t h) { return h ? h->last_cuda_error : 0; }
 int moe_fp8_last_launch_count(moe_fp8_handle_t h) { return h ? h->last_launches : 0; }
 
-// rows_there: event after which hidden_fp8 and hidden_scale may be read (separate-kernel path only), or null.
-static int forward_impl(moe_fp8_handle_t h, int T, const void* hidden_fp8, const float* hidden_scale,
-                        const float* router_logits, const void* routing_bias, const void* w13, const float* w13_scale,
-                        const void* w2, const float* w2_scale, int local_expert_offset, float scaling_factor, void* out,
-                        void* stream_v, cudaEvent_t rows_there) {
+int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const float* hidden_scale,
+                    const float* router_logits, const void* routing_bias, const void* w13, const float* w13_scale,
+                    const void* w2, const float* w2_scale, int local_expert_offset, float scaling_factor, void* out,
+                    void* stream_v) {
     if (!h) return MOE_FP8_ERR_BAD_ARG;
     const moe_fp8_config& c = h->cfg;
     if (T < 0 || T > c.max_tokens) return MOE_FP8_ERR_BAD_ARG;
@@ -586,8 +575,7 @@ static int forward_impl(moe_fp8_handle_t h, int T, const void* hidden_fp8, const
     } else {
         {  // stage 2, continued: placement and gather
             const int grid = min((T + 7) / 8, h->sm_count * 8);
-            if (rows_there && (lerr = cudaStreamWaitEvent(stream, rows_there, 0)) != cudaSuccess) return cuda_fail(h, lerr);
-            MOE_LAUNCH(place_gather_kernel, grid, 256, 0, stream, pdl && !rows_there, T, H, EL, local_expert_offset, row_cap,
+            MOE_LAUNCH(place_gather_kernel, grid, 256, 0, stream, pdl, T, H, EL, local_expert_offset, row_cap,
                        route_count_tokens_per_block(T, EL), c.hidden_scale_layout, static_cast<const int*>(topk_idx),
                        static_cast<const uint8_t*>(hidden_fp8), hidden_scale, m, a1, a1_scale_t, status);
             mark();
@@ -631,14 +619,6 @@ static int forward_impl(moe_fp8_handle_t h, int T, const void* hidden_fp8, const
     h->last_launches = launches;
     h->stage_times_valid = h->stage_timing;
     return MOE_FP8_OK;
-}
-
-int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const float* hidden_scale,
-                    const float* router_logits, const void* routing_bias, const void* w13, const float* w13_scale,
-                    const void* w2, const float* w2_scale, int local_expert_offset, float scaling_factor, void* out,
-                    void* stream_v) {
-    return forward_impl(h, T, hidden_fp8, hidden_scale, router_logits, routing_bias, w13, w13_scale, w2, w2_scale,
-                        local_expert_offset, scaling_factor, out, stream_v, nullptr);
 }
 
 int moe_fp8_debug_set_fault(moe_fp8_handle_t h, int skip_iteration, long long wait_clocks) {
@@ -730,32 +710,14 @@ int moe_fp8_forward_host(moe_fp8_handle_t h, int T, const void* host_hidden_fp8,
     float* d_logits = at<float>(h, h->L.stage_logits);
     void* d_out = at<uint8_t>(h, h->L.stage_out);
     cudaError_t e;
-    // The routing needs the logits only.  Where it is a kernel of its own it runs while the activations, eight times as
-    // many bytes, still come in on a second stream; the gather waits for them.  (us per call, in turn / beside: 459 / 455
-    // at 512 tokens, 917 / 903 at 1172, 1077 / 1067 at 1832.)
-    const bool beside = T > h->fused_max_tokens;
-    if (beside && !h->rows_ready) {  // first use: a stream and two events (host-side objects, no device memory)
-        if ((e = cudaStreamCreateWithFlags(&h->s_rows, cudaStreamNonBlocking)) != cudaSuccess) return cuda_fail(h, e);
-        for (int k = 0; k < 2; ++k)
-            if ((e = cudaEventCreateWithFlags(&h->ev_rows[k], cudaEventDisableTiming)) != cudaSuccess) {
-                if (k) cudaEventDestroy(h->ev_rows[0]);
-                cudaStreamDestroy(h->s_rows);
-                return cuda_fail(h, e);
-            }
-        h->rows_ready = true;
-    }
-    cudaStream_t s_rows = beside ? h->s_rows : stream;
-    // (the staging area may still be read by what was enqueued on `stream` before)
-    if (beside && ((e = cudaEventRecord(h->ev_rows[0], stream)) != cudaSuccess ||
-                   (e = cudaStreamWaitEvent(s_rows, h->ev_rows[0], 0)) != cudaSuccess))
+    if ((e = cudaMemcpyAsync(d_hidden, host_hidden_fp8, Tz * H, cudaMemcpyHostToDevice, stream)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(d_scale, host_hidden_scale, Tz * (H / 128) * 4, cudaMemcpyHostToDevice, stream)) !=
+            cudaSuccess ||
+        (e = cudaMemcpyAsync(d_logits, host_router_logits, Tz * 256 * 4, cudaMemcpyHostToDevice, stream)) !=
+            cudaSuccess)
         return cuda_fail(h, e);
-    if ((e = cudaMemcpyAsync(d_logits, host_router_logits, Tz * 256 * 4, cudaMemcpyHostToDevice, stream)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(d_hidden, host_hidden_fp8, Tz * H, cudaMemcpyHostToDevice, s_rows)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(d_scale, host_hidden_scale, Tz * (H / 128) * 4, cudaMemcpyHostToDevice, s_rows)) != cudaSuccess)
-        return cuda_fail(h, e);
-    if (beside && (e = cudaEventRecord(h->ev_rows[1], s_rows)) != cudaSuccess) return cuda_fail(h, e);
-    int rc = forward_impl(h, T, d_hidden, d_scale, d_logits, routing_bias, w13, w13_scale, w2, w2_scale,
-                          local_expert_offset, scaling_factor, d_out, stream_v, beside ? h->ev_rows[1] : nullptr);
+    int rc = moe_fp8_forward(h, T, d_hidden, d_scale, d_logits, routing_bias, w13, w13_scale, w2, w2_scale,
+                             local_expert_offset, scaling_factor, d_out, stream_v);
     if (rc != MOE_FP8_OK) return rc;
     if ((e = cudaMemcpyAsync(host_out, d_out, Tz * H * 2, cudaMemcpyDeviceToHost, stream)) != cudaSuccess)
         return cuda_fail(h, e);

@@ -169,6 +169,35 @@ def test_host_entry_point_matches_device_entry_point(cuda_device):
     eng.close()
 
 
+@pytest.mark.parametrize("tokens", [300, 20])  # separate kernels | fused kernel
+def test_host_calls_in_a_row_with_other_inputs_each(cuda_device, tokens):
+    # on one handle and on a side stream, the batch before always half as long or twice as long; a forward from hidden
+    # states, which fills the same staging areas, in between
+    wl = _wl(tokens, seed=14)
+    weights = syn.make_inputs(wl, cuda_device)
+    eng = make_engine(wl, cuda_device)
+    side = torch.cuda.Stream(device=cuda_device)
+    r = syn.make_router_inputs(wl, cuda_device)
+    want_hidden = eng.forward_from_hidden({**weights, **r}).clone()
+    torch.cuda.synchronize()
+    for i in range(4):
+        b = syn.make_inputs(_wl(tokens if i % 2 else tokens // 2, seed=15 + i), cuda_device)
+        acts = {k: b[k] for k in ("hidden_fp8", "hidden_scale", "router_logits")}
+        want = eng.forward({**weights, **acts}).cpu()
+        host = {k: v.cpu().pin_memory() for k, v in acts.items()}
+        host_out = torch.empty(want.shape, dtype=torch.bfloat16).pin_memory()
+        with torch.cuda.stream(side):
+            eng.forward_host(host, weights, host_out)
+            got_hidden = eng.forward_from_hidden({**weights, **r})
+            for v in host.values():  # the call has returned: its buffers are the caller's again
+                v.view(torch.uint8).fill_(0xFF)
+        assert torch.equal(want.view(torch.int16), host_out.view(torch.int16)), f"call {i}"
+        side.synchronize()
+        assert eng.status() == 0
+        assert torch.equal(got_hidden.view(torch.int16), want_hidden.view(torch.int16)), f"call {i}"
+    eng.close()
+
+
 def test_forward_on_a_side_stream_and_after_a_change_of_weights(cuda_device):
     # the forward is enqueued on the caller's current stream; the TMA descriptors of the weights are cached
     # per pointer pair and must be rebuilt when other weight tensors are passed
