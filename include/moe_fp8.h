@@ -17,7 +17,8 @@
  *   - The library never allocates, frees or retains caller tensors; scratch
  *     memory is one caller-owned workspace (moe_fp8_set_workspace).
  *   - Functions return 0 on success and a negative MOE_FP8_ERR_* otherwise; on
- *     error nothing has been enqueued.  There is no CPU fallback: without a
+ *     error nothing has been enqueued (except MOE_FP8_ERR_CUDA: what came before
+ *     the CUDA call that failed).  There is no CPU fallback: without a
  *     compute-capability 10.x device moe_fp8_create fails.
  *   - moe_fp8_forward only enqueues work on `stream` and returns; faults found
  *     on the device (a bounded wait that gave up, an out-of-range row) are

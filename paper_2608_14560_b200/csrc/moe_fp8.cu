@@ -385,6 +385,15 @@ int moe_fp8_set_workspace(moe_fp8_handle_t h, void* ws, size_t bytes) {
 int moe_fp8_last_cuda_error(moe_fp8_handle_t h) { return h ? h->last_cuda_error : 0; }
 int moe_fp8_last_launch_count(moe_fp8_handle_t h) { return h ? h->last_launches : 0; }
 
+// The arguments that all entry points pass on to moe_fp8_forward.  Those that enqueue work in front of it look at them
+// first: a rejected call has enqueued nothing.
+static bool layer_args_ok(moe_fp8_handle_t h, const void* routing_bias, const void* w13, const float* w13_scale,
+                          const void* w2, const float* w2_scale, int local_expert_offset) {
+    return local_expert_offset >= 0 && local_expert_offset <= h->cfg.num_experts - h->cfg.num_local_experts &&
+           routing_bias && w13 && w13_scale && w2 && w2_scale && !misaligned(routing_bias) && !misaligned(w13) &&
+           !misaligned(w13_scale) && !misaligned(w2) && !misaligned(w2_scale);
+}
+
 int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const float* hidden_scale,
                     const float* router_logits, const void* routing_bias, const void* w13, const float* w13_scale,
                     const void* w2, const float* w2_scale, int local_expert_offset, float scaling_factor, void* out,
@@ -392,11 +401,7 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
     if (!h) return MOE_FP8_ERR_BAD_ARG;
     const moe_fp8_config& c = h->cfg;
     if (T < 0 || T > c.max_tokens) return MOE_FP8_ERR_BAD_ARG;
-    if (local_expert_offset < 0 || local_expert_offset + c.num_local_experts > c.num_experts)
-        return MOE_FP8_ERR_BAD_ARG;
-    if (!routing_bias || !w13 || !w13_scale || !w2 || !w2_scale || misaligned(routing_bias) || misaligned(w13) ||
-        misaligned(w13_scale) || misaligned(w2) || misaligned(w2_scale))
-        return MOE_FP8_ERR_BAD_ARG;
+    if (!layer_args_ok(h, routing_bias, w13, w13_scale, w2, w2_scale, local_expert_offset)) return MOE_FP8_ERR_BAD_ARG;
     if (T > 0 && (!hidden_fp8 || !hidden_scale || !router_logits || !out || misaligned(hidden_fp8) ||
                   misaligned(hidden_scale) || misaligned(router_logits) || misaligned(out)))
         return MOE_FP8_ERR_BAD_ARG;
@@ -703,6 +708,7 @@ int moe_fp8_forward_host(moe_fp8_handle_t h, int T, const void* host_hidden_fp8,
     if (!h->ws) return MOE_FP8_ERR_NO_WORKSPACE;
     if (T == 0) return moe_fp8_forward(h, 0, nullptr, nullptr, nullptr, routing_bias, w13, w13_scale, w2, w2_scale,
                                        local_expert_offset, scaling_factor, nullptr, stream_v);
+    if (!layer_args_ok(h, routing_bias, w13, w13_scale, w2, w2_scale, local_expert_offset)) return MOE_FP8_ERR_BAD_ARG;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_v);
     const size_t H = h->cfg.hidden, Tz = T;
     uint8_t* d_hidden = at<uint8_t>(h, h->L.stage_hidden);
@@ -734,6 +740,9 @@ int moe_fp8_forward_from_hidden(moe_fp8_handle_t h, int T, const void* hidden_bf
     if (!router_weight || misaligned(router_weight) || (T > 0 && (!hidden_bf16 || misaligned(hidden_bf16))))
         return MOE_FP8_ERR_BAD_ARG;
     if (!h->ws) return MOE_FP8_ERR_NO_WORKSPACE;
+    if (!layer_args_ok(h, routing_bias, w13, w13_scale, w2, w2_scale, local_expert_offset) ||
+        (T > 0 && (!out || misaligned(out))))
+        return MOE_FP8_ERR_BAD_ARG;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_v);
     const int H = h->cfg.hidden, E = h->cfg.num_experts;
     uint8_t* d_hidden = at<uint8_t>(h, h->L.stage_hidden);
@@ -789,6 +798,7 @@ int moe_fp8_forward_host_async(moe_fp8_handle_t h, int T, const void* host_hidde
         return MOE_FP8_ERR_BAD_ARG;
     if (!h->ws) return MOE_FP8_ERR_NO_WORKSPACE;
     if (T == 0) return MOE_FP8_OK;
+    if (!layer_args_ok(h, routing_bias, w13, w13_scale, w2, w2_scale, local_expert_offset)) return MOE_FP8_ERR_BAD_ARG;
     cudaError_t e;
     if (!h->pipe_ready) {  // first use: two copy streams and six events (host-side objects, no device memory)
         if ((e = cudaStreamCreateWithFlags(&h->s_in, cudaStreamNonBlocking)) != cudaSuccess) return cuda_fail(h, e);

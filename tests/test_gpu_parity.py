@@ -198,6 +198,39 @@ def test_host_calls_in_a_row_with_other_inputs_each(cuda_device, tokens):
     eng.close()
 
 
+@pytest.mark.parametrize("tokens", [300, 20])  # separate kernels | fused kernel
+def test_a_rejected_call_has_enqueued_nothing(cuda_device, tokens):
+    # the entry points that copy or compute something in front of the forward: after one that returned an argument
+    # error the staging areas still hold what the last accepted call fed to the forward, and the next call is right
+    wl = _wl(tokens, seed=16)
+    inp = syn.make_inputs(wl, cuda_device)
+    acts = {k: inp[k] for k in ("hidden_fp8", "hidden_scale", "router_logits")}
+    other = {k: v.cpu().pin_memory() for k, v in syn.make_activations(wl, 17, cuda_device).items()}
+    r = {"hidden_bf16": (torch.ones(tokens, 512, device=cuda_device) * 3).bfloat16(),
+         "router_weight": torch.ones(256, 512, device=cuda_device).bfloat16()}
+    host = {k: v.cpu().pin_memory() for k, v in acts.items()}
+    host_out = torch.empty(tokens, 512, dtype=torch.bfloat16).pin_memory()
+    eng = make_engine(wl, cuda_device)
+    want = eng.forward(inp).cpu()
+    shifted = torch.zeros(inp["w2"].numel() + 16, dtype=torch.uint8, device=cuda_device)[1:]
+    for bad in ({"local_expert_offset": 250}, {"local_expert_offset": -1}, {"w2": shifted}, {"w13_scale": None}):
+        for entry in (lambda w: eng.forward_host(other, w, host_out), lambda w: eng.forward_host_async(other, w, host_out),
+                      lambda w: eng.forward_from_hidden({**w, **r})):
+            eng.forward_host(host, inp, host_out)
+            with pytest.raises(MoeFp8Error) as ei:
+                entry({**inp, **bad})
+            assert ei.value.rc == -1
+            torch.cuda.synchronize()
+            fed = eng.debug_export_inputs(tokens)
+            assert torch.equal(fed["router_logits"], acts["router_logits"])
+            assert torch.equal(fed["hidden_fp8"], acts["hidden_fp8"].view(torch.uint8))
+            assert torch.equal(fed["hidden_scale"], acts["hidden_scale"])
+    host_out.zero_()
+    eng.forward_host(host, inp, host_out)
+    assert eng.status() == 0 and torch.equal(host_out.view(torch.int16), want.view(torch.int16))
+    eng.close()
+
+
 def test_forward_on_a_side_stream_and_after_a_change_of_weights(cuda_device):
     # the forward is enqueued on the caller's current stream; the TMA descriptors of the weights are cached
     # per pointer pair and must be rebuilt when other weight tensors are passed
