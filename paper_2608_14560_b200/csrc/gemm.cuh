@@ -215,6 +215,7 @@ struct GemmCtrl {
     uint32_t tmem_slot;
     int abort_flag;
     int split_last;            // fused kernel, K split: this CTA stored the last part of the tile
+    uint32_t gathered;         // fused kernel: stages the gather warp has arrived at
     uint64_t sched_full[SCHED_SLOTS];   // grouped_mlp_kernel: the work list, published tile by tile
     uint64_t sched_rows[SCHED_SLOTS];   // the tile's token rows are in memory
     TileInfo sched[SCHED_SLOTS];
@@ -392,20 +393,21 @@ __device__ __forceinline__ void producer_tiles(const Cta& c, const CUtensorMap* 
             // The tile's A rows are GEMM1's output and must have been stored; its weights need not wait for
             // that, so the B tiles of the first K-blocks go out before the counter is looked at.
             const int npre = kb1 - kb0 < GEO::STAGES ? kb1 - kb0 : GEO::STAGES;
-            for (int k = 0; k < npre && ok; ++k) {
-                ok = claim(it + k);
-                if (ok) load_b(it + k, kb0 + k);
+            int pre = 0;  // stages claimed
+            while (pre < npre && (ok = claim(it + pre))) {
+                load_b(it + pre, kb0 + pre);
+                ++pre;
             }
-            if (!ok) break;
-            if (!wait_counter(f->ready + m_tile, ready_target, c.abort_flag, c.limit)) {
+            if (ok && !wait_counter(f->ready + m_tile, ready_target, c.abort_flag, c.limit)) {
                 raise(ctrl, g.status, DEV_TIMEOUT_READY);
                 ok = false;
-                break;
             }
             fence_proxy_async();  // the rows were stored by other CTAs' copy engines; order our copies behind the acquire
-            for (int k = 0; k < npre; ++k) load_a(it + k, kb0 + k);
-            it += npre;
-            kb = kb0 + npre;
+            // (after a time-out as well, when nobody reads them: a claimed stage is complete with its token rows only, and
+            // drain_after_abort waits for the claimed stages)
+            for (int k = 0; k < pre; ++k) load_a(it + k, kb0 + k);
+            it += pre;
+            kb = kb0 + pre;
         }
         for (; kb < kb1 && ok; ++kb, ++it) {
             ok = claim(it);
@@ -416,26 +418,29 @@ __device__ __forceinline__ void producer_tiles(const Cta& c, const CUtensorMap* 
     }
 }
 
-// Before the producer thread may reach the end of the kernel every copy it issued has to have landed (bounded
-// wait).  On the regular path the MMA issuers have consumed all of them long ago and these waits fall through;
-// after an abort raised by any role they are what keeps the copy engine from writing into shared memory of a
-// CTA that has exited.
+// After an abort, all roles having ended: the copies and MMAs that are still under way have to finish before the CTA
+// gives up its shared and its tensor memory.  The producer thread waits for the stages it claimed last (`it` of them in
+// all; the others were consumed), after making up for the arrivals of a gather warp that stopped before it (`gathered`
+// stages); the issuer threads wait for their own MMAs.  What is waited for is in the hands of the hardware, so the
+// limit is the default one even where a test has shortened that of the roles.  On the regular path the epilogue has waited
+// for every MMA and these for every copy, and nothing is left to wait for.
 template <class GEO>
-__device__ __forceinline__ void producer_drain(const Cta& c, int* status, uint32_t it) {
+__device__ __forceinline__ void drain_after_abort(const Cta& c, int* status, uint32_t it, uint32_t gathered) {
     int zero = 0;
-    const uint32_t n_back = it < GEO::STAGES ? it : GEO::STAGES;
-    for (uint32_t j = it - n_back; j < it; ++j)
-        if (!mbar_wait(smem_u32(&c.ctrl->full[j % GEO::STAGES]), (j / GEO::STAGES) & 1, &zero, c.limit))
-            atomicCAS(status, DEV_OK, DEV_TIMEOUT_DRAIN);
-}
-
-// After an abort: let issued MMAs retire before TMEM is released.
-__device__ __forceinline__ void issuer_drain(const Cta& c, uint32_t mine, bool ok) {
-    if (!ok || *c.abort_flag) {
-        umma_commit(smem_u32(&c.ctrl->drain_bar[mine]));
-        int zero = 0;
-        mbar_wait(smem_u32(&c.ctrl->drain_bar[mine]), 0, &zero, c.limit);
+    if (c.warp == 0 && c.lane == 0) {
+        for (uint32_t j = it < GEO::STAGES ? 0u : it - GEO::STAGES; j < it; ++j) {
+            const uint32_t bar = smem_u32(&c.ctrl->full[j % GEO::STAGES]);
+            if (j >= gathered) mbar_arrive_n(bar, 32);
+            if (!mbar_wait(bar, (j / GEO::STAGES) & 1, &zero)) atomicCAS(status, DEV_OK, DEV_TIMEOUT_DRAIN);
+        }
+    } else if ((c.warp == 1 || c.warp == 2) && c.lane == 0) {
+        const uint32_t bar = smem_u32(&c.ctrl->drain_bar[c.warp - 1]);
+        umma_commit(bar);
+        if (!mbar_wait(bar, 0, &zero)) atomicCAS(status, DEV_OK, DEV_TIMEOUT_DRAIN);
     }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
 }
 
 // ---------------- gather warp (fused kernel) ----------------
@@ -1035,15 +1040,14 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmA2, const __grid_consta
         if (c.warp == 0 && c.lane == 0) {
             producer_tiles<1, GEO>(c, &tmA2, &tmB1, g1, &f, 0, tr1, it, ok, ks1);
             producer_tiles<2, GEO>(c, &tmA2, &tmB2, g2, &f, g1.n_tiles, tr2(), it, ok, ks2);
-            producer_drain<GEO>(c, g1.status, it);
         } else if ((c.warp == 1 || c.warp == 2) && c.lane == 0) {
             issuer_tiles_wm<GEO>(c, g1, tr1, c.warp - 1, it, ok, ks1);
             issuer_tiles_wm<GEO>(c, g2, tr2(), c.warp - 1, it, ok, ks2);
-            issuer_drain(c, c.warp - 1, ok);
         } else if (c.warp == 3) {
             gather_tiles<GEO>(c, g1, f, tr1, it, ok, ks1);
             gather_idle_tiles<GEO>(c, g2, tr2(), it, ok, ks2);
             cp_async_wait_all();  // nothing may still be landing in shared memory when the CTA exits
+            if (c.lane == 0) c.ctrl->gathered = it;
         }
     } else {
         reg_alloc<232>();
@@ -1052,8 +1056,10 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmA2, const __grid_consta
         epilogue_tiles_wm<2, true, GEO>(c, g2, &f, tr2(), it, tile_iter, sync_iter, ok, ks2);
     }
 
+    __syncwarp();
     tc_fence_before();
     __syncthreads();
+    if (*c.abort_flag) drain_after_abort<GEO>(c, g1.status, it, c.ctrl->gathered);
     if (c.warp == 1) {
         __syncwarp();
         tmem_dealloc(c.tmem_base, G_TMEM_COLS);

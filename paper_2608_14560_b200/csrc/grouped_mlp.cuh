@@ -61,8 +61,9 @@ __device__ __forceinline__ TileInfo next_tile_warp(const Cta& c, uint32_t i) {
 // All three maps see the weights as [expert][half][row][K]; a stage takes two boxes of 128 rows.
 // Refilling a freed stage is part of the loop that bounds a large batch, so this thread waits for nothing in global
 // memory: with the ticket and the table entries of the next tile fetched here, a GEMM1 tile took 1 us longer.
+// Returns the number of stages it has claimed.
 template <class GEO>
-__device__ __forceinline__ void mlp_producer(const Cta& c, const CUtensorMap* tmA1, const CUtensorMap* tmA1s,
+__device__ __forceinline__ uint32_t mlp_producer(const Cta& c, const CUtensorMap* tmA1, const CUtensorMap* tmA1s,
                                              const CUtensorMap* tmB1n, const CUtensorMap* tmB1m, const CUtensorMap* tmA2,
                                              const CUtensorMap* tmA2s, const CUtensorMap* tmB2, const MlpArgs& a) {
     GemmCtrl* ctrl = c.ctrl;
@@ -109,9 +110,9 @@ __device__ __forceinline__ void mlp_producer(const Cta& c, const CUtensorMap* tm
         if (!waited || !rows_there) {
             // The token rows may not be there yet, the weights are: those of the first stages go out at once.
             const int npre = num_kb < GEO::STAGES ? num_kb : GEO::STAGES;
-            for (int k = 0; k < npre && ok; ++k) {
-                ok = claim(it + k);
-                if (ok) load_b(it + k, k);
+            while (kb < npre && (ok = claim(it + kb))) {
+                load_b(it + kb, kb);
+                ++kb;
             }
             if (!waited) {
                 pdl_wait();
@@ -121,15 +122,15 @@ __device__ __forceinline__ void mlp_producer(const Cta& c, const CUtensorMap* tm
                 ok = mbar_wait(rows_bar, rows_ph, c.abort_flag, 8 * c.limit);
                 if (!ok) raise(ctrl, a.g1.status, DEV_TIMEOUT_READY);
             }
-            if (!ok) break;
             fence_proxy_async();
-            for (int k = 0; k < npre; ++k) load_a(it + k, k);
-            it += npre;
-            kb = npre;
+            // (after a time-out as well, when nobody reads them: a claimed stage is complete with its token rows only, and
+            // drain_after_abort waits for the claimed stages)
+            for (int k = 0; k < kb; ++k) load_a(it + k, k);
+            it += kb;
         } else if (must_wait) {
             fence_proxy_async();  // stored by other CTAs' copy engines; order our copies behind the barrier
         }
-        for (; kb < num_kb; ++kb, ++it) {
+        for (; kb < num_kb && ok; ++kb, ++it) {
             ok = claim(it);
             if (!ok) break;
             load_b(it, kb);  // (first: it may have to come from HBM, the token rows are in L2)
@@ -137,7 +138,7 @@ __device__ __forceinline__ void mlp_producer(const Cta& c, const CUtensorMap* tm
         }
     }
     if (!waited) pdl_wait();
-    producer_drain<GEO>(c, a.g1.status, it);
+    return it;
 }
 
 // ---------------- MMA issuers (two warps) ----------------
@@ -198,7 +199,6 @@ __device__ __forceinline__ void mlp_issuer(const Cta& c, const MlpArgs& a, uint3
         }
     }
     if (it > mine) bar_sync(ACC_BARRIER + mine, ACC_BARRIER_THREADS);  // the buffer's last hand-over
-    if (c.lane == 0) issuer_drain(c, mine, ok);
 }
 
 // ---------------- factor warp, which is also the tile scheduler ----------------
@@ -598,11 +598,12 @@ grouped_mlp_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_consta
     if (c.warp != 0 && c.warp != 3) pdl_wait();
     c.tmem_base = *reinterpret_cast<volatile uint32_t*>(&c.ctrl->tmem_slot);
     c.limit = a.g1.wait_limit;
+    uint32_t claimed = 0;
 
     if (c.warp < 4) {
         reg_dealloc<56>();
         if (c.warp == 0) {
-            if (c.lane == 0) mlp_producer<GEO>(c, &tmA1, &tmA1s, &tmB1n, &tmB1m, &tmA2, &tmA2s, &tmB2, a);
+            if (c.lane == 0) claimed = mlp_producer<GEO>(c, &tmA1, &tmA1s, &tmB1n, &tmB1m, &tmA2, &tmA2s, &tmB2, a);
         } else if (c.warp == 3) {
             mlp_factors<GEO>(c, a);
         } else {
@@ -616,6 +617,7 @@ grouped_mlp_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_consta
     __syncwarp();
     tc_fence_before();
     __syncthreads();
+    if (*c.abort_flag) drain_after_abort<GEO>(c, a.g1.status, claimed, claimed);
     if (c.warp == 1) {
         __syncwarp();
         tmem_dealloc(c.tmem_base, G_TMEM_COLS);
