@@ -36,11 +36,15 @@ struct MlpArgs {
     int* ready;          // [row tiles] warps that have stored their part, zero at launch
 };
 
-// Entry i of the CTA's work list, as the factor warp published it; the wait is bounded and outlasts every other one.
+// Entry i of the CTA's work list, as the factor warp published it.  A role that gave up here while the others went on
+// would leave them at a named barrier, whose wait has no limit (see mlp_issuer), so this wait has to outlast every chain of
+// waits in front of an entry or the list's end, and its limit is not the one that a test may shorten: with that, a role that
+// looked for its first entry before it was published could take the list for empty.
+constexpr long long SCHED_LIMIT_CLOCKS = 16 * WAIT_LIMIT_CLOCKS;
 __device__ __forceinline__ TileInfo next_tile(const Cta& c, uint32_t i) {
     int zero = 0;
     const uint32_t slot = i % SCHED_SLOTS;
-    if (!mbar_wait(smem_u32(&c.ctrl->sched_full[slot]), (i / SCHED_SLOTS) & 1, &zero, 16 * c.limit)) return TileInfo{};
+    if (!mbar_wait(smem_u32(&c.ctrl->sched_full[slot]), (i / SCHED_SLOTS) & 1, &zero, SCHED_LIMIT_CLOCKS)) return TileInfo{};
     const int4 v = ld_shared_v4(smem_u32(&c.ctrl->sched[slot]));
     return TileInfo{v.x, v.y, v.z, v.w};
 }

@@ -356,7 +356,8 @@ def test_a_wait_that_runs_out_is_reported_and_the_handle_stays_usable(cuda_devic
 
 
 @pytest.mark.parametrize("tokens,eloc", [(9, 32), (48, 32), (200, 32), (300, 32), (2000, 256)])
-def test_an_abort_leaves_nothing_under_way(cuda_device, tokens, eloc):
+@pytest.mark.parametrize("clocks", [1 << 16, 1])  # 1: the roles give up before others have begun, copies still in flight
+def test_an_abort_leaves_nothing_under_way(cuda_device, tokens, eloc, clocks):
     # one launch | fused behind the routing kernel | a launch per GEMM | both GEMMs in one, the last with lists of
     # several tiles per CTA.  The copy producer stops at its first few stages, before and behind a full ring and a tile's
     # end: what was claimed and issued by then has to be waited for (status 5 would say that it was not all there), and the
@@ -367,15 +368,15 @@ def test_an_abort_leaves_nothing_under_way(cuda_device, tokens, eloc):
     want = eng.forward(inp).clone()
     torch.cuda.synchronize()
     assert eng.status() == 0
-    for skip in (0, 1, 2, 3, 4, 5, 6, 7, 9):
-        eng.debug_set_fault(skip_iteration=skip, wait_clocks=1 << 16)
+    for skip in (0, 1, 2, 3, 4, 5, 6, 7, 9) + ((-1,) if clocks == 1 else ()):
+        eng.debug_set_fault(skip_iteration=skip, wait_clocks=clocks)
         eng.forward(inp)
         eng.debug_set_fault(-1, 0)
         got = eng.forward(inp)
         torch.cuda.synchronize()
         assert eng.status() == 0
         assert torch.equal(got.view(torch.int16), want.view(torch.int16)), skip
-        eng.debug_set_fault(skip_iteration=skip, wait_clocks=1 << 16)
+        eng.debug_set_fault(skip_iteration=skip, wait_clocks=clocks)
         eng.forward(inp)
         torch.cuda.synchronize()
         assert eng.status() in (0, 1, 2, 3, 4, 8), skip
