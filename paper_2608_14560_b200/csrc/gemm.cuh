@@ -914,7 +914,10 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
                 last = before == __ldcg(f->tok_nlocal + tok) - 1;
             }
             uint32_t todo = __ballot_sync(0xffffffffu, last);
-            if (todo) __threadfence();
+            if (todo) {
+                __threadfence();
+                __syncwarp();  // (a vote orders no memory: the counting lanes' fences come before all lanes' loads)
+            }
             while (todo) {
                 const int src = __ffs(todo) - 1;
                 todo &= todo - 1;

@@ -324,7 +324,9 @@ __device__ __forceinline__ void mlp_factors(const Cta& c, const MlpArgs& a) {
                     there = wait_counter(a.ready + t.m_tile(), ready_target, c.abort_flag, 4 * c.limit);
                 if (there) mbar_arrive(smem_u32(&ctrl->sched_rows[fi % SCHED_SLOTS]));
             }
-            if (!__shfl_sync(0xffffffffu, there, 0)) {
+            there = __shfl_sync(0xffffffffu, there, 0);
+            __syncwarp();  // a shuffle orders no memory: lane 0 has seen the rows announced, all lanes fetch their scales
+            if (!there) {
                 if (lane == 0) raise(ctrl, a.g1.status, DEV_TIMEOUT_READY);
                 return false;
             }
