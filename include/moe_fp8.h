@@ -206,7 +206,7 @@ int moe_fp8_set_small_batch_fusion(moe_fp8_handle_t h, int enable);
 int moe_fp8_debug_set_k_split(moe_fp8_handle_t h, int enable);
 
 /*
- * Inside the two large-tile GEMM kernels a row tile that holds at most 32 rows (an expert's short last tile) is
+ * Inside the large-tile GEMM kernel a row tile that holds at most 32 rows (an expert's short last tile) is
  * worked on with the operands swapped -- weights on the M side of the MMAs, the 32 token rows on N, a 64-column
  * accumulator -- instead of as a full 128-row tile: same arithmetic, bit-identical results, less tensor and
  * epilogue time.  This hook sets the batch size from which that applies (min_tokens = 0: never).
@@ -216,11 +216,12 @@ int moe_fp8_debug_set_short_tiles(moe_fp8_handle_t h, int min_tokens);
 /*
  * Test hook for the failure path of the bounded device waits (every wait on an mbarrier inside the GEMM
  * kernels gives up after a limit, records a fault code in the status word and lets the kernel return with
- * its tensor memory released).  skip_iteration >= 0: in the next forwards the copy producer of every CTA
- * of the GEMM1 kernel stops before its skip_iteration-th pipeline stage, so the consumers wait for a stage
- * that nothing fills; wait_clocks > 0 shortens the limit of every wait to that many SM clocks (0 restores
- * the default of about a second).  skip_iteration < 0 switches the hook off.  Nothing traps: the forward
- * returns normally, its output is garbage and the status word holds a time-out code (1..5, 8).
+ * its copies landed and its tensor memory released).  skip_iteration >= 0: in the next forwards the copy
+ * producer of every CTA stops before its skip_iteration-th pipeline stage if that belongs to GEMM1, so the
+ * consumers wait for a stage that nothing fills; wait_clocks > 0 shortens the limit of these waits to that
+ * many SM clocks (0 restores the default of about a second).  skip_iteration < 0 switches the hook off.
+ * Nothing traps: the forward returns normally, its output is garbage and the status word holds a time-out
+ * code (1..5, 8): that of the wait that gave up first, in whichever CTA.
  */
 int moe_fp8_debug_set_fault(moe_fp8_handle_t h, int skip_iteration, long long wait_clocks);
 

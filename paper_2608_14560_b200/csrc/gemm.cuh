@@ -3,7 +3,7 @@
 // fused into its epilogue, and GEMM2 [rows,I] x w2[e]^T writing bf16 rows for
 // the combine.
 //
-// One persistent CTA per SM walks a static list of 128 x 256 output tiles.
+// One persistent CTA per SM works through a list of 128 x 256 output tiles (grouped_mlp.cuh says how it comes about).
 //   warp 0      TMA producer.  Per K-block (128 K-bytes = one scale block): the A
 //               tile (128 rows) and the B tile (256 weight rows) into a 4-stage ring
 //               (128-byte swizzle), completion on mbarriers.
@@ -16,7 +16,7 @@
 //               Every K-block starts from zero because its partial sum must be
 //               multiplied by fp32 scales before it joins the running sum.
 //   warp 3      factors: activation scale x weight scale per row and column half,
-//               into an 8-slot ring (factor_tiles).
+//               into an 8-slot ring (mlp_factors).
 //   warps 4-7   epilogue of columns [0,128), warps 8-11 of columns [128,256): read
 //               the partial from TMEM, multiply by a_scale[row,kb] * w_scale[nblk,kb]
 //               with packed fp32 FMAs, accumulate in registers; at the end of the
@@ -90,7 +90,7 @@ constexpr int F_RAW_FLOATS = F_SLOTS * TILE_M + F_SLOTS * F_RUN * 2;
 template <int STAGES_, int A_ROWS_, int SCALE_SLOTS_, int STORE_BYTES_, bool FACTORS_>
 struct Geometry {
     static constexpr int STAGES = STAGES_, A_ROWS = A_ROWS_, SCALE_SLOTS = SCALE_SLOTS_;
-    static constexpr bool FACTORS = FACTORS_;                        // see factor_tiles
+    static constexpr bool FACTORS = FACTORS_;                        // see mlp_factors
     static constexpr int A_BYTES = A_ROWS_ * G_BLOCK_K;
     static constexpr int STAGE_BYTES = A_BYTES + G_B_BYTES;
     static constexpr int SCALE_BYTES = A_ROWS_ * 4;                  // per K-block

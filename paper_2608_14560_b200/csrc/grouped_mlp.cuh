@@ -122,7 +122,7 @@ __device__ __forceinline__ uint32_t mlp_producer(const Cta& c, const CUtensorMap
                 pdl_wait();
                 waited = true;
             }
-            if (ok && !rows_there) {  // (longer than the factor warp's wait for the same rows)
+            if (ok && !rows_there) {  // (8: longer than the factor warp's wait for the same rows)
                 ok = mbar_wait(rows_bar, rows_ph, c.abort_flag, 8 * c.limit);
                 if (!ok) raise(ctrl, a.g1.status, DEV_TIMEOUT_READY);
             }
@@ -320,7 +320,12 @@ __device__ __forceinline__ void mlp_factors(const Cta& c, const MlpArgs& a) {
             publish(false);
             bool there = true;
             if (lane == 0) {
-                if (!m1 && a.phases == 3)  // (longer than the other waits: another CTA's may have to run out first)
+                // (Four limits, so that this warp is not the first to give up when another CTA's roles wait in vain: the
+                // status word then says which wait it was.  The bound on the whole is one limit all the same: meanwhile
+                // this warp holds back its arrivals on done[], and the other roles of the CTA, once they wait for those,
+                // give up after one, which ends this wait as well.  Rows that never come are thus reported as the time-out
+                // of whichever role that is.)
+                if (!m1 && a.phases == 3)
                     there = wait_counter(a.ready + t.m_tile(), ready_target, c.abort_flag, 4 * c.limit);
                 if (there) mbar_arrive(smem_u32(&ctrl->sched_rows[fi % SCHED_SLOTS]));
             }

@@ -181,8 +181,8 @@ __global__ void __launch_bounds__(WARPS * 32) route_count_kernel(
     const int e = tid & (ep - 1), q = tid / ep;
     const bool mine = q < groups && e < E_loc;
     const int b0 = min(nblk, q * per), b1 = min(nblk, b0 + per);
-    // (the first HELD counts of a range stay in registers, which is all of them up to 4096 tokens on 32 experts: one round
-    // trip to L2 instead of two chains of them)
+    // (the first HELD counts of a range stay in registers, which is all of them up to 16384 tokens on 32 experts and 2048
+    // on 256: one round trip to L2 instead of two chains of them)
     constexpr int HELD = 16;
     int* hist = m.block_hist + static_cast<size_t>(b0) * E_loc + e;
     int held[HELD], sum = 0;

@@ -17,7 +17,7 @@ enum : int {
     DEV_TIMEOUT_DRAIN = 5,     // in-flight copies did not land during abort
     DEV_BAD_ROW = 6,           // a computed row index fell outside its buffer
     DEV_BAD_TICKET = 7,        // the last-block ticket counter in the workspace was not zero at launch
-    DEV_TIMEOUT_READY = 8,     // fused kernel: the rows a GEMM2 tile reads were never announced
+    DEV_TIMEOUT_READY = 8,     // the rows a GEMM2 tile reads were never announced (one launch for both GEMMs)
 };
 
 // Clocks a bounded wait spins before it gives up (about a second at 2 GHz).
