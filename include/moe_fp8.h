@@ -214,6 +214,14 @@ int moe_fp8_debug_set_k_split(moe_fp8_handle_t h, int enable);
 int moe_fp8_debug_set_short_tiles(moe_fp8_handle_t h, int min_tokens);
 
 /*
+ * Where both GEMMs run in one launch, a CTA that is through with its own list of GEMM1 tiles takes over the lists of
+ * CTAs that have not started yet (two forwards may share the GPU).  This hook makes that certain: the first `lists`
+ * CTAs leave theirs unclaimed and take none, so that other CTAs work through them (0 switches it off; less than
+ * the number of CTAs, which is the number of SMs).
+ */
+int moe_fp8_debug_set_unclaimed_lists(moe_fp8_handle_t h, int lists);
+
+/*
  * Test hook for the failure path of the bounded device waits (every wait on an mbarrier inside the GEMM
  * kernels gives up after a limit, records a fault code in the status word and lets the kernel return with
  * its copies landed and its tensor memory released).  skip_iteration >= 0: in the next forwards the copy

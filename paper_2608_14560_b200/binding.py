@@ -20,7 +20,7 @@ EXPORTS = (
     "moe_fp8_get_stage_times", "moe_fp8_expert_histogram_static", "moe_fp8_debug_set_fault",
     "moe_fp8_debug_sigmoid", "moe_fp8_forward_from_hidden", "moe_fp8_debug_export_inputs",
     "moe_fp8_set_small_batch_fusion", "moe_fp8_forward_host_async", "moe_fp8_host_sync",
-    "moe_fp8_debug_set_short_tiles", "moe_fp8_debug_set_k_split",
+    "moe_fp8_debug_set_short_tiles", "moe_fp8_debug_set_k_split", "moe_fp8_debug_set_unclaimed_lists",
 )
 
 
@@ -91,6 +91,8 @@ def load_library() -> C.CDLL:
         lib.moe_fp8_debug_set_k_split.restype = C.c_int
         lib.moe_fp8_debug_set_short_tiles.argtypes = [vp, C.c_int]
         lib.moe_fp8_debug_set_short_tiles.restype = C.c_int
+        lib.moe_fp8_debug_set_unclaimed_lists.argtypes = [vp, C.c_int]
+        lib.moe_fp8_debug_set_unclaimed_lists.restype = C.c_int
         lib.moe_fp8_debug_set_fault.argtypes = [vp, C.c_int, C.c_longlong]
         lib.moe_fp8_debug_set_fault.restype = C.c_int
         lib.moe_fp8_debug_sigmoid.argtypes = [C.c_int, fp, fp, vp]
@@ -247,6 +249,11 @@ class MoeFp8:
         """moe_fp8_debug_set_short_tiles: batch size from which row tiles of at most 32 rows run with the weights
         on the M side of the MMAs inside the large-tile GEMM kernels (0: never)."""
         self._check(self.lib.moe_fp8_debug_set_short_tiles(self.handle, int(min_tokens)))
+
+    def debug_set_unclaimed_lists(self, lists: int):
+        """moe_fp8_debug_set_unclaimed_lists: the first `lists` CTAs of the one launch for both GEMMs leave their
+        GEMM1 tiles to the other CTAs (0: off)."""
+        self._check(self.lib.moe_fp8_debug_set_unclaimed_lists(self.handle, int(lists)))
 
     def debug_set_fault(self, skip_iteration: int = -1, wait_clocks: int = 0):
         """moe_fp8_debug_set_fault (test hook of the bounded-wait failure path)."""

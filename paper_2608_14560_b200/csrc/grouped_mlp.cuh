@@ -34,6 +34,7 @@ struct MlpArgs {
     int phases;          // bit 0: GEMM1's tiles, bit 1: GEMM2's; both: a GEMM2 tile waits for its rows
     int* claimed;        // [grid] lists of GEMM1 tiles somebody works on, zero at launch (both GEMMs only)
     int* ready;          // [row tiles] warps that have stored their part, zero at launch
+    int left_open;       // test hook: the first CTAs, which leave their lists of GEMM1 tiles to the others (0 outside of tests)
 };
 
 // Entry i of the CTA's work list, as the factor warp published it.  A role that gave up here while the others went on
@@ -241,13 +242,16 @@ __device__ __forceinline__ void mlp_factors(const Cta& c, const MlpArgs& a) {
     const int extra = r1 * 16 <= grid * 12 && r1 > 0 ? a.g1.num_kb / a.g2.num_kb : 0, first2 = extra * (grid - r1);
     const int turn = static_cast<int>(blockIdx.x) - r1 + (late ? grid : 0);
     int round = late ? extra : 0;
-    if (a.phases == 3) {
-        int taken = 0;
-        if (lane == 0) taken = atomicExch(a.claimed + blockIdx.x, 1);
-        if (__shfl_sync(0xffffffffu, taken, 0)) id1 = n1;  // (somebody else works on it)
-    }
     uint32_t published = 0;
     int last_key = 1;
+    if (a.phases == 3) {
+        int taken = 0;
+        if (static_cast<int>(blockIdx.x) < a.left_open)
+            taken = 1, last_key = 2;  // (and it takes none of another CTA)
+        else if (lane == 0)
+            taken = atomicExch(a.claimed + blockIdx.x, 1);
+        if (__shfl_sync(0xffffffffu, taken, 0)) id1 = n1;  // (somebody else works on it)
+    }
     auto publish = [&](bool end) {  // the next tile of the list, or its end
         if (a.phases == 3 && id1 >= n1 && !end && (last_key & 3) == 1) {
             // the end of a list of GEMM1 tiles: go on with one that nobody has claimed, if there is any

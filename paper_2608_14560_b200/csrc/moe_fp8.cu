@@ -127,6 +127,7 @@ struct moe_fp8_handle_s {
     cudaEvent_t ev[NUM_STAGES_MAX + 1];
     int fused_max_tokens;   // batches of at most this many tokens take the fused kernel (0: never)
     bool k_split;           // fused kernel: very small batches may cut a tile's K range over several CTAs
+    int lists_left_open;    // test hook, see moe_fp8_debug_set_unclaimed_lists
     int short_tile_min_tokens;   // batches of at least this many tokens run short row tiles with the weights on M (0: never)
     unsigned long long fused_calls;
     // moe_fp8_forward_host_async: copy streams and the events that order the two staging sets
@@ -587,7 +588,7 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
         }
         // stage 3: GEMM1 + SwiGLU + re-quantisation, GEMM2
         if (h->short_tile_min_tokens > 0 && T >= h->short_tile_min_tokens) g1.wm_rows = g2.wm_rows = WM_TOKENS;
-        MlpArgs a = {g1, g2, 3, m.mlp_claimed, m.mlp_ready};
+        MlpArgs a = {g1, g2, 3, m.mlp_claimed, m.mlp_ready, h->lists_left_open};
         auto mlp = [&](int phases) {
             a.phases = phases;
             return launch(grouped_mlp_kernel, m.mlp_grid, G_THREADS, GeomFull::SMEM_BYTES, stream, pdl, h->tm_a1, h->tm_a1_small,
@@ -636,6 +637,12 @@ int moe_fp8_debug_set_fault(moe_fp8_handle_t h, int skip_iteration, long long wa
 int moe_fp8_debug_set_k_split(moe_fp8_handle_t h, int enable) {
     if (!h) return MOE_FP8_ERR_BAD_ARG;
     h->k_split = enable != 0;
+    return MOE_FP8_OK;
+}
+
+int moe_fp8_debug_set_unclaimed_lists(moe_fp8_handle_t h, int lists) {
+    if (!h || lists < 0 || lists >= std::min(h->sm_count, MLP_MAX_GRID)) return MOE_FP8_ERR_BAD_ARG;
+    h->lists_left_open = lists;
     return MOE_FP8_OK;
 }
 

@@ -529,6 +529,36 @@ def test_one_launch_for_both_gemms(cuda_device, dims, tokens, kw):
     eng.close()
 
 
+@pytest.mark.parametrize("tokens,eloc,skew", [(300, 8, False),     # at most one GEMM1 tile in a list
+                                              (1200, 48, False),   # one or two
+                                              (1200, 96, True),    # two and three, with short and full row tiles
+                                              (1000, 256, False)])  # six and seven
+def test_lists_of_gemm1_tiles_that_other_ctas_take_over(cuda_device, tokens, eloc, skew):
+    # CTAs that have not started when others are through with their tiles, made certain: 1, 40 (beyond the first 32
+    # entries of the table) and all but one of the CTAs leave their lists open.  The CTA that takes one over announces
+    # the rows of its own and of the adopted lists, and everybody's GEMM2 tiles wait for them.
+    dims = syn.LayerDims(hidden=512, intermediate=512, num_local_experts=eloc)
+    wl = _wl(tokens, dims, seed=1100 + eloc, skew=skew)
+    inp = syn.make_inputs(wl, cuda_device)
+    eng = make_engine(wl, cuda_device)
+    want = eng.forward(inp).clone()
+    torch.cuda.synchronize()
+    assert eng.last_launch_count() == 4 and eng.status() == 0
+    sms = torch.cuda.get_device_properties(cuda_device).multi_processor_count
+    for lists in (1, 40, sms - 1):
+        eng.debug_set_unclaimed_lists(lists)
+        for _ in range(3):
+            got = eng.forward(inp)
+        torch.cuda.synchronize()
+        assert eng.status() == 0, lists
+        assert torch.equal(got.view(torch.int16), want.view(torch.int16)), lists
+    with pytest.raises(MoeFp8Error):
+        eng.debug_set_unclaimed_lists(sms)
+    eng.debug_set_unclaimed_lists(0)
+    run_and_compare(wl, cuda_device, inp=inp, eng=eng, sample_tokens=_sample(tokens, 64, 1))
+    eng.close()
+
+
 def test_two_handles_on_two_streams_share_the_gpu(cuda_device):
     # kernels whose CTAs wait for one another, from two streams at a time: a CTA may only depend on CTAs that run
     wls = [_wl(1500, seed=71), _wl(700, syn.LayerDims(hidden=1024, intermediate=512, num_local_experts=32), seed=72)]
