@@ -97,7 +97,11 @@ int moe_fp8_set_workspace(moe_fp8_handle_t h, void* dev_workspace, size_t bytes)
  *
  * All pointers are device pointers, 16-byte aligned; nothing is copied or kept beyond the call's kernels.
  * Forwards on one handle share its workspace: their kernels must not overlap on the GPU (one stream, or
- * streams ordered with events); use one handle per concurrent stream otherwise.
+ * streams ordered with events); use one handle per concurrent stream otherwise.  The CTAs of the fused kernel
+ * of small batches, one per SM, wait for one another and therefore have to be resident together.  That is so
+ * beside other work of the same priority, whose launches are placed one after the other; kernels of another
+ * priority that keep SMs from a launch half placed until one of its waits runs out (a code in the status word)
+ * are to be kept apart from it, or the fused kernel switched off (moe_fp8_set_small_batch_fusion).
  */
 int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const float* hidden_scale,
                     const float* router_logits, const void* routing_bias, const void* w13,

@@ -579,6 +579,33 @@ def test_two_handles_on_two_streams_share_the_gpu(cuda_device):
         engs[k].close()
 
 
+@pytest.mark.parametrize("sizes", [(9, 14), (48, 70), (12, 60), (16, 700), (75, 1500)])
+def test_fused_batches_on_two_streams(cuda_device, sizes):
+    # the fused kernel beside another fused one and beside the joint GEMM launch: its CTAs wait for one another, and its
+    # forwards follow each other closely (programmatic launches).  The waits give up early, so that a batch that only
+    # got some of its CTAs would show as a time-out and not as a slow pass.
+    wls = [_wl(t, syn.LayerDims(hidden=1024, intermediate=512, num_local_experts=32), seed=73 + t) for t in sizes]
+    inps = [syn.make_inputs(w, cuda_device) for w in wls]
+    engs = [make_engine(w, cuda_device) for w in wls]
+    want = [e.forward(i).clone() for e, i in zip(engs, inps)]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(device=cuda_device) for _ in wls]
+    for e in engs:
+        e.debug_set_fault(-1, 1 << 26)  # a few tens of milliseconds
+    for _ in range(4):
+        got = [[], []]
+        for _ in range(25):
+            for k in range(2):
+                with torch.cuda.stream(streams[k]):
+                    got[k].append(engs[k].forward(inps[k]))
+        torch.cuda.synchronize()
+        for k in range(2):
+            assert engs[k].status() == 0
+            assert all(torch.equal(g.view(torch.int16), want[k].view(torch.int16)) for g in got[k])
+    for e in engs:
+        e.close()
+
+
 # ---- routing + counts + row tables in one launch, placement in the gather: block sizes and group splits ---------
 @pytest.mark.parametrize("tokens,eloc,off", [(1, 32, 0), (7, 1, 3), (9, 64, 64), (129, 65, 20), (1023, 64, 0), (1024, 3, 5),
                                              (1025, 32, 32), (1025, 200, 56), (4999, 17, 0), (8193, 256, 0)])
