@@ -250,7 +250,9 @@ int moe_fp8_debug_sigmoid(int n, const float* x, float* y, void* stream);
  * destroys them.  Off by default.
  */
 int moe_fp8_set_stage_timing(moe_fp8_handle_t h, int enable);
-/* Number of stages and the name of stage i ("route_topk", ..., "combine"). */
+/* Number of stages and the name of stage i.  A stage that a forward has no launch for (the two GEMMs and the joint
+ * "grouped_mlp" exclude each other, "fused_small" all but the routing) takes 0 ms; so do "count", "scan" and "place",
+ * which are part of the launches of "route_topk" and "gather_rows" at every batch size. */
 int moe_fp8_num_stages(void);
 const char* moe_fp8_stage_name(int i);
 /* Waits for the events of the last forward and writes the device time of each

@@ -104,7 +104,11 @@ WsLayout make_layout(const moe_fp8_config& c) {
 
 }  // namespace
 
-constexpr int NUM_STAGES_MAX = 10;
+// Stages of the timing hook, numbered for callers, not in the order of the launches.  The routing kernels count, scan and
+// place as well: those three have no time of their own.
+enum Stage { ST_ROUTE, ST_COUNT, ST_SCAN, ST_PLACE, ST_GATHER, ST_GEMM1, ST_GEMM2, ST_COMBINE, ST_FUSED_SMALL, ST_GROUPED_MLP, NUM_STAGES };
+const char* const STAGE_NAMES[NUM_STAGES] = {"route_topk", "count", "scan", "place", "gather_rows", "gemm1_swiglu_quant",
+                                             "gemm2", "combine", "fused_small", "grouped_mlp"};
 
 struct moe_fp8_handle_s {
     moe_fp8_config cfg;
@@ -124,7 +128,8 @@ struct moe_fp8_handle_s {
     bool stage_times_valid;
     int fault_skip_it;         // test hook, see moe_fp8_debug_set_fault
     long long fault_wait_limit;
-    cudaEvent_t ev[NUM_STAGES_MAX + 1];
+    cudaEvent_t ev[NUM_STAGES + 1];   // in front of the first launch, and behind each one
+    int ev_count, ev_stage[NUM_STAGES + 1];   // of the last forward: events recorded, the stage that ends at each
     int fused_max_tokens;   // batches of at most this many tokens take the fused kernel (0: never)
     bool k_split;           // fused kernel: very small batches may cut a tile's K range over several CTAs
     int lists_left_open;    // test hook, see moe_fp8_debug_set_unclaimed_lists
@@ -229,9 +234,6 @@ PermuteMeta meta_of(moe_fp8_handle_t h) {
 }
 
 constexpr int PDL_MAX_TOKENS = 2048;
-constexpr int NUM_STAGES = 10;
-const char* const STAGE_NAMES[NUM_STAGES] = {"route_topk", "count", "scan", "place", "gather_rows",
-                                             "gemm1_swiglu_quant", "gemm2", "grouped_mlp", "combine", "fused_small"};
 
 bool misaligned(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) != 0; }
 
@@ -444,9 +446,11 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
     const bool pdl = !h->stage_timing && T <= PDL_MAX_TOKENS;
 
     // No memset: the first kernel clears the status word, and the ticket counter returns to zero by itself.
-    int ev_i = 0;
-    auto mark = [&]() {
-        if (h->stage_timing) cudaEventRecord(h->ev[ev_i++], stream);
+    h->ev_count = 0;
+    auto mark = [&](int stage) {  // behind the launch of a stage
+        if (!h->stage_timing) return;
+        h->ev_stage[h->ev_count] = stage;
+        cudaEventRecord(h->ev[h->ev_count++], stream);
     };
     // The first launch that fails ends the call: nothing further is enqueued behind it.
     cudaError_t lerr = cudaSuccess;
@@ -457,7 +461,7 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
         ++launches;                                       \
     } while (0)
     h->stage_times_valid = false;
-    mark();
+    mark(-1);
     // Batches of at most fused_max_tokens tokens: gather, both GEMMs and the combine in one kernel; up to
     // F_ROUTE_MAX_TOKENS that kernel also routes and permutes (every CTA for itself: one launch per forward).
     const bool fused = T <= h->fused_max_tokens;
@@ -471,28 +475,19 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
     }
 
     if (route_in_fused) {
-        mark();
-        mark();
-        mark();
-        mark();
+        // no launch of its own
     } else if (fused) {  // routing in parallel blocks, the last one to finish does stage 2 up to the gather
         const int grid = min((T + 7) / 8, h->sm_count * 8);
         MOE_LAUNCH(route_permute_kernel, grid, P_TAIL_THREADS, route_permute_smem_bytes(T, EL), stream, false, T, EL,
                    local_expert_offset, row_cap, router_logits, static_cast<const __nv_bfloat16*>(routing_bias),
                    scaling_factor, topk_idx, topk_w, m, status + 1, status);
-        mark();
-        mark();
-        mark();
-        mark();
+        mark(ST_ROUTE);
     } else {  // routing, counts and row tables; the placement follows with the gather
         const int tpb = route_count_tokens_per_block(T, EL), grid = (T + tpb - 1) / tpb;
         const auto kernel = tpb == 8 ? route_count_kernel<8> : route_count_kernel<32>;
         MOE_LAUNCH(kernel, grid, tpb * 32, 0, stream, false, T, EL, local_expert_offset, router_logits,
                    static_cast<const __nv_bfloat16*>(routing_bias), scaling_factor, topk_idx, topk_w, m, status + 1, status);
-        mark();
-        mark();
-        mark();
-        mark();
+        mark(ST_ROUTE);
     }
     // the two GEMMs' arguments
     GemmArgs g1, g2;
@@ -569,22 +564,17 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
         f.meta = m;
         f.counters_next = counters_next;
         f.num_counters = static_cast<int>(h->L.num_counters);
-        mark();  // gather_rows
-        mark();  // gemm1
-        mark();  // gemm2
-        mark();  // grouped_mlp
-        mark();  // combine
         MOE_LAUNCH(fused_small_kernel, h->sm_count, G_THREADS, GeomSmall::SMEM_BYTES, stream, pdl, h->tm_a2_small,
                    h->tm_w13_m, h->tm_w2, g1, g2, f);
         ++h->fused_calls;  // only a kernel that runs zeroes the other counter set
-        mark();
+        mark(ST_FUSED_SMALL);
     } else {
         {  // stage 2, continued: placement and gather
             const int grid = min((T + 7) / 8, h->sm_count * 8);
             MOE_LAUNCH(place_gather_kernel, grid, 256, 0, stream, pdl, T, H, EL, local_expert_offset, row_cap,
                        route_count_tokens_per_block(T, EL), c.hidden_scale_layout, static_cast<const int*>(topk_idx),
                        static_cast<const uint8_t*>(hidden_fp8), hidden_scale, m, a1, a1_scale_t, status);
-            mark();
+            mark(ST_GATHER);
         }
         // stage 3: GEMM1 + SwiGLU + re-quantisation, GEMM2
         if (h->short_tile_min_tokens > 0 && T >= h->short_tile_min_tokens) g1.wm_rows = g2.wm_rows = WM_TOKENS;
@@ -596,28 +586,24 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
         };
         const long long slots = static_cast<long long>(T) * R_TOPK * EL / R_EXPERTS;
         if (T > MLP_SPLIT_MAX_TOKENS && slots <= MLP_JOINT_MAX_SLOTS) {
-            mark();  // gemm1
-            mark();  // gemm2
             if ((lerr = mlp(3)) != cudaSuccess) return cuda_fail(h, lerr);
             ++launches;
-            mark();
+            mark(ST_GROUPED_MLP);
         } else {
             if ((lerr = mlp(1)) != cudaSuccess) return cuda_fail(h, lerr);
             ++launches;
-            mark();
+            mark(ST_GEMM1);
             if ((lerr = mlp(2)) != cudaSuccess) return cuda_fail(h, lerr);
             ++launches;
-            mark();
-            mark();  // grouped_mlp
+            mark(ST_GEMM2);
         }
         {  // stage 4: weighted combine back to token order
             const int grid = min(T, h->sm_count * 16);
             MOE_LAUNCH(combine_kernel, grid, 256, 0, stream, pdl, T, H, static_cast<const int*>(m.slot_to_row),
                        static_cast<const float*>(topk_w), reinterpret_cast<const uint8_t*>(y),
                        static_cast<__nv_bfloat16*>(out));
-            mark();
+            mark(ST_COMBINE);
         }
-        mark();  // fused_small (not used on this path)
     }
 #undef MOE_LAUNCH
     const cudaError_t e = cudaGetLastError();
@@ -694,12 +680,15 @@ const char* moe_fp8_stage_name(int i) { return (i >= 0 && i < NUM_STAGES) ? STAG
 int moe_fp8_get_stage_times(moe_fp8_handle_t h, float* host_ms, int n) {
     if (!h || !host_ms || n < 0) return MOE_FP8_ERR_BAD_ARG;
     if (!h->stage_timing || !h->stage_times_valid) return MOE_FP8_ERR_BAD_ARG;
-    cudaError_t e = cudaEventSynchronize(h->ev[NUM_STAGES]);
+    cudaError_t e = cudaEventSynchronize(h->ev[h->ev_count - 1]);
     if (e != cudaSuccess) return cuda_fail(h, e);
     const int k = n < NUM_STAGES ? n : NUM_STAGES;
-    for (int i = 0; i < k; ++i) {
-        e = cudaEventElapsedTime(&host_ms[i], h->ev[i], h->ev[i + 1]);
+    for (int i = 0; i < k; ++i) host_ms[i] = 0.0f;
+    for (int i = 1; i < h->ev_count; ++i) {
+        float ms = 0.0f;
+        e = cudaEventElapsedTime(&ms, h->ev[i - 1], h->ev[i]);
         if (e != cudaSuccess) return cuda_fail(h, e);
+        if (h->ev_stage[i] < k) host_ms[h->ev_stage[i]] = ms;
     }
     return k;
 }

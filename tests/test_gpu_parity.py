@@ -384,6 +384,30 @@ def test_an_abort_leaves_nothing_under_way(cuda_device, tokens, eloc, clocks):
     eng.close()
 
 
+def test_stage_times_name_the_launches_of_a_forward(cuda_device):
+    gemms = {"route_topk", "gather_rows", "gemm1_swiglu_quant", "gemm2", "combine"}
+    joint = {"route_topk", "gather_rows", "grouped_mlp", "combine"}
+    eng = make_engine(_wl(300), cuda_device)
+    # (callers may keep the numbers)
+    assert eng.stage_names()[:9] == ["route_topk", "count", "scan", "place", "gather_rows", "gemm1_swiglu_quant", "gemm2",
+                                     "combine", "fused_small"]
+    eng.set_stage_timing(True)
+    for tokens, stages in ((9, {"fused_small"}), (40, {"route_topk", "fused_small"}), (200, gemms), (300, joint), (9, {"fused_small"})):
+        inp = syn.make_inputs(_wl(tokens, seed=tokens), cuda_device)
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        eng.forward(inp)
+        b.record()
+        times = eng.get_stage_times()
+        torch.cuda.synchronize()
+        assert {k for k, v in times.items() if v > 0} == stages and eng.last_launch_count() == len(stages)
+        assert sum(times.values()) <= a.elapsed_time(b) + 1e-3
+    eng.set_stage_timing(False)
+    with pytest.raises(MoeFp8Error):
+        eng.get_stage_times()
+    eng.close()
+
+
 # ---- the layer started from bf16 hidden states (router projection + input quantisation in front) ----------
 def _from_hidden_case(wl, device, sample_tokens=None, **kw):
     d = wl.dims
