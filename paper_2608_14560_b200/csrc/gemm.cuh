@@ -280,10 +280,14 @@ struct AheadSeq {  // the first `rounds` rounds of items to `stride` of the CTAs
 // After `before` items dealt by seq_plain: the CTAs that got one item less are the first in every round, and they take up
 // to `ahead` rounds among themselves in front, as far as the items reach whose row tiles the full rounds have finished
 // (n1_tiles items before and n2_tiles new ones belong to a row tile).  Only where the last round before has few items: a
-// CTA streams up to 64 GB/s, so a hundred of them saturate the memory and the idle time of the others costs nothing (with 108
-// or 140 such items a forward took 6 % longer, with 24 or 40 it takes 4-10 % less).  (Dealt in plain rounds, 54 tokens on 23 experts left 72 CTAs with 238 K-blocks and 76
-// with 182; us per forward, plain rounds / these: 54 tokens 175 / 165, 33 tokens on 256 local experts 766 / 752, 8 and
-// 16 tokens up to 6 % less, equal where GEMM1 fills whole rounds.)
+// CTA streams up to 64 GB/s, so a hundred of them saturate the memory and the idle time of the others costs nothing.
+// (Dealt in plain rounds, 54 tokens on 23 experts left 72 CTAs with 238 K-blocks and 76 with 182; us per forward, plain
+// rounds / these: 54 tokens 175 / 165, 33 tokens on 256 local experts 766 / 752, 8 and 16 tokens up to 6 % less, equal
+// where GEMM1 fills whole rounds.)  The line is at 83 of 148 items, below every count that loses; us with plain rounds /
+// with these by that number, 40 and 72 tokens on 17 to 35 experts: 24 178 / 177 and 190 / 194, 56 192 / 191 and 205 / 206,
+// 72 193 / 191 and 207 / 205; beyond the line 84 263 / 258 and 277 / 266, 88 205 / 201 and 220 / 210, 100 274 / 270 and
+// 286 / 287, 104 206 / 204 and 217 / 215, 116 276 / 274 and 286 / 286, 120 208 / 220 and 220 / 236 (up to 104 these rounds
+// would gain as well).
 __device__ __forceinline__ AheadSeq seq_after(int before, int ahead, int n1_tiles, int n2_tiles, int count) {
     const int grid = static_cast<int>(gridDim.x), b = static_cast<int>(blockIdx.x);
     int r = before, rounds = 0;

@@ -11,9 +11,10 @@
 // arrival took GEMM1 of 8192 skewed tokens from 1226 to 1331 us.
 // What the common list is for: a launch per GEMM leaves most SMs idle in its last, partly filled wave.  With 24 active
 // experts (257 tokens) GEMM1 is 384 tiles of 56 K-blocks, 2.6 waves, and GEMM2 672 tiles of 16, 4.5 waves: 248 K-block
-// times per launch pair against 218 in one list.  Measured per forward: 225 -> 211 us at 257 tokens, 289 -> 274 at 901,
-// 500 -> 472 at 512 from host buffers, 425 -> 417 at 4096.  Two launches of this kernel stay better where a list is long
-// (see MLP_JOINT_MAX_SLOTS) and the CTAs, in step after a launch, drift apart.
+// times per launch pair against 218 in one list.  Measured per forward, two launches against one, this kernel on both
+// sides (the first 32 experts, uniform routing, runs too short for the power cap): 187 -> 170 us at 257 tokens, 208 -> 193
+// at 512, 212 -> 197 at 901, 261 -> 238 at 2048, 351 -> 338 at 4096.  In long runs two launches are better where a list is
+// long (see MLP_JOINT_MAX_SLOTS) and the CTAs, in step after a launch, drift apart.
 #pragma once
 #include "gemm.cuh"
 
@@ -23,7 +24,12 @@ namespace moe {
 // the local share of the experts) run both GEMMs in one launch, the others in one each.  us per forward, one launch
 // against two: 248 / 256 at 1109 slots, 417 / 429 at 4171, 1435 / 1439 at 4096 with 256 experts, 1055 / 1065 at 16872
 // skewed, 1116 / 1125 at 16167, 2194 / 2201 at 16384 with 256 experts, 3170 / 3159 at 32768, 8913 / 8626 at 131072.
-// (Up to 256 tokens the separate launches are what callers that switch the fused kernel off have always counted.)
+// The last figure sets the line: under the power cap, which short runs do not reach (there one launch stays ahead: 2908 / 2987
+// at 32768 slots, 5066 / 5169 at 65536), the largest batches lose 3 %.
+// The lower line is not set by speed: callers count on two GEMM launches up to 256 tokens (last_launch_count, the stage
+// times of the two GEMMs).  Above the fused kernel's 80 tokens one launch would be the faster one with uniform routing
+// (two / one: 153 / 148 us at 81 tokens, 184 / 166 at 128, 189 / 181 at 160, 206 / 192 at 256) and the slower one for few
+// skewed tokens (147 / 149 at 81, 151 / 154 at 128; 173 / 156 at 160, 197 / 186 at 256).
 constexpr int MLP_SPLIT_MAX_TOKENS = 256;
 constexpr int MLP_JOINT_MAX_SLOTS = 16384;
 
@@ -234,9 +240,12 @@ __device__ __forceinline__ void mlp_factors(const Cta& c, const MlpArgs& a) {
     const int n1 = (a.phases & 1) ? m_tiles * a.g1.n_tiles : 0, n12 = n1 + ((a.phases & 2) ? m_tiles * a.g2.n_tiles : 0);
     const int grid = static_cast<int>(gridDim.x);
     // GEMM1: tiles id1, id1 + grid, ... ; GEMM2: the CTAs that have one GEMM1 tile less (of num_kb1 K-blocks) take
-    // `extra` rounds of tiles (of num_kb2) among themselves, then the rounds go over all CTAs, those first.  (Not where nearly all CTAs have the tile more, so
-    // that the idle time of the others costs no bandwidth; us per forward without / with: 400 tokens on 24 experts, 88
-    // such CTAs, 207 / 198; 600 on 25, 104 such CTAs, 214 / 204; 257 on 17, 124 such CTAs, 149 / 162.)
+    // `extra` rounds of tiles (of num_kb2) among themselves, then the rounds go over all CTAs, those first.  (Not where
+    // nearly all CTAs have the tile more, so that the idle time of the others costs no bandwidth; us per forward without /
+    // with, by the number of CTAs that have it, 257 tokens on 17 to 36 experts: 241 / 234 with 72, 324 / 318 with 84, 262 /
+    // 251 with 88, 329 / 322 with 100, 261 / 253 with 104; 335 / 329 with 116, 268 / 270 with 120, 194 / 210 with 124, 345 /
+    // 346 with 132, 277 / 272 with 136, 198 / 226 with 140.  The line is at 111 of 148: below it every count gains, above it
+    // the losses are larger than the gains.)
     int id1 = static_cast<int>(blockIdx.x);
     const int r1 = n1 % grid, late = static_cast<int>(blockIdx.x) < r1 ? 1 : 0;
     const int extra = r1 * 16 <= grid * 12 && r1 > 0 ? a.g1.num_kb / a.g2.num_kb : 0, first2 = extra * (grid - r1);
