@@ -632,10 +632,11 @@ def test_fused_batches_on_two_streams(cuda_device, sizes):
 
 # ---- routing + counts + row tables in one launch, placement in the gather: block sizes and group splits ---------
 @pytest.mark.parametrize("tokens,eloc,off", [(1, 32, 0), (7, 1, 3), (9, 64, 64), (129, 65, 20), (1023, 64, 0), (1024, 3, 5),
-                                             (1025, 32, 32), (1025, 200, 56), (4999, 17, 0), (8193, 256, 0)])
+                                             (1025, 32, 32), (1025, 200, 56), (4999, 17, 0), (8193, 256, 0),
+                                             (256, 256, 0), (257, 129, 100), (512, 128, 128), (513, 65, 0)])
 def test_permutation_at_the_edges_of_its_blocks(cuda_device, tokens, eloc, off):
-    # blocks of 8 tokens (up to 1024 tokens and 64 local experts) and of 32, the last block ragged; local expert
-    # counts on both sides of a power of two split the last block's threads into 1 to 32 groups
+    # blocks of 8 tokens (up to 1024 tokens, 512 with more than 64 local experts and 256 with more than 128) and of 32, the
+    # last block ragged; local expert counts on both sides of a power of two split the last block's threads into 1 to 32 groups
     dims = dataclasses.replace(syn.LayerDims(hidden=256, intermediate=128), num_local_experts=eloc)
     wl = _wl(tokens, dims, seed=40 + tokens, local_expert_offset=off)
     eng = make_engine(wl, cuda_device)
