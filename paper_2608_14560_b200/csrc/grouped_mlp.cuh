@@ -34,6 +34,7 @@ constexpr int MLP_SPLIT_MAX_TOKENS = 256;
 constexpr int MLP_JOINT_MAX_SLOTS = 16384;
 
 constexpr int MLP_MAX_GRID = 1024;   // capacity of `claimed`
+constexpr int FRONT_MIN_KB = 16;     // K-blocks of a GEMM2 tile for the rounds in front, see mlp_factors
 
 struct MlpArgs {
     GemmArgs g1, g2;
@@ -248,7 +249,14 @@ __device__ __forceinline__ void mlp_factors(const Cta& c, const MlpArgs& a) {
     // the losses are larger than the gains.)
     int id1 = static_cast<int>(blockIdx.x);
     const int r1 = n1 % grid, late = static_cast<int>(blockIdx.x) < r1 ? 1 : 0;
-    const int extra = r1 * 16 <= grid * 12 && r1 > 0 ? a.g1.num_kb / a.g2.num_kb : 0, first2 = extra * (grid - r1);
+    // Only with GEMM2 tiles of at least 16 K-blocks (intermediate size 2048 and more), and no more rounds than there are
+    // GEMM2 tiles whose rows the full GEMM1 rounds have finished: shorter GEMM2 tiles cost more than their K-blocks say, and
+    // a tile whose rows come from the last GEMM1 round is waited for.  (us per forward without / with as many rounds as K-block
+    // counts allow: 7168 x 384, 3 experts, no full GEMM1 round, 103 / 133; 7168 x 1024, 27 to 32 experts, 168 to 186 / 184
+    // to 208; 7168 x 512, 189 / 209; 4096 x 1024, 111 / 118; 2048 x 512, 76 / 84.)
+    const int reach = (n1 - r1) / a.g1.n_tiles * a.g2.n_tiles / (grid - r1);
+    const bool front = r1 > 0 && r1 * 16 <= grid * 12 && a.g2.num_kb >= FRONT_MIN_KB;
+    const int extra = front ? min(a.g1.num_kb / a.g2.num_kb, reach) : 0, first2 = extra * (grid - r1);
     const int turn = static_cast<int>(blockIdx.x) - r1 + (late ? grid : 0);
     int round = late ? extra : 0;
     uint32_t published = 0;

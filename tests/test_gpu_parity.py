@@ -583,6 +583,35 @@ def test_lists_of_gemm1_tiles_that_other_ctas_take_over(cuda_device, tokens, elo
     eng.close()
 
 
+def _route_round_robin(inp, tokens, active, away=0):
+    # token t on eight experts in turn, of the first `active` ones and `away` experts of other ranks
+    ids = torch.tensor(list(range(active)) + list(range(256 - away, 256)))
+    idx = ids[(torch.arange(tokens)[:, None] * 8 + torch.arange(8)[None]) % len(ids)]
+    inp["router_logits"][:] = -8.0
+    inp["router_logits"].scatter_(1, idx.to(inp["router_logits"].device), 6.0)
+    inp["routing_bias"][:] = 0
+
+
+@pytest.mark.parametrize("active", [4, 9, 10, 16, 19, 25, 28])  # one row tile each: 16 GEMM1 and 28 GEMM2 tiles
+def test_gemm2_rounds_in_front_of_the_joint_launch(cuda_device, active):
+    # fewer GEMM1 tiles than CTAs (4, 9: 64 and 144), fewer rounds in reach than wanted (10), as many as wanted and not
+    # one more (19), more (25, 28), all but a few CTAs without the last GEMM1 tile or with it; and the same again with
+    # lists that other CTAs take over
+    wl = _wl(257, syn.DSV3, seed=1200 + active)
+    inp = syn.make_inputs(wl, cuda_device)
+    _route_round_robin(inp, 257, active, away=40 - active)
+    eng = make_engine(wl, cuda_device, poison=False)
+    run_and_compare(wl, cuda_device, inp=inp, eng=eng, sample_tokens=_sample(257, 24, active))
+    assert eng.last_launch_count() == 4
+    assert int((eng.debug_export(257, rows=False)["expert_count"] > 0).sum()) == active
+    want = eng.forward(inp).clone()
+    eng.debug_set_unclaimed_lists(50)
+    got = eng.forward(inp)
+    torch.cuda.synchronize()
+    assert eng.status() == 0 and torch.equal(got.view(torch.int16), want.view(torch.int16))
+    eng.close()
+
+
 def test_two_handles_on_two_streams_share_the_gpu(cuda_device):
     # kernels whose CTAs wait for one another, from two streams at a time: a CTA may only depend on CTAs that run
     wls = [_wl(1500, seed=71), _wl(700, syn.LayerDims(hidden=1024, intermediate=512, num_local_experts=32), seed=72)]
