@@ -188,6 +188,13 @@ struct FusedArgs {
     int split;                    // 1: the split may be used by this call
     int ahead;                    // GEMM2 tiles that take the time of a GEMM1 tile, see seq_after
 };
+// A GEMM2 tile of the fused kernel, however few its K-blocks, takes the time of about 18: its weights come in six stages
+// deep in front of its rows, its stores, its counters and the combine behind it.  Best number of rounds in front (0 to 6
+// measured, 16 to 64 tokens, five numbers of spare CTAs each; us per forward without / with it / with one per
+// K-block ratio): 2 to 3 with GEMM1 tiles of 56 K-blocks (7168 x 1024 159 / 152 / 175, x 512 182 / 167 / 206, x 256
+// 210 / 196 / 259), 1 with 32 (4096 x 2048 248 / 243 / 252, x 1024 100 / 97 / 102, x 512 115 / 110 / 133), none with 16
+// (2048 x 1024 68 / 68 / 72, x 512 68 / 68 / 85).
+constexpr int FRONT_TILE_KB = 18;
 constexpr int SPLIT_MAX_TOKENS = 4;                       // rows of a tile whose K range may be split
 constexpr int SPLIT_MAX_TILES = 74;                       // a split needs at least two CTAs per tile
 constexpr int SPLIT_RAW_FLOATS = 2 * SPLIT_MAX_TOKENS * 128;  // per tile and K-block

@@ -545,7 +545,7 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
         f.raw[0] = at<float>(h, h->L.raw1);
         f.raw[1] = at<float>(h, h->L.raw2);
         f.split = h->k_split ? 1 : 0;
-        f.ahead = g1.num_kb / g2.num_kb;
+        f.ahead = g1.num_kb / std::max(g2.num_kb, FRONT_TILE_KB);
         // the fused kernel works on sub-tiles of at most 32 rows
         g1.num_m_tiles = g2.num_m_tiles = m.num_st;
         g1.tile_expert = g2.tile_expert = m.st_expert;

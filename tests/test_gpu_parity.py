@@ -771,6 +771,26 @@ def test_fused_kernel_work_lists_around_full_rounds_of_ctas(cuda_device, active)
     eng.close()
 
 
+@pytest.mark.parametrize("hidden,inter", [(7168, 256), (4096, 256), (2048, 256)])  # three, one and no rounds in front
+@pytest.mark.parametrize("active", [75, 79, 94, 115, 148])  # two GEMM1 tiles each: 2, 10, 40, 82 and no spare ones
+def test_gemm2_rounds_in_front_of_the_fused_kernel(cuda_device, hidden, inter, active):
+    dims = syn.LayerDims(hidden=hidden, intermediate=inter, num_local_experts=160)
+    wl = _wl(30, dims, seed=1300 + active)
+    inp = syn.make_inputs(wl, cuda_device)
+    _route_round_robin(inp, 30, active)
+    eng = make_engine(wl, cuda_device, poison=False)
+    eng.set_small_batch_fusion(False)
+    want = eng.forward(inp).clone()
+    eng.set_small_batch_fusion(True)
+    for _ in range(2):
+        got = eng.forward(inp).clone()
+    torch.cuda.synchronize()
+    assert eng.status() == 0 and eng.last_launch_count() == 2
+    assert torch.equal(got.view(torch.int16), want.view(torch.int16))
+    assert int((eng.debug_export(30, rows=False)["expert_count"] > 0).sum()) == active
+    eng.close()
+
+
 @pytest.mark.parametrize("tokens,launches,eloc", [(16, 1, 32), (48, 2, 32), (3, 1, 256)])  # 3 tokens: K split
 def test_a_wait_that_runs_out_in_the_fused_small_batch_kernel(cuda_device, tokens, launches, eloc):
     wl = _wl(tokens, dataclasses.replace(SMALL, num_local_experts=eloc), seed=43)
