@@ -189,8 +189,13 @@ __global__ void __launch_bounds__(WARPS * 32) route_count_kernel(
     const bool mine = q < groups && e < E_loc;
     const int b0 = min(nblk, q * per), b1 = min(nblk, b0 + per);
     // (the first HELD counts of a range stay in registers, which is all of them up to 16384 tokens on 32 experts and 2048
-    // on 256: one round trip to L2 instead of two chains of them)
+    // on 256: one round trip to L2 instead of two chains of them.  With blocks of 8 tokens the next HELD do as well, and that is
+    // all there can be: left to the loops behind, what remains after whole batches of loads goes one by one, 38.0
+    // against 31 us per forward at 457 tokens on 65 experts.)
     constexpr int HELD = 16;
+    constexpr bool ALL_HELD = WARPS == 8;
+    int held2[HELD];
+    const bool more = ALL_HELD && per > HELD;  // (the same for the whole block)
     int* hist = m.block_hist + static_cast<size_t>(b0) * E_loc + e;
     int held[HELD], sum = 0;
     if (mine) {
@@ -198,8 +203,14 @@ __global__ void __launch_bounds__(WARPS * 32) route_count_kernel(
         for (int i = 0; i < HELD; ++i) held[i] = b0 + i < b1 ? __ldcg(hist + static_cast<size_t>(i) * E_loc) : 0;
 #pragma unroll
         for (int i = 0; i < HELD; ++i) sum += held[i];
+        if (more) {
+#pragma unroll
+            for (int i = 0; i < HELD; ++i) held2[i] = b0 + HELD + i < b1 ? __ldcg(hist + static_cast<size_t>(HELD + i) * E_loc) : 0;
+#pragma unroll
+            for (int i = 0; i < HELD; ++i) sum += held2[i];
+        }
 #pragma unroll 16
-        for (int i = HELD; i < b1 - b0; ++i) sum += __ldcg(hist + static_cast<size_t>(i) * E_loc);
+        for (int i = HELD; !ALL_HELD && i < b1 - b0; ++i) sum += __ldcg(hist + static_cast<size_t>(i) * E_loc);
     }
     s_part[tid] = sum;
     for (int i = tid; i < P_MAX_LOCAL; i += THREADS) s_cnt[i] = 0;
@@ -213,8 +224,15 @@ __global__ void __launch_bounds__(WARPS * 32) route_count_kernel(
             if (b0 + i < b1) hist[static_cast<size_t>(i) * E_loc] = base;
             base += held[i];
         }
+        if (more) {
+#pragma unroll
+            for (int i = 0; i < HELD; ++i) {
+                if (b0 + HELD + i < b1) hist[static_cast<size_t>(HELD + i) * E_loc] = base;
+                base += held2[i];
+            }
+        }
 #pragma unroll 16
-        for (int i = HELD; i < b1 - b0; ++i) {
+        for (int i = HELD; !ALL_HELD && i < b1 - b0; ++i) {
             const int c = __ldcg(hist + static_cast<size_t>(i) * E_loc);
             hist[static_cast<size_t>(i) * E_loc] = base;
             base += c;
