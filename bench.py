@@ -39,13 +39,15 @@ W2_BYTES_PER_EXPERT = 7168 * 2048 + 56 * 16 * 4
 FP8_DATASHEET_TFLOPS = 4500.0
 HBM_DATASHEET_GBS = 8000.0
 # Measured DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch divided by the algorithmic
-# bytes of the same launch, from the committed ncu captures (see profiles/): the weight-streaming regime was
-# captured on the T = 8 and T = 64 workloads (fused kernel) and on the T = 1024 workload (the two GEMM kernels)
-# themselves, the tensor-bound regime on a reduced case (32 local experts) whose traffic is scaled to a full
-# launch by the algorithmic bytes, since both grow with the experts and rows.
+# bytes of the same launch, from the committed ncu captures (profiles/fused_kernel_dsv3_T8_E32.md,
+# launches_dsv3_T64_E32.md, traffic_grouped_mlp_*.md): in the weight-streaming regime the T = 8 and T = 64 workloads
+# (fused kernel) and the T = 1024 workload (both GEMMs in one launch) themselves and 200 tokens (a launch per
+# GEMM), in the tensor-bound regime the skewed T = 8192 workload itself (one launch) and T = 16384 with 64
+# local experts (a launch per GEMM), whose traffic is scaled to a full launch by the algorithmic bytes, since both
+# grow with the experts and rows.
 NCU_TRAFFIC_RATIO = {
-    ("hbm", "gemm1_swiglu_quant"): 1.04, ("hbm", "gemm2"): 1.02,
-    ("tensor", "gemm1_swiglu_quant"): 1.31, ("tensor", "gemm2"): 0.99,
+    ("hbm", "gemm1_swiglu_quant"): 1.01, ("hbm", "gemm2"): 1.00, ("hbm", "grouped_mlp"): 1.02,
+    ("tensor", "gemm1_swiglu_quant"): 1.34, ("tensor", "gemm2"): 1.07, ("tensor", "grouped_mlp"): 1.09,
     ("hbm", "fused_small"): 1.00,
 }
 METRIC = "fused FP8 MoE forward throughput (tokens/s; TFLOPS and roofline fraction alongside)"
@@ -301,8 +303,8 @@ def run_cuda_config(wl, device, steps, warmup, peaks, peak_kind, want_e2e=True, 
                            "frac_of_datasheet": ach / HBM_DATASHEET_GBS, "peak_source": f"{peak_kind} copy bandwidth"}
     ratio = NCU_TRAFFIC_RATIO.get((res["roofline"]["bound"], dom))
     res["roofline"]["traffic"] = None if ratio is None else ratio * kern_bytes
-    res["roofline"]["traffic_source"] = ("ncu capture of this kernel on a smaller case of the same regime, scaled "
-                                         "to this launch by its algorithmic bytes")
+    res["roofline"]["traffic_source"] = None if ratio is None else (
+        "ncu capture of this kernel in the same regime, scaled to this launch by its algorithmic bytes")
     res["roofline"]["algorithmic_bytes_per_launch"] = kern_bytes
     res["roofline"]["algorithmic_flops_per_launch"] = kern_flops
     res["roofline"]["kernel_ms"] = stage_avg[dom]
