@@ -220,8 +220,8 @@ int moe_fp8_debug_set_short_tiles(moe_fp8_handle_t h, int min_tokens);
 /*
  * Where both GEMMs run in one launch, a CTA that is through with its own list of GEMM1 tiles takes over the lists of
  * CTAs that have not started yet (two forwards may share the GPU).  This hook makes that certain: the first `lists`
- * CTAs leave theirs unclaimed and take none, so that other CTAs work through them (0 switches it off; less than
- * the number of CTAs, which is the number of SMs).
+ * CTAs never take their own, so that other CTAs work through them (0 switches it off; less than the number of CTAs,
+ * which is the number of SMs).
  */
 int moe_fp8_debug_set_unclaimed_lists(moe_fp8_handle_t h, int lists);
 

@@ -252,7 +252,7 @@ class MoeFp8:
 
     def debug_set_unclaimed_lists(self, lists: int):
         """moe_fp8_debug_set_unclaimed_lists: the first `lists` CTAs of the one launch for both GEMMs leave their
-        GEMM1 tiles to the other CTAs (0: off)."""
+        own GEMM1 tiles to the other CTAs (0: off)."""
         self._check(self.lib.moe_fp8_debug_set_unclaimed_lists(self.handle, int(lists)))
 
     def debug_set_fault(self, skip_iteration: int = -1, wait_clocks: int = 0):

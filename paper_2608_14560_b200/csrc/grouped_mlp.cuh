@@ -39,9 +39,8 @@ constexpr int FRONT_MIN_KB = 16;     // K-blocks of a GEMM2 tile for the rounds 
 struct MlpArgs {
     GemmArgs g1, g2;
     int phases;          // bit 0: GEMM1's tiles, bit 1: GEMM2's; both: a GEMM2 tile waits for its rows
-    int* claimed;        // [grid] lists of GEMM1 tiles somebody works on, zero at launch (both GEMMs only)
+    int* claimed;        // [grid] the lists of GEMM1 tiles, LIST_OPEN (or LIST_LEFT) at launch (both GEMMs only)
     int* ready;          // [row tiles] warps that have stored their part, zero at launch
-    int left_open;       // test hook: the first CTAs, which leave their lists of GEMM1 tiles to the others (0 outside of tests)
 };
 
 // Entry i of the CTA's work list, as the factor warp published it.  A role that gave up here while the others went on
@@ -259,28 +258,26 @@ __device__ __forceinline__ void mlp_factors(const Cta& c, const MlpArgs& a) {
     const int extra = front ? min(a.g1.num_kb / a.g2.num_kb, reach) : 0, first2 = extra * (grid - r1);
     const int turn = static_cast<int>(blockIdx.x) - r1 + (late ? grid : 0);
     int round = late ? extra : 0;
+    if (a.phases == 3) {
+        int was = LIST_OPEN;
+        if (lane == 0) was = atomicCAS(a.claimed + blockIdx.x, LIST_OPEN, LIST_CLAIMED);
+        if (__shfl_sync(0xffffffffu, was, 0) != LIST_OPEN) id1 = n1;  // (somebody else works on it, or will)
+    }
     uint32_t published = 0;
     int last_key = 1;
-    if (a.phases == 3) {
-        int taken = 0;
-        if (static_cast<int>(blockIdx.x) < a.left_open)
-            taken = 1, last_key = 2;  // (and it takes none of another CTA)
-        else if (lane == 0)
-            taken = atomicExch(a.claimed + blockIdx.x, 1);
-        if (__shfl_sync(0xffffffffu, taken, 0)) id1 = n1;  // (somebody else works on it)
-    }
     auto publish = [&](bool end) {  // the next tile of the list, or its end
         if (a.phases == 3 && id1 >= n1 && !end && (last_key & 3) == 1) {
             // the end of a list of GEMM1 tiles: go on with one that nobody has claimed, if there is any
             for (int v0 = 0; v0 < grid && id1 >= n1; v0 += 32) {
                 const int v = v0 + lane;
-                uint32_t open = __ballot_sync(0xffffffffu, v < grid && v < n1 && __ldcg(a.claimed + v) == 0);
+                const bool other = v < grid && v < n1 && v != static_cast<int>(blockIdx.x);
+                uint32_t open = __ballot_sync(0xffffffffu, other && __ldcg(a.claimed + v) != LIST_CLAIMED);
                 while (open && id1 >= n1) {
                     const int u = v0 + __ffs(open) - 1;
                     open &= open - 1;
-                    int taken = 0;
-                    if (lane == 0) taken = atomicExch(a.claimed + u, 1);
-                    if (!__shfl_sync(0xffffffffu, taken, 0)) id1 = u;
+                    int was = LIST_CLAIMED;
+                    if (lane == 0) was = atomicExch(a.claimed + u, LIST_CLAIMED);
+                    if (__shfl_sync(0xffffffffu, was, 0) != LIST_CLAIMED) id1 = u;
                 }
             }
         }

@@ -222,6 +222,7 @@ PermuteMeta meta_of(moe_fp8_handle_t h) {
     m.mlp_ready = at<int>(h, h->L.mlp_ready);
     m.mlp_claimed = at<int>(h, h->L.mlp_claimed);
     m.mlp_grid = std::min(h->sm_count, MLP_MAX_GRID);
+    m.mlp_left = h->lists_left_open;
     m.slot_to_row = at<int>(h, h->L.slot_to_row);
     m.row_to_slot = at<int>(h, h->L.row_to_slot);
     m.row_token = at<int>(h, h->L.row_token);
@@ -578,7 +579,7 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
         }
         // stage 3: GEMM1 + SwiGLU + re-quantisation, GEMM2
         if (h->short_tile_min_tokens > 0 && T >= h->short_tile_min_tokens) g1.wm_rows = g2.wm_rows = WM_TOKENS;
-        MlpArgs a = {g1, g2, 3, m.mlp_claimed, m.mlp_ready, h->lists_left_open};
+        MlpArgs a = {g1, g2, 3, m.mlp_claimed, m.mlp_ready};
         auto mlp = [&](int phases) {
             a.phases = phases;
             return launch(grouped_mlp_kernel, m.mlp_grid, G_THREADS, GeomFull::SMEM_BYTES, stream, pdl, h->tm_a1, h->tm_a1_small,

@@ -17,6 +17,8 @@
 namespace moe {
 
 constexpr int TILE_M = 128;              // GEMM tile height (rows)
+// A list of GEMM1 tiles in `mlp_claimed`: open to all, being worked on, open to all but its own CTA.
+constexpr int LIST_OPEN = 0, LIST_CLAIMED = 1, LIST_LEFT = 2;
 
 struct PermuteMeta {
     int* block_hist;     // [nblk, E_loc] per-block counts, turned into per-block bases by the last block
@@ -30,6 +32,7 @@ struct PermuteMeta {
     int* mlp_ready;      // [max_m_tiles] grouped_mlp_kernel's counters, zeroed with the tables: parts of GEMM1 stored,
     int* mlp_claimed;    // [mlp_grid] and lists of tiles claimed
     int mlp_grid;
+    int mlp_left;        // test hook: the first lists, which their own CTAs leave to the others (0 outside of tests)
     int* slot_to_row;    // [T*8] padded row of each slot, -1 when the slot's expert is not local
     int* row_to_slot;    // [T*8] canonical row -> slot id (first S entries valid)
     int* row_token;      // [row_cap] padded row -> token (valid rows only)
@@ -92,7 +95,7 @@ __device__ __forceinline__ void scan_experts(int E_loc, int* s_cnt, int* s_pad, 
             m.mlp_ready[t0 + i] = 0;
         }
     }
-    for (int v = tid; v < m.mlp_grid; v += blockDim.x) m.mlp_claimed[v] = 0;
+    for (int v = tid; v < m.mlp_grid; v += blockDim.x) m.mlp_claimed[v] = v < m.mlp_left ? LIST_LEFT : LIST_OPEN;
     if (tid == 0) {  // entries past E_loc count nothing, so entry E_loc already holds the totals
         m.expert_offset[E_loc] = s_cnt[E_loc];
         m.padded_offset[E_loc] = s_pad[E_loc];

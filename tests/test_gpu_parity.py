@@ -559,7 +559,7 @@ def test_one_launch_for_both_gemms(cuda_device, dims, tokens, kw):
                                               (1000, 256, False)])  # six and seven
 def test_lists_of_gemm1_tiles_that_other_ctas_take_over(cuda_device, tokens, eloc, skew):
     # CTAs that have not started when others are through with their tiles, made certain: 1, 40 (beyond the first 32
-    # entries of the table) and all but one of the CTAs leave their lists open.  The CTA that takes one over announces
+    # entries of the table) and all but one of the CTAs never take their own lists.  The CTA that takes one over announces
     # the rows of its own and of the adopted lists, and everybody's GEMM2 tiles wait for them.
     dims = syn.LayerDims(hidden=512, intermediate=512, num_local_experts=eloc)
     wl = _wl(tokens, dims, seed=1100 + eloc, skew=skew)
