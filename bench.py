@@ -39,8 +39,7 @@ W2_BYTES_PER_EXPERT = 7168 * 2048 + 56 * 16 * 4
 FP8_DATASHEET_TFLOPS = 4500.0
 HBM_DATASHEET_GBS = 8000.0
 # Measured DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch divided by the algorithmic
-# bytes of the same launch, from the committed ncu captures (profiles/fused_kernel_dsv3_T8_E32.md,
-# launches_dsv3_T64_E32.md, traffic_grouped_mlp_*.md): in the weight-streaming regime the T = 8 and T = 64 workloads
+# bytes of the same launch, from the committed ncu captures (see profiles/): in the weight-streaming regime the T = 8 and T = 64 workloads
 # (fused kernel) and the T = 1024 workload (both GEMMs in one launch) themselves and 200 tokens (a launch per
 # GEMM), in the tensor-bound regime the skewed T = 8192 workload itself (one launch) and T = 16384 with 64
 # local experts (a launch per GEMM), whose traffic is scaled to a full launch by the algorithmic bytes, since both
