@@ -149,6 +149,7 @@ struct GemmArgs {
     const int* tile_row0;     // fused kernel: first padded row of each (sub-)tile; else null: tile * TILE_M
     int wm_rows;              // grouped_mlp_kernel: row tiles with at most this many rows (0 or 32) run with the
                               // weights on the M side of the MMAs, see epilogue_tile_wm
+    int* ready;               // GEMM1 in one launch with GEMM2: [row tiles] warps that have stored their part, zero at launch
     const float* a_scale_t;   // [num_kb, row_cap]
     const float* w_scale;     // [E_loc, w_rows/128, num_kb]
     uint8_t* out_fp8;         // GEMM1: [row_cap, I] e4m3
@@ -216,7 +217,8 @@ struct GemmCtrl {
     uint64_t full[G_MAX_STAGES];   // stage filled (TMA transaction bytes)
     uint64_t done[G_MAX_STAGES];   // the MMAs that read the stage have finished: stage free AND accumulator ready
     uint64_t tmem_empty[G_MAX_STAGES];   // accumulator buffers: two, or one per stage (weights-on-M roles)
-    uint64_t amax_bar[2];
+    uint64_t amax_bar;         // all epilogue warps have their row maxima in the exchange area (weights on M)
+    uint64_t amax_quad[4];     // the same for the two warps that share a quadrant's rows (full row tiles)
     uint64_t drain_bar[2];
     uint64_t sync_bar[2];      // fused kernel: rendezvous of the epilogue warps at the end of a tile
     uint32_t tmem_slot;
@@ -241,6 +243,24 @@ __host__ __device__ __forceinline__ size_t y_block_offset(int r, int c16, int n_
     const int n = c16 / 16, half = (c16 % 16) / 8, q = c16 % 8;
     return (((static_cast<size_t>(m_tile) * n_tiles + n) * 2 + half) * 4 + quad) * 8192 + q * 1024 + lane * 32;
 }
+
+// An epilogue warp's turns at the row-maximum exchange.  Bit 0: which half of the exchange area the next GEMM1 tile uses
+// (they take turns, so that a warp may be in the next tile while another one still reads); bits 1 and 2: the phases of
+// amax_bar and amax_quad.
+struct AmaxTurn {
+    uint32_t bits;
+    __device__ __forceinline__ uint32_t area() const { return bits & 1; }
+    __device__ __forceinline__ uint32_t all() const { return (bits >> 1) & 1; }
+    __device__ __forceinline__ uint32_t quad() const { return (bits >> 2) & 1; }
+};
+template <bool B>
+struct Bool {
+    static constexpr bool value = B;
+};
+
+// x * sigmoid(x) with the hardware exp2 and reciprocal approximations (a few ulp): a tile's tail runs while the tensor pipe
+// idles, so its instruction count matters.
+__device__ __forceinline__ float silu_fast(float x) { return __fdividef(x, 1.0f + __expf(-x)); }
 
 // The CTA's carve-up of shared memory and the values every role needs.
 struct Cta {
@@ -338,8 +358,8 @@ __device__ __forceinline__ void gemm_cta_setup(Cta& c, uint8_t* smem_raw, int fu
             mbar_init(smem_u32(&ctrl->done[s]), GEO::FACTORS ? 2 : 1);  // the MMAs' commit; the factor warp
         }
         for (int b = 0; b < G_MAX_STAGES; ++b) mbar_init(smem_u32(&ctrl->tmem_empty[b]), G_EPI_WARPS);
-        mbar_init(smem_u32(&ctrl->amax_bar[0]), G_EPI_WARPS * 32);
-        mbar_init(smem_u32(&ctrl->amax_bar[1]), G_EPI_WARPS * 32);
+        mbar_init(smem_u32(&ctrl->amax_bar), G_EPI_WARPS);
+        for (int q = 0; q < 4; ++q) mbar_init(smem_u32(&ctrl->amax_quad[q]), 2);
         mbar_init(smem_u32(&ctrl->drain_bar[0]), 1);
         mbar_init(smem_u32(&ctrl->drain_bar[1]), 1);
         mbar_init(smem_u32(&ctrl->sync_bar[0]), G_EPI_WARPS * 32);
@@ -590,11 +610,9 @@ __device__ __forceinline__ void issuer_tiles_wm(const Cta& c, const GemmArgs& g,
 // the epilogue 1-2 us per tile, and the fence of an announcement about 400 clocks, so tiles are announced together: those
 // before in the tails of the last two tiles of a list, the last one behind it.
 struct Announce {
-    int* ready;       // [row tiles]; null: nobody waits (one GEMM per launch)
-    int n_tiles, stride;
-    int id, count;    // tiles id, id + stride, ... (row tile * n_tiles + column tile)
+    int id, count;    // tiles id, id + grid, ... (row tile * n_tiles + column tile)
     // The whole warp; the staging of the warp's last bulk store may be written again afterwards.
-    __device__ __forceinline__ void settle(int lane, bool announce) {
+    __device__ __forceinline__ void settle(int lane, bool announce, int* ready, int n_tiles) {
         if (!announce || count == 0) {
             if (lane == 0) bulk_wait_read_all();
             __syncwarp();
@@ -604,11 +622,10 @@ struct Announce {
         fence_proxy_async();
         __syncwarp();
         __threadfence();
-        for (int k = lane; k < count; k += 32) atomicAdd(ready + (id + k * stride) / n_tiles, 1);
+        for (int k = lane; k < count; k += 32) atomicAdd(ready + (id + k * static_cast<int>(gridDim.x)) / n_tiles, 1);
         count = 0;
     }
     __device__ __forceinline__ void add(int tile) {
-        if (ready == nullptr) return;
         if (count == 0) id = tile;
         ++count;
     }
@@ -629,7 +646,7 @@ struct Announce {
 // the unsplit tile uses, and finishes the tile.  Every fp32 operation is the one of the unsplit tile.
 template <int MODE, bool FUSED, class GEO, bool SHARED, bool SPLIT = false>
 __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g, const FusedArgs* f, int m_tile, int n,
-                                                 uint32_t& it, uint32_t& tile_iter, uint32_t& sync_iter, int kb0 = 0,
+                                                 uint32_t& it, AmaxTurn& turn, uint32_t& sync_iter, int kb0 = 0,
                                                  int kb1 = -1, int parts = 1, Announce* announce = nullptr,
                                                  bool settle = false) {
     static_assert(!SPLIT || FUSED, "only the fused kernel cuts K ranges");
@@ -640,7 +657,7 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
     // (lane l of quadrant q holds weight row 32 q + l of each 128-row block)
     const uint32_t t_lane = c.tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + th * 16;
     const size_t row_cap = static_cast<size_t>(g.row_cap);
-    uint32_t* amax_x = reinterpret_cast<uint32_t*>(c.amax_x);   // [2 parities][256]: [2 token halves][4 quadrants][16] used
+    uint32_t* amax_x = reinterpret_cast<uint32_t*>(c.amax_x);   // [2 turns][256]: [2 token halves][4 quadrants][16] used
     const int num_kb = g.num_kb;
     const int e = SHARED ? __ldcg(g.tile_expert + m_tile) : tile_expert_of(c, g, m_tile);
     const int rows_valid = SHARED ? __ldcg(g.tile_rows + m_tile) : tile_rows_of(c, g, m_tile);
@@ -803,7 +820,7 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
     const size_t row0 = static_cast<size_t>(tile_row0) + th * 16;  // padded row of this thread's token 0
     const uint32_t wst_off = (warp - 4) * (SHARED ? G_STORE_WARP_BYTES : 512);  // this warp's staging
     if (SHARED) {  // the warp's last TMA store may still be reading the area
-        announce->settle(lane, settle);
+        announce->settle(lane, settle, g.ready, g.n_tiles);
     }
     const int valid = min(16, rows_valid - th * 16);                     // tokens of this thread that exist
     if (MODE == 1) {
@@ -819,14 +836,11 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
         }
 #pragma unroll
         for (int t = 0; t < 16; ++t) {
-            const float gt = acc[t];
-            cc[t] = __fdividef(gt, 1.0f + __expf(-gt)) * acc[16 + t];
+            cc[t] = silu_fast(acc[t]) * acc[16 + t];
             // |x| as an integer orders like the float: the warp's maximum over its 32 output columns
             wmax[t] = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(cc[t])));
         }
-        const uint32_t par = tile_iter & 1;
-        // (inside the half of the exchange area that belongs to this parity in the other orientation as well)
-        uint32_t* xq = amax_x + par * (2 * TILE_M) + th * 64;
+        uint32_t* xq = amax_x + turn.area() * (2 * TILE_M) + th * 64;
         {
             uint32_t mine = 0;
 #pragma unroll
@@ -834,13 +848,14 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
                 if (lane == t) mine = wmax[t];
             if (lane < 16) xq[quad * 16 + lane] = mine;
         }
-        const uint32_t xbar = smem_u32(&ctrl->amax_bar[par]);
-        mbar_arrive(xbar);
-        if (!__all_sync(0xffffffffu, mbar_wait(xbar, (tile_iter >> 1) & 1, c.abort_flag, c.limit))) {
+        const uint32_t xbar = smem_u32(&ctrl->amax_bar);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(xbar);
+        if (!__all_sync(0xffffffffu, mbar_wait(xbar, turn.all(), c.abort_flag, c.limit))) {
             if (lane == 0) raise(ctrl, g.status, DEV_TIMEOUT_EPILOGUE);
             return false;
         }
-        ++tile_iter;
+        turn.bits ^= 3;
         // lane t < 16 owns the scale of token t's 128-column block; everybody fetches its reciprocal
         float my_sc = 1.0f, my_inv = 1.0f;
         if (lane < 16) {
@@ -977,16 +992,16 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
 
 template <int MODE, bool FUSED, class GEO, class SEQ>
 __device__ __forceinline__ void epilogue_tiles_wm(const Cta& c, const GemmArgs& g, const FusedArgs* f, const SEQ& seq,
-                                                  uint32_t& it, uint32_t& tile_iter, uint32_t& sync_iter, bool& ok,
+                                                  uint32_t& it, AmaxTurn& turn, uint32_t& sync_iter, bool& ok,
                                                   KSplit ks) {
     for (int j = 0, item; ok && (item = seq.at(j)) < seq.count; ++j) {
         const int tile = item / ks.parts, kb0 = (item - tile * ks.parts) * ks.len;
         const int m_tile = tile / g.n_tiles, n = tile - m_tile * g.n_tiles;
         // (two instantiations, so that the unsplit tile's loop carries nothing of the split)
         ok = (FUSED && MODE == 1 && ks.parts > 1)
-                 ? epilogue_tile_wm<MODE, FUSED, GEO, false, FUSED && MODE == 1>(c, g, f, m_tile, n, it, tile_iter, sync_iter, kb0,
+                 ? epilogue_tile_wm<MODE, FUSED, GEO, false, FUSED && MODE == 1>(c, g, f, m_tile, n, it, turn, sync_iter, kb0,
                                                                                 min(g.num_kb, kb0 + ks.len), ks.parts)
-                 : epilogue_tile_wm<MODE, FUSED, GEO, false, false>(c, g, f, m_tile, n, it, tile_iter, sync_iter);
+                 : epilogue_tile_wm<MODE, FUSED, GEO, false, false>(c, g, f, m_tile, n, it, turn, sync_iter);
     }
 }
 
@@ -1065,9 +1080,10 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmA2, const __grid_consta
         }
     } else {
         reg_alloc<232>();
-        uint32_t tile_iter = 0, sync_iter = 0;
-        epilogue_tiles_wm<1, true, GEO>(c, g1, &f, tr1, it, tile_iter, sync_iter, ok, ks1);
-        epilogue_tiles_wm<2, true, GEO>(c, g2, &f, tr2(), it, tile_iter, sync_iter, ok, ks2);
+        uint32_t sync_iter = 0;
+        AmaxTurn turn{0};
+        epilogue_tiles_wm<1, true, GEO>(c, g1, &f, tr1, it, turn, sync_iter, ok, ks1);
+        epilogue_tiles_wm<2, true, GEO>(c, g2, &f, tr2(), it, turn, sync_iter, ok, ks2);
     }
 
     __syncwarp();

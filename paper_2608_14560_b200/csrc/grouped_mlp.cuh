@@ -40,9 +40,12 @@ struct MlpArgs {
     GemmArgs g1, g2;
     int phases;          // bit 0: GEMM1's tiles, bit 1: GEMM2's; both: a GEMM2 tile waits for its rows
     int* claimed;        // [grid] the lists of GEMM1 tiles, LIST_OPEN (or LIST_LEFT) at launch (both GEMMs only)
-    int* ready;          // [row tiles] warps that have stored their part, zero at launch
 };
 
+__device__ __forceinline__ TileInfo read_tile(const Cta& c, uint32_t i) {  // an entry that has been waited for
+    const int4 v = ld_shared_v4(smem_u32(&c.ctrl->sched[i % SCHED_SLOTS]));
+    return TileInfo{v.x, v.y, v.z, v.w};
+}
 // Entry i of the CTA's work list, as the factor warp published it.  A role that gave up here while the others went on
 // would leave them at a named barrier, whose wait has no limit (see mlp_issuer), so this wait has to outlast every chain of
 // waits in front of an entry or the list's end, and its limit is not the one that a test may shorten: with that, a role that
@@ -52,8 +55,7 @@ __device__ __forceinline__ TileInfo next_tile(const Cta& c, uint32_t i) {
     int zero = 0;
     const uint32_t slot = i % SCHED_SLOTS;
     if (!mbar_wait(smem_u32(&c.ctrl->sched_full[slot]), (i / SCHED_SLOTS) & 1, &zero, SCHED_LIMIT_CLOCKS)) return TileInfo{};
-    const int4 v = ld_shared_v4(smem_u32(&c.ctrl->sched[slot]));
-    return TileInfo{v.x, v.y, v.z, v.w};
+    return read_tile(c, i);
 }
 // The same by a whole warp: all lanes see the entry or none does.
 __device__ __forceinline__ TileInfo next_tile_warp(const Cta& c, uint32_t i) {
@@ -344,7 +346,7 @@ __device__ __forceinline__ void mlp_factors(const Cta& c, const MlpArgs& a) {
                 // give up after one, which ends this wait as well.  Rows that never come are thus reported as the time-out
                 // of whichever role that is.)
                 if (!m1 && a.phases == 3)
-                    there = wait_counter(a.ready + t.m_tile(), ready_target, c.abort_flag, 4 * c.limit);
+                    there = wait_counter(a.g1.ready + t.m_tile(), ready_target, c.abort_flag, 4 * c.limit);
                 if (there) mbar_arrive(smem_u32(&ctrl->sched_rows[fi % SCHED_SLOTS]));
             }
             there = __shfl_sync(0xffffffffu, there, 0);
@@ -422,24 +424,52 @@ __device__ __forceinline__ void mlp_factors(const Cta& c, const MlpArgs& a) {
 // acc[0..64) += v * f with packed fp32 FMAs: one instruction, two independent round-to-nearest FMAs, the bits of the
 // scalar form.  Beside scalar FMAs the MMA issuers, which share the schedulers with the epilogue warps, needed 955
 // clocks per K-block in a probe of this loop, beside packed ones 672 (602 beside an epilogue without FMAs).
+template <bool FIRST>
 __device__ __forceinline__ void fma64(float* acc, const float (&v)[64], float f) {
     const uint64_t p = pack_f32x2(__float_as_uint(f), __float_as_uint(f));
 #pragma unroll
     for (int j = 0; j < 64; j += 2) {
         const uint64_t a = fma_f32x2(pack_f32x2(__float_as_uint(v[j]), __float_as_uint(v[j + 1])), p,
-                                     pack_f32x2(__float_as_uint(acc[j]), __float_as_uint(acc[j + 1])));
+                                     FIRST ? 0ull : pack_f32x2(__float_as_uint(acc[j]), __float_as_uint(acc[j + 1])));
         acc[j] = __uint_as_float(static_cast<uint32_t>(a));
         acc[j + 1] = __uint_as_float(static_cast<uint32_t>(a >> 32));
     }
 }
 
 // ---------------- epilogue warps ----------------
+// bf16 rows out in a tile-blocked layout: block (row tile, column tile, half, quadrant) holds a warp's 32 rows x 128
+// columns as [8 column groups][32 rows][16 bf16], so every warp store instruction writes 1 KB of contiguous memory (32
+// bytes per lane).  `p` is where the first of four groups goes.
+__device__ __forceinline__ void store_rows64(uint8_t* p, const float* acc) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        uint32_t w[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const __nv_bfloat162 pr = __floats2bfloat162_rn(acc[q * 16 + 2 * i], acc[q * 16 + 2 * i + 1]);
+            w[i] = *reinterpret_cast<const uint32_t*>(&pr);
+        }
+        st_global_v8(p + q * 1024, w);
+    }
+}
+
 // GEMM1: gate/up projection + SwiGLU + re-quantisation; tmOut describes the e4m3 output [row_cap, I] for 64-byte x
-// 32-row TMA stores.  GEMM2: down projection, bf16 rows out in the tile-blocked layout.  One full row tile; false: a
-// wait gave up (the code is in the status word) and `it` stands at the K-block whose buffer was not handed back.
+// 32-row TMA stores.  GEMM2: down projection, bf16 rows out in the tile-blocked layout.  One full row tile, entry i of the
+// list; false: a wait gave up (the code is in the status word) and `it` stands at the K-block whose buffer was not handed
+// back.  Otherwise `t` is the next entry.
+// The MMAs run two K-blocks ahead and then wait for this function to come round, so what lies between the last K-block of
+// a tile and the first of the next is lost beyond about 1700 clocks (it was 5600 of GEMM1's 51 000 and 1800 of GEMM2's
+// 14 600).  Hence no clearing of the sums, an exchange of maxima between the two warps concerned and not among all eight,
+// the next entry read beside it (GEMM2: not behind all of the stores, which hold up every later access to shared memory),
+// and the halves of the weights taken in the order gate, up instead of changing places behind the loop.
+// The loop has 192 of its 224 registers in its two arrays: what it does not need, the tile's entry for one, is fetched again
+// behind it.  Spilling decides here: forms with 110 to 380 bytes of spilled registers instead of 20 were 2 to 8 % slower,
+// tiles of the other orientation included.
+// us of the GEMM launches before / this form: 8192 skewed tokens on 32 experts 1536 / 1432, 4096 tokens 399 / 387, 8192 tokens
+// on 256 experts 3926 / 3674.  What is left of the tails is 1 % (the SwiGLU left out altogether: 1416, 382).
 template <int MODE, class GEO>
-__device__ __forceinline__ bool mlp_epilogue_tile(const Cta& c, const CUtensorMap* tmOut, const GemmArgs& g, const TileInfo& t,
-                                                  uint32_t& it, uint32_t& tile_iter, Announce& announce) {
+__device__ __forceinline__ bool mlp_epilogue_tile(const Cta& c, const CUtensorMap* tmOut, const GemmArgs& g, uint32_t i,
+                                                  TileInfo& t, uint32_t& it, AmaxTurn& turn, Announce& announce) {
     static_assert(GEO::A_ROWS == TILE_M && GEO::STORE_BYTES == G_EPI_WARPS * G_STORE_WARP_BYTES, "full row tiles");
     GemmCtrl* ctrl = c.ctrl;
     const int warp = c.warp, lane = c.lane;
@@ -447,19 +477,17 @@ __device__ __forceinline__ bool mlp_epilogue_tile(const Cta& c, const CUtensorMa
     const int half = widx >> 2;              // which 128-column half of the tile
     const int quad = warp & 3;               // TMEM lane quadrant this warp may read
     const int r_in_tile = quad * 32 + lane;  // accumulator row == TMEM lane
-    const uint32_t t_lane = c.tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + half * G_HALF_N;
-    const size_t row_cap = static_cast<size_t>(g.row_cap);
-    float* amax_x = c.amax_x;
-    uint8_t* stage = c.store_stage + widx * G_STORE_WARP_BYTES;  // staging of this warp's GEMM1 rows
-    const int num_kb = g.num_kb, m_tile = t.m_tile(), n = t.n, rows_valid = t.rows;
-    const size_t row = static_cast<size_t>(m_tile) * TILE_M + r_in_tile;
-    // GEMM1: of this warpgroup's 128 columns, [0,64) are gate and [64,128) the matching up columns; GEMM2: one factor
-    const uint32_t factors = smem_u32(c.scale_ring + r_in_tile + (MODE == 1 ? 0 : half * GEO::A_ROWS));
+    // GEMM1: of this warpgroup's 128 columns, one half of 64 are gate columns (they go to acc[0..64)) and the other the
+    // matching up columns, each with its own factor; GEMM2: one factor
+    const uint32_t swap = MODE == 1 && g.up_first ? 1 : 0;
+    const uint32_t t_lane = c.tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + half * G_HALF_N + swap * 64;
+    const uint32_t factors = smem_u32(c.scale_ring + r_in_tile + (MODE == 1 ? swap : half) * GEO::A_ROWS);
+    const uint32_t second = 64 - swap * 128, second_f = (GEO::A_ROWS - swap * 2 * GEO::A_ROWS) * 4;
     float acc[128];
-#pragma unroll
-    for (int j = 0; j < 128; ++j) acc[j] = 0.0f;
 
-    for (int kb = 0; kb < num_kb; ++kb, ++it) {
+    // One K-block; the first one starts the sums (nothing has to be cleared between two tiles).
+    auto k_block = [&](auto first) -> bool {
+        constexpr bool FIRST = decltype(first)::value;
         const uint32_t s = it % GEO::STAGES, ph = (it / GEO::STAGES) & 1, buf = it & 1;
         // Every lane polls (a single polling lane plus a broadcast was measured 2.5 % slower); the vote
         // keeps the warp converged when a wait gives up: either all lanes go on or none does.
@@ -473,130 +501,122 @@ __device__ __forceinline__ bool mlp_epilogue_tile(const Cta& c, const CUtensorMa
         tmem_ld32_issue(col, v);
         tmem_ld32_issue(col + 32, v + 32);
         const uint32_t slot = factors + (it % GEO::SCALE_SLOTS) * 2 * GEO::A_ROWS * 4;
-        const float f0 = ld_shared_f32(slot), f1 = MODE == 1 ? ld_shared_f32(slot + GEO::A_ROWS * 4) : f0;
+        const float f0 = ld_shared_f32(slot), f1 = MODE == 1 ? ld_shared_f32(slot + second_f) : f0;
         tmem_wait_ld(v);
-        fma64(acc, v, f0);
-        tmem_ld32_issue(col + 64, v);
-        tmem_ld32_issue(col + 96, v + 32);
+        fma64<FIRST>(acc, v, f0);
+        tmem_ld32_issue(col + second, v);
+        tmem_ld32_issue(col + second + 32, v + 32);
         tmem_wait_ld(v);
         tc_fence_before();
         bar_arrive(ACC_BARRIER + buf, ACC_BARRIER_THREADS);
-        fma64(acc + 64, v, f1);
-    }
+        fma64<FIRST>(acc + 64, v, f1);
+        ++it;
+        return true;
+    };
+    const uint32_t end = it + g.num_kb;
+    if (!k_block(Bool<true>{})) return false;
+    while (it != end)
+        if (!k_block(Bool<false>{})) return false;
 
-    if (MODE == 1) {
-        // The staging area of this warp was handed to the TMA engine at the end of the previous tile;
-        // by now (a whole tile later) that copy has long landed, so this wait does not stall.
-        announce.settle(lane, t.key & TileInfo::LAST_TWO);
-        const int sw = (lane >> 1) & 3;  // 64-byte swizzle: 16-byte chunk index ^= bits 7..8 of the address
-        // SwiGLU on this thread's 64 columns, then the row's 128-wide amax across the two halves
-        float cc[64];
-        float amax = 0.0f;
-        if (g.up_first) {
+    t = read_tile(c, i);
+    const int m_tile = t.m_tile(), n = t.n, rows_valid = t.rows;
+    if (MODE == 2) {
+        uint8_t* blk = reinterpret_cast<uint8_t*>(g.out_bf16) +
+                       (((static_cast<size_t>(m_tile) * g.n_tiles + n) * 2 + half) * 4 + quad) * 8192 + lane * 32;
+        if (quad * 32 < rows_valid) store_rows64(blk, acc);
+        t = next_tile_warp(c, i + 1);  // (not behind all of the stores)
+        if (quad * 32 < rows_valid) store_rows64(blk + 4096, acc + 64);
+        return true;
+    }
+    const size_t row_cap = static_cast<size_t>(g.row_cap);
+    const size_t row = static_cast<size_t>(m_tile) * TILE_M + r_in_tile;
+    uint8_t* stage = c.store_stage + widx * G_STORE_WARP_BYTES;  // staging of this warp's GEMM1 rows
+    // The staging area of this warp was handed to the TMA engine at the end of the previous tile; by now (a whole tile
+    // later) that copy has long landed, so this wait does not stall.
+    announce.settle(lane, t.key & TileInfo::LAST_TWO, g.ready, g.n_tiles);
+    const int sw = (lane >> 1) & 3;  // 64-byte swizzle: 16-byte chunk index ^= bits 7..8 of the address
+    // SwiGLU on this thread's 64 columns, then the row's 128-wide amax across the two halves
+    float cc[64];
+    float amax = 0.0f;
 #pragma unroll
-            for (int j = 0; j < 64; ++j) {
-                const float x = acc[j];
-                acc[j] = acc[64 + j];
-                acc[64 + j] = x;
+    for (int j = 0; j < 64; ++j) {
+        cc[j] = silu_fast(acc[j]) * acc[64 + j];
+        amax = fmaxf(amax, fabsf(cc[j]));
+    }
+    // The two warps of these 32 rows exchange their maxima.
+    float* ax = c.amax_x + turn.area() * 2 * TILE_M;
+    ax[half * TILE_M + r_in_tile] = amax;
+    const uint32_t xbar = smem_u32(&ctrl->amax_quad[quad]);
+    __syncwarp();
+    if (lane == 0) mbar_arrive(xbar);
+    t = next_tile_warp(c, i + 1);
+    if (!__all_sync(0xffffffffu, mbar_wait(xbar, turn.quad(), c.abort_flag, c.limit))) {
+        if (lane == 0) raise(ctrl, g.status, DEV_TIMEOUT_EPILOGUE);
+        return false;
+    }
+    turn.bits ^= 5;
+    amax = fmaxf(amax, *reinterpret_cast<volatile float*>(&ax[(half ^ 1) * TILE_M + r_in_tile]));
+    const float sc = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, 448.0f);
+    const float inv_sc = __frcp_rn(sc);
+    if (quad * 32 < rows_valid) {
+        // e4m3 rows out: 32 rows x 64 bytes per warp, staged with the 64-byte swizzle, one TMA store
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            uint32_t w[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int j = q * 16 + k * 4;
+                const uint32_t lo = __nv_cvt_float2_to_fp8x2(
+                    make_float2(cc[j] * inv_sc, cc[j + 1] * inv_sc), __NV_SATFINITE, __NV_E4M3);
+                const uint32_t hi = __nv_cvt_float2_to_fp8x2(
+                    make_float2(cc[j + 2] * inv_sc, cc[j + 3] * inv_sc), __NV_SATFINITE, __NV_E4M3);
+                w[k] = lo | (hi << 16);
             }
+            *reinterpret_cast<uint4*>(stage + lane * 64 + ((q ^ sw) << 4)) =
+                make_uint4(w[0], w[1], w[2], w[3]);
         }
-#pragma unroll
-        for (int j = 0; j < 64; ++j) {
-            // silu(g) * u with the hardware exp2 and reciprocal approximations (a few ulp): the
-            // tile's tail runs while the tensor pipe idles, so its instruction count matters.
-            const float gt = acc[j];
-            cc[j] = __fdividef(gt, 1.0f + __expf(-gt)) * acc[64 + j];
-            amax = fmaxf(amax, fabsf(cc[j]));
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+            tma_store_2d(tmOut, smem_u32(stage), n * 128 + half * 64, m_tile * TILE_M + quad * 32);
+            bulk_commit_group();
         }
-        const uint32_t par = tile_iter & 1;
-        amax_x[(par * 2 + half) * TILE_M + r_in_tile] = amax;
-        const uint32_t xbar = smem_u32(&ctrl->amax_bar[par]);
-        mbar_arrive(xbar);
-        if (!__all_sync(0xffffffffu, mbar_wait(xbar, (tile_iter >> 1) & 1, c.abort_flag, c.limit))) {
-            if (lane == 0) raise(ctrl, g.status, DEV_TIMEOUT_EPILOGUE);
-            return false;
-        }
-        ++tile_iter;
-        amax = fmaxf(amax,
-                     *reinterpret_cast<volatile float*>(&amax_x[(par * 2 + (half ^ 1)) * TILE_M + r_in_tile]));
-        const float sc = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, 448.0f);
-        const float inv_sc = __frcp_rn(sc);
-        if (quad * 32 < rows_valid) {
-            // e4m3 rows out: 32 rows x 64 bytes per warp, staged with the 64-byte swizzle, one TMA store
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                uint32_t w[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int j = q * 16 + i * 4;
-                    const uint32_t lo = __nv_cvt_float2_to_fp8x2(
-                        make_float2(cc[j] * inv_sc, cc[j + 1] * inv_sc), __NV_SATFINITE, __NV_E4M3);
-                    const uint32_t hi = __nv_cvt_float2_to_fp8x2(
-                        make_float2(cc[j + 2] * inv_sc, cc[j + 3] * inv_sc), __NV_SATFINITE, __NV_E4M3);
-                    w[i] = lo | (hi << 16);
-                }
-                *reinterpret_cast<uint4*>(stage + lane * 64 + ((q ^ sw) << 4)) =
-                    make_uint4(w[0], w[1], w[2], w[3]);
-            }
-            fence_async_smem();
-            __syncwarp();
-            if (lane == 0) {
-                tma_store_2d(tmOut, smem_u32(stage), n * 128 + half * 64, m_tile * TILE_M + quad * 32);
-                bulk_commit_group();
-            }
-            if (half == 0 && r_in_tile < rows_valid)
-                g.out_scale_t[static_cast<size_t>(n) * row_cap + row] = sc;
-        }
-    } else {
-        // bf16 rows out in a tile-blocked layout: block (row tile, column tile, half, quadrant) holds
-        // this warp's 32 rows x 128 columns as [8 column groups][32 rows][16 bf16], so every warp
-        // store instruction writes 1 KB of contiguous memory (32 bytes per lane).
-        if (quad * 32 < rows_valid) {
-            uint8_t* blk = reinterpret_cast<uint8_t*>(g.out_bf16) +
-                           (((static_cast<size_t>(m_tile) * g.n_tiles + n) * 2 + half) * 4 + quad) * 8192 +
-                           lane * 32;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                uint32_t w[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const __nv_bfloat162 pr = __floats2bfloat162_rn(acc[q * 16 + 2 * i], acc[q * 16 + 2 * i + 1]);
-                    w[i] = *reinterpret_cast<const uint32_t*>(&pr);
-                }
-                st_global_v8(blk + q * 1024, w);
-            }
-        }
+        if (half == 0 && r_in_tile < rows_valid)
+            g.out_scale_t[static_cast<size_t>(n) * row_cap + row] = sc;
     }
     return true;
 }
 
 template <class GEO>
 __device__ __forceinline__ void mlp_epilogue(const Cta& c, const CUtensorMap* tmOut, const MlpArgs& a) {
-    uint32_t it = 0, tile_iter = 0, unused = 0;
+    uint32_t it = 0, unused = 0;
+    AmaxTurn turn{0};
     bool ok = true;
-    Announce announce{a.phases == 3 ? a.ready : nullptr, a.g1.n_tiles, static_cast<int>(gridDim.x), 0, 0};
-    for (uint32_t i = 0;; ++i) {
-        const TileInfo t = next_tile_warp(c, i);
-        if (t.mode() == 0) break;
+    Announce announce{0, 0};
+    TileInfo t = next_tile_warp(c, 0);
+    for (uint32_t i = 0; t.mode() != 0; ++i) {
         const uint32_t end = it + (t.mode() == 1 ? a.g1.num_kb : a.g2.num_kb);
+        const bool wm = t.rows <= a.g1.wm_rows;
+        const int tile = t.m_tile() * a.g1.n_tiles + t.n;  // (GEMM1)
+        const bool last = t.key & TileInfo::LAST;
         if (ok) {
-            const bool wm = t.rows <= a.g1.wm_rows;
             if (t.mode() == 1) {
-                ok = wm ? epilogue_tile_wm<1, false, GEO, true>(c, a.g1, nullptr, t.m_tile(), t.n, it, tile_iter, unused, 0, -1, 1,
+                ok = wm ? epilogue_tile_wm<1, false, GEO, true>(c, a.g1, nullptr, t.m_tile(), t.n, it, turn, unused, 0, -1, 1,
                                                                 &announce, t.key & TileInfo::LAST_TWO)
-                        : mlp_epilogue_tile<1, GEO>(c, tmOut, a.g1, t, it, tile_iter, announce);
+                        : mlp_epilogue_tile<1, GEO>(c, tmOut, a.g1, i, t, it, turn, announce);
                 if (ok) {
-                    announce.add(t.m_tile() * a.g1.n_tiles + t.n);
-                    if (t.key & TileInfo::LAST) announce.settle(c.lane, true);  // somebody may be waiting for it
+                    if (a.phases == 3) announce.add(tile);
+                    if (last) announce.settle(c.lane, true, a.g1.ready, a.g1.n_tiles);  // somebody may be waiting for it
                 }
             } else {
-                ok = wm ? epilogue_tile_wm<2, false, GEO, true>(c, a.g2, nullptr, t.m_tile(), t.n, it, tile_iter, unused, 0, -1, 1,
+                ok = wm ? epilogue_tile_wm<2, false, GEO, true>(c, a.g2, nullptr, t.m_tile(), t.n, it, turn, unused, 0, -1, 1,
                                                                 &announce, false)
-                        : mlp_epilogue_tile<2, GEO>(c, tmOut, a.g2, t, it, tile_iter, announce);
+                        : mlp_epilogue_tile<2, GEO>(c, tmOut, a.g2, i, t, it, turn, announce);
             }
         }
         // After an abort: the hand-overs this warp still owes, waiting for the issuer so that no turn is taken twice.
         for (; it < end; ++it) bar_sync(ACC_BARRIER + (it & 1), ACC_BARRIER_THREADS);
+        if (!ok || wm) t = next_tile_warp(c, i + 1);
     }
     if (c.lane == 0) bulk_wait_all();
 }

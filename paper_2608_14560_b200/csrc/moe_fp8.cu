@@ -579,7 +579,8 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
         }
         // stage 3: GEMM1 + SwiGLU + re-quantisation, GEMM2
         if (h->short_tile_min_tokens > 0 && T >= h->short_tile_min_tokens) g1.wm_rows = g2.wm_rows = WM_TOKENS;
-        MlpArgs a = {g1, g2, 3, m.mlp_claimed, m.mlp_ready};
+        g1.ready = m.mlp_ready;
+        MlpArgs a = {g1, g2, 3, m.mlp_claimed};
         auto mlp = [&](int phases) {
             a.phases = phases;
             return launch(grouped_mlp_kernel, m.mlp_grid, G_THREADS, GeomFull::SMEM_BYTES, stream, pdl, h->tm_a1, h->tm_a1_small,
