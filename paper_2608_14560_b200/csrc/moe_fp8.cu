@@ -600,8 +600,10 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
             mark(ST_GEMM2);
         }
         {  // stage 4: weighted combine back to token order
-            const int grid = min(T, h->sm_count * 16);
-            MOE_LAUNCH(combine_kernel, grid, 256, 0, stream, pdl, T, H, static_cast<const int*>(m.slot_to_row),
+            const int groups = H / 16, parts = (groups + COMBINE_MAX_THREADS - 1) / COMBINE_MAX_THREADS;
+            const int threads = ((groups + parts - 1) / parts + 31) / 32 * 32;
+            const dim3 grid(min(T, h->sm_count * COMBINE_BLOCKS_PER_SM), parts);
+            MOE_LAUNCH(combine_kernel, grid, threads, 0, stream, pdl, T, H, static_cast<const int*>(m.slot_to_row),
                        static_cast<const float*>(topk_w), reinterpret_cast<const uint8_t*>(y),
                        static_cast<__nv_bfloat16*>(out));
             mark(ST_COMBINE);
