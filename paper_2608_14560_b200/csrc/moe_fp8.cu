@@ -235,6 +235,12 @@ PermuteMeta meta_of(moe_fp8_handle_t h) {
 }
 
 constexpr int PDL_MAX_TOKENS = 2048;
+// Beyond that the GEMMs alone, behind the gather: their CTAs set up and ask for the first weights on the SMs that have
+// finished gathering.  Up to this many expected local slots (tokens x 8 x the local share of the experts); us per forward on 32
+// experts without / with: uniform routing 309.0 / 300.7 at 2500 tokens, 437.6 / 435.5 at 4096, 423.7 / 418.6 at 6000 (another
+// draw); skewed 711.6 / 712.2 at 3000, 1071 / 1075 at 4096, 1584 / 1597 at 8192; 3950 / 3955 at 8192 on 256 experts.  The other
+// kernels gain nothing there (gather 0 to + 1.3 % with skewed routing, combine 0 to + 0.6 %).
+constexpr long long PDL_MLP_MAX_SLOTS = 6144;
 
 bool misaligned(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) != 0; }
 
@@ -445,6 +451,8 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
     // removes 10-13 us of launch gaps from a small batch; on large batches the early-resident blocks of the
     // next kernel cost the running GEMM about 6 %, so it is limited to the launch-latency-bound regime.
     const bool pdl = !h->stage_timing && T <= PDL_MAX_TOKENS;
+    const long long slots = static_cast<long long>(T) * R_TOPK * EL / R_EXPERTS;  // expected local ones
+    const bool pdl_mlp = pdl || (!h->stage_timing && slots <= PDL_MLP_MAX_SLOTS);
 
     // No memset: the first kernel clears the status word, and the ticket counter returns to zero by itself.
     h->ev_count = 0;
@@ -583,10 +591,9 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
         MlpArgs a = {g1, g2, 3, m.mlp_claimed};
         auto mlp = [&](int phases) {
             a.phases = phases;
-            return launch(grouped_mlp_kernel, m.mlp_grid, G_THREADS, GeomFull::SMEM_BYTES, stream, pdl, h->tm_a1, h->tm_a1_small,
+            return launch(grouped_mlp_kernel, m.mlp_grid, G_THREADS, GeomFull::SMEM_BYTES, stream, pdl_mlp, h->tm_a1, h->tm_a1_small,
                           h->tm_w13_n, h->tm_w13_m, h->tm_a2_store, h->tm_a2, h->tm_a2_small, h->tm_w2, a);
         };
-        const long long slots = static_cast<long long>(T) * R_TOPK * EL / R_EXPERTS;
         if (T > MLP_SPLIT_MAX_TOKENS && slots <= MLP_JOINT_MAX_SLOTS) {
             if ((lerr = mlp(3)) != cudaSuccess) return cuda_fail(h, lerr);
             ++launches;
