@@ -1,14 +1,18 @@
 // The expert MLP (stage 3 of the Fused MoE description) of batches beyond the fused kernel's range: GEMM1 with SwiGLU and
 // re-quantisation and GEMM2, in one launch.  Roles and their loop: see gemm.cuh.
 //
-// Every CTA has a list of tiles, GEMM1's first: CTA b takes GEMM1 tiles b, b + grid, ... and then its GEMM2 tiles, of
-// which CTAs with one GEMM1 tile less get more.  A GEMM2 tile starts once GEMM1's column tiles of its row tile have been
-// announced (bounded wait).  So that no CTA ever depends on one that has not started -- two such kernels may share the
+// Every CTA has a list of tiles, GEMM1's first: CTA b takes GEMM1 tiles b, b + grid, ... and then GEMM2 tiles from a counter
+// until there are none.  A GEMM2 tile starts once GEMM1's column tiles of its row tile have been announced (bounded wait).  So that no CTA ever depends on one that has not started -- two such kernels may share the
 // GPU from different streams --, a CTA claims its list of GEMM1 tiles when it starts, and before its first GEMM2 tile it
 // works through the lists nobody has claimed: every GEMM1 tile it may then wait for is in the hands of a running CTA.
-// Fixed lists, not a counter that hands out tiles: neighbouring tiles share operands, and CTAs that read the same lines
+// Fixed lists for GEMM1, not a counter that hands out tiles: neighbouring tiles share operands, and CTAs that read the same lines
 // at the same time get them out of L2 faster (loads-only kernel: 26 against 17 TB/s).  Tiles handed out in order of
-// arrival took GEMM1 of 8192 skewed tokens from 1226 to 1331 us.
+// arrival took GEMM1 of 8192 skewed tokens from 1226 to 1331 us.  For GEMM2 the counter is the better way, or an equal one: row
+// tiles differ in time and CTAs in their share of the memory's rate, and dealt in rounds, with up to three rounds in front
+// for the CTAs with one GEMM1 tile less, the last CTA ended 12 us (6 %) behind the middle one at 257 tokens, now 5.  us per forward
+// dealt / counter: 194.0 / 193.4 at 100 tokens, 139.9 / 137.0 at 150 skewed, 205.7 / 202.2 at 257, 204.7 / 202.0 at 400, 223.1 /
+// 221.5 at 901, 251.5 / 248.8 at 1500, 436.5 / 433.4 at 4096, 1589 / 1591 at 8192 skewed; on 256 experts 1184 / 1178 at 300, 1405 /
+// 1394 at 1000, 4006 / 4001 at 8192.
 // What the common list is for: a launch per GEMM leaves most SMs idle in its last, partly filled wave.  With 24 active
 // experts (257 tokens) GEMM1 is 384 tiles of 56 K-blocks, 2.6 waves, and GEMM2 672 tiles of 16, 4.5 waves: 248 K-block
 // times per launch pair against 218 in one list.  Measured per forward, two launches against one, this kernel on both
@@ -33,13 +37,12 @@ namespace moe {
 constexpr int MLP_SPLIT_MAX_TOKENS = 256;
 constexpr int MLP_JOINT_MAX_SLOTS = 16384;
 
-constexpr int MLP_MAX_GRID = 1024;   // capacity of `claimed`
-constexpr int FRONT_MIN_KB = 16;     // K-blocks of a GEMM2 tile for the rounds in front, see mlp_factors
-
+constexpr int MLP_MAX_GRID = 1023;   // lists that `claimed` has room for
 struct MlpArgs {
     GemmArgs g1, g2;
     int phases;          // bit 0: GEMM1's tiles, bit 1: GEMM2's; both: a GEMM2 tile waits for its rows
-    int* claimed;        // [grid] the lists of GEMM1 tiles, LIST_OPEN (or LIST_LEFT) at launch (both GEMMs only)
+    int* claimed;        // [grid] the lists of GEMM1 tiles, LIST_OPEN (or LIST_LEFT) at launch (both GEMMs only), and
+                         // the next GEMM2 tile, zero at launch
 };
 
 __device__ __forceinline__ TileInfo read_tile(const Cta& c, uint32_t i) {  // an entry that has been waited for
@@ -241,25 +244,9 @@ __device__ __forceinline__ void mlp_factors(const Cta& c, const MlpArgs& a) {
     const int m_tiles = __ldcg(a.g1.num_m_tiles);
     const int n1 = (a.phases & 1) ? m_tiles * a.g1.n_tiles : 0, n12 = n1 + ((a.phases & 2) ? m_tiles * a.g2.n_tiles : 0);
     const int grid = static_cast<int>(gridDim.x);
-    // GEMM1: tiles id1, id1 + grid, ... ; GEMM2: the CTAs that have one GEMM1 tile less (of num_kb1 K-blocks) take
-    // `extra` rounds of tiles (of num_kb2) among themselves, then the rounds go over all CTAs, those first.  (Not where
-    // nearly all CTAs have the tile more, so that the idle time of the others costs no bandwidth; us per forward without /
-    // with, by the number of CTAs that have it, 257 tokens on 17 to 36 experts: 241 / 234 with 72, 324 / 318 with 84, 262 /
-    // 251 with 88, 329 / 322 with 100, 261 / 253 with 104; 335 / 329 with 116, 268 / 270 with 120, 194 / 210 with 124, 345 /
-    // 346 with 132, 277 / 272 with 136, 198 / 226 with 140.  The line is at 111 of 148: below it every count gains, above it
-    // the losses are larger than the gains.)
+    // GEMM1: tiles id1, id1 + grid, ... ; GEMM2: whichever is next when this CTA needs one (a ticket, drawn when it enters
+    // the tile before).
     int id1 = static_cast<int>(blockIdx.x);
-    const int r1 = n1 % grid, late = static_cast<int>(blockIdx.x) < r1 ? 1 : 0;
-    // Only with GEMM2 tiles of at least 16 K-blocks (intermediate size 2048 and more), and no more rounds than there are
-    // GEMM2 tiles whose rows the full GEMM1 rounds have finished: shorter GEMM2 tiles cost more than their K-blocks say, and
-    // a tile whose rows come from the last GEMM1 round is waited for.  (us per forward without / with as many rounds as K-block
-    // counts allow: 7168 x 384, 3 experts, no full GEMM1 round, 103 / 133; 7168 x 1024, 27 to 32 experts, 168 to 186 / 184
-    // to 208; 7168 x 512, 189 / 209; 4096 x 1024, 111 / 118; 2048 x 512, 76 / 84.)
-    const int reach = (n1 - r1) / a.g1.n_tiles * a.g2.n_tiles / (grid - r1);
-    const bool front = r1 > 0 && r1 * 16 <= grid * 12 && a.g2.num_kb >= FRONT_MIN_KB;
-    const int extra = front ? min(a.g1.num_kb / a.g2.num_kb, reach) : 0, first2 = extra * (grid - r1);
-    const int turn = static_cast<int>(blockIdx.x) - r1 + (late ? grid : 0);
-    int round = late ? extra : 0;
     if (a.phases == 3) {
         int was = LIST_OPEN;
         if (lane == 0) was = atomicCAS(a.claimed + blockIdx.x, LIST_OPEN, LIST_CLAIMED);
@@ -287,9 +274,10 @@ __device__ __forceinline__ void mlp_factors(const Cta& c, const MlpArgs& a) {
         if (id1 < n1) {
             id = id1;
             id1 += grid;
-        } else {
-            id = n1 + (round < extra ? round * (grid - r1) + turn : first2 + (round - extra) * grid + turn);
-            ++round;
+        } else if ((a.phases & 2) && !end) {
+            int ticket = 0;
+            if (lane == 0) ticket = atomicAdd(a.claimed + grid, 1);
+            id = n1 + __shfl_sync(0xffffffffu, ticket, 0);
         }
         const bool live = !end && id < n12;
         const bool first = id < n1;

@@ -63,7 +63,7 @@ WsLayout make_layout(const moe_fp8_config& c) {
     L.tile_rows = take(static_cast<size_t>(L.max_m_tiles) * 4);
     L.num_m_tiles = take(4);
     L.mlp_ready = take(static_cast<size_t>(L.max_m_tiles) * 4);
-    L.mlp_claimed = take(MLP_MAX_GRID * 4);
+    L.mlp_claimed = take((MLP_MAX_GRID + 1) * 4);
     L.slot_to_row = take(slots * 4);
     L.row_to_slot = take(slots * 4);
     L.row_token = take(rc * 4);

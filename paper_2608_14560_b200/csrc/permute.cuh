@@ -30,7 +30,7 @@ struct PermuteMeta {
     int* tile_rows;      // [max_m_tiles] valid rows in each row tile (1..TILE_M)
     int* num_m_tiles;    // [1]
     int* mlp_ready;      // [max_m_tiles] grouped_mlp_kernel's counters, zeroed with the tables: parts of GEMM1 stored,
-    int* mlp_claimed;    // [mlp_grid] and lists of tiles claimed
+    int* mlp_claimed;    // [mlp_grid] lists of tiles claimed, [1] GEMM2 tiles handed out
     int mlp_grid;
     int mlp_left;        // test hook: the first lists, which their own CTAs leave to the others (0 outside of tests)
     int* slot_to_row;    // [T*8] padded row of each slot, -1 when the slot's expert is not local
@@ -96,7 +96,9 @@ __device__ __forceinline__ void scan_experts(int E_loc, int* s_cnt, int* s_pad, 
         }
     }
     for (int v = tid; v < m.mlp_grid; v += blockDim.x) m.mlp_claimed[v] = v < m.mlp_left ? LIST_LEFT : LIST_OPEN;
-    if (tid == 0) {  // entries past E_loc count nothing, so entry E_loc already holds the totals
+    if (tid == 0) {
+        m.mlp_claimed[m.mlp_grid] = 0;
+        // entries past E_loc count nothing, so entry E_loc already holds the totals
         m.expert_offset[E_loc] = s_cnt[E_loc];
         m.padded_offset[E_loc] = s_pad[E_loc];
     }
@@ -572,7 +574,9 @@ __device__ __forceinline__ void route_permute_in_cta(int* scratch, CtaTiles& til
             m.st_rows[t0] = total;
         }
     }
-    if (tid == 0) {  // entries past E_loc count nothing, so entry E_loc already holds the totals
+    if (tid == 0) {
+        m.mlp_claimed[m.mlp_grid] = 0;
+        // entries past E_loc count nothing, so entry E_loc already holds the totals
         tiles.count = s_pad[E_loc] / TILE_M;
         *m.num_m_tiles = s_pad[E_loc] / TILE_M;
         *m.num_st = s_pad[E_loc] / TILE_M;
