@@ -319,8 +319,8 @@ int moe_fp8_create(const moe_fp8_config* cfg, moe_fp8_handle_t* out) {
     e = cudaFuncSetAttribute(fused_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GeomSmall::SMEM_BYTES);
     if (e != cudaSuccess) return MOE_FP8_ERR_CUDA;
     e = set_router_smem<2, 1, 4, 4, 256, 8>();
+    if (e == cudaSuccess) e = set_router_smem<2, 1, 4, 4, 512, 4>();
     if (e == cudaSuccess) e = set_router_smem<2, 2, 8, 8, 256, 2>();
-    if (e == cudaSuccess) e = set_router_smem<2, 2, 16, 8, 512, 2>();
     if (e != cudaSuccess) return MOE_FP8_ERR_CUDA;
     e = cudaFuncSetAttribute(route_permute_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(route_permute_smem_bytes(P_TAIL_MAX_TOKENS, P_MAX_LOCAL)));
@@ -759,12 +759,12 @@ int moe_fp8_forward_from_hidden(moe_fp8_handle_t h, int T, const void* hidden_bf
         const __nv_bfloat16* x = static_cast<const __nv_bfloat16*>(hidden_bf16);
         const __nv_bfloat16* wr = static_cast<const __nv_bfloat16*>(router_weight);
         cudaError_t e;
-        if (T <= RP_SMALL_MAX_TOKENS)
-            e = launch_router<2, 1, 4, 4, 256, 8>(T, H, E, x, wr, d_logits, stream);
-        else if (T < RP_LARGE_MIN_TOKENS || H % 512 != 0)
+        if (T > RP_SMALL_MAX_TOKENS)
             e = launch_router<2, 2, 8, 8, 256, 2>(T, H, E, x, wr, d_logits, stream);
+        else if (H % 512 == 0)
+            e = launch_router<2, 1, 4, 4, 512, 4>(T, H, E, x, wr, d_logits, stream);
         else
-            e = launch_router<2, 2, 16, 8, 512, 2>(T, H, E, x, wr, d_logits, stream);
+            e = launch_router<2, 1, 4, 4, 256, 8>(T, H, E, x, wr, d_logits, stream);
         if (e != cudaSuccess) return cuda_fail(h, e);
         const long long blocks = (static_cast<long long>(T) * (H / 128) + 7) / 8;
         e = launch(quantize_rows_kernel, static_cast<int>(std::min<long long>(blocks, h->sm_count * 16LL)), 256, 0, stream,

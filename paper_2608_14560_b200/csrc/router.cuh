@@ -24,15 +24,16 @@ namespace moe {
 // dimension spread over its lanes, a CTA WT x WE such warps; rows come in through a ring of S stages of KC elements
 // (cp.async).  x [T, H] and w [E, H] bf16, H a multiple of KC, E a multiple of WE * ME.
 //
-// Large batches are bound by the fp32 pipes (2 x 7168 x 256 FLOP per token, 36 TFMA/s measured for packed and for scalar
-// FMAs) and the issue slots around the FMAs.  ldmatrix hands a lane its words of four rows in one instruction (16
-// single-word loads per 64 elements and 8 x 8 tile before, 4 now); the packed FMA does two tokens at a time.  Small ones
-// are bound by latency and the number of warps that stream the 3.7 MB of weights.  Hence three shapes (us, loads in 32
-// single words and two stages before / this kernel):
-//   8 x 8 per warp, 2 x 2 warps   many small CTAs balance the SMs: 257 tokens 73 / 36, 1024 139 / 99, 2048 270 / 186
-//   16 x 8, 2 x 2 warps           fewer words per FMA, for batches that fill the GPU anyway: 2048 tokens 182, 8192
-//                                 926 / 669 (8 x 8: 704), 61 % of the pipes
-//   4 x 4, 2 x 1 warps            eight stages in flight per warp: 16 tokens 26 / 14, 64 tokens 24 / 17
+// Large batches are bound by the fp32 pipes (2 x 7168 x 256 FLOP per token) and the issue slots around the FMAs.  The FMA
+// with bf16 factors takes its words as they are, with nothing to convert and no factor to put into both halves of a pair:
+// alone it runs at 25.7 TFMA/s on the chip, the packed fp32 FMA at 32.2 and at 27.3 beside the conversions for an 8 x 8 tile,
+// but in this kernel it is the faster one (packed / this: 94.9 / 83.3 us at 1024 tokens; one of each per word 86.8).  ldmatrix
+// hands a lane its words of four rows in one instruction.  Small batches are bound by latency and the number of warps that
+// stream the 3.7 MB of weights.  Hence two shapes (us, packed fp32 FMAs / this kernel):
+//   8 x 8 per warp, 2 x 2 warps   many small CTAs balance the SMs: 257 tokens 33.5 / 29.4, 1024 94.9 / 83.3, 8192 660 (16 x 8
+//                                 per warp) / 627, 24.0 TFMA/s; with the bf16 FMA 16 x 8 is slower (662)
+//   4 x 4, 2 x 1 warps            many loads in flight per warp: 16 tokens 11.2 / 8.9, 64 tokens 15.2 / 11.1 in rows of 512
+//                                 elements, four stages (256, eight stages: 9.6 and 13.5); equal to 8 x 8 at 128 tokens
 template <int WT, int WE, int MT, int ME, int KC, int S>
 struct RouterShape {
     static constexpr int ROWS_T = WT * MT, ROWS_E = WE * ME, THREADS = WT * WE * 32, ROWS = ROWS_T + ROWS_E;
@@ -40,7 +41,6 @@ struct RouterShape {
     static_assert(MT % 4 == 0 && ME % 4 == 0 && KC % 64 == 0, "rows are read four at a time, in runs of 64 elements");
 };
 constexpr int RP_SMALL_MAX_TOKENS = 64;    // 4 x 4 up to here
-constexpr int RP_LARGE_MIN_TOKENS = 2048;  // 16 x 8 from here
 
 template <int WT, int WE, int MT, int ME, int KC, int S>
 __global__ void __launch_bounds__(WT * WE * 32)
@@ -79,13 +79,11 @@ router_logits_kernel(int T, int H, int E, const __nv_bfloat16* __restrict__ x, c
         cp_async_commit();
     };
 
-    // Accumulators as pairs of tokens (2 i, 2 i + 1) for the packed fp32 FMA: one instruction, two independent
-    // round-to-nearest FMAs, so every sum is bit for bit the one of the scalar form.
-    uint64_t acc[MT / 2][ME];
+    float acc[MT][ME];
 #pragma unroll
-    for (int i = 0; i < MT / 2; ++i)
+    for (int i = 0; i < MT; ++i)
 #pragma unroll
-        for (int j = 0; j < ME; ++j) acc[i][j] = 0ull;
+        for (int j = 0; j < ME; ++j) acc[i][j] = 0.0f;
 
 #pragma unroll
     for (int i = 0; i < S - 1; ++i) stage(i);
@@ -99,16 +97,13 @@ router_logits_kernel(int T, int H, int E, const __nv_bfloat16* __restrict__ x, c
         const uint32_t base = smem0 + (kc % S) * ROWS * ROW_BYTES;
 #pragma unroll
         for (int run = 0; run < KC / 64; ++run) {
-            uint64_t xl[MT / 2], xh[MT / 2];  // elements 2l / 2l+1 of the run for two tokens each
+            uint32_t xr[MT];  // elements 2l, 2l+1 of the run
 #pragma unroll
             for (int q = 0; q < MT / 4; ++q) {
                 uint32_t r[4];
                 ldmatrix_x4(base + x_off + q * 4 * ROW_BYTES + run * 128, r);
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    xl[2 * q + i] = pack_f32x2(r[2 * i] << 16, r[2 * i + 1] << 16);
-                    xh[2 * q + i] = pack_f32x2(r[2 * i] & 0xffff0000u, r[2 * i + 1] & 0xffff0000u);
-                }
+                for (int i = 0; i < 4; ++i) xr[4 * q + i] = r[i];
             }
 #pragma unroll
             for (int q = 0; q < ME / 4; ++q) {
@@ -116,12 +111,10 @@ router_logits_kernel(int T, int H, int E, const __nv_bfloat16* __restrict__ x, c
                 ldmatrix_x4(base + w_off + q * 4 * ROW_BYTES + run * 128, r);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const uint64_t wl = pack_f32x2(r[j] << 16, r[j] << 16);
-                    const uint64_t wh = pack_f32x2(r[j] & 0xffff0000u, r[j] & 0xffff0000u);
 #pragma unroll
-                    for (int i = 0; i < MT / 2; ++i) acc[i][4 * q + j] = fma_f32x2(xl[i], wl, acc[i][4 * q + j]);  // element 2l
+                    for (int i = 0; i < MT; ++i) acc[i][4 * q + j] = fma_bf16_lo(xr[i], r[j], acc[i][4 * q + j]);  // element 2l
 #pragma unroll
-                    for (int i = 0; i < MT / 2; ++i) acc[i][4 * q + j] = fma_f32x2(xh[i], wh, acc[i][4 * q + j]);  // then 2l+1
+                    for (int i = 0; i < MT; ++i) acc[i][4 * q + j] = fma_bf16_hi(xr[i], r[j], acc[i][4 * q + j]);  // then 2l+1
                 }
             }
         }
@@ -132,7 +125,7 @@ router_logits_kernel(int T, int H, int E, const __nv_bfloat16* __restrict__ x, c
     for (int i = 0; i < MT; ++i)
 #pragma unroll
         for (int j = 0; j < ME; ++j) {
-            float v = __uint_as_float(static_cast<uint32_t>((i & 1) ? acc[i / 2][j] >> 32 : acc[i / 2][j]));
+            float v = acc[i][j];
 #pragma unroll
             for (int d = 16; d >= 1; d >>= 1) v = __fadd_rn(v, __shfl_xor_sync(0xffffffffu, v, d));
             const int t = t0 + wt * MT + i;

@@ -457,6 +457,13 @@ def test_from_hidden_at_the_edges_of_the_projection_shapes(cuda_device, tokens, 
     _from_hidden_case(_wl(tokens, dims, seed=600 + tokens), cuda_device, sample_tokens=_sample(tokens, 64, tokens))
 
 
+@pytest.mark.parametrize("tokens,hidden", [(1, 512), (63, 1024), (64, 2560)])
+def test_from_hidden_of_small_batches_in_chunks_of_512(cuda_device, tokens, hidden):
+    # fewer chunks than pipeline stages (1 and 2 of 4) and one more
+    dims = syn.LayerDims(hidden=hidden, intermediate=128, num_local_experts=32)
+    _from_hidden_case(_wl(tokens, dims, seed=650 + tokens), cuda_device)
+
+
 def test_from_hidden_transposed_scale_layout(cuda_device):
     _from_hidden_case(_wl(77, seed=59), cuda_device, hidden_scale_layout=1)
 
