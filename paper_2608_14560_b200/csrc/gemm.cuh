@@ -70,7 +70,7 @@ constexpr int G_THREADS = 384;                          // 4 control warps + 8 e
 constexpr int G_EPI_WARPS = 8;
 constexpr int G_STORE_WARP_BYTES = 2048;                // per-warp staging: 32 rows x 64 B (swizzled)
 constexpr int G_AMAX_BYTES = 2 * 2 * TILE_M * 4;               // GEMM1 row-amax exchange
-constexpr int G_CTRL_BYTES = 768;
+constexpr int G_CTRL_BYTES = 832;
 constexpr uint32_t G_TMEM_COLS = 512;
 // grouped_mlp_kernel: named barrier ACC_BARRIER + b hands accumulator buffer b from the epilogue warps (which
 // arrive) back to its issuer warp (which waits).
@@ -220,7 +220,10 @@ struct GemmCtrl {
     uint64_t amax_bar;         // all epilogue warps have their row maxima in the exchange area (weights on M)
     uint64_t amax_quad[4];     // the same for the two warps that share a quadrant's rows (full row tiles)
     uint64_t drain_bar[2];
-    uint64_t sync_bar[2];      // fused kernel: rendezvous of the epilogue warps at the end of a tile
+    uint64_t sync_bar;         // fused kernel, K split: rendezvous of the epilogue warps
+    uint64_t group_amax[2];    // fused kernel, by epilogue group: row maxima are in the exchange area,
+    uint64_t group_sync[2];    // rendezvous at the end of a tile,
+    uint64_t group_turn[2];    // the other group has read the last accumulator of the tile before
     uint32_t tmem_slot;
     int abort_flag;
     int split_last;            // fused kernel, K split: this CTA stored the last part of the tile
@@ -362,8 +365,12 @@ __device__ __forceinline__ void gemm_cta_setup(Cta& c, uint8_t* smem_raw, int fu
         for (int q = 0; q < 4; ++q) mbar_init(smem_u32(&ctrl->amax_quad[q]), 2);
         mbar_init(smem_u32(&ctrl->drain_bar[0]), 1);
         mbar_init(smem_u32(&ctrl->drain_bar[1]), 1);
-        mbar_init(smem_u32(&ctrl->sync_bar[0]), G_EPI_WARPS * 32);
-        mbar_init(smem_u32(&ctrl->sync_bar[1]), G_EPI_WARPS * 32);
+        mbar_init(smem_u32(&ctrl->sync_bar), G_EPI_WARPS);
+        for (int q = 0; q < 2; ++q) {
+            mbar_init(smem_u32(&ctrl->group_amax[q]), G_EPI_WARPS / 2);
+            mbar_init(smem_u32(&ctrl->group_sync[q]), G_EPI_WARPS / 2);
+            mbar_init(smem_u32(&ctrl->group_turn[q]), G_EPI_WARPS / 2);
+        }
         for (int i = 0; i < SCHED_SLOTS; ++i) {
             mbar_init(smem_u32(&ctrl->sched_full[i]), 2);
             mbar_init(smem_u32(&ctrl->sched_rows[i]), 1);
@@ -544,13 +551,14 @@ __device__ __forceinline__ void gather_idle_tiles(const Cta& c, const GemmArgs& 
     }
 }
 
-// Rendezvous of all epilogue threads (an mbarrier, because its wait is bounded: a plain barrier would hold the
-// arrived warps for ever if another warp had given up).  Orders the arrived threads' earlier writes before the
-// later reads of those that leave.  `n` counts the rendezvous of this thread so far.
-__device__ __forceinline__ bool epilogue_rendezvous(const Cta& c, uint32_t& n) {
-    const uint32_t bar = smem_u32(&c.ctrl->sync_bar[n & 1]);
-    mbar_arrive(bar);
-    const bool ok = __all_sync(0xffffffffu, mbar_wait(bar, (n >> 1) & 1, c.abort_flag, c.limit));
+// Rendezvous of epilogue warps at barrier `bar` (an mbarrier, because its wait is bounded: a plain barrier would hold the
+// arrived warps for ever if another warp had given up).  Orders the arrived threads' earlier writes before the later
+// reads, and before the later fences and atomics, of those that leave.  `n` counts the rendezvous of this thread so far.
+__device__ __forceinline__ bool epilogue_rendezvous(const Cta& c, uint64_t* bar, uint32_t& n) {
+    const uint32_t b = smem_u32(bar);
+    __syncwarp();
+    if (c.lane == 0) mbar_arrive(b);
+    const bool ok = __all_sync(0xffffffffu, mbar_wait(b, n & 1, c.abort_flag, c.limit));
     ++n;
     return ok;
 }
@@ -561,8 +569,9 @@ __device__ __forceinline__ bool epilogue_rendezvous(const Cta& c, uint32_t& n) {
 // operands are swapped instead: the 256 weight rows of the tile are the M side (two MMAs of M = 128 per K
 // step), the 32 token rows the N side.  An accumulator is then 128 lanes x 32 columns per weight-row block,
 // 64 columns per K-block: every stage gets an accumulator buffer of its own (6 x 64 of the 512 columns),
-// so the hand-over latencies overlap six deep, and every epilogue thread owns one weight row (an output
-// column) for 16 tokens -- 32 loads and 32 FMAs per K-block instead of 128, evenly over all eight warps.
+// so the hand-over latencies overlap six deep, and an epilogue thread owns one weight row (an output
+// column) of both blocks for the tile's 32 tokens, the four warps of a group taking a tile together and the two
+// groups the tiles in turn (epilogue_tile_group).
 // Element for element the arithmetic is the one of the other orientation.
 static_assert(G_MAX_STAGES * WM_BUF_COLS <= static_cast<int>(G_TMEM_COLS), "one accumulator buffer per stage");
 
@@ -631,25 +640,26 @@ struct Announce {
     }
 };
 
+// A tile with the weights on M by all eight epilogue warps: a thread owns one weight row of each block for 16 tokens.
 // MODE 1: weight-row block 0 = 128 gate rows, block 1 = the matching 128 up rows; SwiGLU, re-quantisation per
-//         token over the tile's 128 output columns, e4m3 bytes and scales out, tile announced in f->ready.
-// MODE 2: blocks 0 / 1 = output columns [0,128) / [128,256) of the tile; bf16 out in the tile-blocked layout,
-//         then the per-(token, column tile) counters and the combine of the tokens this CTA completes.
-// One tile; false: a wait gave up (the code is in the status word).  SHARED: the tile runs inside the large-tile
-// kernel, between tiles of the other orientation -- its accumulators are the first 64 columns of the two
-// 256-column buffers of that kernel, handed over through the same two barriers, and its staging is the first
-// 512 bytes of the warp's own TMA staging area.
-// SPLIT (fused kernel, batches of at most SPLIT_MAX_TOKENS tokens with few tiles, parts > 1): this call covers the
+//         token over the tile's 128 output columns, e4m3 bytes and scales out.
+// MODE 2: blocks 0 / 1 = output columns [0,128) / [128,256) of the tile; bf16 out in the tile-blocked layout.
+// False: a wait gave up (the code is in the status word).
+// Without SPLIT the tile runs inside the large-tile kernel, between tiles of the other orientation -- its accumulators are
+// the first 64 columns of the two 256-column buffers of that kernel, handed over through the same two barriers, and its
+// staging is the first 512 bytes of the warp's own TMA staging area.
+// SPLIT (fused kernel, GEMM1, batches of at most SPLIT_MAX_TOKENS tokens with few tiles): this call covers the
 // K-blocks [kb0, kb1) only.  It stores every K-block's partial sums as they come out of the tensor memory, not
 // yet multiplied by the scales; the CTA that stores the last part of a tile -- found with a counter, nobody
 // waits -- then runs the whole promotion from the stored partial sums, K-block after K-block in the one order
 // the unsplit tile uses, and finishes the tile.  Every fp32 operation is the one of the unsplit tile.
-template <int MODE, bool FUSED, class GEO, bool SHARED, bool SPLIT = false>
+template <int MODE, bool SPLIT, class GEO>
 __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g, const FusedArgs* f, int m_tile, int n,
                                                  uint32_t& it, AmaxTurn& turn, uint32_t& sync_iter, int kb0 = 0,
                                                  int kb1 = -1, int parts = 1, Announce* announce = nullptr,
                                                  bool settle = false) {
-    static_assert(!SPLIT || FUSED, "only the fused kernel cuts K ranges");
+    static_assert(!SPLIT || MODE == 1, "only GEMM1's K range is cut");
+    constexpr bool SHARED = !SPLIT;
     GemmCtrl* ctrl = c.ctrl;
     const int warp = c.warp, lane = c.lane;
     const int th = (warp - 4) >> 2;          // which 16 of the tile's 32 token rows
@@ -659,18 +669,7 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
     const size_t row_cap = static_cast<size_t>(g.row_cap);
     uint32_t* amax_x = reinterpret_cast<uint32_t*>(c.amax_x);   // [2 turns][256]: [2 token halves][4 quadrants][16] used
     const int num_kb = g.num_kb;
-    const int e = SHARED ? __ldcg(g.tile_expert + m_tile) : tile_expert_of(c, g, m_tile);
     const int rows_valid = SHARED ? __ldcg(g.tile_rows + m_tile) : tile_rows_of(c, g, m_tile);
-    const int sblocks = g.w_rows_per_expert / 128;
-    const float* ws0;  // weight-scale rows of block 0 / block 1
-    const float* ws1;
-    if (MODE == 1) {
-        ws0 = g.w_scale + (static_cast<size_t>(e) * sblocks + n) * num_kb;
-        ws1 = g.w_scale + (static_cast<size_t>(e) * sblocks + g.up_row0 / 128 + n) * num_kb;
-    } else {
-        ws0 = g.w_scale + (static_cast<size_t>(e) * sblocks + 2 * n) * num_kb;
-        ws1 = ws0 + num_kb;
-    }
     float acc[32];  // [0,16): block 0, [16,32): block 1, for tokens 16 th .. 16 th + 15
 #pragma unroll
     for (int j = 0; j < 32; ++j) acc[j] = 0.0f;
@@ -681,17 +680,7 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
     if (SPLIT)
         raw = reinterpret_cast<float4*>(f->raw[MODE - 1] + static_cast<size_t>(m_tile * g.n_tiles + n) * num_kb * SPLIT_RAW_FLOATS) +
               quad * 32 + lane;
-    float s0 = 0.0f, s1 = 0.0f;
-    if (!SHARED) {
-        s0 = __ldg(ws0 + kb0);
-        s1 = __ldg(ws1 + kb0);
-    }
     for (int kb = kb0; kb < kb_end; ++kb, ++it) {
-        const float w0 = s0, w1 = s1;
-        if (!SHARED && kb + 1 < kb_end) {
-            s0 = __ldg(ws0 + kb + 1);
-            s1 = __ldg(ws1 + kb + 1);
-        }
         const uint32_t s = it % GEO::STAGES, ph = (it / GEO::STAGES) & 1;
         if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctrl->done[s]), ph, c.abort_flag, c.limit))) {
             if (lane == 0) raise(ctrl, g.status, DEV_TIMEOUT_EPILOGUE);
@@ -706,18 +695,6 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
             for (int q = 0; q < 4; ++q) {
                 *reinterpret_cast<float4*>(f0 + 4 * q) = fp[q];
                 *reinterpret_cast<float4*>(f1 + 4 * q) = fp[GEO::A_ROWS / 4 + q];
-            }
-        } else {
-            const float4* sp = reinterpret_cast<const float4*>(c.scale_ring + (it % GEO::SCALE_SLOTS) * GEO::A_ROWS + th * 16);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float4 x = sp[q];
-                const float sa[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    f0[4 * q + i] = sa[i] * w0;
-                    f1[4 * q + i] = sa[i] * w1;
-                }
             }
         }
         float v[32];
@@ -746,7 +723,7 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
     if (SPLIT) {
         // count this part; the last one goes on, the others are done with the tile
         __threadfence();
-        if (!epilogue_rendezvous(c, sync_iter)) {
+        if (!epilogue_rendezvous(c, &ctrl->sync_bar, sync_iter)) {
             if (lane == 0) raise(ctrl, g.status, DEV_TIMEOUT_EPILOGUE);
             return false;
         }
@@ -755,7 +732,7 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
             const int before = atomicAdd(f->part_done[MODE - 1] + m_tile * g.n_tiles + n, 1);
             *reinterpret_cast<volatile int*>(&ctrl->split_last) = (before == parts - 1);
         }
-        if (!epilogue_rendezvous(c, sync_iter)) {
+        if (!epilogue_rendezvous(c, &ctrl->sync_bar, sync_iter)) {
             if (lane == 0) raise(ctrl, g.status, DEV_TIMEOUT_EPILOGUE);
             return false;
         }
@@ -782,9 +759,11 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
             }
             sa_s[i] = v;
         }
+        const float* ws0 = g.w_scale + (static_cast<size_t>(tile_expert_of(c, g, m_tile)) * (g.w_rows_per_expert / 128) + n) * num_kb;
+        const float* ws1 = ws0 + static_cast<size_t>(g.up_row0 / 128) * num_kb;
         for (int i = threadIdx.x - 128; i < 2 * num_kb; i += G_EPI_WARPS * 32)
             w_s[i] = __ldg((i < num_kb ? ws0 : ws1 - num_kb) + i);
-        if (!epilogue_rendezvous(c, sync_iter)) {
+        if (!epilogue_rendezvous(c, &ctrl->sync_bar, sync_iter)) {
             if (lane == 0) raise(ctrl, g.status, DEV_TIMEOUT_EPILOGUE);
             return false;
         }
@@ -805,7 +784,7 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
         }
         float4* xchg = reinterpret_cast<float4*>(c.store_stage);  // [128 weight rows]: half 0's warps read their own staging
         if (th == 1) xchg[quad * 32 + lane] = a4;
-        if (!epilogue_rendezvous(c, sync_iter)) {
+        if (!epilogue_rendezvous(c, &ctrl->sync_bar, sync_iter)) {
             if (lane == 0) raise(ctrl, g.status, DEV_TIMEOUT_EPILOGUE);
             return false;
         }
@@ -883,11 +862,11 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
         // (The rows are read by copy engines, of other CTAs or of the next kernel: plain stores here,
         // asynchronous-proxy loads there.)
         fence_proxy_async();
-        if (FUSED) {
+        if (SPLIT) {
             // Announce the tile: every thread's stores are fenced before the epilogue warps meet, and the
             // announcing thread fences once more behind the barrier.
             __threadfence();
-            if (!epilogue_rendezvous(c, sync_iter)) {
+            if (!epilogue_rendezvous(c, &ctrl->sync_bar, sync_iter)) {
                 if (lane == 0) raise(ctrl, g.status, DEV_TIMEOUT_EPILOGUE);
                 return false;
             }
@@ -917,91 +896,238 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
                 __syncwarp();
             }
         }
-        // Stage 4 without a kernel of its own.  Once the tile is stored and fenced, the thread of each valid
-        // row bumps the counter of (its token, this column tile); whoever brings it to the token's number of
-        // local slots knows that all of the token's rows for these 256 columns are in memory and sums
-        // them, in routing order, exactly as combine_kernel does.
-        if (!FUSED) return true;  // (one GEMM per launch: the combine is a kernel of its own)
-        __threadfence();
-        if (!epilogue_rendezvous(c, sync_iter)) {
-            if (lane == 0) raise(ctrl, g.status, DEV_TIMEOUT_EPILOGUE);
-            return false;
+    }
+    return true;
+}
+
+// acc[t] += v[t] * (sa[t] * w) for 16 tokens, packed: each product and each FMA rounds like the scalar one.
+__device__ __forceinline__ void promote16(float* acc, const float* v, const float4* sa, float w) {
+    const uint64_t ww = pack_f32x2(__float_as_uint(w), __float_as_uint(w));
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float4 x = sa[q];
+        const uint64_t f[2] = {mul_f32x2(pack_f32x2(__float_as_uint(x.x), __float_as_uint(x.y)), ww),
+                               mul_f32x2(pack_f32x2(__float_as_uint(x.z), __float_as_uint(x.w)), ww)};
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int t = 4 * q + 2 * k;
+            const uint64_t a = fma_f32x2(pack_f32x2(__float_as_uint(v[t]), __float_as_uint(v[t + 1])), f[k],
+                                         pack_f32x2(__float_as_uint(acc[t]), __float_as_uint(acc[t + 1])));
+            acc[t] = __uint_as_float(static_cast<uint32_t>(a));
+            acc[t + 1] = __uint_as_float(static_cast<uint32_t>(a >> 32));
         }
-        {
-            // epilogue warp w looks after the rows w, w + 8, w + 16, w + 24 of the tile (lanes 0..3), so up
-            // to eight completed tokens are summed at the same time
-            int tok = -1;
-            bool last = false;
-            const int r_mine = (warp - 4) + 8 * lane;
-            if (lane < 4 && r_mine < rows_valid) {
-                tok = row_token_of(c, f->row_token, m_tile, tile_row0, r_mine);
-                __threadfence();
-                const int before = atomicAdd(f->tok_done + static_cast<size_t>(tok) * g.n_tiles + n, 1);
-                last = before == __ldcg(f->tok_nlocal + tok) - 1;
+    }
+}
+
+// A tile of the fused kernel by one of its two epilogue groups of four warps, which take the CTA's tiles in turn: a thread owns
+// one weight row of each block for all 32 tokens.  A tile's tail is a chain of round trips to L2 (rows stored, fence, counter,
+// combine) of 4 to 8 us while the memory is busy, as long as a GEMM2 tile's loop; with all eight warps on every tile nothing
+// was read from the stages meanwhile, six stages held 6 to 8 us of the tile's stream, and all CTAs were in their tails together.
+// Now the tail runs beside the other group's tile.  us per forward, eight warps on every tile / two groups: 70.9 / 67.6 at 4
+// tokens, 82.0 / 80.0 at 8, 125.1 / 115.4 at 16, 130.3 / 121.4 at 32, 162.1 / 153.9 at 54, 166.4 / 160.3 at 80, 124.4 / 115.7 at 64
+// skewed, 726 / 701 at 33 on 256 experts.  Element for element the arithmetic is that of epilogue_tile_wm.
+// `k` numbers the CTA's tiles.  Scales and tables are asked for before the group's turn comes.
+template <int MODE, class GEO>
+__device__ __forceinline__ bool epilogue_tile_group(const Cta& c, const GemmArgs& g, const FusedArgs& f, int m_tile, int n, uint32_t k,
+                                                    uint32_t& it, uint32_t& amax_iter, uint32_t& sync_iter) {
+    GemmCtrl* ctrl = c.ctrl;
+    const int lane = c.lane, quad = c.warp & 3, group = (c.warp - 4) >> 2;
+    const uint32_t t_lane = c.tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
+    const size_t row_cap = static_cast<size_t>(g.row_cap);
+    const int num_kb = g.num_kb;
+    const int e = tile_expert_of(c, g, m_tile), rows_valid = tile_rows_of(c, g, m_tile), tile_row0 = tile_row0_of(c, g, m_tile);
+    const bool swap = MODE == 1 && g.up_first;  // acc[0..32) is the gate block's either way
+    const float* ws0 = g.w_scale + (static_cast<size_t>(e) * (g.w_rows_per_expert / 128) + (MODE == 1 ? n : 2 * n)) * num_kb;
+    const float* ws1 = ws0 + static_cast<size_t>(MODE == 1 ? g.up_row0 / 128 : 1) * num_kb;
+    if (swap) {
+        const float* w = ws0;
+        ws0 = ws1;
+        ws1 = w;
+    }
+    const uint32_t col0 = swap ? WM_TOKENS : 0, col1 = WM_TOKENS - col0;
+    float s0 = __ldg(ws0), s1 = __ldg(ws1);
+    // MODE 2: warp `quad` looks after the rows quad, quad + 4, ... of the tile (lanes 0..7): their tokens and how many rows each has
+    int tok = -1, tok_rows = 0;
+    if (MODE == 2 && lane < 8 && quad + 4 * lane < rows_valid) {
+        tok = row_token_of(c, f.row_token, m_tile, tile_row0, quad + 4 * lane);
+        tok_rows = __ldcg(f.tok_nlocal + tok);
+    }
+    auto timed_out = [&]() {
+        if (lane == 0) raise(ctrl, g.status, DEV_TIMEOUT_EPILOGUE);
+        return false;
+    };
+    // The other group has read the last accumulator of the tile before: from here on no stage is more than one phase behind.
+    if (k > 0 && !__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctrl->group_turn[group]), ((k - 1) >> 1) & 1, c.abort_flag, c.limit)))
+        return timed_out();
+
+    float acc[64];  // [0,32): block 0 (the gate rows), [32,64): block 1
+#pragma unroll
+    for (int j = 0; j < 64; ++j) acc[j] = 0.0f;
+    for (int kb = 0; kb < num_kb; ++kb, ++it) {
+        const float w0 = s0, w1 = s1;
+        if (kb + 1 < num_kb) {
+            s0 = __ldg(ws0 + kb + 1);
+            s1 = __ldg(ws1 + kb + 1);
+        }
+        const uint32_t s = it % GEO::STAGES, ph = (it / GEO::STAGES) & 1;
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctrl->done[s]), ph, c.abort_flag, c.limit))) return timed_out();
+        tc_fence_after();
+        float v[64];
+        tmem_ld32_issue(t_lane + s * WM_BUF_COLS + col0, v);
+        tmem_ld32_issue(t_lane + s * WM_BUF_COLS + col1, v + 32);
+        tmem_wait_ld(v);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_n(smem_u32(&ctrl->tmem_empty[s]), 2);  // (for a warp of each group)
+        // the MMAs of this K-block have finished, hence its stage -- tokens, weights and scales -- had landed
+        const float4* sp = reinterpret_cast<const float4*>(c.scale_ring + (it % GEO::SCALE_SLOTS) * GEO::A_ROWS);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float4 sa[4] = {sp[4 * h], sp[4 * h + 1], sp[4 * h + 2], sp[4 * h + 3]};
+            promote16(acc + 16 * h, v + 16 * h, sa, w0);
+            promote16(acc + 32 + 16 * h, v + 32 + 16 * h, sa, w1);
+        }
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_u32(&ctrl->group_turn[group ^ 1]));
+
+    uint8_t* wst = c.store_stage + (c.warp - 4) * 512;  // this warp's staging
+    if (MODE == 1) {
+        float cc[32];
+        uint32_t mine = 0;
+#pragma unroll
+        for (int t = 0; t < 32; ++t) {
+            cc[t] = silu_fast(acc[t]) * acc[32 + t];
+            // |x| as an integer orders like the float: the warp's maximum over its 32 output columns
+            const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(cc[t])));
+            if (lane == t) mine = m;
+        }
+        uint32_t* xq = reinterpret_cast<uint32_t*>(c.amax_x) + group * 128;  // [4 quadrants][32 tokens]
+        xq[quad * 32 + lane] = mine;
+        if (!epilogue_rendezvous(c, &ctrl->group_amax[group], amax_iter)) return timed_out();
+        // lane t owns the scale of token t's 128-column block; everybody fetches its reciprocal
+        const volatile uint32_t* xv = xq + lane;
+        const float amax = __uint_as_float(max(max(xv[0], xv[32]), max(xv[64], xv[96])));
+        const float my_sc = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, 448.0f), my_inv = __frcp_rn(my_sc);
+        // Narrow global stores are slow (a warp's 32 single bytes cost tens of clocks): the codes are
+        // transposed through this warp's 512 bytes of staging, [16 tokens][32 columns], and leave as
+        // 16-byte stores -- lane l carries 16 columns of token l / 2.
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (h * 16 >= rows_valid) break;
+#pragma unroll
+            for (int t = 0; t < 16; ++t) {
+                const float inv_sc = __shfl_sync(0xffffffffu, my_inv, h * 16 + t);
+                wst[t * 32 + lane] = static_cast<uint8_t>(__nv_cvt_float_to_fp8(cc[h * 16 + t] * inv_sc, __NV_SATFINITE, __NV_E4M3));
             }
-            uint32_t todo = __ballot_sync(0xffffffffu, last);
-            if (todo) {
-                __threadfence();
-                __syncwarp();  // (a vote orders no memory: the counting lanes' fences come before all lanes' loads)
+            __syncwarp();
+            const int t = h * 16 + (lane >> 1);
+            if (t < rows_valid)
+                *reinterpret_cast<uint4*>(g.out_fp8 + (static_cast<size_t>(tile_row0) + t) * g.out_cols + n * 128 + quad * 32 + (lane & 1) * 16) =
+                    *reinterpret_cast<const uint4*>(wst + (lane >> 1) * 32 + (lane & 1) * 16);
+            __syncwarp();
+        }
+        if (quad == 0 && lane < rows_valid) g.out_scale_t[static_cast<size_t>(n) * row_cap + tile_row0 + lane] = my_sc;
+        // Announce the tile.  (The rows are read by copy engines of other CTAs: plain stores here, asynchronous-proxy loads
+        // there.)  The announcing thread's fence comes behind the rendezvous and covers the stores of all.
+        fence_proxy_async();
+        if (!epilogue_rendezvous(c, &ctrl->group_sync[group], sync_iter)) return timed_out();
+        if (quad == 0 && lane == 0) {
+            __threadfence();
+            atomicAdd(f.ready + m_tile, 1);
+        }
+    } else {
+        // bf16 out through this warp's 512 bytes of staging, eight tokens x 32 columns at a time, so that
+        // the rows leave as 16-byte stores: lane l carries 8 columns of token l / 4 (half of a 32-byte
+        // group of the tile-blocked layout)
+        __nv_bfloat16* bst = reinterpret_cast<__nv_bfloat16*>(wst);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            if (h * 8 >= rows_valid) break;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+#pragma unroll
+                for (int t = 0; t < 8; ++t) bst[t * 32 + lane] = __float2bfloat16_rn(acc[j * 32 + h * 8 + t]);
+                __syncwarp();
+                const int t = h * 8 + (lane >> 2), ch0 = quad * 32 + (lane & 3) * 8;
+                if (t < rows_valid)
+                    *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(g.out_bf16) +
+                                              y_block_offset(tile_row0 + t, n * 16 + j * 8 + (ch0 >> 4), g.n_tiles) + (ch0 & 15) * 2) =
+                        *reinterpret_cast<const uint4*>(bst + (lane >> 2) * 32 + (lane & 3) * 8);
+                __syncwarp();
             }
-            while (todo) {
-                const int src = __ffs(todo) - 1;
-                todo &= todo - 1;
-                const int t = __shfl_sync(0xffffffffu, tok, src);
-                // lane l owns columns n*256 + 8 l .. + 8: half of the 32-byte group n*16 + l/2.  All loads
-                // first, then the sum in routing order.
-                const int4 ra = __ldcg(reinterpret_cast<const int4*>(f->slot_to_row) + 2 * t);
-                const int4 rb = __ldcg(reinterpret_cast<const int4*>(f->slot_to_row) + 2 * t + 1);
-                const float4 wa = __ldcg(reinterpret_cast<const float4*>(f->topk_w) + 2 * t);
-                const float4 wb = __ldcg(reinterpret_cast<const float4*>(f->topk_w) + 2 * t + 1);
-                const int rr[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
-                const float ww[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
-                uint4 u[8];
+        }
+        // Stage 4 without a kernel of its own.  Once the tile is stored, the thread of each valid row fences and bumps the
+        // counter of (its token, this column tile); whoever brings it to the token's number of local slots knows that all of
+        // the token's rows for these 256 columns are in memory and sums them, in routing order, exactly as combine_kernel does.
+        if (!epilogue_rendezvous(c, &ctrl->group_sync[group], sync_iter)) return timed_out();
+        bool last = false;
+        if (tok >= 0) {
+            __threadfence();
+            last = atomicAdd(f.tok_done + static_cast<size_t>(tok) * g.n_tiles + n, 1) == tok_rows - 1;
+        }
+        uint32_t todo = __ballot_sync(0xffffffffu, last);
+        if (todo) {
+            __threadfence();
+            __syncwarp();  // (a vote orders no memory: the counting lanes' fences come before all lanes' loads)
+        }
+        while (todo) {
+            const int src = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const int t = __shfl_sync(0xffffffffu, tok, src);
+            // lane l owns columns n*256 + 8 l .. + 8: half of the 32-byte group n*16 + l/2.  All loads
+            // first, then the sum in routing order.
+            const int4 ra = __ldcg(reinterpret_cast<const int4*>(f.slot_to_row) + 2 * t);
+            const int4 rb = __ldcg(reinterpret_cast<const int4*>(f.slot_to_row) + 2 * t + 1);
+            const float4 wa = __ldcg(reinterpret_cast<const float4*>(f.topk_w) + 2 * t);
+            const float4 wb = __ldcg(reinterpret_cast<const float4*>(f.topk_w) + 2 * t + 1);
+            const int rr[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
+            const float ww[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+            uint4 u[8];
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    if (rr[j] >= 0)
-                        u[j] = __ldcg(reinterpret_cast<const uint4*>(
-                            reinterpret_cast<const uint8_t*>(g.out_bf16) +
-                            y_block_offset(rr[j], n * 16 + (lane >> 1), g.n_tiles) + (lane & 1) * 16));
-                float o[8];
+            for (int j = 0; j < 8; ++j)
+                if (rr[j] >= 0)
+                    u[j] = __ldcg(reinterpret_cast<const uint4*>(
+                        reinterpret_cast<const uint8_t*>(g.out_bf16) +
+                        y_block_offset(rr[j], n * 16 + (lane >> 1), g.n_tiles) + (lane & 1) * 16));
+            float o[8];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) o[i] = 0.0f;
+            for (int i = 0; i < 8; ++i) o[i] = 0.0f;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    if (rr[j] < 0) continue;
-                    const uint32_t uu[4] = {u[j].x, u[j].y, u[j].z, u[j].w};
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        o[2 * i] = fmaf(ww[j], __uint_as_float(uu[i] << 16), o[2 * i]);
-                        o[2 * i + 1] = fmaf(ww[j], __uint_as_float(uu[i] & 0xffff0000u), o[2 * i + 1]);
-                    }
-                }
-                uint32_t p[4];
+            for (int j = 0; j < 8; ++j) {
+                if (rr[j] < 0) continue;
+                const uint32_t uu[4] = {u[j].x, u[j].y, u[j].z, u[j].w};
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const __nv_bfloat162 pr = __floats2bfloat162_rn(o[2 * i], o[2 * i + 1]);
-                    p[i] = *reinterpret_cast<const uint32_t*>(&pr);
+                    o[2 * i] = fmaf(ww[j], __uint_as_float(uu[i] << 16), o[2 * i]);
+                    o[2 * i + 1] = fmaf(ww[j], __uint_as_float(uu[i] & 0xffff0000u), o[2 * i + 1]);
                 }
-                *reinterpret_cast<uint4*>(f->out + static_cast<size_t>(t) * f->H + n * G_TILE_N + lane * 8) =
-                    make_uint4(p[0], p[1], p[2], p[3]);
             }
+            uint32_t p[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const __nv_bfloat162 pr = __floats2bfloat162_rn(o[2 * i], o[2 * i + 1]);
+                p[i] = *reinterpret_cast<const uint32_t*>(&pr);
+            }
+            *reinterpret_cast<uint4*>(f.out + static_cast<size_t>(t) * f.H + n * G_TILE_N + lane * 8) =
+                make_uint4(p[0], p[1], p[2], p[3]);
         }
     }
     return true;
 }
 
-template <int MODE, bool FUSED, class GEO, class SEQ>
-__device__ __forceinline__ void epilogue_tiles_wm(const Cta& c, const GemmArgs& g, const FusedArgs* f, const SEQ& seq,
-                                                  uint32_t& it, AmaxTurn& turn, uint32_t& sync_iter, bool& ok,
-                                                  KSplit ks) {
-    for (int j = 0, item; ok && (item = seq.at(j)) < seq.count; ++j) {
-        const int tile = item / ks.parts, kb0 = (item - tile * ks.parts) * ks.len;
+// The tiles of one GEMM, those of this warp's group; `k` goes on from GEMM to GEMM.
+template <int MODE, class GEO, class SEQ>
+__device__ __forceinline__ void epilogue_tiles_group(const Cta& c, const GemmArgs& g, const FusedArgs& f, const SEQ& seq, uint32_t& k,
+                                                     uint32_t& it, uint32_t& amax_iter, uint32_t& sync_iter, bool& ok) {
+    const uint32_t group = (c.warp - 4) >> 2;
+    for (int j = 0, tile; ok && (tile = seq.at(j)) < seq.count; ++j, ++k) {
+        if ((k & 1) != group) {
+            it += g.num_kb;
+            continue;
+        }
         const int m_tile = tile / g.n_tiles, n = tile - m_tile * g.n_tiles;
-        // (two instantiations, so that the unsplit tile's loop carries nothing of the split)
-        ok = (FUSED && MODE == 1 && ks.parts > 1)
-                 ? epilogue_tile_wm<MODE, FUSED, GEO, false, FUSED && MODE == 1>(c, g, f, m_tile, n, it, turn, sync_iter, kb0,
-                                                                                min(g.num_kb, kb0 + ks.len), ks.parts)
-                 : epilogue_tile_wm<MODE, FUSED, GEO, false, false>(c, g, f, m_tile, n, it, turn, sync_iter);
+        ok = epilogue_tile_group<MODE, GEO>(c, g, f, m_tile, n, k, it, amax_iter, sync_iter);
     }
 }
 
@@ -1065,7 +1191,7 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmA2, const __grid_consta
     bool ok = true;
 
     if (c.warp < 4) {
-        reg_dealloc<40>();
+        reg_dealloc<56>();
         if (c.warp == 0 && c.lane == 0) {
             producer_tiles<1, GEO>(c, &tmA2, &tmB1, g1, &f, 0, tr1, it, ok, ks1);
             producer_tiles<2, GEO>(c, &tmA2, &tmB2, g2, &f, g1.n_tiles, tr2(), it, ok, ks2);
@@ -1079,11 +1205,20 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmA2, const __grid_consta
             if (c.lane == 0) c.ctrl->gathered = it;
         }
     } else {
-        reg_alloc<232>();
-        uint32_t sync_iter = 0;
-        AmaxTurn turn{0};
-        epilogue_tiles_wm<1, true, GEO>(c, g1, &f, tr1, it, turn, sync_iter, ok, ks1);
-        epilogue_tiles_wm<2, true, GEO>(c, g2, &f, tr2(), it, turn, sync_iter, ok, ks2);
+        reg_alloc<224>();
+        uint32_t k = 0, amax_iter = 0, sync_iter = 0;
+        if (ks1.parts > 1) {  // (one part of a tile at most; all eight warps)
+            uint32_t joint_iter = 0;
+            AmaxTurn turn{0};
+            if (tr1.at(0) < n1) {
+                const int tile = tr1.at(0) / ks1.parts, kb0 = (tr1.at(0) - tile * ks1.parts) * ks1.len;
+                ok = epilogue_tile_wm<1, true, GEO>(c, g1, &f, tile / g1.n_tiles, tile % g1.n_tiles, it, turn, joint_iter, kb0,
+                                                    min(g1.num_kb, kb0 + ks1.len), ks1.parts);
+            }
+        } else {
+            epilogue_tiles_group<1, GEO>(c, g1, f, tr1, k, it, amax_iter, sync_iter, ok);
+        }
+        epilogue_tiles_group<2, GEO>(c, g2, f, tr2(), k, it, amax_iter, sync_iter, ok);
     }
 
     __syncwarp();

@@ -589,7 +589,7 @@ __device__ __forceinline__ void mlp_epilogue(const Cta& c, const CUtensorMap* tm
         const bool last = t.key & TileInfo::LAST;
         if (ok) {
             if (t.mode() == 1) {
-                ok = wm ? epilogue_tile_wm<1, false, GEO, true>(c, a.g1, nullptr, t.m_tile(), t.n, it, turn, unused, 0, -1, 1,
+                ok = wm ? epilogue_tile_wm<1, false, GEO>(c, a.g1, nullptr, t.m_tile(), t.n, it, turn, unused, 0, -1, 1,
                                                                 &announce, t.key & TileInfo::LAST_TWO)
                         : mlp_epilogue_tile<1, GEO>(c, tmOut, a.g1, i, t, it, turn, announce);
                 if (ok) {
@@ -597,7 +597,7 @@ __device__ __forceinline__ void mlp_epilogue(const Cta& c, const CUtensorMap* tm
                     if (last) announce.settle(c.lane, true, a.g1.ready, a.g1.n_tiles);  // somebody may be waiting for it
                 }
             } else {
-                ok = wm ? epilogue_tile_wm<2, false, GEO, true>(c, a.g2, nullptr, t.m_tile(), t.n, it, turn, unused, 0, -1, 1,
+                ok = wm ? epilogue_tile_wm<2, false, GEO>(c, a.g2, nullptr, t.m_tile(), t.n, it, turn, unused, 0, -1, 1,
                                                                 &announce, false)
                         : mlp_epilogue_tile<2, GEO>(c, tmOut, a.g2, i, t, it, turn, announce);
             }

@@ -332,6 +332,13 @@ __device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c
     return d;
 }
 
+// (a.lo * b.lo, a.hi * b.hi), each rounded to nearest even.
+__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
 // ---- bf16 x bf16 + fp32 -------------------------------------------------------
 // a * b + c with the low / high bf16 halves of two words as factors: the product is exact, one rounding to nearest even, so
 // these are the bits of the fp32 FMA on the converted factors.

@@ -798,6 +798,24 @@ def test_gemm2_rounds_in_front_of_the_fused_kernel(cuda_device, hidden, inter, a
     eng.close()
 
 
+@pytest.mark.parametrize("hidden,inter,gate_first", [(256, 128, True), (256, 384, False), (768, 128, False)])
+def test_fused_kernel_groups_take_turns_at_tiles_shorter_than_the_pipeline(cuda_device, hidden, inter, gate_first):
+    # 1 to 6 K-blocks per tile against 6 stages, several tiles per CTA in both GEMMs, sub-tiles of more than 16 rows
+    dims = syn.LayerDims(hidden=hidden, intermediate=inter, num_local_experts=256)
+    for tokens in (14, 80):
+        wl = _wl(tokens, dims, seed=1500 + hidden + inter + tokens, skew=tokens == 80)
+        inp = syn.make_inputs(wl, cuda_device)
+        eng = make_engine(wl, cuda_device, poison=False, gate_first=gate_first)
+        eng.set_small_batch_fusion(False)
+        want = eng.forward(inp).clone()
+        eng.set_small_batch_fusion(True)
+        got = eng.forward(inp).clone()
+        torch.cuda.synchronize()
+        assert eng.status() == 0 and eng.last_launch_count() == (1 if tokens <= 16 else 2)
+        assert torch.equal(got.view(torch.int16), want.view(torch.int16))
+        eng.close()
+
+
 @pytest.mark.parametrize("tokens,launches,eloc", [(16, 1, 32), (48, 2, 32), (3, 1, 256)])  # 3 tokens: K split
 def test_a_wait_that_runs_out_in_the_fused_small_batch_kernel(cuda_device, tokens, launches, eloc):
     wl = _wl(tokens, dataclasses.replace(SMALL, num_local_experts=eloc), seed=43)
