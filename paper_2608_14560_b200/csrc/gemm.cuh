@@ -34,7 +34,7 @@
 //   fused_small_kernel          small batches (the host decides up to which size): the gather of stage 2, GEMM1, GEMM2
 //               and the weighted combine of stage 4 in ONE launch, with the operands swapped (weights on the
 //               M side of the MMA, the tile's at most 32 token rows on the N side; see "weights on M" below).
-//               Every CTA first works through its GEMM1 tiles, then its GEMM2 tiles.  Warp 3 gathers the (few)
+//               Every CTA first works through its GEMM1 tiles, then takes GEMM2 tiles from a counter.  Warp 3 gathers the (few)
 //               token rows of a GEMM1 tile straight from the token-major input with cp.async.  A GEMM2 tile
 //               starts once a counter in global memory says that all GEMM1 column tiles of its row tile have
 //               been stored (bounded wait; GEMM1 tiles never wait for another CTA and precede the GEMM2 tiles
@@ -54,8 +54,6 @@
 #include "ptx.cuh"
 
 namespace moe {
-
-
 
 // The two MMA issuer threads take the even and the odd K-blocks.  A thread must see EVERY phase of a barrier it
 // waits on (a parity wait cannot tell the wanted phase from the one two earlier), so a stage must always fall
@@ -187,15 +185,8 @@ struct FusedArgs {
     float* raw[2];
     int* part_done[2];            // [tiles] per GEMM, zero at launch (part of the counter set)
     int split;                    // 1: the split may be used by this call
-    int ahead;                    // GEMM2 tiles that take the time of a GEMM1 tile, see seq_after
+    int* ticket;                  // the next GEMM2 tile, zero at launch (part of the counter set)
 };
-// A GEMM2 tile of the fused kernel, however few its K-blocks, takes the time of about 18: its weights come in six stages
-// deep in front of its rows, its stores, its counters and the combine behind it.  Best number of rounds in front (0 to 6
-// measured, 16 to 64 tokens, five numbers of spare CTAs each; us per forward without / with it / with one per
-// K-block ratio): 2 to 3 with GEMM1 tiles of 56 K-blocks (7168 x 1024 159 / 152 / 175, x 512 182 / 167 / 206, x 256
-// 210 / 196 / 259), 1 with 32 (4096 x 2048 248 / 243 / 252, x 1024 100 / 97 / 102, x 512 115 / 110 / 133), none with 16
-// (2048 x 1024 68 / 68 / 72, x 512 68 / 68 / 85).
-constexpr int FRONT_TILE_KB = 18;
 constexpr int SPLIT_MAX_TOKENS = 4;                       // rows of a tile whose K range may be split
 constexpr int SPLIT_MAX_TILES = 74;                       // a split needs at least two CTAs per tile
 constexpr int SPLIT_RAW_FLOATS = 2 * SPLIT_MAX_TOKENS * 128;  // per tile and K-block
@@ -228,7 +219,7 @@ struct GemmCtrl {
     int abort_flag;
     int split_last;            // fused kernel, K split: this CTA stored the last part of the tile
     uint32_t gathered;         // fused kernel: stages the gather warp has arrived at
-    uint64_t sched_full[SCHED_SLOTS];   // grouped_mlp_kernel: the work list, published tile by tile
+    uint64_t sched_full[SCHED_SLOTS];   // the work list, published tile by tile (fused kernel: GEMM2's part of it)
     uint64_t sched_rows[SCHED_SLOTS];   // the tile's token rows are in memory
     TileInfo sched[SCHED_SLOTS];
 };
@@ -300,33 +291,38 @@ struct PlainSeq {  // the items in turn to all CTAs
 __device__ __forceinline__ PlainSeq seq_plain(int count) {
     return PlainSeq{static_cast<int>(blockIdx.x), static_cast<int>(gridDim.x), count};
 }
-struct AheadSeq {  // the first `rounds` rounds of items to `stride` of the CTAs, the later ones to all
-    int turn, skip, rounds, stride, grid, count;
-    __device__ __forceinline__ int at(int j) const {
-        j += skip;
-        return j < rounds ? j * stride + turn : rounds * stride + (j - rounds) * grid + turn;
+// The fused kernel's GEMM2 tiles come from a counter: the producer draws a ticket shortly before it needs the next tile and
+// publishes it for the other roles, entry by entry.  The GEMM1 tiles, one round more for some CTAs, and the memory's rate, which
+// is not the same for all, leave the CTAs at different times otherwise.  us per forward, dealt in rounds (with rounds in front where
+// few CTAs had a GEMM1 tile more) / from the counter: 37.1 / 35.9 at 1 token, 79.6 / 78.4 at 8, 114.4 / 110.2 at 16, 117.8 / 111.8 at 24,
+// 120.4 / 121.4 at 32, 158 / 153 at 28 (21 experts), 152.3 / 147.7 at 54, 114.4 / 109.8 at 64 skewed, 700 / 679 at 33 on 256 experts;
+// two handles with the same binary differ by up to 1 % there.
+struct Tickets {  // producer thread
+    int* counter;
+    int next;      // the drawn one; a draw in flight costs nothing until this is looked at
+    bool drawn;
+    __device__ __forceinline__ void draw() {
+        if (!drawn) next = atomicAdd(counter, 1);
+        drawn = true;
     }
 };
-// After `before` items dealt by seq_plain: the CTAs that got one item less are the first in every round, and they take up
-// to `ahead` rounds among themselves in front, as far as the items reach whose row tiles the full rounds have finished
-// (n1_tiles items before and n2_tiles new ones belong to a row tile).  Only where the last round before has few items: a
-// CTA streams up to 64 GB/s, so a hundred of them saturate the memory and the idle time of the others costs nothing.
-// (Dealt in plain rounds, 54 tokens on 23 experts left 72 CTAs with 238 K-blocks and 76 with 182; us per forward, plain
-// rounds / these: 54 tokens 175 / 165, 33 tokens on 256 local experts 766 / 752, 8 and 16 tokens up to 6 % less, equal
-// where GEMM1 fills whole rounds.)  The line is at 83 of 148 items, below every count that loses; us with plain rounds /
-// with these by that number, 40 and 72 tokens on 17 to 35 experts: 24 178 / 177 and 190 / 194, 56 192 / 191 and 205 / 206,
-// 72 193 / 191 and 207 / 205; beyond the line 84 263 / 258 and 277 / 266, 88 205 / 201 and 220 / 210, 100 274 / 270 and
-// 286 / 287, 104 206 / 204 and 217 / 215, 116 276 / 274 and 286 / 286, 120 208 / 220 and 220 / 236 (up to 104 these rounds
-// would gain as well).
-__device__ __forceinline__ AheadSeq seq_after(int before, int ahead, int n1_tiles, int n2_tiles, int count) {
-    const int grid = static_cast<int>(gridDim.x), b = static_cast<int>(blockIdx.x);
-    int r = before, rounds = 0;
-    if (before >= grid) {  // (below, the smallest batches, no division delays the first weights of the second phase)
-        r = before % grid;
-        if (r && r * 16 <= grid * 9) rounds = min(ahead, (before - r) / n1_tiles * n2_tiles / (grid - r));
+template <bool WARP>
+struct TicketSeq {  // the other roles; WARP: called by whole warps, whose lanes see all the same
+    const Cta& c;
+    int* status;
+    int count;
+    // Entry j; `count` at the end of the list or when the wait gave up.
+    __device__ __forceinline__ int at(int j) const {
+        const uint32_t slot = static_cast<uint32_t>(j) % SCHED_SLOTS;
+        bool ok = mbar_wait(smem_u32(&c.ctrl->sched_full[slot]), (static_cast<uint32_t>(j) / SCHED_SLOTS) & 1, c.abort_flag, c.limit);
+        if (WARP) ok = __all_sync(0xffffffffu, ok);
+        if (!ok) {
+            if (!WARP || c.lane == 0) raise(c.ctrl, status, DEV_TIMEOUT_PRODUCER);
+            return count;
+        }
+        return ld_shared_s32(smem_u32(&c.ctrl->sched[slot].key));
     }
-    return b < r ? AheadSeq{b - r + grid, rounds, rounds, grid - r, grid, count} : AheadSeq{b - r, 0, rounds, grid - r, grid, count};
-}
+};
 
 // Very small batches of the fused kernel: a tile's K range is cut into `parts` pieces of `len` K-blocks that
 // different CTAs work on (see epilogue_tile_wm).  parts = 1: a work item is a whole tile.
@@ -372,7 +368,7 @@ __device__ __forceinline__ void gemm_cta_setup(Cta& c, uint8_t* smem_raw, int fu
             mbar_init(smem_u32(&ctrl->group_turn[q]), G_EPI_WARPS / 2);
         }
         for (int i = 0; i < SCHED_SLOTS; ++i) {
-            mbar_init(smem_u32(&ctrl->sched_full[i]), 2);
+            mbar_init(smem_u32(&ctrl->sched_full[i]), GEO::FACTORS ? 2 : 1);  // (two arrivals: see mlp_factors)
             mbar_init(smem_u32(&ctrl->sched_rows[i]), 1);
         }
         ctrl->abort_flag = 0;
@@ -388,14 +384,27 @@ __device__ __forceinline__ void gemm_cta_setup(Cta& c, uint8_t* smem_raw, int fu
 // tmB: boxes of 128 weight rows of [expert][half][row][K]; MODE 1 takes gate[0,128) | up[0,128) of the tile's 128 columns ("gate" and "up"
 // change places with gate_first = 0), MODE 2 256 consecutive rows.  MODE 1: the token rows and the scales come from
 // the gather warp instead; MODE 2: the tile's token rows are GEMM1's output and must have been stored.
-template <int MODE, class GEO, class SEQ>
+template <int MODE, class GEO>
 __device__ __forceinline__ void producer_tiles(const Cta& c, const CUtensorMap* tmA, const CUtensorMap* tmB,
-                                               const GemmArgs& g, const FusedArgs* f, int ready_target, const SEQ& seq,
-                                               uint32_t& it, bool& ok, KSplit ks) {
+                                               const GemmArgs& g, const FusedArgs* f, int ready_target, PlainSeq seq,
+                                               Tickets& tickets, uint32_t& it, bool& ok, KSplit ks) {
     GemmCtrl* ctrl = c.ctrl;
-    for (int j = 0, item; ok && (item = seq.at(j)) < seq.count; ++j) {
+    for (int j = 0;; ++j) {
+        int item = MODE == 1 ? seq.at(j) : 0;
+        if (MODE == 2) {  // the next ticket, published for the other roles; one past the last tile ends the list
+            tickets.draw();
+            tickets.drawn = false;
+            item = min(tickets.next, seq.count);
+            const uint32_t slot = static_cast<uint32_t>(j) % SCHED_SLOTS;
+            *reinterpret_cast<volatile int*>(&ctrl->sched[slot].key) = item;
+            mbar_arrive(smem_u32(&ctrl->sched_full[slot]));
+        }
+        if (item >= seq.count) break;
         const int tile = item / ks.parts, kb0 = (item - tile * ks.parts) * ks.len;
         const int kb1 = min(g.num_kb, kb0 + ks.len);
+        // The ticket for the tile behind this one is drawn when the last stages are being refilled: not earlier, so that a CTA
+        // that waits for rows takes no tile from one that does not, and early enough to have come when it is needed.
+        const int draw_kb = MODE == 2 || seq.at(j + 1) >= seq.count ? max(kb0, kb1 - GEO::STAGES) : kb1;
         const int m_tile = tile / g.n_tiles, n = tile - m_tile * g.n_tiles;
         const int e = tile_expert_of(c, g, m_tile), wrow = n * (MODE == 1 ? 128 : G_TILE_N);
         const int row0 = tile_row0_of(c, g, m_tile);
@@ -452,7 +461,9 @@ __device__ __forceinline__ void producer_tiles(const Cta& c, const CUtensorMap* 
             if (!ok) break;
             load_b(it, kb);
             if (MODE == 2) load_a(it, kb);
+            if (kb >= draw_kb) tickets.draw();
         }
+        if (!ok) break;
     }
 }
 
@@ -1183,24 +1194,23 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmA2, const __grid_consta
     // (GEMM2's K range is too short for it: counting the parts and the finisher's pass over the stored partial sums
     // cost 5-6 us per tile, which 16 K-blocks do not win back; measured 1-2 us slower)
     const KSplit ks2 = ksplit_none(g2.num_kb);
-    const int n1 = m_tiles * g1.n_tiles * ks1.parts, n2 = m_tiles * g2.n_tiles * ks2.parts;
+    const int n1 = m_tiles * g1.n_tiles * ks1.parts, n2 = m_tiles * g2.n_tiles;
     const PlainSeq tr1 = seq_plain(n1);
-    // (set up behind the GEMM1 phase, where nobody waits for it)
-    auto tr2 = [&]() { return seq_after(n1, f.ahead, g1.n_tiles, g2.n_tiles, n2); };
     uint32_t it = 0;
     bool ok = true;
 
     if (c.warp < 4) {
         reg_dealloc<56>();
         if (c.warp == 0 && c.lane == 0) {
-            producer_tiles<1, GEO>(c, &tmA2, &tmB1, g1, &f, 0, tr1, it, ok, ks1);
-            producer_tiles<2, GEO>(c, &tmA2, &tmB2, g2, &f, g1.n_tiles, tr2(), it, ok, ks2);
+            Tickets tickets{f.ticket, 0, false};
+            producer_tiles<1, GEO>(c, &tmA2, &tmB1, g1, &f, 0, tr1, tickets, it, ok, ks1);
+            if (ok) producer_tiles<2, GEO>(c, &tmA2, &tmB2, g2, &f, g1.n_tiles, seq_plain(n2), tickets, it, ok, ks2);
         } else if ((c.warp == 1 || c.warp == 2) && c.lane == 0) {
             issuer_tiles_wm<GEO>(c, g1, tr1, c.warp - 1, it, ok, ks1);
-            issuer_tiles_wm<GEO>(c, g2, tr2(), c.warp - 1, it, ok, ks2);
+            issuer_tiles_wm<GEO>(c, g2, TicketSeq<false>{c, g1.status, n2}, c.warp - 1, it, ok, ks2);
         } else if (c.warp == 3) {
             gather_tiles<GEO>(c, g1, f, tr1, it, ok, ks1);
-            gather_idle_tiles<GEO>(c, g2, tr2(), it, ok, ks2);
+            gather_idle_tiles<GEO>(c, g2, TicketSeq<true>{c, g1.status, n2}, it, ok, ks2);
             cp_async_wait_all();  // nothing may still be landing in shared memory when the CTA exits
             if (c.lane == 0) c.ctrl->gathered = it;
         }
@@ -1218,7 +1228,7 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmA2, const __grid_consta
         } else {
             epilogue_tiles_group<1, GEO>(c, g1, f, tr1, k, it, amax_iter, sync_iter, ok);
         }
-        epilogue_tiles_group<2, GEO>(c, g2, f, tr2(), k, it, amax_iter, sync_iter, ok);
+        epilogue_tiles_group<2, GEO>(c, g2, f, TicketSeq<true>{c, g1.status, n2}, k, it, amax_iter, sync_iter, ok);
     }
 
     __syncwarp();

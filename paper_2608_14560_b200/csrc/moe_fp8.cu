@@ -79,7 +79,7 @@ WsLayout make_layout(const moe_fp8_config& c) {
     // (a batch the fused kernel takes has at most EL + F_MAX_TOKENS * 8 / 32 sub-tiles)
     // (then the parts stored per tile by the K split of very small batches, per GEMM)
     L.num_counters = std::min<size_t>(L.max_st, EL + F_MAX_TOKENS / 4) + static_cast<size_t>(F_MAX_TOKENS) * (H / G_TILE_N) +
-                     2 * SPLIT_MAX_TILES;
+                     2 * SPLIT_MAX_TILES + 1;
     L.counters = take(2 * L.num_counters * 4);
     L.raw1 = take(static_cast<size_t>(SPLIT_MAX_TILES) * (H / 128) * SPLIT_RAW_FLOATS * 4);
     L.raw2 = take(static_cast<size_t>(SPLIT_MAX_TILES) * (I / 128) * SPLIT_RAW_FLOATS * 4);
@@ -548,13 +548,13 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
         f.topk_w = topk_w;
         f.tok_nlocal = m.tok_nlocal;
         f.ready = counters;
-        f.tok_done = counters + (h->L.num_counters - 2 * SPLIT_MAX_TILES - static_cast<size_t>(F_MAX_TOKENS) * (H / G_TILE_N));
-        f.part_done[0] = counters + (h->L.num_counters - 2 * SPLIT_MAX_TILES);
+        f.ticket = counters + (h->L.num_counters - 1);
+        f.part_done[0] = f.ticket - 2 * SPLIT_MAX_TILES;
+        f.tok_done = f.part_done[0] - static_cast<size_t>(F_MAX_TOKENS) * (H / G_TILE_N);
         f.part_done[1] = f.part_done[0] + SPLIT_MAX_TILES;
         f.raw[0] = at<float>(h, h->L.raw1);
         f.raw[1] = at<float>(h, h->L.raw2);
         f.split = h->k_split ? 1 : 0;
-        f.ahead = g1.num_kb / std::max(g2.num_kb, FRONT_TILE_KB);
         // the fused kernel works on sub-tiles of at most 32 rows
         g1.num_m_tiles = g2.num_m_tiles = m.num_st;
         g1.tile_expert = g2.tile_expert = m.st_expert;
