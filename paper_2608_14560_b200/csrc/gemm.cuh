@@ -482,10 +482,12 @@ __device__ __forceinline__ void drain_after_abort(const Cta& c, int* status, uin
             if (j >= gathered) mbar_arrive_n(bar, 32);
             if (!mbar_wait(bar, (j / GEO::STAGES) & 1, &zero)) atomicCAS(status, DEV_OK, DEV_TIMEOUT_DRAIN);
         }
-    } else if ((c.warp == 1 || c.warp == 2) && c.lane == 0) {
-        const uint32_t bar = smem_u32(&c.ctrl->drain_bar[c.warp - 1]);
-        umma_commit(bar);
-        if (!mbar_wait(bar, 0, &zero)) atomicCAS(status, DEV_OK, DEV_TIMEOUT_DRAIN);
+    } else if (c.warp == 1 || c.warp == 2) {
+        if (GEO::FACTORS ? elect_one() : c.lane == 0) {  // the thread that issued the MMAs
+            const uint32_t bar = smem_u32(&c.ctrl->drain_bar[c.warp - 1]);
+            umma_commit(bar);
+            if (!mbar_wait(bar, 0, &zero)) atomicCAS(status, DEV_OK, DEV_TIMEOUT_DRAIN);
+        }
     }
     __syncwarp();
     tc_fence_before();

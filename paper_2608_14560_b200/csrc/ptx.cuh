@@ -367,6 +367,14 @@ __device__ __forceinline__ float fma_bf16_hi(uint32_t a, uint32_t b, float c) {
     return d;
 }
 
+// ---- one lane of a converged warp ------------------------------------------------
+// True for one lane, always the same one; the compiler knows that what follows is done by a single thread.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 // ---- registers --------------------------------------------------------------
 template <int N>
 __device__ __forceinline__ void reg_alloc() {
