@@ -30,17 +30,21 @@ namespace moe {
 // skewed, 1116 / 1125 at 16167, 2194 / 2201 at 16384 with 256 experts, 3170 / 3159 at 32768, 8913 / 8626 at 131072.
 // The last figure sets the line: under the power cap, which short runs do not reach (there one launch stays ahead: 2908 / 2987
 // at 32768 slots, 5066 / 5169 at 65536), the largest batches lose 3 %.
+// Two launches overlap up to PDL_MAX_TOKENS tokens: a CTA of the second one starts on an SM that has finished its GEMM1 tiles, all
+// CTAs of the first one run by then (they allow the second launch when they start), and its tiles wait for the announcements
+// of their rows like those of the one launch.  us per forward, one launch after the
+// other / overlapping: 191.4 / 179.3 at 81 tokens, 195.9 / 184.5 at 128, 196.5 / 182.6 at 160, 208.5 / 205.1 at 200, 208.9 / 205.1 at
+// 256; skewed 138.0 / 128.4 at 81, 175.6 / 159.2 at 200; on 256 experts 1187 / 1172 at 256.
 // The lower line is not set by speed: callers count on two GEMM launches up to 256 tokens (last_launch_count, the stage
-// times of the two GEMMs).  Above the fused kernel's 80 tokens one launch would be the faster one with uniform routing
-// (two / one: 153 / 148 us at 81 tokens, 184 / 166 at 128, 189 / 181 at 160, 206 / 192 at 256) and the slower one for few
-// skewed tokens (147 / 149 at 81, 151 / 154 at 128; 173 / 156 at 160, 197 / 186 at 256).
+// times of the two GEMMs).
 constexpr int MLP_SPLIT_MAX_TOKENS = 256;
 constexpr int MLP_JOINT_MAX_SLOTS = 16384;
 
 constexpr int MLP_MAX_GRID = 1023;   // lists that `claimed` has room for
 struct MlpArgs {
     GemmArgs g1, g2;
-    int phases;          // bit 0: GEMM1's tiles, bit 1: GEMM2's; both: a GEMM2 tile waits for its rows
+    int phases;          // bit 0: GEMM1's tiles, bit 1: GEMM2's
+    int by_row;          // a GEMM2 tile waits for the announcements of its rows: both GEMMs in one launch, or in two that overlap
     int* claimed;        // [grid] the lists of GEMM1 tiles, LIST_OPEN (or LIST_LEFT) at launch (both GEMMs only), and
                          // the next GEMM2 tile, zero at launch
 };
@@ -84,7 +88,7 @@ __device__ __forceinline__ uint32_t mlp_producer(const Cta& c, const CUtensorMap
                                              const CUtensorMap* tmA2s, const CUtensorMap* tmB2, const MlpArgs& a) {
     GemmCtrl* ctrl = c.ctrl;
     uint32_t it = 0;
-    bool ok = true, waited = false;  // waited: the kernels before this one have finished
+    bool ok = true, waited = a.phases == 2 && a.by_row;  // waited: the kernels before this one have finished (or need not have)
     for (uint32_t i = 0; ok; ++i) {
         const TileInfo cur = next_tile(c, i);
         if (cur.mode() == 0) break;
@@ -120,7 +124,7 @@ __device__ __forceinline__ uint32_t mlp_producer(const Cta& c, const CUtensorMap
             tma_load_2d(c.smem_base + s * GEO::STAGE_BYTES, tA, kb * G_BLOCK_K, row0, smem_u32(&ctrl->full[s]));
         };
         const uint32_t rows_bar = smem_u32(&ctrl->sched_rows[i % SCHED_SLOTS]), rows_ph = (i / SCHED_SLOTS) & 1;
-        const bool must_wait = !m1 && a.phases == 3;
+        const bool must_wait = !m1 && a.by_row;
         bool rows_there = !must_wait || mbar_test(rows_bar, rows_ph);
         int kb = 0;
         if (!waited || !rows_there) {
@@ -300,7 +304,7 @@ __device__ __forceinline__ void mlp_factors(const Cta& c, const MlpArgs& a) {
         ++published;
     };
     publish(false);
-    pdl_wait();
+    if (a.phases != 2 || !a.by_row) pdl_wait();
     // The fetch cursor: K-blocks fetched, tile, K-block in it, K-blocks left of the run.  Past the last tile of a GEMM it
     // goes on fetching the last K-block's scales, which nobody reads, so that the regular step has no branch for it.
     uint32_t fit = 0, fi = 0, frun = 0;
@@ -334,7 +338,7 @@ __device__ __forceinline__ void mlp_factors(const Cta& c, const MlpArgs& a) {
                 // this warp holds back its arrivals on done[], and the other roles of the CTA, once they wait for those,
                 // give up after one, which ends this wait as well.  Rows that never come are thus reported as the time-out
                 // of whichever role that is.)
-                if (!m1 && a.phases == 3)
+                if (!m1 && a.by_row)
                     there = wait_counter(a.g1.ready + t.m_tile(), ready_target, c.abort_flag, 4 * c.limit);
                 if (there) mbar_arrive(smem_u32(&ctrl->sched_rows[fi % SCHED_SLOTS]));
             }
@@ -594,7 +598,7 @@ __device__ __forceinline__ void mlp_epilogue(const Cta& c, const CUtensorMap* tm
                                                                 &announce, t.key & TileInfo::LAST_TWO)
                         : mlp_epilogue_tile<1, GEO>(c, tmOut, a.g1, i, t, it, turn, announce);
                 if (ok) {
-                    if (a.phases == 3) announce.add(tile);
+                    if (a.by_row) announce.add(tile);
                     if (last) announce.settle(c.lane, true, a.g1.ready, a.g1.n_tiles);  // somebody may be waiting for it
                 }
             } else {
@@ -633,7 +637,8 @@ grouped_mlp_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_consta
     // kernels before this one (warps 0 and 3 wait for them by themselves: weights and tile tables are there already,
     // see place_gather_kernel).
     pdl_launch_dependents();
-    if (c.warp != 0 && c.warp != 3) pdl_wait();
+    const bool overlaps = a.phases == 2 && a.by_row;  // with the GEMM1 launch before it, see MLP_SPLIT_MAX_TOKENS
+    if (c.warp != 0 && c.warp != 3 && !overlaps) pdl_wait();
     c.tmem_base = *reinterpret_cast<volatile uint32_t*>(&c.ctrl->tmem_slot);
     c.limit = a.g1.wait_limit;
     uint32_t claimed = 0;
@@ -653,6 +658,7 @@ grouped_mlp_kernel(const __grid_constant__ CUtensorMap tmA1, const __grid_consta
     }
 
     __syncwarp();
+    if (overlaps) pdl_wait();  // (so that whoever follows finds GEMM1's launch finished as well)
     tc_fence_before();
     __syncthreads();
     if (*c.abort_flag) drain_after_abort<GEO>(c, a.g1.status, claimed, claimed);

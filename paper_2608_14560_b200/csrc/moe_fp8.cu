@@ -588,13 +588,14 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
         // stage 3: GEMM1 + SwiGLU + re-quantisation, GEMM2
         if (h->short_tile_min_tokens > 0 && T >= h->short_tile_min_tokens) g1.wm_rows = g2.wm_rows = WM_TOKENS;
         g1.ready = m.mlp_ready;
-        MlpArgs a = {g1, g2, 3, m.mlp_claimed};
+        const bool joint = T > MLP_SPLIT_MAX_TOKENS && slots <= MLP_JOINT_MAX_SLOTS;
+        MlpArgs a = {g1, g2, 3, joint || pdl, m.mlp_claimed};
         auto mlp = [&](int phases) {
             a.phases = phases;
             return launch(grouped_mlp_kernel, m.mlp_grid, G_THREADS, GeomFull::SMEM_BYTES, stream, pdl_mlp, h->tm_a1, h->tm_a1_small,
                           h->tm_w13_n, h->tm_w13_m, h->tm_a2_store, h->tm_a2, h->tm_a2_small, h->tm_w2, a);
         };
-        if (T > MLP_SPLIT_MAX_TOKENS && slots <= MLP_JOINT_MAX_SLOTS) {
+        if (joint) {
             if ((lerr = mlp(3)) != cudaSuccess) return cuda_fail(h, lerr);
             ++launches;
             mark(ST_GROUPED_MLP);

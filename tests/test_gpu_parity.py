@@ -798,6 +798,28 @@ def test_gemm2_rounds_in_front_of_the_fused_kernel(cuda_device, hidden, inter, a
     eng.close()
 
 
+@pytest.mark.parametrize("tokens,skew", [(81, False), (81, True), (200, True), (256, False)])
+def test_two_gemm_launches_that_overlap(cuda_device, tokens, skew):
+    # GEMM2's launch starts while GEMM1's still runs and waits row tile by row tile; batches in a row on one handle, with
+    # and without stage timing (which keeps the launches apart)
+    eng = make_engine(_wl(tokens), cuda_device)
+    ref = make_engine(_wl(tokens), cuda_device)
+    ref.set_small_batch_fusion(256)
+    inps = [syn.make_inputs(_wl(tokens, seed=1700 + tokens + k, skew=skew), cuda_device) for k in range(3)]
+    want = [ref.forward(i).clone() for i in inps]
+    got = [eng.forward(inps[k % 3]).clone() for k in range(9)]
+    eng.set_stage_timing(True)
+    got += [eng.forward(i).clone() for i in inps]
+    eng.set_stage_timing(False)
+    got += [eng.forward(i).clone() for i in inps]
+    torch.cuda.synchronize()
+    assert eng.status() == 0 and ref.status() == 0 and eng.last_launch_count() == 5
+    for k, g in enumerate(got):
+        assert torch.equal(g.view(torch.int16), want[k % 3].view(torch.int16)), k
+    eng.close()
+    ref.close()
+
+
 @pytest.mark.parametrize("hidden,inter,gate_first", [(256, 128, True), (256, 384, False), (768, 128, False)])
 def test_fused_kernel_groups_take_turns_at_tiles_shorter_than_the_pipeline(cuda_device, hidden, inter, gate_first):
     # 1 to 6 K-blocks per tile against 6 stages, several tiles per CTA in both GEMMs, sub-tiles of more than 16 rows
