@@ -1079,9 +1079,17 @@ __device__ __forceinline__ bool epilogue_tile_group(const Cta& c, const GemmArgs
             last = atomicAdd(f.tok_done + static_cast<size_t>(tok) * g.n_tiles + n, 1) == tok_rows - 1;
         }
         uint32_t todo = __ballot_sync(0xffffffffu, last);
-        if (todo) {
-            __threadfence();
-            __syncwarp();  // (a vote orders no memory: the counting lanes' fences come before all lanes' loads)
+        if (!todo) return true;
+        __threadfence();
+        __syncwarp();  // (a vote orders no memory: the counting lanes' fences come before all lanes' loads)
+        // the rows and weights of all tokens at once, each by the lane that counted it: one round trip instead of one per token
+        int4 ra = make_int4(-1, -1, -1, -1), rb = ra;
+        float4 wa = make_float4(0.f, 0.f, 0.f, 0.f), wb = wa;
+        if (last) {
+            ra = __ldcg(reinterpret_cast<const int4*>(f.slot_to_row) + 2 * tok);
+            rb = __ldcg(reinterpret_cast<const int4*>(f.slot_to_row) + 2 * tok + 1);
+            wa = __ldcg(reinterpret_cast<const float4*>(f.topk_w) + 2 * tok);
+            wb = __ldcg(reinterpret_cast<const float4*>(f.topk_w) + 2 * tok + 1);
         }
         while (todo) {
             const int src = __ffs(todo) - 1;
@@ -1089,12 +1097,13 @@ __device__ __forceinline__ bool epilogue_tile_group(const Cta& c, const GemmArgs
             const int t = __shfl_sync(0xffffffffu, tok, src);
             // lane l owns columns n*256 + 8 l .. + 8: half of the 32-byte group n*16 + l/2.  All loads
             // first, then the sum in routing order.
-            const int4 ra = __ldcg(reinterpret_cast<const int4*>(f.slot_to_row) + 2 * t);
-            const int4 rb = __ldcg(reinterpret_cast<const int4*>(f.slot_to_row) + 2 * t + 1);
-            const float4 wa = __ldcg(reinterpret_cast<const float4*>(f.topk_w) + 2 * t);
-            const float4 wb = __ldcg(reinterpret_cast<const float4*>(f.topk_w) + 2 * t + 1);
-            const int rr[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
-            const float ww[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+            int rr[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
+            float ww[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                rr[j] = __shfl_sync(0xffffffffu, rr[j], src);
+                ww[j] = __shfl_sync(0xffffffffu, ww[j], src);
+            }
             uint4 u[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j)
