@@ -405,6 +405,7 @@ __device__ __forceinline__ void producer_tiles(const Cta& c, const CUtensorMap* 
         // The ticket for the tile behind this one is drawn when the last stages are being refilled: not earlier, so that a CTA
         // that waits for rows takes no tile from one that does not, and early enough to have come when it is needed.
         const int draw_kb = MODE == 2 || seq.at(j + 1) >= seq.count ? max(kb0, kb1 - GEO::STAGES) : kb1;
+        if (MODE == 2 && kb1 - kb0 <= GEO::STAGES) tickets.draw();  // (all of its stages go out at once)
         const int m_tile = tile / g.n_tiles, n = tile - m_tile * g.n_tiles;
         const int e = tile_expert_of(c, g, m_tile), wrow = n * (MODE == 1 ? 128 : G_TILE_N);
         const int row0 = tile_row0_of(c, g, m_tile);
