@@ -405,7 +405,8 @@ __device__ __forceinline__ void producer_tiles(const Cta& c, const CUtensorMap* 
         // The ticket for the tile behind this one is drawn when the last stages are being refilled: not earlier, so that a CTA
         // that waits for rows takes no tile from one that does not, and early enough to have come when it is needed.
         const int draw_kb = MODE == 2 || seq.at(j + 1) >= seq.count ? max(kb0, kb1 - GEO::STAGES) : kb1;
-        if (MODE == 2 && kb1 - kb0 <= GEO::STAGES) tickets.draw();  // (all of its stages go out at once)
+        // (a tile all of whose stages go out at once: now, where there are enough tiles for everybody)
+        if (MODE == 2 && kb1 - kb0 <= GEO::STAGES && seq.count > 2 * seq.stride) tickets.draw();
         const int m_tile = tile / g.n_tiles, n = tile - m_tile * g.n_tiles;
         const int e = tile_expert_of(c, g, m_tile), wrow = n * (MODE == 1 ? 128 : G_TILE_N);
         const int row0 = tile_row0_of(c, g, m_tile);
@@ -1009,11 +1010,15 @@ __device__ __forceinline__ bool epilogue_tile_group(const Cta& c, const GemmArgs
         float cc[32];
         uint32_t mine = 0;
 #pragma unroll
-        for (int t = 0; t < 32; ++t) {
-            cc[t] = silu_fast(acc[t]) * acc[32 + t];
-            // |x| as an integer orders like the float: the warp's maximum over its 32 output columns
-            const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(cc[t])));
-            if (lane == t) mine = m;
+        for (int h = 0; h < 2; ++h) {
+            if (h * 16 >= rows_valid) break;  // (most tiles of a decode batch have no more than 16 rows)
+#pragma unroll
+            for (int t = 16 * h; t < 16 * h + 16; ++t) {
+                cc[t] = silu_fast(acc[t]) * acc[32 + t];
+                // |x| as an integer orders like the float: the warp's maximum over its 32 output columns
+                const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(cc[t])));
+                if (lane == t) mine = m;
+            }
         }
         uint32_t* xq = reinterpret_cast<uint32_t*>(c.amax_x) + group * 128;  // [4 quadrants][32 tokens]
         xq[quad * 32 + lane] = mine;
