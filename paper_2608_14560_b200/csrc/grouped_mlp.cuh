@@ -197,7 +197,11 @@ __device__ __forceinline__ void mlp_issuer(const Cta& c, const MlpArgs& a, uint3
                 ok = __shfl_sync(0xffffffffu, ok, 0);
                 if (!ok && c.lane == 0) raise(ctrl, a.g1.status, DEV_TIMEOUT_MMA_SMEM);
             }
-            if (it >= G_ACC_BUFS) bar_sync(ACC_BARRIER + mine, ACC_BARRIER_THREADS);
+            // (orders the issuing lane behind lane 0, which has seen the stage land; a shuffle orders no memory)
+            if (it >= G_ACC_BUFS)
+                bar_sync(ACC_BARRIER + mine, ACC_BARRIER_THREADS);
+            else
+                __syncwarp();
             if (!ok) continue;
             tc_fence_after();
             // (by a lane chosen by its number, eight MMAs of a short tile took 850 clocks to issue, now 690)

@@ -590,6 +590,23 @@ def test_lists_of_gemm1_tiles_that_other_ctas_take_over(cuda_device, tokens, elo
     eng.close()
 
 
+@pytest.mark.parametrize("tokens", [90, 300])  # a launch per GEMM | both in one
+def test_first_k_blocks_of_a_launch(cuda_device, tokens):
+    # the first K-block of either issuer warp is the only one without an accumulator hand-over in front; here they are whole
+    # GEMM1 tiles (two K-blocks), every CTA has one at most, and other rows lie in shared memory from the batch before
+    dims = syn.LayerDims(hidden=256, intermediate=256, num_local_experts=32)
+    inps = [syn.make_inputs(_wl(tokens, dims, seed=1150 + tokens + k), cuda_device) for k in range(2)]
+    eng = make_engine(_wl(tokens, dims), cuda_device)
+    for k, inp in enumerate(inps):
+        run_and_compare(_wl(tokens, dims, seed=1150 + tokens + k), cuda_device, inp=inp, eng=eng)
+    want = [eng.forward(i).clone() for i in inps]
+    got = [eng.forward(inps[k % 2]).clone() for k in range(100)]
+    torch.cuda.synchronize()
+    assert eng.status() == 0
+    assert all(torch.equal(g.view(torch.int16), want[k % 2].view(torch.int16)) for k, g in enumerate(got))
+    eng.close()
+
+
 def _route_round_robin(inp, tokens, active, away=0):
     # token t on eight experts in turn, of the first `active` ones and `away` experts of other ranks
     ids = torch.tensor(list(range(active)) + list(range(256 - away, 256)))
