@@ -2,7 +2,7 @@
 // re-quantisation and GEMM2, in one launch.  Roles and their loop: see gemm.cuh.
 //
 // Every CTA has a list of tiles, GEMM1's first: CTA b takes GEMM1 tiles b, b + grid, ... and then GEMM2 tiles from a counter
-// until there are none.  A GEMM2 tile starts once GEMM1's column tiles of its row tile have been announced (bounded wait).  So that no CTA ever depends on one that has not started -- two such kernels may share the
+// until there are none (the first one is dealt where tiles are few, see mlp_first_tile_dealt).  A GEMM2 tile starts once GEMM1's column tiles of its row tile have been announced (bounded wait).  So that no CTA ever depends on one that has not started -- two such kernels may share the
 // GPU from different streams --, a CTA claims its list of GEMM1 tiles when it starts, and before its first GEMM2 tile it
 // works through the lists nobody has claimed: every GEMM1 tile it may then wait for is in the hands of a running CTA.
 // Fixed lists for GEMM1, not a counter that hands out tiles: neighbouring tiles share operands, and CTAs that read the same lines
@@ -40,13 +40,26 @@ namespace moe {
 constexpr int MLP_SPLIT_MAX_TOKENS = 256;
 constexpr int MLP_JOINT_MAX_SLOTS = 16384;
 
+// GEMM2 tiles that are dealt, one to every CTA (all or none); the later ones come from the counter.  With the counter alone a CTA
+// that waits for its first rows has already drawn a second tile, and where there are not many of them others have none.  Dealt
+// in one launch where there is no tile of GEMM1 or of GEMM2 for every CTA; in a launch of its own where there is no GEMM2 tile for
+// every CTA and a tile is longer than the ring of stages: short ones are better off on the CTAs that start first.  us per forward
+// from the counter / with one dealt: 7168 x 2048, 8 experts, 300 tokens 66.6 / 60.9, 3 experts, 600 tokens 72.8 / 66.9; 2048 x 2048,
+// 16 experts, 200 skewed 54.9 / 50.4; 512 x 2048, 64 experts, 100 tokens 53.2 / 49.5; 2048 x 1024, 16 experts, 400 tokens 38.4 / 35.0;
+// 768 x 768, 32 experts, 256 skewed 31.8 / 29.3.  Beyond the lines: 1024 x 1024, 64 experts, 114 tokens 48.8 / 50.6; 512 x 512, 100
+// experts, 92 tokens 30.9 / 32.3; 7168 x 2048, 32 experts, 901 tokens 194.3 / 195.1.
+__device__ __forceinline__ bool mlp_first_tile_dealt(bool joint, int m_tiles, const GemmArgs& g1, const GemmArgs& g2, int grid) {
+    const bool few1 = m_tiles * g1.n_tiles <= grid, few2 = m_tiles * g2.n_tiles <= grid;
+    return joint ? few1 || few2 : few2 && g2.num_kb > GeomFull::STAGES;
+}
+
 constexpr int MLP_MAX_GRID = 1023;   // lists that `claimed` has room for
 struct MlpArgs {
     GemmArgs g1, g2;
     int phases;          // bit 0: GEMM1's tiles, bit 1: GEMM2's
     int by_row;          // a GEMM2 tile waits for the announcements of its rows: both GEMMs in one launch, or in two that overlap
     int* claimed;        // [grid] the lists of GEMM1 tiles, LIST_OPEN (or LIST_LEFT) at launch (both GEMMs only), and
-                         // the next GEMM2 tile, zero at launch
+                         // the next GEMM2 tile behind the dealt ones, zero at launch
 };
 
 __device__ __forceinline__ TileInfo read_tile(const Cta& c, uint32_t i) {  // an entry that has been waited for
@@ -251,9 +264,14 @@ __device__ __forceinline__ void mlp_factors(const Cta& c, const MlpArgs& a) {
     const int m_tiles = __ldcg(a.g1.num_m_tiles);
     const int n1 = (a.phases & 1) ? m_tiles * a.g1.n_tiles : 0, n12 = n1 + ((a.phases & 2) ? m_tiles * a.g2.n_tiles : 0);
     const int grid = static_cast<int>(gridDim.x);
-    // GEMM1: tiles id1, id1 + grid, ... ; GEMM2: whichever is next when this CTA needs one (a ticket, drawn when it enters
-    // the tile before).
+    // GEMM1: tiles id1, id1 + grid, ... ; GEMM2: the dealt one, if any, then whichever is next when this CTA needs one (a ticket,
+    // drawn when it enters the tile before).
     int id1 = static_cast<int>(blockIdx.x);
+    int id2 = ~0;  // GEMM2: the dealt tile, or ~(number of dealt tiles)
+    if (mlp_first_tile_dealt(a.phases == 3, m_tiles, a.g1, a.g2, grid)) {
+        const int late = n1 % grid;  // CTAs with one GEMM1 tile more: they come last
+        id2 = id1 < late ? id1 + grid - late : id1 - late;
+    }
     if (a.phases == 3) {
         int was = LIST_OPEN;
         if (lane == 0) was = atomicCAS(a.claimed + blockIdx.x, LIST_OPEN, LIST_CLAIMED);
@@ -283,8 +301,13 @@ __device__ __forceinline__ void mlp_factors(const Cta& c, const MlpArgs& a) {
             id1 += grid;
         } else if ((a.phases & 2) && !end) {
             int ticket = 0;
-            if (lane == 0) ticket = atomicAdd(a.claimed + grid, 1);
-            id = n1 + __shfl_sync(0xffffffffu, ticket, 0);
+            if (id2 >= 0) {
+                id = n1 + id2;
+                id2 = ~grid;
+            } else {
+                if (lane == 0) ticket = atomicAdd(a.claimed + grid, 1);
+                id = n1 + ~id2 + __shfl_sync(0xffffffffu, ticket, 0);
+            }
         }
         const bool live = !end && id < n12;
         const bool first = id < n1;

@@ -636,6 +636,30 @@ def test_gemm2_rounds_in_front_of_the_joint_launch(cuda_device, active):
     eng.close()
 
 
+@pytest.mark.parametrize("hidden,inter,active", [(512, 256, 73), (512, 256, 74), (512, 256, 75),   # two and two tiles each
+                                                 (256, 512, 37), (256, 512, 38), (256, 512, 148), (256, 512, 149),  # four and one
+                                                 (1024, 128, 37), (1024, 128, 38), (1024, 128, 148), (1024, 128, 149)])  # one and four
+def test_gemm2_tiles_dealt_and_from_the_counter(cuda_device, hidden, inter, active):
+    # tiles of either GEMM on both sides of one for each of 148 CTAs: a launch per GEMM, overlapping | both GEMMs in one, and that
+    # with lists that other CTAs take over
+    dims = syn.LayerDims(hidden=hidden, intermediate=inter, num_local_experts=160)
+    eng = make_engine(_wl(300, dims), cuda_device)
+    for tokens, launches in ((100, 5), (300, 4)):
+        wl = _wl(tokens, dims, seed=1250 + tokens + active)
+        inp = syn.make_inputs(wl, cuda_device)
+        _route_round_robin(inp, tokens, active)
+        run_and_compare(wl, cuda_device, inp=inp, eng=eng, sample_tokens=_sample(tokens, 48, active), check_rows="tiles")
+        assert eng.last_launch_count() == launches
+        assert int((eng.debug_export(tokens, rows=False)["expert_count"] > 0).sum()) == active
+        want = eng.forward(inp).clone()
+        eng.debug_set_unclaimed_lists(50)
+        got = [eng.forward(inp).clone() for _ in range(3)]
+        torch.cuda.synchronize()
+        assert eng.status() == 0 and all(torch.equal(g.view(torch.int16), want.view(torch.int16)) for g in got)
+        eng.debug_set_unclaimed_lists(0)
+    eng.close()
+
+
 def test_two_handles_on_two_streams_share_the_gpu(cuda_device):
     # kernels whose CTAs wait for one another, from two streams at a time: a CTA may only depend on CTAs that run
     wls = [_wl(1500, seed=71), _wl(700, syn.LayerDims(hidden=1024, intermediate=512, num_local_experts=32), seed=72)]
