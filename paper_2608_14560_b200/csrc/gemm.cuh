@@ -1215,7 +1215,9 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmA2, const __grid_consta
     uint32_t it = 0;
     bool ok = true;
 
-    if (c.warp < 4) {
+    if (m_tiles == 0) {
+        // no token has a local expert: the roles would only tell one another so (6.8 against 5.7 us per forward)
+    } else if (c.warp < 4) {
         reg_dealloc<56>();
         if (c.warp == 0 && c.lane == 0) {
             Tickets tickets{f.ticket, 0, false};

@@ -104,6 +104,24 @@ def test_no_token_routes_locally(cuda_device):
     assert st["S"] == 0
 
 
+@pytest.mark.parametrize("tokens", [1, 16, 17, 80])  # one launch | behind the routing kernel
+def test_fused_kernel_without_a_tile_between_batches_that_have_some(cuda_device, tokens):
+    inp = syn.make_inputs(_wl(tokens, seed=19), cuda_device)
+    none = dict(inp, router_logits=inp["router_logits"].clone())
+    none["router_logits"][:, :32] = -20.0
+    eng = make_engine(_wl(tokens), cuda_device)
+    run_and_compare(_wl(tokens, seed=19), cuda_device, inp=inp, eng=eng)
+    want = eng.forward(inp).clone()
+    for n in (1, 2, 3):  # (the two counter sets take turns)
+        for _ in range(n):
+            out = torch.full_like(want, float("nan"))
+            eng.forward(none, out)
+            assert not out.view(torch.int16).any()
+        got = eng.forward(inp).clone()
+        assert eng.status() == 0 and torch.equal(got.view(torch.int16), want.view(torch.int16))
+    eng.close()
+
+
 def test_every_token_on_the_same_experts(cuda_device):
     wl = _wl(300, seed=2)
     inp = syn.make_inputs(wl, cuda_device)
