@@ -167,7 +167,7 @@ struct FusedArgs {
     const int* slot_to_row;       // [T*8]
     const float* topk_w;          // [T*8]
     const int* tok_nlocal;        // [T] local slots of each token
-    int* ready;                   // [row tiles] GEMM1 column tiles stored, zero at launch
+    int* ready;                   // [row tiles] GEMM1 column tiles stored, two per tile (one for each epilogue group), zero at launch
     int* tok_done;                // [T, H/256] GEMM2 rows stored per (token, column tile), zero at launch
     __nv_bfloat16* out;           // bf16 [T, H]
     // Routing and permutation inside the kernel (route != 0): every CTA computes stages 1 and 2 for itself.
@@ -886,7 +886,7 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
             }
             if (warp == 4 && lane == 0) {
                 __threadfence();
-                atomicAdd(f->ready + m_tile, 1);
+                atomicAdd(f->ready + m_tile, 2);
             }
         }
     } else {
@@ -934,15 +934,22 @@ __device__ __forceinline__ void promote16(float* acc, const float* v, const floa
 }
 
 // A tile of the fused kernel by one of its two epilogue groups of four warps, which take the CTA's tiles in turn: a thread owns
-// one weight row of each block for all 32 tokens.  A tile's tail is a chain of round trips to L2 (rows stored, fence, counter,
+// one weight row of each block for all 32 tokens, 16 at a time.  A tile's tail is a chain of round trips to L2 (rows stored, fence, counter,
 // combine) of 4 to 8 us while the memory is busy, as long as a GEMM2 tile's loop; with all eight warps on every tile nothing
 // was read from the stages meanwhile, six stages held 6 to 8 us of the tile's stream, and all CTAs were in their tails together.
 // Now the tail runs beside the other group's tile.  us per forward, eight warps on every tile / two groups: 70.9 / 67.6 at 4
 // tokens, 82.0 / 80.0 at 8, 125.1 / 115.4 at 16, 130.3 / 121.4 at 32, 162.1 / 153.9 at 54, 166.4 / 160.3 at 80, 124.4 / 115.7 at 64
 // skewed, 726 / 701 at 33 on 256 experts.  Element for element the arithmetic is that of epilogue_tile_wm.
-// `k` numbers the CTA's tiles.  Scales and tables are asked for before the group's turn comes.
+// Sixteen rows that do not exist are not read.  `halved`: both groups are on the tile, each with 16 of its rows to promote, store, count
+// and combine; neither waits for the other.  Where a CTA has one tile there is no other group's tail to hide, and four warps on more than
+// 16 rows take longer than eight (weights in L2; us per forward, eight warps on every tile before there were groups / never halved /
+// halved: 256 x 256, 70 skewed tokens 25.6 / 27.8 / 24.4; 1024 x 768, 30 skewed 29.9 / 31.8 / 28.5; 1536 x 256, 27 skewed 28.5 / 30.2 / 27;
+// 2048 x 512, 40 skewed 33.8 / 35 / 31.4).  Halved whatever the number of tiles, 7168 x 512 with 64 experts and 60 skewed tokens takes
+// 80.7 instead of 75.5, 1024 x 1024 with 128 experts and 80 skewed 54.0 instead of 48.3; up to two tiles per CTA 54.3 there.
+// us per forward before / with the rows that exist alone: 53.9 / 51.1 at 8 tokens, 70.2 / 68.3 at 16, 110 / 109 at 54.
+// Scales and tables are asked for before the group's turn comes.  `turn`: phase of the barrier to wait for, -1: none.
 template <int MODE, class GEO>
-__device__ __forceinline__ bool epilogue_tile_group(const Cta& c, const GemmArgs& g, const FusedArgs& f, int m_tile, int n, uint32_t k,
+__device__ __forceinline__ bool epilogue_tile_group(const Cta& c, const GemmArgs& g, const FusedArgs& f, int m_tile, int n, bool halved, int turn,
                                                     uint32_t& it, uint32_t& amax_iter, uint32_t& sync_iter) {
     GemmCtrl* ctrl = c.ctrl;
     const int lane = c.lane, quad = c.warp & 3, group = (c.warp - 4) >> 2;
@@ -950,6 +957,7 @@ __device__ __forceinline__ bool epilogue_tile_group(const Cta& c, const GemmArgs
     const size_t row_cap = static_cast<size_t>(g.row_cap);
     const int num_kb = g.num_kb;
     const int e = tile_expert_of(c, g, m_tile), rows_valid = tile_rows_of(c, g, m_tile), tile_row0 = tile_row0_of(c, g, m_tile);
+    const int halves = halved ? 1 << group : rows_valid > 16 ? 3 : 1;  // bit h: this group's warps look after the rows [16 h, 16 h + 16)
     const bool swap = MODE == 1 && g.up_first;  // acc[0..32) is the gate block's either way
     const float* ws0 = g.w_scale + (static_cast<size_t>(e) * (g.w_rows_per_expert / 128) + (MODE == 1 ? n : 2 * n)) * num_kb;
     const float* ws1 = ws0 + static_cast<size_t>(MODE == 1 ? g.up_row0 / 128 : 1) * num_kb;
@@ -960,9 +968,10 @@ __device__ __forceinline__ bool epilogue_tile_group(const Cta& c, const GemmArgs
     }
     const uint32_t col0 = swap ? WM_TOKENS : 0, col1 = WM_TOKENS - col0;
     float s0 = __ldg(ws0), s1 = __ldg(ws1);
-    // MODE 2: warp `quad` looks after the rows quad, quad + 4, ... of the tile (lanes 0..7): their tokens and how many rows each has
+    // MODE 2: warp `quad` looks after the group's rows among quad, quad + 4, ... of the tile (lanes 0..7): their tokens and how many rows
+    // each has
     int tok = -1, tok_rows = 0;
-    if (MODE == 2 && lane < 8 && quad + 4 * lane < rows_valid) {
+    if (MODE == 2 && lane < 8 && quad + 4 * lane < rows_valid && (halves >> (lane >> 2) & 1)) {
         tok = row_token_of(c, f.row_token, m_tile, tile_row0, quad + 4 * lane);
         tok_rows = __ldcg(f.tok_nlocal + tok);
     }
@@ -971,7 +980,7 @@ __device__ __forceinline__ bool epilogue_tile_group(const Cta& c, const GemmArgs
         return false;
     };
     // The other group has read the last accumulator of the tile before: from here on no stage is more than one phase behind.
-    if (k > 0 && !__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctrl->group_turn[group]), ((k - 1) >> 1) & 1, c.abort_flag, c.limit)))
+    if (turn >= 0 && !__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctrl->group_turn[group]), turn, c.abort_flag, c.limit)))
         return timed_out();
 
     float acc[64];  // [0,32): block 0 (the gate rows), [32,64): block 1
@@ -986,24 +995,26 @@ __device__ __forceinline__ bool epilogue_tile_group(const Cta& c, const GemmArgs
         const uint32_t s = it % GEO::STAGES, ph = (it / GEO::STAGES) & 1;
         if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&ctrl->done[s]), ph, c.abort_flag, c.limit))) return timed_out();
         tc_fence_after();
-        float v[64];
-        tmem_ld32_issue(t_lane + s * WM_BUF_COLS + col0, v);
-        tmem_ld32_issue(t_lane + s * WM_BUF_COLS + col1, v + 32);
-        tmem_wait_ld(v);
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_n(smem_u32(&ctrl->tmem_empty[s]), 2);  // (for a warp of each group)
         // the MMAs of this K-block have finished, hence its stage -- tokens, weights and scales -- had landed
         const float4* sp = reinterpret_cast<const float4*>(c.scale_ring + (it % GEO::SCALE_SLOTS) * GEO::A_ROWS);
+        const uint32_t t_buf = t_lane + s * WM_BUF_COLS;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
+            if (!(halves >> h & 1)) continue;
+            float v[32];
+            tmem_ld16x2(t_buf + col0 + 16 * h, t_buf + col1 + 16 * h, v);
             const float4 sa[4] = {sp[4 * h], sp[4 * h + 1], sp[4 * h + 2], sp[4 * h + 3]};
-            promote16(acc + 16 * h, v + 16 * h, sa, w0);
-            promote16(acc + 32 + 16 * h, v + 32 + 16 * h, sa, w1);
+            promote16(acc + 16 * h, v, sa, w0);
+            promote16(acc + 32 + 16 * h, v + 16, sa, w1);
         }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_n(smem_u32(&ctrl->tmem_empty[s]), halved ? 1 : 2);  // (2: for a warp of each group)
     }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(smem_u32(&ctrl->group_turn[group ^ 1]));
+    if (!halved) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&ctrl->group_turn[group ^ 1]));
+    }
 
     uint8_t* wst = c.store_stage + (c.warp - 4) * 512;  // this warp's staging
     if (MODE == 1) {
@@ -1011,7 +1022,7 @@ __device__ __forceinline__ bool epilogue_tile_group(const Cta& c, const GemmArgs
         uint32_t mine = 0;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            if (h * 16 >= rows_valid) break;  // (most tiles of a decode batch have no more than 16 rows)
+            if (!(halves >> h & 1)) continue;  // (most tiles of a decode batch have no more than 16 rows)
 #pragma unroll
             for (int t = 16 * h; t < 16 * h + 16; ++t) {
                 cc[t] = silu_fast(acc[t]) * acc[32 + t];
@@ -1032,7 +1043,7 @@ __device__ __forceinline__ bool epilogue_tile_group(const Cta& c, const GemmArgs
         // 16-byte stores -- lane l carries 16 columns of token l / 2.
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            if (h * 16 >= rows_valid) break;
+            if (!(halves >> h & 1)) continue;
 #pragma unroll
             for (int t = 0; t < 16; ++t) {
                 const float inv_sc = __shfl_sync(0xffffffffu, my_inv, h * 16 + t);
@@ -1045,14 +1056,15 @@ __device__ __forceinline__ bool epilogue_tile_group(const Cta& c, const GemmArgs
                     *reinterpret_cast<const uint4*>(wst + (lane >> 1) * 32 + (lane & 1) * 16);
             __syncwarp();
         }
-        if (quad == 0 && lane < rows_valid) g.out_scale_t[static_cast<size_t>(n) * row_cap + tile_row0 + lane] = my_sc;
+        if (quad == 0 && lane < rows_valid && (halves >> (lane >> 4) & 1))
+            g.out_scale_t[static_cast<size_t>(n) * row_cap + tile_row0 + lane] = my_sc;
         // Announce the tile.  (The rows are read by copy engines of other CTAs: plain stores here, asynchronous-proxy loads
         // there.)  The announcing thread's fence comes behind the rendezvous and covers the stores of all.
         fence_proxy_async();
         if (!epilogue_rendezvous(c, &ctrl->group_sync[group], sync_iter)) return timed_out();
         if (quad == 0 && lane == 0) {
             __threadfence();
-            atomicAdd(f.ready + m_tile, 1);
+            atomicAdd(f.ready + m_tile, halved ? 1 : 2);
         }
     } else {
         // bf16 out through this warp's 512 bytes of staging, eight tokens x 32 columns at a time, so that
@@ -1061,7 +1073,7 @@ __device__ __forceinline__ bool epilogue_tile_group(const Cta& c, const GemmArgs
         __nv_bfloat16* bst = reinterpret_cast<__nv_bfloat16*>(wst);
 #pragma unroll
         for (int h = 0; h < 4; ++h) {
-            if (h * 8 >= rows_valid) break;
+            if (!(halves >> (h >> 1) & 1) || h * 8 >= rows_valid) continue;
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
 #pragma unroll
@@ -1143,18 +1155,26 @@ __device__ __forceinline__ bool epilogue_tile_group(const Cta& c, const GemmArgs
     return true;
 }
 
-// The tiles of one GEMM, those of this warp's group; `k` goes on from GEMM to GEMM.
+// The tiles of one GEMM.  `few`: no more tiles than CTAs, so that the other group would have nothing to do meanwhile; tiles of more
+// than 16 rows are then halved.  `k` numbers the tiles that a group takes alone, from GEMM to GEMM; `behind`: this group has passed one by
+// since its own last one.
 template <int MODE, class GEO, class SEQ>
-__device__ __forceinline__ void epilogue_tiles_group(const Cta& c, const GemmArgs& g, const FusedArgs& f, const SEQ& seq, uint32_t& k,
-                                                     uint32_t& it, uint32_t& amax_iter, uint32_t& sync_iter, bool& ok) {
+__device__ __forceinline__ void epilogue_tiles_group(const Cta& c, const GemmArgs& g, const FusedArgs& f, const SEQ& seq, bool few, uint32_t& k,
+                                                     bool& behind, uint32_t& it, uint32_t& amax_iter, uint32_t& sync_iter, bool& ok) {
     const uint32_t group = (c.warp - 4) >> 2;
-    for (int j = 0, tile; ok && (tile = seq.at(j)) < seq.count; ++j, ++k) {
-        if ((k & 1) != group) {
+    for (int j = 0, tile; ok && (tile = seq.at(j)) < seq.count; ++j) {
+        const int m_tile = tile / g.n_tiles, n = tile - m_tile * g.n_tiles;
+        const bool halved = few && tile_rows_of(c, g, m_tile) > 16;
+        const uint32_t before = k;
+        if (!halved) ++k;
+        if (!halved && (before & 1) != group) {
             it += g.num_kb;
+            behind = true;
             continue;
         }
-        const int m_tile = tile / g.n_tiles, n = tile - m_tile * g.n_tiles;
-        ok = epilogue_tile_group<MODE, GEO>(c, g, f, m_tile, n, k, it, amax_iter, sync_iter);
+        const int turn = behind ? static_cast<int>(((before - 1) >> 1) & 1) : -1;
+        behind = false;
+        ok = epilogue_tile_group<MODE, GEO>(c, g, f, m_tile, n, halved, turn, it, amax_iter, sync_iter);
     }
 }
 
@@ -1222,7 +1242,7 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmA2, const __grid_consta
         if (c.warp == 0 && c.lane == 0) {
             Tickets tickets{f.ticket, 0, false};
             producer_tiles<1, GEO>(c, &tmA2, &tmB1, g1, &f, 0, tr1, tickets, it, ok, ks1);
-            if (ok) producer_tiles<2, GEO>(c, &tmA2, &tmB2, g2, &f, g1.n_tiles, seq_plain(n2), tickets, it, ok, ks2);
+            if (ok) producer_tiles<2, GEO>(c, &tmA2, &tmB2, g2, &f, 2 * g1.n_tiles, seq_plain(n2), tickets, it, ok, ks2);
         } else if ((c.warp == 1 || c.warp == 2) && c.lane == 0) {
             issuer_tiles_wm<GEO>(c, g1, tr1, c.warp - 1, it, ok, ks1);
             issuer_tiles_wm<GEO>(c, g2, TicketSeq<false>{c, g1.status, n2}, c.warp - 1, it, ok, ks2);
@@ -1235,6 +1255,7 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmA2, const __grid_consta
     } else {
         reg_alloc<224>();
         uint32_t k = 0, amax_iter = 0, sync_iter = 0;
+        bool behind = false;
         if (ks1.parts > 1) {  // (one part of a tile at most; all eight warps)
             uint32_t joint_iter = 0;
             AmaxTurn turn{0};
@@ -1244,9 +1265,9 @@ fused_small_kernel(const __grid_constant__ CUtensorMap tmA2, const __grid_consta
                                                     min(g1.num_kb, kb0 + ks1.len), ks1.parts);
             }
         } else {
-            epilogue_tiles_group<1, GEO>(c, g1, f, tr1, k, it, amax_iter, sync_iter, ok);
+            epilogue_tiles_group<1, GEO>(c, g1, f, tr1, n1 <= grid, k, behind, it, amax_iter, sync_iter, ok);
         }
-        epilogue_tiles_group<2, GEO>(c, g2, f, TicketSeq<true>{c, g1.status, n2}, k, it, amax_iter, sync_iter, ok);
+        epilogue_tiles_group<2, GEO>(c, g2, f, TicketSeq<true>{c, g1.status, n2}, n2 <= grid, k, behind, it, amax_iter, sync_iter, ok);
     }
 
     __syncwarp();

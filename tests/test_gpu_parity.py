@@ -897,6 +897,32 @@ def test_fused_kernel_groups_take_turns_at_tiles_shorter_than_the_pipeline(cuda_
         eng.close()
 
 
+@pytest.mark.parametrize("hidden,inter,active", [(512, 256, 5), (1024, 128, 37), (1024, 128, 38), (256, 512, 37), (256, 512, 38)])
+@pytest.mark.parametrize("tokens", [16, 17, 33, 70])
+def test_fused_kernel_tiles_of_one_group_and_of_both(cuda_device, hidden, inter, active, tokens):
+    # tiles for at most every CTA in both GEMMs, in GEMM1 only and in GEMM2 only, or one too many; sub-tiles of 16, 17, 32 and 1,
+    # 32, 32 and 6 rows (three experts that every token goes to) beside short ones
+    dims = syn.LayerDims(hidden=hidden, intermediate=inter, num_local_experts=160)
+    wl = _wl(tokens, dims, seed=1550 + tokens + active)
+    inp = syn.make_inputs(wl, cuda_device)
+    _route_round_robin(inp, tokens, active - 3 if active > 11 else active)
+    if active > 11:
+        rest = torch.arange(tokens)[:, None] * 5 % (active - 3) + torch.arange(5)[None]
+        idx = torch.cat([torch.arange(active - 3, active).expand(tokens, 3), rest % (active - 3)], 1)
+        inp["router_logits"][:] = -8.0
+        inp["router_logits"].scatter_(1, idx.to(cuda_device), 6.0)
+    eng = make_engine(wl, cuda_device)
+    eng.set_small_batch_fusion(False)
+    want = eng.forward(inp).clone()
+    eng.set_small_batch_fusion(True)
+    got = [eng.forward(inp).clone() for _ in range(4)]
+    torch.cuda.synchronize()
+    assert eng.status() == 0 and eng.last_launch_count() == (1 if tokens <= 16 else 2)
+    assert all(torch.equal(g.view(torch.int16), want.view(torch.int16)) for g in got)
+    run_and_compare(wl, cuda_device, inp=inp, eng=eng, check_rows="tiles")
+    eng.close()
+
+
 @pytest.mark.parametrize("tokens,launches,eloc", [(16, 1, 32), (48, 2, 32), (3, 1, 256)])  # 3 tokens: K split
 def test_a_wait_that_runs_out_in_the_fused_small_batch_kernel(cuda_device, tokens, launches, eloc):
     wl = _wl(tokens, dataclasses.replace(SMALL, num_local_experts=eloc), seed=43)
