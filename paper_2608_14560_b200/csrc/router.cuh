@@ -33,14 +33,18 @@ namespace moe {
 //   8 x 8 per warp, 2 x 2 warps   many small CTAs balance the SMs: 257 tokens 33.5 / 29.4, 1024 94.9 / 83.3, 8192 660 (16 x 8
 //                                 per warp) / 627, 24.0 TFMA/s; with the bf16 FMA 16 x 8 is slower (662)
 //   4 x 4, 2 x 1 warps            many loads in flight per warp: 16 tokens 11.2 / 8.9, 64 tokens 15.2 / 11.1 in rows of 512
-//                                 elements, four stages (256, eight stages: 9.6 and 13.5); equal to 8 x 8 at 128 tokens
+//                                 elements, four stages (256, eight stages: 9.6 and 13.5)
+// The line lies where they are equal.  us per forward from hidden states with 8 x 8 / 4 x 4, hidden 7168: without local rows 28.1 /
+// 26.8 at 80 tokens, 33.7 / 32.8 at 96, 34.6 / 34.3 at 128, 34.9 / 35.0 at 144; 32 experts of 7168 x 2048 158.0 / 145.4 at 72, 202.6 / 196.7 at
+// 100, 161.0 / 152.5 at 128; hidden 2048 34.1 / 33.1 at 100, 34.5 / 33.8 at 128, 37.2 / 37.8 at 200; hidden 512 26.5 / 25.7 at 100, 20.4 / 20.8
+// at 200.
 template <int WT, int WE, int MT, int ME, int KC, int S>
 struct RouterShape {
     static constexpr int ROWS_T = WT * MT, ROWS_E = WE * ME, THREADS = WT * WE * 32, ROWS = ROWS_T + ROWS_E;
     static constexpr int SMEM_BYTES = S * ROWS * KC * 2;
     static_assert(MT % 4 == 0 && ME % 4 == 0 && KC % 64 == 0, "rows are read four at a time, in runs of 64 elements");
 };
-constexpr int RP_SMALL_MAX_TOKENS = 64;    // 4 x 4 up to here
+constexpr int RP_SMALL_MAX_TOKENS = 128;   // 4 x 4 up to here
 
 template <int WT, int WE, int MT, int ME, int KC, int S>
 __global__ void __launch_bounds__(WT * WE * 32)

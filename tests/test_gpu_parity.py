@@ -466,11 +466,11 @@ def test_from_hidden_small_layer(cuda_device, tokens):
     _from_hidden_case(_wl(tokens, seed=60 + tokens), cuda_device)
 
 
-@pytest.mark.parametrize("tokens,hidden", [(3, 256), (64, 768), (65, 256), (257, 512), (2047, 256), (2048, 256), (2049, 512),
-                                           (2053, 1280)])
+@pytest.mark.parametrize("tokens,hidden", [(3, 256), (64, 768), (65, 256), (127, 1280), (128, 768), (128, 512), (129, 768), (129, 512),
+                                           (257, 512), (2047, 256), (2048, 256), (2049, 512), (2053, 1280)])
 def test_from_hidden_at_the_edges_of_the_projection_shapes(cuda_device, tokens, hidden):
-    # the three warp tiles of the projection with ragged last tiles, K from fewer chunks than pipeline stages up, and a
-    # hidden size that the largest shape's chunks do not divide
+    # the two warp tiles of the projection (up to 128 tokens and above) with ragged last tiles, K from fewer chunks than pipeline
+    # stages up, and hidden sizes that the chunks of 512 do not divide
     dims = syn.LayerDims(hidden=hidden, intermediate=128, num_local_experts=32)
     _from_hidden_case(_wl(tokens, dims, seed=600 + tokens), cuda_device, sample_tokens=_sample(tokens, 64, tokens))
 
