@@ -180,10 +180,10 @@ struct FusedArgs {
     PermuteMeta meta;
     int* counters_next;           // the counter set of the NEXT fused call, zeroed by CTA 0 of this one
     int num_counters;
-    // K split of very small batches (T <= SPLIT_MAX_TOKENS, few tiles): the parts of a tile store their per-K-block
-    // partial sums here, [tile][K-block][weight-row block][128 rows][4 tokens] fp32 per GEMM, and count themselves
-    float* raw[2];
-    int* part_done[2];            // [tiles] per GEMM, zero at launch (part of the counter set)
+    // K split of very small batches (GEMM1, T <= SPLIT_MAX_TOKENS, few tiles): the parts of a tile store their per-K-block
+    // partial sums here, [tile][K-block][weight-row block][128 rows][4 tokens] fp32, and count themselves
+    float* raw;
+    int* part_done;               // [tiles] zero at launch (part of the counter set)
     int split;                    // 1: the split may be used by this call
     int* ticket;                  // the next GEMM2 tile, zero at launch (part of the counter set)
 };
@@ -693,7 +693,7 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
     const int tile_row0 = SHARED ? m_tile * TILE_M : tile_row0_of(c, g, m_tile);
     float4* raw = nullptr;  // this tile's stored partial sums (four tokens each): this thread's weight row
     if (SPLIT)
-        raw = reinterpret_cast<float4*>(f->raw[MODE - 1] + static_cast<size_t>(m_tile * g.n_tiles + n) * num_kb * SPLIT_RAW_FLOATS) +
+        raw = reinterpret_cast<float4*>(f->raw + static_cast<size_t>(m_tile * g.n_tiles + n) * num_kb * SPLIT_RAW_FLOATS) +
               quad * 32 + lane;
     for (int kb = kb0; kb < kb_end; ++kb, ++it) {
         const uint32_t s = it % GEO::STAGES, ph = (it / GEO::STAGES) & 1;
@@ -745,7 +745,7 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
         }
         if (warp == 4 && lane == 0) {
             __threadfence();
-            const int before = atomicAdd(f->part_done[MODE - 1] + m_tile * g.n_tiles + n, 1);
+            const int before = atomicAdd(f->part_done + m_tile * g.n_tiles + n, 1);
             *reinterpret_cast<volatile int*>(&ctrl->split_last) = (before == parts - 1);
         }
         if (!epilogue_rendezvous(c, &ctrl->sync_bar, sync_iter)) {
@@ -765,13 +765,9 @@ __device__ __forceinline__ bool epilogue_tile_wm(const Cta& c, const GemmArgs& g
             const int kb = i / SPLIT_MAX_TOKENS, t = i - kb * SPLIT_MAX_TOKENS;
             float v = 0.0f;
             if (t < rows_valid) {
-                if (MODE == 1) {
-                    const int tok = row_token_of(c, f->row_token, m_tile, tile_row0, t);
-                    v = __ldcg(f->scale_layout ? f->hidden_scale + static_cast<size_t>(kb) * f->T + tok
-                                               : f->hidden_scale + static_cast<size_t>(tok) * num_kb + kb);
-                } else {
-                    v = __ldcg(g.a_scale_t + static_cast<size_t>(kb) * row_cap + tile_row0 + t);
-                }
+                const int tok = row_token_of(c, f->row_token, m_tile, tile_row0, t);
+                v = __ldcg(f->scale_layout ? f->hidden_scale + static_cast<size_t>(kb) * f->T + tok
+                                           : f->hidden_scale + static_cast<size_t>(tok) * num_kb + kb);
             }
             sa_s[i] = v;
         }

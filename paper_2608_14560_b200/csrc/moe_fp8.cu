@@ -31,7 +31,7 @@ inline size_t align_up(size_t x, size_t a = WS_ALIGN) { return (x + a - 1) / a *
 
 struct WsLayout {
     size_t topk_idx, topk_w, slot_rank, block_hist, expert_count, expert_offset, padded_offset, tile_expert, tile_rows,
-        num_m_tiles, mlp_ready, mlp_claimed, slot_to_row, row_to_slot, row_token, tok_nlocal, st_expert, st_row0, st_rows, num_st, counters, num_counters, max_st, raw1, raw2, status, a1, a1_scale_t, a2, a2_scale_t, y, stage_hidden,
+        num_m_tiles, mlp_ready, mlp_claimed, slot_to_row, row_to_slot, row_token, tok_nlocal, st_expert, st_row0, st_rows, num_st, counters, num_counters, max_st, split_raw, status, a1, a1_scale_t, a2, a2_scale_t, y, stage_hidden,
         stage_scale, stage_logits, stage_out, stage2_hidden, stage2_scale, stage2_logits, stage2_out, total;
     int row_cap, max_m_tiles, max_blocks;
 };
@@ -77,12 +77,11 @@ WsLayout make_layout(const moe_fp8_config& c) {
     L.st_rows = take(L.max_st * 4);
     L.num_st = take(4);
     // (a batch the fused kernel takes has at most EL + F_MAX_TOKENS * 8 / 32 sub-tiles)
-    // (then the parts stored per tile by the K split of very small batches, per GEMM)
+    // (then the parts stored per tile by the K split of very small batches, and the tickets)
     L.num_counters = std::min<size_t>(L.max_st, EL + F_MAX_TOKENS / 4) + static_cast<size_t>(F_MAX_TOKENS) * (H / G_TILE_N) +
-                     2 * SPLIT_MAX_TILES + 1;
+                     SPLIT_MAX_TILES + 1;
     L.counters = take(2 * L.num_counters * 4);
-    L.raw1 = take(static_cast<size_t>(SPLIT_MAX_TILES) * (H / 128) * SPLIT_RAW_FLOATS * 4);
-    L.raw2 = take(static_cast<size_t>(SPLIT_MAX_TILES) * (I / 128) * SPLIT_RAW_FLOATS * 4);
+    L.split_raw = take(static_cast<size_t>(SPLIT_MAX_TILES) * (H / 128) * SPLIT_RAW_FLOATS * 4);
     L.status = take(8);  // device status word, then the ticket counter of route_permute_kernel
     L.a1 = take(rc * H);
     L.a1_scale_t = take(rc * (H / 128) * 4);
@@ -549,11 +548,9 @@ int moe_fp8_forward(moe_fp8_handle_t h, int T, const void* hidden_fp8, const flo
         f.tok_nlocal = m.tok_nlocal;
         f.ready = counters;
         f.ticket = counters + (h->L.num_counters - 1);
-        f.part_done[0] = f.ticket - 2 * SPLIT_MAX_TILES;
-        f.tok_done = f.part_done[0] - static_cast<size_t>(F_MAX_TOKENS) * (H / G_TILE_N);
-        f.part_done[1] = f.part_done[0] + SPLIT_MAX_TILES;
-        f.raw[0] = at<float>(h, h->L.raw1);
-        f.raw[1] = at<float>(h, h->L.raw2);
+        f.part_done = f.ticket - SPLIT_MAX_TILES;
+        f.tok_done = f.part_done - static_cast<size_t>(F_MAX_TOKENS) * (H / G_TILE_N);
+        f.raw = at<float>(h, h->L.split_raw);
         f.split = h->k_split ? 1 : 0;
         // the fused kernel works on sub-tiles of at most 32 rows
         g1.num_m_tiles = g2.num_m_tiles = m.num_st;

@@ -574,9 +574,7 @@ __device__ __forceinline__ void route_permute_in_cta(int* scratch, CtaTiles& til
             m.st_rows[t0] = total;
         }
     }
-    if (tid == 0) {
-        m.mlp_claimed[m.mlp_grid] = 0;
-        // entries past E_loc count nothing, so entry E_loc already holds the totals
+    if (tid == 0) {  // entries past E_loc count nothing, so entry E_loc already holds the totals
         tiles.count = s_pad[E_loc] / TILE_M;
         *m.num_m_tiles = s_pad[E_loc] / TILE_M;
         *m.num_st = s_pad[E_loc] / TILE_M;
