@@ -376,7 +376,7 @@ def test_a_wait_that_runs_out_is_reported_and_the_handle_stays_usable(cuda_devic
 @pytest.mark.parametrize("tokens,eloc", [(9, 32), (48, 32), (200, 32), (300, 32), (2000, 256)])
 @pytest.mark.parametrize("clocks", [1 << 16, 1])  # 1: the roles give up before others have begun, copies still in flight
 def test_an_abort_leaves_nothing_under_way(cuda_device, tokens, eloc, clocks):
-    # one launch | fused behind the routing kernel | a launch per GEMM | both GEMMs in one, the last with lists of
+    # one launch | fused behind the routing kernel | a launch per GEMM, overlapping | both GEMMs in one, the last with lists of
     # several tiles per CTA.  The copy producer stops at its first few stages, before and behind a full ring and a tile's
     # end: what was claimed and issued by then has to be waited for (status 5 would say that it was not all there), and the
     # forward that follows at once, whose CTAs get the shared and tensor memory, must be right
@@ -635,10 +635,10 @@ def _route_round_robin(inp, tokens, active, away=0):
 
 
 @pytest.mark.parametrize("active", [4, 9, 10, 16, 19, 25, 28])  # one row tile each: 16 GEMM1 and 28 GEMM2 tiles
-def test_gemm2_rounds_in_front_of_the_joint_launch(cuda_device, active):
-    # fewer GEMM1 tiles than CTAs (4, 9: 64 and 144), fewer rounds in reach than wanted (10), as many as wanted and not
-    # one more (19), more (25, 28), all but a few CTAs without the last GEMM1 tile or with it; and the same again with
-    # lists that other CTAs take over
+def test_joint_launch_by_the_number_of_row_tiles(cuda_device, active):
+    # fewer GEMM1 tiles than 148 CTAs (4, 9: 64 and 144, the first GEMM2 tile of every CTA dealt), one, two and three rounds of
+    # them, all but a few CTAs without the last one (10: 160 tiles, 19: 304) or with it (16, 25, 28); and the same again with lists that
+    # other CTAs take over
     wl = _wl(257, syn.DSV3, seed=1200 + active)
     inp = syn.make_inputs(wl, cuda_device)
     _route_round_robin(inp, 257, active, away=40 - active)
@@ -698,10 +698,10 @@ def test_two_handles_on_two_streams_share_the_gpu(cuda_device):
         engs[k].close()
 
 
-@pytest.mark.parametrize("sizes", [(9, 14), (48, 70), (12, 60), (16, 700), (75, 1500)])
+@pytest.mark.parametrize("sizes", [(9, 14), (48, 70), (12, 60), (16, 700), (75, 1500), (100, 200), (12, 150), (200, 1500)])
 def test_fused_batches_on_two_streams(cuda_device, sizes):
-    # the fused kernel beside another fused one and beside the joint GEMM launch: its CTAs wait for one another, and its
-    # forwards follow each other closely (programmatic launches).  The waits give up early, so that a batch that only
+    # the fused kernel beside another fused one, beside two GEMM launches that overlap and beside the joint one, and the latter two
+    # beside each other: CTAs wait for one another, and the forwards follow each other closely (programmatic launches).  The waits give up early, so that a batch that only
     # got some of its CTAs would show as a time-out and not as a slow pass.
     wls = [_wl(t, syn.LayerDims(hidden=1024, intermediate=512, num_local_experts=32), seed=73 + t) for t in sizes]
     inps = [syn.make_inputs(w, cuda_device) for w in wls]
@@ -837,9 +837,13 @@ def test_fused_kernel_work_lists_around_full_rounds_of_ctas(cuda_device, active)
     eng.close()
 
 
-@pytest.mark.parametrize("hidden,inter", [(7168, 256), (4096, 256), (2048, 256)])  # three, one and no rounds in front
-@pytest.mark.parametrize("active", [75, 79, 94, 115, 148])  # two GEMM1 tiles each: 2, 10, 40, 82 and no spare ones
-def test_gemm2_rounds_in_front_of_the_fused_kernel(cuda_device, hidden, inter, active):
+@pytest.mark.parametrize("hidden,inter,active",
+                         # two GEMM1 tiles each (2, 10, 40, 82 CTAs and none with one more), 28, 16 and 8 short GEMM2 tiles
+                         [(h, 256, a) for h in (7168, 4096, 2048) for a in (75, 79, 94, 115, 148)]
+                         # two GEMM2 tiles each: fewer than 148 CTAs, one, just at and above two for every CTA, of six K-blocks (all
+                         # stages go out at once) and of seven
+                         + [(512, i, a) for i in (768, 896) for a in (20, 74, 75, 147, 148, 149)])
+def test_gemm2_tiles_of_the_fused_kernel_come_from_a_counter(cuda_device, hidden, inter, active):
     dims = syn.LayerDims(hidden=hidden, intermediate=inter, num_local_experts=160)
     wl = _wl(30, dims, seed=1300 + active)
     inp = syn.make_inputs(wl, cuda_device)
@@ -857,14 +861,17 @@ def test_gemm2_rounds_in_front_of_the_fused_kernel(cuda_device, hidden, inter, a
     eng.close()
 
 
-@pytest.mark.parametrize("tokens,skew", [(81, False), (81, True), (200, True), (256, False)])
-def test_two_gemm_launches_that_overlap(cuda_device, tokens, skew):
+@pytest.mark.parametrize("tokens,skew,dims", [(81, False, SMALL), (81, True, SMALL), (200, True, SMALL), (256, False, SMALL),
+                                              (150, False, syn.LayerDims(512, 512, num_local_experts=256)),
+                                              (200, True, syn.LayerDims(512, 1024, num_local_experts=100))])
+def test_two_gemm_launches_that_overlap(cuda_device, tokens, skew, dims):
     # GEMM2's launch starts while GEMM1's still runs and waits row tile by row tile; batches in a row on one handle, with
-    # and without stage timing (which keeps the launches apart)
-    eng = make_engine(_wl(tokens), cuda_device)
-    ref = make_engine(_wl(tokens), cuda_device)
+    # and without stage timing (which keeps the launches apart).  The two larger layers have lists of three and more GEMM1 tiles,
+    # whose rows are announced together, and the skewed one short and full row tiles in them.
+    eng = make_engine(_wl(tokens, dims), cuda_device)
+    ref = make_engine(_wl(tokens, dims), cuda_device)
     ref.set_small_batch_fusion(256)
-    inps = [syn.make_inputs(_wl(tokens, seed=1700 + tokens + k, skew=skew), cuda_device) for k in range(3)]
+    inps = [syn.make_inputs(_wl(tokens, dims, seed=1700 + tokens + k, skew=skew), cuda_device) for k in range(3)]
     want = [ref.forward(i).clone() for i in inps]
     got = [eng.forward(inps[k % 3]).clone() for k in range(9)]
     eng.set_stage_timing(True)
