@@ -187,7 +187,6 @@ template <class GEO>
 __device__ __forceinline__ void mlp_issuer(const Cta& c, const MlpArgs& a, uint32_t mine) {
     GemmCtrl* ctrl = c.ctrl;
     const uint32_t idesc = umma_idesc_f8(TILE_M, G_TILE_N), idesc_wm = umma_idesc_f8(TILE_M, WM_TOKENS);
-    const int leader = elected_lane();
     uint32_t it = 0;
     bool ok = true;
     for (uint32_t i = 0;; ++i) {
@@ -207,12 +206,15 @@ __device__ __forceinline__ void mlp_issuer(const Cta& c, const MlpArgs& a, uint3
             const uint64_t b_desc = umma_desc_sw128(a_addr + GEO::A_BYTES);
             const uint32_t d_tmem = c.tmem_base + mine * G_TILE_N;
             if (ok) {
-                // (by the lane that issues the MMAs: a shuffle orders no memory)
-                if (elect_one()) ok = mbar_wait(smem_u32(&ctrl->full[s]), ph, c.abort_flag, c.limit);
-                ok = __shfl_sync(0xffffffffu, ok, leader);
+                if (c.lane == 0) ok = mbar_wait(smem_u32(&ctrl->full[s]), ph, c.abort_flag, c.limit);
+                ok = __shfl_sync(0xffffffffu, ok, 0);
                 if (!ok && c.lane == 0) raise(ctrl, a.g1.status, DEV_TIMEOUT_MMA_SMEM);
             }
-            if (it >= G_ACC_BUFS) bar_sync(ACC_BARRIER + mine, ACC_BARRIER_THREADS);
+            // (orders the issuing lane behind lane 0, which has seen the stage land; a shuffle orders no memory)
+            if (it >= G_ACC_BUFS)
+                bar_sync(ACC_BARRIER + mine, ACC_BARRIER_THREADS);
+            else
+                __syncwarp();
             if (!ok) continue;
             tc_fence_after();
             // (by a lane chosen by its number, eight MMAs of a short tile took 850 clocks to issue, now 690)

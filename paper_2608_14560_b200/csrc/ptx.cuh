@@ -374,12 +374,6 @@ __device__ __forceinline__ bool elect_one() {
     asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
     return p != 0;
 }
-// Which lane that is.
-__device__ __forceinline__ int elected_lane() {
-    uint32_t l;
-    asm volatile("{\n\t.reg .pred P;\n\telect.sync %0|P, 0xffffffff;\n\t}" : "=r"(l));
-    return static_cast<int>(l);
-}
 
 // ---- registers --------------------------------------------------------------
 template <int N>
