@@ -206,15 +206,11 @@ __device__ __forceinline__ void mlp_issuer(const Cta& c, const MlpArgs& a, uint3
             const uint64_t b_desc = umma_desc_sw128(a_addr + GEO::A_BYTES);
             const uint32_t d_tmem = c.tmem_base + mine * G_TILE_N;
             if (ok) {
-                if (c.lane == 0) ok = mbar_wait(smem_u32(&ctrl->full[s]), ph, c.abort_flag, c.limit);
-                ok = __shfl_sync(0xffffffffu, ok, 0);
+                // (by all lanes, the one that issues the MMAs among them)
+                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&ctrl->full[s]), ph, c.abort_flag, c.limit));
                 if (!ok && c.lane == 0) raise(ctrl, a.g1.status, DEV_TIMEOUT_MMA_SMEM);
             }
-            // (orders the issuing lane behind lane 0, which has seen the stage land; a shuffle orders no memory)
-            if (it >= G_ACC_BUFS)
-                bar_sync(ACC_BARRIER + mine, ACC_BARRIER_THREADS);
-            else
-                __syncwarp();
+            if (it >= G_ACC_BUFS) bar_sync(ACC_BARRIER + mine, ACC_BARRIER_THREADS);
             if (!ok) continue;
             tc_fence_after();
             // (by a lane chosen by its number, eight MMAs of a short tile took 850 clocks to issue, now 690)
