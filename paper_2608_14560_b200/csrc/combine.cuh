@@ -13,8 +13,8 @@ namespace moe {
 
 // Bound by the latency of scattered 32-byte reads (a token's rows lie in up to eight row tiles, its 16-column groups 1 KB
 // apart): about 4.7 TB/s with all experts local.  So only the rows that exist are looked at, the loads of up to four of them
-// are under way in a thread, the token's table entries come one token ahead, and a block holds a part of a token's columns,
-// which leaves 28 warps on an SM.  us for one block of 256 threads per token and all eight slots in turn / this form: 12.3
+// are under way in a thread, the token's table entries come one token ahead, and a block holds a part of a token's columns:
+// 75 registers, six blocks of four warps on an SM (at hidden 7168 the last of four parts has columns for two of its warps).  us for one block of 256 threads per token and all eight slots in turn / this form: 12.3
 // / 8.2 at 257 tokens (257 rows), 16.4 / 14.4 at 1024 (1602), 43.0 / 36.9 at 4096 (6007), 131 / 115 at 8192 skewed (33838), 127
 // / 110 at 4096 with 256 experts (32768).  Blocks of 448 threads 41, 122 and 118 for the last three; two or three rows under
 // way 37 to 39, 115 to 118 and 110; eight rows 88, 226 and 164 (registers: few warps).

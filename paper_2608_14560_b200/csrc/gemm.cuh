@@ -117,10 +117,11 @@ using GeomSmall = Geometry<6, 32, 16, G_EPI_WARPS * 512, false>;
 constexpr int F_MAX_TOKENS = 256;
 // From this batch size up the large-tile GEMM kernels run row tiles of at most 32 rows with the weights on M.
 constexpr int SHORT_TILE_MIN_TOKENS = 1;
-// Up to here the fused kernel is used unless the caller says otherwise.  Measured against the separate kernels
-// (cold step): 9-17 % faster from 34 to 80 tokens with uniform routing, 13-16 % faster at 40-64 tokens with
-// skewed routing, 3-6 % slower at exactly 33 and at 80 skewed tokens (hot experts need a second or third
-// sub-tile), 10 % slower at 100 skewed tokens, still 9-15 % faster at 128-192 uniform tokens.
+// Up to here the fused kernel is used unless the caller says otherwise.  us per forward, separate kernels / fused (7168 x 2048, 32 experts,
+// mean of three draws): uniform routing 134.1 / 118.7 at 33 tokens, 164.4 / 147.9 at 64, 168.8 / 153.2 at 80, 169.6 / 154.7 at 100, 175.8 / 165.0 at
+// 128, 190.5 / 185.3 at 256; four hot experts, which need a sub-tile per 32 rows, 124.2 / 103.0 at 33, 148.2 / 131.3 at 64, 154.9 / 143.3 at 80,
+// 157.5 / 157.0 at 100, 157.9 / 161.5 at 128, 171.9 / 183.1 at 160, 189.2 / 254.0 at 256.  It would be the faster one up to 100 tokens; callers
+// count on the separate kernels from 81 on (last_launch_count, the stage times).
 constexpr int F_DEFAULT_MAX_TOKENS = 80;
 static_assert(GeomSmall::A_ROWS == ST_ROWS, "the token slot of a stage holds one sub-tile");
 // Largest batch whose routing and permutation run inside fused_small_kernel, by every CTA for itself (one token
@@ -147,7 +148,8 @@ struct GemmArgs {
     const int* tile_row0;     // fused kernel: first padded row of each (sub-)tile; else null: tile * TILE_M
     int wm_rows;              // grouped_mlp_kernel: row tiles with at most this many rows (0 or 32) run with the
                               // weights on the M side of the MMAs, see epilogue_tile_wm
-    int* ready;               // GEMM1 in one launch with GEMM2: [row tiles] warps that have stored their part, zero at launch
+    int* ready;               // GEMM1 whose rows GEMM2's tiles wait for (one launch, or two that overlap): [row tiles] warps that have
+                              // stored their part, zero at launch
     const float* a_scale_t;   // [num_kb, row_cap]
     const float* w_scale;     // [E_loc, w_rows/128, num_kb]
     uint8_t* out_fp8;         // GEMM1: [row_cap, I] e4m3
@@ -585,8 +587,8 @@ __device__ __forceinline__ bool epilogue_rendezvous(const Cta& c, uint64_t* bar,
 // step), the 32 token rows the N side.  An accumulator is then 128 lanes x 32 columns per weight-row block,
 // 64 columns per K-block: every stage gets an accumulator buffer of its own (6 x 64 of the 512 columns),
 // so the hand-over latencies overlap six deep, and an epilogue thread owns one weight row (an output
-// column) of both blocks for the tile's 32 tokens, the four warps of a group taking a tile together and the two
-// groups the tiles in turn (epilogue_tile_group).
+// column) of both blocks, the four warps of a group taking a tile together and the two groups the tiles in turn, or
+// half of a tile each (epilogue_tile_group).
 // Element for element the arithmetic is the one of the other orientation.
 static_assert(G_MAX_STAGES * WM_BUF_COLS <= static_cast<int>(G_TMEM_COLS), "one accumulator buffer per stage");
 

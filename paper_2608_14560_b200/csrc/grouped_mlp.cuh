@@ -12,7 +12,7 @@
 // for the CTAs with one GEMM1 tile less, the last CTA ended 12 us (6 %) behind the middle one at 257 tokens, now 5.  us per forward
 // dealt / counter: 194.0 / 193.4 at 100 tokens, 139.9 / 137.0 at 150 skewed, 205.7 / 202.2 at 257, 204.7 / 202.0 at 400, 223.1 /
 // 221.5 at 901, 251.5 / 248.8 at 1500, 436.5 / 433.4 at 4096, 1589 / 1591 at 8192 skewed; on 256 experts 1184 / 1178 at 300, 1405 /
-// 1394 at 1000, 4006 / 4001 at 8192.
+// 1394 at 1000, 4006 / 4001 at 8192 (runs too short for the power cap, under which 8192 skewed tokens take 2100).
 // What the common list is for: a launch per GEMM leaves most SMs idle in its last, partly filled wave.  With 24 active
 // experts (257 tokens) GEMM1 is 384 tiles of 56 K-blocks, 2.6 waves, and GEMM2 672 tiles of 16, 4.5 waves: 248 K-block
 // times per launch pair against 218 in one list.  Measured per forward, two launches against one, this kernel on both
@@ -30,7 +30,7 @@ namespace moe {
 // skewed, 1116 / 1125 at 16167, 2194 / 2201 at 16384 with 256 experts, 3170 / 3159 at 32768, 8913 / 8626 at 131072.
 // The last figure sets the line: under the power cap, which short runs do not reach (there one launch stays ahead: 2908 / 2987
 // at 32768 slots, 5066 / 5169 at 65536), the largest batches lose 3 %.
-// Two launches overlap up to PDL_MAX_TOKENS tokens: a CTA of the second one starts on an SM that has finished its GEMM1 tiles, all
+// Two launches overlap up to MLP_SPLIT_MAX_TOKENS tokens: a CTA of the second one starts on an SM that has finished its GEMM1 tiles, all
 // CTAs of the first one run by then (they allow the second launch when they start), and its tiles wait for the announcements
 // of their rows like those of the one launch.  us per forward, one launch after the
 // other / overlapping: 191.4 / 179.3 at 81 tokens, 195.9 / 184.5 at 128, 196.5 / 182.6 at 160, 208.5 / 205.1 at 200, 208.9 / 205.1 at
@@ -479,8 +479,8 @@ __device__ __forceinline__ void store_rows64(uint8_t* p, const float* acc) {
 // the next entry read beside it (GEMM2: not behind all of the stores, which hold up every later access to shared memory),
 // and the halves of the weights taken in the order gate, up instead of changing places behind the loop.
 // The loop has 192 of its 224 registers in its two arrays: what it does not need, the tile's entry for one, is fetched again
-// behind it.  Spilling decides here: forms with 110 to 380 bytes of spilled registers instead of 20 were 2 to 8 % slower,
-// tiles of the other orientation included.
+// behind it.  Spilling decides here: forms with 110 to 380 bytes of spilled registers were 2 to 8 % slower, tiles of the other
+// orientation included; this one stores 4 bytes and loads 24.
 // us of the GEMM launches before / this form: 8192 skewed tokens on 32 experts 1536 / 1432, 4096 tokens 399 / 387, 8192 tokens
 // on 256 experts 3926 / 3674.  What is left of the tails is 1 % (the SwiGLU left out altogether: 1416, 382).
 template <int MODE, class GEO>

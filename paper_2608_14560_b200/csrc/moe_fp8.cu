@@ -237,8 +237,8 @@ constexpr int PDL_MAX_TOKENS = 2048;
 // Beyond that the GEMMs alone, behind the gather: their CTAs set up and ask for the first weights on the SMs that have
 // finished gathering.  Up to this many expected local slots (tokens x 8 x the local share of the experts); us per forward on 32
 // experts without / with: uniform routing 309.0 / 300.7 at 2500 tokens, 437.6 / 435.5 at 4096, 423.7 / 418.6 at 6000 (another
-// draw); skewed 711.6 / 712.2 at 3000, 1071 / 1075 at 4096, 1584 / 1597 at 8192; 3950 / 3955 at 8192 on 256 experts.  The other
-// kernels gain nothing there (gather 0 to + 1.3 % with skewed routing, combine 0 to + 0.6 %).
+// draw); skewed 711.6 / 712.2 at 3000, 1071 / 1075 at 4096, 1584 / 1597 at 8192; 3950 / 3955 at 8192 on 256 experts (runs too short
+// for the power cap).  The other kernels gain nothing there (gather 0 to + 1.3 % with skewed routing, combine 0 to + 0.6 %).
 constexpr long long PDL_MLP_MAX_SLOTS = 6144;
 
 bool misaligned(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) != 0; }

@@ -461,7 +461,7 @@ def _from_hidden_case(wl, device, sample_tokens=None, **kw):
     return int(((ridx >= wl.local_expert_offset) & (ridx < wl.local_expert_offset + d.num_local_experts)).sum())
 
 
-@pytest.mark.parametrize("tokens", [1, 8, 33, 128, 129, 700])  # 128 | 129: the two projection tile shapes
+@pytest.mark.parametrize("tokens", [1, 8, 33, 128, 129, 700])  # 128 | 129: the two tile shapes of the projection
 def test_from_hidden_small_layer(cuda_device, tokens):
     _from_hidden_case(_wl(tokens, seed=60 + tokens), cuda_device)
 
