@@ -187,6 +187,11 @@ template <class GEO>
 __device__ __forceinline__ void mlp_issuer(const Cta& c, const MlpArgs& a, uint32_t mine) {
     GemmCtrl* ctrl = c.ctrl;
     const uint32_t idesc = umma_idesc_f8(TILE_M, G_TILE_N), idesc_wm = umma_idesc_f8(TILE_M, WM_TOKENS);
+    // Lanes that wait for the stages: the one that issues the MMAs in any case (a shuffle from another one orders no memory).  All of
+    // them, without a branch around the wait, are 1 to 1.5 % faster up to MLP_JOINT_MAX_SLOTS (us per forward one lane / all: 185.0 / 182.2
+    // at 257 tokens, 223.8 / 221.5 at 901, 415.9 / 411.6 at 4096, equal at 8192 skewed); beyond, at the power cap, 32 polling lanes cost
+    // more than they save (7440 / 7545 at 16384 tokens on 256 experts).
+    const bool waits = a.by_row || elect_one();
     uint32_t it = 0;
     bool ok = true;
     for (uint32_t i = 0;; ++i) {
@@ -206,8 +211,8 @@ __device__ __forceinline__ void mlp_issuer(const Cta& c, const MlpArgs& a, uint3
             const uint64_t b_desc = umma_desc_sw128(a_addr + GEO::A_BYTES);
             const uint32_t d_tmem = c.tmem_base + mine * G_TILE_N;
             if (ok) {
-                // (by all lanes, the one that issues the MMAs among them)
-                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&ctrl->full[s]), ph, c.abort_flag, c.limit));
+                if (waits) ok = mbar_wait(smem_u32(&ctrl->full[s]), ph, c.abort_flag, c.limit);
+                ok = __all_sync(0xffffffffu, ok);
                 if (!ok && c.lane == 0) raise(ctrl, a.g1.status, DEV_TIMEOUT_MMA_SMEM);
             }
             if (it >= G_ACC_BUFS) bar_sync(ACC_BARRIER + mine, ACC_BARRIER_THREADS);
