@@ -270,10 +270,11 @@ __device__ __forceinline__ void mlp_factors(const Cta& c, const MlpArgs& a) {
     // GEMM1: tiles id1, id1 + grid, ... ; GEMM2: the dealt one, if any, then whichever is next when this CTA needs one (a ticket,
     // drawn when it enters the tile before).
     int id1 = static_cast<int>(blockIdx.x);
-    int id2 = ~0;  // GEMM2: the dealt tile, or ~(number of dealt tiles)
+    int drawn = -1, dealt = 0;  // GEMM2: the dealt tile (a ticket that has been drawn already); the number of dealt tiles
     if (mlp_first_tile_dealt(a.phases == 3, m_tiles, a.g1, a.g2, grid)) {
         const int late = n1 % grid;  // CTAs with one GEMM1 tile more: they come last
-        id2 = id1 < late ? id1 + grid - late : id1 - late;
+        drawn = id1 < late ? id1 + grid - late : id1 - late;
+        dealt = grid;
     }
     if (a.phases == 3) {
         int was = LIST_OPEN;
@@ -303,14 +304,10 @@ __device__ __forceinline__ void mlp_factors(const Cta& c, const MlpArgs& a) {
             id = id1;
             id1 += grid;
         } else if ((a.phases & 2) && !end) {
-            int ticket = 0;
-            if (id2 >= 0) {
-                id = n1 + id2;
-                id2 = ~grid;
-            } else {
-                if (lane == 0) ticket = atomicAdd(a.claimed + grid, 1);
-                id = n1 + ~id2 + __shfl_sync(0xffffffffu, ticket, 0);
-            }
+            int ticket = drawn;
+            if (lane == 0 && drawn < 0) ticket = dealt + atomicAdd(a.claimed + grid, 1);
+            drawn = -1;
+            id = n1 + __shfl_sync(0xffffffffu, ticket, 0);
         }
         const bool live = !end && id < n12;
         const bool first = id < n1;
