@@ -482,7 +482,7 @@ __device__ __forceinline__ void store_rows64(uint8_t* p, const float* acc) {
 // and the halves of the weights taken in the order gate, up instead of changing places behind the loop.
 // The loop has 192 of its 224 registers in its two arrays: what it does not need, the tile's entry for one, is fetched again
 // behind it.  Spilling decides here: forms with 110 to 380 bytes of spilled registers were 2 to 8 % slower, tiles of the other
-// orientation included; this one stores 4 bytes and loads 24.
+// orientation included; this one stores 12 bytes and loads 28.
 // us of the GEMM launches before / this form: 8192 skewed tokens on 32 experts 1536 / 1432, 4096 tokens 399 / 387, 8192 tokens
 // on 256 experts 3926 / 3674.  What is left of the tails is 1 % (the SwiGLU left out altogether: 1416, 382).
 template <int MODE, class GEO>
